@@ -219,6 +219,11 @@ struct tree_ot_handle {
   Task* d_btasks[2] = {nullptr, nullptr};
   int32_t* d_queue = nullptr;              // [colour][slot][2] work-queue counters
   int32_t rec_ob = kRecOut;                // recomputed-cost output block (autotuned)
+  int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
+  bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
+  std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
+  int32_t item_begin[2][4] = {}, item_count[2][4] = {};  // per dimension
+  FactItem* d_items[2] = {nullptr, nullptr};
   int32_t grid_mult = 0;                   // 0: occupancy-derived grid; else CTAs per SM (autotuned)
   int32_t rec_variant = 0;                 // recomputed-cost kernel register budget (autotuned)
   int32_t dense_tma = 0;                   // stored-cost tasks on the bulk-copy staged kernel
@@ -244,6 +249,8 @@ struct tree_ot_handle {
   double *d_resid_acc = nullptr, *d_resid_dedge = nullptr, *d_res_sum = nullptr, *d_marg = nullptr;
   double *d_edge_tc = nullptr, *d_edge_mass = nullptr;
   float *d_hh = nullptr, *d_hl = nullptr, *d_ah = nullptr, *d_al = nullptr, *d_coords = nullptr;
+  float4 *d_slot_x = nullptr, *d_grp = nullptr;  // compact groups of the support points (group.cu)
+  float2* d_slot_q = nullptr;
   float *d_coords_hi = nullptr, *d_coords_lo = nullptr;  // coordinates split hi + lo (exact distances)
   uint32_t* d_cmax = nullptr;              // per problem max |coordinate| (split scratch)
   int32_t* d_exact = nullptr;              // per problem: exact squared distances (recomputed costs)
@@ -300,7 +307,7 @@ struct tree_ot_handle {
   cudaStream_t hstream = nullptr;
   cudaGraphExec_t graph = nullptr;
   int graph_len = 0;
-  int apply_grid[kApplySlots] = {1, 1, 1, 1};
+  int apply_grid[kApplySlots] = {1, 1, 1, 1, 1, 1, 1};
   int sms = 1;
 
   bool have_check = false;
@@ -353,6 +360,11 @@ void prof_span(tree_ot_handle* h, int cat, int i0, int i1) {
 }
 cudaEvent_t prof_event(tree_ot_handle* h, int i) { return i >= 0 ? h->prof_ev[i] : nullptr; }
 
+// directed edges whose recomputed-cost apply runs in factored form
+bool fact_edge(const tree_ot_handle* h, const DEdgeD& d) {
+  return h->nodes[d.owner].gs > 0 && h->nodes[d.nbr].n >= kGroupMin;
+}
+
 // Apply tasks of both colours, grouped by kernel slot.  rec_ob: largest output
 // block of a recomputed-cost task (256, 512 or 1024 outputs); a task with fewer
 // outputs runs its CTA as G warp groups splitting the reduction points.
@@ -383,6 +395,17 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
         for (int32_t o0 = 0; o0 < own.n; o0 += kColCols)
           tl.push_back(Task{(int32_t)di, TASK_COL, o0, std::min(kColCols, own.n - o0), s * kColRows,
                             std::min(kColRows, nbn.n - s * kColRows), s, 0});
+    } else if (fact_edge(h, d)) {
+      // slots of the owner's groups against all of the neighbour's points, 2^split warps of a CTA per block of 64;
+      // the exact-distance kernel reads the same range as plain outputs, with G warp groups of at most
+      // 1024 / G outputs
+      const int32_t ob = (8 >> h->fact_split) * 64;
+      for (int32_t o0 = 0; o0 < own.n; o0 += ob) {
+        const int32_t oc = std::min(ob, own.n - o0);
+        int32_t G = 1;
+        while (G < 8 && kRecOut / (2 * G) >= oc) G *= 2;
+        tl.push_back(Task{(int32_t)di, TASK_FACT + h->fact_split, o0, oc, 0, nbn.n, 0, G});
+      }
     } else {
       for (int32_t o0 = 0; o0 < own.n; o0 += rec_ob) {
         const int32_t oc = std::min(rec_ob, own.n - o0);
@@ -398,8 +421,8 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
   // dimension); recomputed tasks go largest first for the work queue
   for (int c = 0; c < 2; ++c) {
     auto slot_of = [&](const Task& t) {
-      if (h->fp64 || t.kind != TASK_RECOMP) return 0;
-      return (int)h->probs[h->dedges[t.dedge].prob].dim;
+      if (h->fp64 || t.kind < TASK_RECOMP) return 0;
+      return (int)h->probs[h->dedges[t.dedge].prob].dim + (t.kind >= TASK_FACT ? 3 : 0);
     };
     auto cost_of = [&](const Task& t) { return (int64_t)t.ocount * t.rcount; };
     std::stable_sort(h->tasks[c].begin(), h->tasks[c].end(), [&](const Task& x, const Task& y) {
@@ -434,6 +457,9 @@ ApplyArgs apply_args(tree_ot_handle* h, int colour) {
   a.coords = h->d_coords;
   a.coords_hi = h->d_coords_hi;
   a.coords_lo = h->d_coords_lo;
+  a.slot_x = h->d_slot_x;
+  a.slot_q = h->d_slot_q;
+  a.grp = h->d_grp;
   a.exact = h->d_exact;
   a.any_exact = h->any_exact;
   a.part32 = h->d_part32;
@@ -534,8 +560,9 @@ int launch_absorb_step(tree_ot_handle* h, cudaStream_t s) {
   return TREE_OT_OK;
 }
 
-// only_stored: just the stored-cost (slot 0) kernel, for timing it
-int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, bool only_stored = false) {
+// which kernels an apply launches: all, or one family of them (for timing it)
+enum ApplySet { APPLY_ALL, APPLY_STORED, APPLY_DIFF, APPLY_FACT };
+int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, ApplySet set = APPLY_ALL) {
   ApplyArgs a = apply_args(h, colour);
   if (h->fp64) {
     const int grid = std::max(1, std::min<int>(a.ntasks, h->apply_grid[0]));
@@ -545,9 +572,10 @@ int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, bool only_stored
     prof_span(h, TREE_OT_PROF_APPLY_FP64, p0, prof_mark(h, s));
     return TREE_OT_OK;
   }
-  for (int slot = 0; slot < (only_stored ? 1 : kApplySlots); ++slot) {
+  for (int slot = 0; slot < kApplySlots; ++slot) {
     const int32_t cnt = h->slot_count[colour][slot];
     if (cnt == 0) continue;
+    if (set != APPLY_ALL && set != (slot == 0 ? APPLY_STORED : slot <= 3 ? APPLY_DIFF : APPLY_FACT)) continue;
     a.tasks = h->d_tasks[colour] + h->slot_begin[colour][slot];
     a.ntasks = cnt;
     a.queue = h->d_queue + 2 * (colour * kApplySlots + slot);
@@ -560,13 +588,29 @@ int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, bool only_stored
       continue;
     }
     int cap = slot == 0 ? h->apply_grid[0] : h->rec_grid[h->rec_variant][slot];
-    if (slot > 0 && h->grid_mult > 0) cap = h->sms * h->grid_mult;
-    const int grid = std::max(1, std::min<int>(cnt, cap));
-    cudaError_t e = launch_apply_f32(a, slot, slot == 0 ? 0 : h->rec_variant, grid, s);
+    if (slot > 0 && slot <= 3 && h->grid_mult > 0) cap = h->sms * h->grid_mult;
+    int work = cnt, variant = slot == 0 ? 0 : h->rec_variant;
+    // both forms in one launch: slot 3 + D's tasks follow slot D's (no other dimension in the handle)
+    const bool both = h->both_forms && set == APPLY_ALL && !a.any_exact && slot > 0;
+    if (both && slot > 3 && h->slot_count[colour][slot - 3] > 0) continue;  // taken by that launch
+    if (both && slot <= 3 && h->slot_count[colour][slot + 3] > 0) {
+      a.ntasks += h->slot_count[colour][slot + 3];
+      work = a.ntasks;
+      variant = kBothForms;
+      cap = h->rec_grid[0][slot];
+    } else if (slot > 3) {
+      variant = h->fact_split > 0 ? 1 : 0;
+      cap = a.any_exact ? h->rec_grid[0][slot - 3] : h->rec_grid[variant][slot];
+      a.items = h->d_items[colour] + h->item_begin[colour][slot - 3];
+      a.nitems = h->item_count[colour][slot - 3];
+      if (!a.any_exact && variant == 0) work = (a.nitems + 3) / 4;  // four warps per CTA
+    }
+    const int grid = std::max(1, std::min<int>(work, cap));
+    cudaError_t e = launch_apply_f32(a, slot, variant, grid, s);
     if (e != cudaSuccess) return cuda_fail(e, "edge apply launch");
     prof_span(h, slot == 0 ? TREE_OT_PROF_APPLY_STORED : TREE_OT_PROF_APPLY_RECOMPUTE, p0, prof_mark(h, s));
   }
-  if (h->lowp && !only_stored && !h->btasks[colour].empty()) {
+  if (h->lowp && set == APPLY_ALL && !h->btasks[colour].empty()) {
     a.tasks = h->d_btasks[colour];
     a.ntasks = (int32_t)h->btasks[colour].size();
     const int grid = std::max(1, std::min<int>(a.ntasks, h->bf16_grid));
@@ -575,7 +619,7 @@ int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, bool only_stored
     if (e != cudaSuccess) return cuda_fail(e, "absorbed apply launch");
     prof_span(h, TREE_OT_PROF_APPLY_BF16, p0, prof_mark(h, s));
   }
-  if (!only_stored)
+  if (set == APPLY_ALL)
     for (const auto& g : h->sk) {
       const int p0 = prof_mark(h, s), m0 = prof_take(h), m1 = prof_take(h);
       cudaError_t e = launch_sk(g.args[colour], g.args[colour].use_tc ? &g.maps[colour] : nullptr, s,
@@ -644,7 +688,8 @@ int launch_forest_chunk(tree_ot_handle* h, int G, bool retire, cudaStream_t s) {
   for (int c = 0; c < 2; ++c) {
     f.ap[c] = apply_args(h, c);
     f.ap[c].tasks = h->d_tasks[c] + h->slot_begin[c][h->forest_D];
-    f.ap[c].ntasks = h->slot_count[c][h->forest_D];
+    // the factored tasks follow the others: no other dimension's lie between
+    f.ap[c].ntasks = h->slot_count[c][h->forest_D] + h->slot_count[c][h->forest_D + 3];
     f.nd[c] = node_args(h, c, retire);
   }
   f.cnt = h->d_fcnt;
@@ -975,7 +1020,7 @@ void fill_result(tree_ot_handle* h, tree_ot_result* res, int p) {
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mu;
 struct TuneCfg {
-  int32_t ob, gm, variant;
+  int32_t ob, gm, variant, split, both;
 };
 std::map<uint64_t, TuneCfg> g_tune_cache;
 
@@ -991,6 +1036,7 @@ uint64_t shape_signature(const tree_ot_handle* h) {
     mix((uint64_t)h->nodes[d.nbr].n);
     mix((uint64_t)h->probs[d.prob].dim);
     mix((uint64_t)h->nodes[d.owner].colour);
+    mix((uint64_t)h->nodes[d.owner].gs);
   }
   return sig;
 }
@@ -1005,60 +1051,123 @@ int upload_tasks(tree_ot_handle* h, cudaStream_t s) {
   return TREE_OT_OK;
 }
 
-int autotune_recompute(tree_ot_handle* h, cudaStream_t s) {
-  bool any = false;
+// one timing of both colours' applies with the current configuration (warm-up, then two of each)
+int time_applies(tree_ot_handle* h, cudaStream_t s, ApplySet set, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
+  for (int rep = 0; rep < 3; ++rep) {
+    if (rep == 1) CUDA_TRY(cudaEventRecord(e0, s));
+    RC_TRY(launch_apply(h, 0, s, set));
+    RC_TRY(launch_apply(h, 1, s, set));
+  }
+  CUDA_TRY(cudaEventRecord(e1, s));
+  CUDA_TRY(cudaEventSynchronize(e1));
+  CUDA_TRY(cudaEventElapsedTime(ms, e0, e1));
+  return TREE_OT_OK;
+}
+
+int apply_tune(tree_ot_handle* h, const TuneCfg& cfg, cudaStream_t s) {
+  h->both_forms = cfg.both != 0;
+  h->fact_split = cfg.split;
+  h->grid_mult = cfg.gm;
+  h->rec_variant = cfg.variant;
+  build_apply_tasks(h, cfg.ob);
+  return upload_tasks(h, s);
+}
+
+// every recomputed-cost task of one dimension (its two slots are then adjacent in the task lists)
+bool one_dimension(const tree_ot_handle* h) {
+  int D = 0;
   for (int c = 0; c < 2; ++c)
-    for (int slot = 1; slot < kApplySlots; ++slot) any = any || h->slot_count[c][slot] > 0;
-  if (!any) return TREE_OT_OK;
+    for (int slot = 1; slot < kApplySlots; ++slot) {
+      if (h->slot_count[c][slot] == 0) continue;
+      const int dim = slot > 3 ? slot - 3 : slot;
+      if (D && D != dim) return false;
+      D = dim;
+    }
+  return D > 0;
+}
+
+int tune_applies(tree_ot_handle* h, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1, bool diff, bool fact,
+                 TuneCfg* cfg) {
+  // factored form: warps per group (1: the per-warp queue)
+  float best = 1e30f, ms = 0.f;
+  for (int32_t lw = 0; fact && lw < 4; ++lw) {
+    h->fact_split = lw;
+    build_apply_tasks(h, cfg->ob);
+    RC_TRY(upload_tasks(h, s));
+    RC_TRY(time_applies(h, s, APPLY_FACT, e0, e1, &ms));
+    if (ms > 1.3f * best) break;  // more warps per group only get slower from here
+    if (ms < best) {
+      best = ms;
+      cfg->split = lw;
+    }
+  }
+  h->fact_split = cfg->split;
+  // difference form: output block, register budget and grid
+  best = 1e30f;
+  for (int32_t ob : {1024, 512, 256}) {
+    if (!diff) break;
+    build_apply_tasks(h, ob);
+    RC_TRY(upload_tasks(h, s));
+    for (int32_t v = 0; v < 3; ++v) {
+      h->grid_mult = v == 2 ? 1 : 0;
+      h->rec_variant = v == 1 ? 1 : 0;
+      RC_TRY(time_applies(h, s, APPLY_DIFF, e0, e1, &ms));
+      if (ms < best) {
+        best = ms;
+        cfg->ob = ob;
+        cfg->gm = h->grid_mult;
+        cfg->variant = h->rec_variant;
+      }
+    }
+  }
+  if (!diff || !fact || !one_dimension(h)) return TREE_OT_OK;
+  // both forms in one launch against one launch each: pays where each alone leaves the GPU half empty
+  RC_TRY(apply_tune(h, *cfg, s));
+  float two = 0.f;
+  RC_TRY(time_applies(h, s, APPLY_ALL, e0, e1, &two));
+  if (two > 0.4f) return TREE_OT_OK;  // 0.1 ms per apply: both launches fill the GPU
+  const TuneCfg sep = *cfg;
+  h->both_forms = true;
+  for (int32_t ob : {1024, 512, 256})
+    for (int32_t lw = 0; lw < 4; ++lw) {
+      h->fact_split = lw;
+      build_apply_tasks(h, ob);
+      RC_TRY(upload_tasks(h, s));
+      RC_TRY(time_applies(h, s, APPLY_ALL, e0, e1, &ms));
+      if (ms > 1.5f * two) break;
+      if (ms < (cfg->both ? best : two)) {
+        best = ms;
+        cfg->ob = ob;
+        cfg->split = lw;
+        cfg->both = 1;
+      }
+    }
+  if (!cfg->both) *cfg = sep;
+  return TREE_OT_OK;
+}
+
+int autotune_recompute(tree_ot_handle* h, cudaStream_t s) {
+  bool diff = false, fact = false;
+  for (int c = 0; c < 2; ++c)
+    for (int slot = 1; slot < kApplySlots; ++slot) (slot > 3 ? fact : diff) |= h->slot_count[c][slot] > 0;
+  if (!diff && !fact) return TREE_OT_OK;
   const uint64_t sig = shape_signature(h);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_cache.find(sig);
-    if (it != g_tune_cache.end()) {
-      build_apply_tasks(h, it->second.ob);
-      h->grid_mult = it->second.gm;
-      h->rec_variant = it->second.variant;
-      return upload_tasks(h, s);
-    }
+    if (it != g_tune_cache.end()) return apply_tune(h, it->second, s);
   }
   cudaEvent_t e0, e1;
   CUDA_TRY(cudaEventCreate(&e0));
   CUDA_TRY(cudaEventCreate(&e1));
-  float best = 1e30f;
-  TuneCfg best_cfg{kRecOut, 0, 0};
-  for (int32_t ob : {1024, 512, 256}) {
-    build_apply_tasks(h, ob);
-    RC_TRY(upload_tasks(h, s));
-    for (int32_t cfg = 0; cfg < 3; ++cfg) {
-      const int32_t gm = cfg == 2 ? 1 : 0;
-      const int32_t variant = cfg == 1 ? 1 : 0;
-      h->grid_mult = gm;
-      h->rec_variant = variant;
-      RC_TRY(launch_apply(h, 0, s));  // warm-up
-      RC_TRY(launch_apply(h, 1, s));
-      CUDA_TRY(cudaEventRecord(e0, s));
-      for (int rep = 0; rep < 2; ++rep) {
-        RC_TRY(launch_apply(h, 0, s));
-        RC_TRY(launch_apply(h, 1, s));
-      }
-      CUDA_TRY(cudaEventRecord(e1, s));
-      CUDA_TRY(cudaEventSynchronize(e1));
-      float ms = 0.f;
-      CUDA_TRY(cudaEventElapsedTime(&ms, e0, e1));
-      if (ms < best) {
-        best = ms;
-        best_cfg = {ob, gm, variant};
-      }
-    }
-  }
+  TuneCfg cfg{kRecOut, 0, 0, 0, 0};
+  const int rc = tune_applies(h, s, e0, e1, diff, fact, &cfg);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  build_apply_tasks(h, best_cfg.ob);
-  h->grid_mult = best_cfg.gm;
-  h->rec_variant = best_cfg.variant;
-  RC_TRY(upload_tasks(h, s));
+  if (rc) return rc;
+  RC_TRY(apply_tune(h, cfg, s));
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  g_tune_cache[sig] = best_cfg;
+  g_tune_cache[sig] = cfg;
   return TREE_OT_OK;
 }
 
@@ -1114,8 +1223,8 @@ int autotune_dense(tree_ot_handle* h, cudaStream_t s) {
     h->dense_tma = tma;
     for (int rep = 0; rep < 4; ++rep) {
       if (rep == 1) CUDA_TRY(cudaEventRecord(e0, s));
-      RC_TRY(launch_apply(h, 0, s, true));
-      RC_TRY(launch_apply(h, 1, s, true));
+      RC_TRY(launch_apply(h, 0, s, APPLY_STORED));
+      RC_TRY(launch_apply(h, 1, s, APPLY_STORED));
     }
     CUDA_TRY(cudaEventRecord(e1, s));
     CUDA_TRY(cudaEventSynchronize(e1));
@@ -1215,6 +1324,103 @@ int plan_shared_kernels(tree_ot_handle* h, const tree_ot_problem* probs, int32_t
     if (!g.cols[0].empty() || !g.cols[1].empty()) kept.push_back(std::move(g));
   h->sk = std::move(kept);
   h->sk_prob = ok;
+  return TREE_OT_OK;
+}
+
+// Compact groups of the support points of squared-Euclidean problems (group.cu): measures the groups of
+// 64, 32, 16 and 8 points of every node, picks each node's size by kGroupKappa, sorts the points and sets the
+// directed edges in factored form to a single reduction split (nodes and dedges are uploaded again after).
+int plan_groups(tree_ot_handle* h, cudaStream_t s) {
+  if (h->fp64) return TREE_OT_OK;
+  std::vector<GroupWork> work;
+  for (size_t j = 0; j < h->nodes.size(); ++j) {
+    const NodeD& nd = h->nodes[j];
+    if (nd.coord_off < 0 || nd.n < kGroupMin || h->probs[nd.prob].cost_kind != TREE_OT_COST_SQEUCLID) continue;
+    for (int32_t x0 = 0; x0 < nd.n; x0 += kGroupChunk)
+      work.push_back(GroupWork{(int32_t)j, x0, std::min(kGroupChunk, nd.n - x0)});
+  }
+  if (work.empty()) return TREE_OT_OK;
+  GroupWork* d_work = nullptr;
+  float* d_meas = nullptr;
+  std::vector<float> meas(kGroupSizes * work.size());
+  const int32_t nw = (int32_t)work.size();
+  cudaError_t e = cudaMalloc((void**)&d_work, sizeof(GroupWork) * work.size());
+  if (e == cudaSuccess) e = cudaMalloc((void**)&d_meas, sizeof(float) * meas.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(d_work, work.data(), sizeof(GroupWork) * work.size(), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, d_meas, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(meas.data(), d_meas, sizeof(float) * meas.size(), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  int rc = e == cudaSuccess ? TREE_OT_OK : cuda_fail(e, "measuring the point groups");
+  int64_t slots = 0;
+  for (size_t i = 0; rc == TREE_OT_OK && i < work.size();) {
+    NodeD& nd = h->nodes[work[i].node];
+    double r2[kGroupSizes] = {};
+    size_t k = i;
+    for (; k < work.size() && work[k].node == work[i].node; ++k)
+      for (int v = 0; v < kGroupSizes; ++v) r2[v] += meas[kGroupSizes * k + v];
+    for (int v = 0; v < kGroupSizes && nd.gs == 0; ++v) {
+      const int32_t gs = 64 >> v, ng = (nd.n + gs - 1) / gs;
+      if (h->probs[nd.prob].s2_scaled * (r2[v] / ng) <= kGroupKappa[v]) nd.gs = gs;
+    }
+    if (nd.gs) {
+      nd.slot_off = slots;
+      slots += align_up(nd.n, 64);
+    }
+    i = k;
+  }
+  if (rc == TREE_OT_OK && slots > 0 &&
+      !((rc = h->alloc(&h->d_slot_x, slots)) || (rc = h->alloc(&h->d_slot_q, slots)) ||
+        (rc = h->alloc(&h->d_grp, 3 * (slots / 8))))) {
+    e = cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
+                             h->d_grp, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) rc = cuda_fail(e, "building the point groups");
+  }
+  cudaFree(d_work);
+  cudaFree(d_meas);
+  if (rc) return rc;
+  for (size_t di = 0; di < h->dedges.size(); ++di) {
+    DEdgeD& d = h->dedges[di];
+    if (!fact_edge(h, d)) continue;
+    d.nsplit = 1;
+    const NodeD &own = h->nodes[d.owner], &nbn = h->nodes[d.nbr];
+    const ProbD& pd = h->probs[d.prob];
+    for (int32_t o0 = 0; o0 < own.n; o0 += 64) {
+      FactItem it{};
+      it.slot0 = own.slot_off + o0;
+      it.part_off = d.part_off;
+      it.off = d.off;
+      it.rev_off = d.rev_off;
+      it.coord_nbr = nbn.coord_off;
+      it.nrow = std::min(64, own.n - o0);
+      it.n_nbr = nbn.n;
+      it.dedge = (int32_t)di;
+      it.prob = d.prob;
+      it.gs = own.gs;
+      it.shi = pd.s2_scaled;
+      it.slo = pd.s2_scaled_lo;
+      h->items[own.colour].push_back(it);
+    }
+  }
+  for (int c = 0; c < 2; ++c) {
+    auto& v = h->items[c];
+    auto dim = [&](const FactItem& x) { return h->probs[x.prob].dim; };
+    std::stable_sort(v.begin(), v.end(), [&](const FactItem& x, const FactItem& y) {
+      if (dim(x) != dim(y)) return dim(x) < dim(y);
+      return (int64_t)x.nrow * x.n_nbr > (int64_t)y.nrow * y.n_nbr;
+    });
+    for (const FactItem& x : v) ++h->item_count[c][dim(x)];
+    for (int k = 1; k < 4; ++k) h->item_begin[c][k] = h->item_begin[c][k - 1] + h->item_count[c][k - 1];
+    if (v.empty()) continue;
+    RC_TRY(h->alloc(&h->d_items[c], (int64_t)v.size()));
+    CUDA_TRY(cudaMemcpyAsync(h->d_items[c], v.data(), sizeof(FactItem) * v.size(), cudaMemcpyHostToDevice, s));
+  }
+  CUDA_TRY(cudaStreamSynchronize(s));
+  build_apply_tasks(h, kRecOut);
   return TREE_OT_OK;
 }
 
@@ -1325,14 +1531,15 @@ int setup_forest(tree_ot_handle* h, cudaStream_t s) {
     if (h->slot_count[c][0] > 0) return TREE_OT_OK;
     for (int slot = 1; slot < kApplySlots; ++slot) {
       if (h->slot_count[c][slot] == 0) continue;
-      if (D && D != slot) return TREE_OT_OK;
-      D = slot;
+      const int dim = slot > 3 ? slot - 3 : slot;
+      if (D && D != dim) return TREE_OT_OK;
+      D = dim;
     }
   }
   if (D == 0) return TREE_OT_OK;
   std::vector<int32_t> cnt(4 * (size_t)h->nprob, 0);
   for (int c = 0; c < 2; ++c) {
-    for (int32_t i = 0; i < h->slot_count[c][D]; ++i)
+    for (int32_t i = 0; i < h->slot_count[c][D] + h->slot_count[c][D + 3]; ++i)
       ++cnt[4 * h->dedges[h->tasks[c][h->slot_begin[c][D] + i].dedge].prob + c];
     for (const NodeChunk& ch : h->chunks[c]) ++cnt[4 * h->nodes[ch.node].prob + 2 + c];
   }
@@ -1641,10 +1848,13 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   }
   h->nzchunks = chunk_base;
 
-  // device task arrays are sized for the finest output blocking the autotuner may pick
+  // device task arrays are sized for the finest output blocking the autotuner may pick, in either form
+  // of the recomputed-cost apply (an edge in factored form takes at most n / 64 tasks)
   build_apply_tasks(h, 256);
-  h->task_cap[0] = (int64_t)h->tasks[0].size();
-  h->task_cap[1] = (int64_t)h->tasks[1].size();
+  for (int c = 0; c < 2; ++c) h->task_cap[c] = (int64_t)h->tasks[c].size();
+  for (const DEdgeD& d : h->dedges)
+    if (!h->fp64 && h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
+      h->task_cap[h->nodes[d.owner].colour] += (h->nodes[d.owner].n + 63) / 64;
   build_apply_tasks(h, kRecOut);
   // absorbed BF16 phase: apply tasks per colour and absorption blocks (stored-cost edges only)
   h->lowp = o.apply_mode == TREE_OT_APPLY_BF16 && !h->fp64;
@@ -1721,7 +1931,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       (rc = h->alloc(&h->d_Z, NN)) || (rc = h->alloc(&h->d_rho, NN)) || (rc = h->alloc(&h->d_logg, h->node_len)) ||
       (rc = h->alloc(&h->d_mu, h->node_len)) || (rc = h->alloc(&h->d_lgf, h->node_len)) ||
       (rc = h->alloc(&h->d_coords, h->coord_len)) ||
-      (rc = h->alloc(&h->d_coords_hi, h->coord_len)) || (rc = h->alloc(&h->d_coords_lo, h->coord_len)) ||
+      (rc = h->alloc(&h->d_coords_hi, h->coord_len + 4)) || (rc = h->alloc(&h->d_coords_lo, h->coord_len + 4)) ||
       (rc = h->alloc(&h->d_cmax, num_probs)) || (rc = h->alloc(&h->d_exact, num_probs)) ||
       (rc = h->alloc(&h->d_zpart, h->nzchunks)) || (rc = h->alloc(&h->d_resid_acc, ND)) ||
       (rc = h->alloc(&h->d_resid_dedge, ND)) || (rc = h->alloc(&h->d_res_sum, (int64_t)kResidRing * num_probs)) ||
@@ -1756,6 +1966,38 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       if ((rc = h->alloc(&ed.K, (int64_t)ed.na * ed.ldk))) return bail(rc);
     }
   }
+  auto up = [&](void* dst, const void* src, size_t bytes) -> int {
+    if (bytes == 0) return TREE_OT_OK;
+    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
+    return e == cudaSuccess ? TREE_OT_OK : cuda_fail(e, "cudaMemcpyAsync(upload)");
+  };
+
+  // coordinates
+  for (int32_t p = 0; p < num_probs; ++p) {
+    const tree_ot_problem& P = probs[p];
+    const ProbD& pd = h->probs[p];
+    if (!P.coords || pd.dim == 0) continue;
+    const cudaMemcpyKind kind =
+        (P.flags & TREE_OT_INPUT_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    for (int32_t j = 0; j < P.num_nodes; ++j) {
+      const NodeD& nd = h->nodes[h->prob_node_base[p] + j];
+      cudaError_t e = cudaMemcpyAsync(h->d_coords + nd.coord_off, P.coords[j], sizeof(float) * nd.n * pd.dim, kind, s);
+      if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMemcpyAsync(coords)"));
+    }
+  }
+  if (h->coord_len > 0) {  // the split and the grouping need the node and problem tables on the device
+    if ((rc = up(h->d_probs, h->probs.data(), sizeof(ProbD) * h->probs.size())) ||
+        (rc = up(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size())))
+      return bail(rc);
+    // the factored apply loads points in pairs: padding after a support reads as zeros
+    cudaError_t e = cudaMemsetAsync(h->d_coords_hi, 0, sizeof(float) * (h->coord_len + 4), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_coords_lo, 0, sizeof(float) * (h->coord_len + 4), s);
+    if (e == cudaSuccess)
+      e = launch_split_coords(h->d_coords, h->d_nodes, (int32_t)h->nodes.size(), h->d_probs, h->d_cmax,
+                                        num_probs, h->d_coords_hi, h->d_coords_lo, s);
+    if (e != cudaSuccess) return bail(cuda_fail(e, "coordinate split"));
+    if ((rc = plan_groups(h, s))) return bail(rc);
+  }
   if ((rc = setup_shared_kernels(h, s))) return bail(rc);
   if (!h->fp64) {  // host-resolved records of the fixed leaves' chunks, per colour
     std::vector<SkRefD> skref(h->dedges.size(), SkRefD{nullptr, nullptr, nullptr});
@@ -1782,12 +2024,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       if (ce != cudaSuccess) return bail(cuda_fail(ce, "upload fixed-leaf chunk records"));
     }
   }
-
-  auto up = [&](void* dst, const void* src, size_t bytes) -> int {
-    if (bytes == 0) return TREE_OT_OK;
-    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s);
-    return e == cudaSuccess ? TREE_OT_OK : cuda_fail(e, "cudaMemcpyAsync(upload)");
-  };
 
   // node vectors: log gamma and mu (FP64)
   {
@@ -1816,19 +2052,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
         (rc = up(h->d_lgf, lgf.data(), sizeof(float4) * lgf.size())))
       return bail(rc);
     CUDA_TRY(cudaStreamSynchronize(s));
-  }
-  // coordinates
-  for (int32_t p = 0; p < num_probs; ++p) {
-    const tree_ot_problem& P = probs[p];
-    const ProbD& pd = h->probs[p];
-    if (!P.coords || pd.dim == 0) continue;
-    const cudaMemcpyKind kind =
-        (P.flags & TREE_OT_INPUT_DEVICE) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    for (int32_t j = 0; j < P.num_nodes; ++j) {
-      const NodeD& nd = h->nodes[h->prob_node_base[p] + j];
-      cudaError_t e = cudaMemcpyAsync(h->d_coords + nd.coord_off, P.coords[j], sizeof(float) * nd.n * pd.dim, kind, s);
-      if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMemcpyAsync(coords)"));
-    }
   }
   // dense costs: borrow aligned device matrices, otherwise copy into a padded buffer
   CUDA_TRY(cudaMemsetAsync(h->d_scan, 0, sizeof(int32_t), s));
@@ -1883,11 +2106,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       (rc = up(h->d_chunks[1], h->chunks[1].data(), sizeof(NodeChunk) * h->chunks[1].size())) ||
       (rc = up(h->d_check_tasks, h->check_tasks.data(), sizeof(Task) * h->check_tasks.size())))
     return bail(rc);
-  if (h->coord_len > 0) {  // needs the node and problem tables on the device
-    cudaError_t e = launch_split_coords(h->d_coords, h->d_nodes, (int32_t)h->nodes.size(), h->d_probs, h->d_cmax,
-                                        num_probs, h->d_coords_hi, h->d_coords_lo, s);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "coordinate split"));
-  }
   if (h->lowp && ((rc = up(h->d_btasks[0], h->btasks[0].data(), sizeof(Task) * h->btasks[0].size())) ||
                   (rc = up(h->d_btasks[1], h->btasks[1].data(), sizeof(Task) * h->btasks[1].size())) ||
                   (rc = up(h->d_atasks, h->atasks.data(), sizeof(Task) * h->atasks.size()))))

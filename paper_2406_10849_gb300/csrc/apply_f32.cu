@@ -33,7 +33,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
-#include "recomp_task.cuh"
+#include "fact_task.cuh"
 
 namespace treeot {
 
@@ -242,11 +242,15 @@ __global__ void __launch_bounds__(kApplyThreads, 2) apply_dense_kernel(ApplyArgs
 // Tasks come from a work queue (an atomic counter; tasks are sorted by cost on
 // the host), so uneven edges of a batch of trees balance across the CTAs.  The
 // last CTA to leave resets the counter for the next launch.
-// EXACT: some problems run the exact-distance variant (A.exact); instantiated
-// separately so the plain kernel keeps its register budget.
-template <int D, int MINB, bool EXACT>
+// MODE 0: the difference form alone.  MODE 1: both forms' tasks, and some
+// problems run the exact-distance variant (A.exact).  MODE 2: both forms' tasks
+// in one launch, for handles whose two launches would each leave the GPU half
+// empty (the autotuner times it).  Instantiated separately so that the plain
+// kernel keeps its register budget.
+template <int D, int MINB, int MODE>
 __global__ void __launch_bounds__(kApplyThreads, MINB) apply_recomp_kernel(ApplyArgs A) {
-  __shared__ __align__(16) float sm[16 * kApplyThreads + 2 * 4 * kApplyThreads];  // 24 KB
+  // 24 KB of the difference form's staging; the factored form's where it runs (28 KB)
+  __shared__ __align__(16) float sm[MODE == 0 ? 24 * kApplyThreads : kFactSmemFloats];
   __shared__ int s_ti;
   // every problem retired or in a BF16 phase: nothing to apply (the same for every CTA; the
   // work queue is then untouched and stays reset)
@@ -260,11 +264,77 @@ __global__ void __launch_bounds__(kApplyThreads, MINB) apply_recomp_kernel(Apply
     const Task t = A.tasks[ti];
     const int prob = A.dedges[t.dedge].prob;
     if (A.done[prob] || A.lowp[prob] == 1) continue;  // retired, or in a BF16 phase
-    if (EXACT && A.exact[prob])  // block-uniform: refined past the plain recomputation's floor
+    if (MODE == 1 && A.exact[prob])  // block-uniform: refined past the plain recomputation's floor
       recomp_task_exact<D>(A, t, sm);
+    else if (MODE != 0 && t.kind >= TASK_FACT)
+      fact_dispatch<D>(A, t, sm);
     else
       recomp_task<D>(A, t, sm);
   }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&A.queue[1], 1) == (int)gridDim.x - 1) {
+      A.queue[0] = 0;
+      A.queue[1] = 0;
+      __threadfence();
+    }
+  }
+}
+
+// The factored form (fact_task.cuh) in kernels of its own: it needs fewer
+// registers than the difference form, and more warps hide the MUFU's latency.
+// SHARED: tasks of the CTA, whose warps share blocks of outputs (small handles).
+template <int D>
+__global__ void __launch_bounds__(kApplyThreads, 2) apply_fact_shared_kernel(ApplyArgs A) {
+  __shared__ __align__(16) float sm[kFactSmemFloats];
+  if (A.fp32_live && *((volatile const int32_t*)A.fp32_live) <= 0) return;
+  for (int ti = blockIdx.x; ti < A.ntasks; ti += gridDim.x) {
+    const Task t = A.tasks[ti];
+    const int prob = A.dedges[t.dedge].prob;
+    if (A.done[prob] || A.lowp[prob] == 1) continue;  // retired, or in a BF16 phase
+    fact_dispatch<D>(A, t, sm);
+    __syncthreads();
+  }
+}
+
+// One block of 64 outputs per item, an item per warp, from a queue sorted by cost.  Warps run
+// on their own (no CTA barrier): while a warp works on an item, the next item's
+// record is on its way into a register and the ticket after that is being taken,
+// so the chain queue -> record -> block does not stall it.
+constexpr int kFactThreads = 128, kFactCtas = 4;  // 16 warps per SM (20 measured the same)
+template <int D>
+__global__ void __launch_bounds__(kFactThreads, kFactCtas) apply_fact_kernel(ApplyArgs A) {
+  constexpr int kWarps = kFactThreads / 32, kWords = sizeof(FactItem) / 4;
+  static_assert(kWords <= 32, "a record is loaded one word per lane");
+  __shared__ __align__(16) float sm[kWarps * kFactWarp];
+  __shared__ __align__(16) int32_t s_rec[kWarps][kWords];
+  if (A.fp32_live && *((volatile const int32_t*)A.fp32_live) <= 0) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the first two tickets follow from the warp's place; the queue counts from there
+  const int nwarps = gridDim.x * kWarps;
+  int cur = blockIdx.x * kWarps + warp, nxt = cur + nwarps;
+  int32_t word = 0;
+  if (cur < A.nitems && lane < kWords) word = reinterpret_cast<const int32_t*>(A.items + cur)[lane];
+  while (cur < A.nitems) {  // warp-uniform
+    __syncwarp();
+    if (lane < kWords) s_rec[warp][lane] = word;
+    __syncwarp();
+    int ticket = 0;
+    if (lane == 0) ticket = atomicAdd(&A.queue[0], 1);
+    if (nxt < A.nitems && lane < kWords) word = reinterpret_cast<const int32_t*>(A.items + nxt)[lane];
+    const FactItem& it = *reinterpret_cast<const FactItem*>(s_rec[warp]);
+    if (!A.done[it.prob] && A.lowp[it.prob] != 1) {  // not retired, nor in a BF16 phase
+      if (it.gs == 64)
+        fact_block<D, 64, false>(A, it, sm, warp, 0);
+      else if (it.gs == 32)
+        fact_block<D, 32, false>(A, it, sm, warp, 0);
+      else
+        fact_block<D, 16, false>(A, it, sm, warp, 0);
+    }
+    cur = nxt;
+    nxt = 2 * nwarps + __shfl_sync(0xffffffffu, ticket, 0);
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&A.queue[1], 1) == (int)gridDim.x - 1) {
@@ -403,12 +473,23 @@ __global__ void noalloc_merge_kernel(const float2* part, int32_t n_rows, int32_t
 template <int D, int MINB>
 int occ_recomp() {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, apply_recomp_kernel<D, MINB, false>, kApplyThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, apply_recomp_kernel<D, MINB, 0>, kApplyThreads, 0);
+  return n > 0 ? n : 1;
+}
+
+template <int D>
+int occ_fact(int shared) {
+  int n = 0;
+  if (shared)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, apply_fact_shared_kernel<D>, kApplyThreads, 0);
+  else
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, apply_fact_kernel<D>, kFactThreads, 0);
   return n > 0 ? n : 1;
 }
 
 int apply_ctas_per_sm(int slot, int variant) {
   int n = 0;
+  if (slot > 3) return slot == 4 ? occ_fact<1>(variant) : slot == 5 ? occ_fact<2>(variant) : occ_fact<3>(variant);
   if (slot == 0) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, apply_dense_kernel, kApplyThreads, 0);
     return n > 0 ? n : 1;
@@ -422,18 +503,34 @@ cudaError_t launch_apply_f32(const ApplyArgs& a, int slot, int variant, int grid
   if (slot == 0) {
     apply_dense_kernel<<<grid, kApplyThreads, 0, s>>>(a);
   } else if (a.any_exact) {
-    // rare (after certification): the 2-CTA register budget, whatever the tuned variant
-    if (slot == 1) apply_recomp_kernel<1, 2, true><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 2) apply_recomp_kernel<2, 2, true><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 3) apply_recomp_kernel<3, 2, true><<<grid, kApplyThreads, 0, s>>>(a);
+    // rare (after certification): the 2-CTA register budget, whatever the tuned variant; takes both
+    // forms' tasks
+    if (slot > 3) slot -= 3;
+    if (slot == 1) apply_recomp_kernel<1, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 2) apply_recomp_kernel<2, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 3) apply_recomp_kernel<3, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
+  } else if (variant == kBothForms) {  // a: the tasks of both forms
+    if (slot == 1) apply_recomp_kernel<1, 2, 2><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 2) apply_recomp_kernel<2, 2, 2><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 3) apply_recomp_kernel<3, 2, 2><<<grid, kApplyThreads, 0, s>>>(a);
+  } else if (slot > 3) {
+    if (variant) {  // warps share blocks
+      if (slot == 4) apply_fact_shared_kernel<1><<<grid, kApplyThreads, 0, s>>>(a);
+      if (slot == 5) apply_fact_shared_kernel<2><<<grid, kApplyThreads, 0, s>>>(a);
+      if (slot == 6) apply_fact_shared_kernel<3><<<grid, kApplyThreads, 0, s>>>(a);
+    } else {
+      if (slot == 4) apply_fact_kernel<1><<<grid, kFactThreads, 0, s>>>(a);
+      if (slot == 5) apply_fact_kernel<2><<<grid, kFactThreads, 0, s>>>(a);
+      if (slot == 6) apply_fact_kernel<3><<<grid, kFactThreads, 0, s>>>(a);
+    }
   } else if (variant == 0) {
-    if (slot == 1) apply_recomp_kernel<1, 2, false><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 2) apply_recomp_kernel<2, 2, false><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 3) apply_recomp_kernel<3, 2, false><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 1) apply_recomp_kernel<1, 2, 0><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 2) apply_recomp_kernel<2, 2, 0><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 3) apply_recomp_kernel<3, 2, 0><<<grid, kApplyThreads, 0, s>>>(a);
   } else {
-    if (slot == 1) apply_recomp_kernel<1, 3, false><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 2) apply_recomp_kernel<2, 3, false><<<grid, kApplyThreads, 0, s>>>(a);
-    if (slot == 3) apply_recomp_kernel<3, 3, false><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 1) apply_recomp_kernel<1, 3, 0><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 2) apply_recomp_kernel<2, 3, 0><<<grid, kApplyThreads, 0, s>>>(a);
+    if (slot == 3) apply_recomp_kernel<3, 3, 0><<<grid, kApplyThreads, 0, s>>>(a);
   }
   return cudaGetLastError();
 }

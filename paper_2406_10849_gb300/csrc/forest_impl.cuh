@@ -6,7 +6,7 @@
 
 #include "forest.h"
 #include "node_chunk.cuh"
-#include "recomp_task.cuh"
+#include "fact_task.cuh"
 
 namespace treeot {
 namespace {
@@ -67,6 +67,8 @@ __device__ __forceinline__ int apply_item(const ForestArgs& F, const ApplyArgs& 
   if (go == 1) {
     if (EXACT && A.exact[p])
       recomp_task_exact<D>(A, task, sm);
+    else if (task.kind >= TASK_FACT)
+      fact_dispatch<D>(A, task, sm);
     else
       recomp_task<D>(A, task, sm);
   }
@@ -109,7 +111,7 @@ __device__ __forceinline__ int node_item(const ForestArgs& F, const NodeArgs& N,
 template <int D, bool EXACT, int MINB>
 __global__ void __launch_bounds__(kApplyThreads, MINB) forest_kernel(ForestArgs F) {
   extern __shared__ __align__(16) unsigned char node_sm[];
-  __shared__ __align__(16) float sm[16 * kApplyThreads + 2 * 4 * kApplyThreads];  // apply staging, 24 KB
+  __shared__ __align__(16) float sm[kFactSmemFloats];  // apply staging, 28 KB
   __shared__ double red[kNodeThreads / 32];
   __shared__ int s_t;
   const int tid = threadIdx.x;

@@ -45,6 +45,8 @@ enum TaskKind : int32_t {
   TASK_ROW = 0,     // stored matrix, owner is the row node: reduce along a row
   TASK_COL = 1,     // stored matrix, owner is the column node: reduce down columns
   TASK_RECOMP = 2,  // squared-Euclidean cost recomputed from coordinates
+  TASK_FACT = 4,    // 4 .. 7: the same in factored form, outputs are slots of the owner's groups, 2^(kind - 4)
+                    // warps share a group
 };
 
 struct DEdgeD {
@@ -77,7 +79,21 @@ struct NodeD {
   int32_t colour;
   int32_t chunk_base;   // node-update chunks of this node: zpart[chunk_base .. +nchunks)
   int32_t nchunks;
+  int64_t slot_off;     // compact groups of the points (group.cu): first slot (a multiple of 64)
+  int32_t gs;           // points per group (64, 32 or 16), 0 = not grouped
+  int32_t pad;
 };
+
+// A chunk of at most kGroupChunk consecutive points of a node, sorted into compact groups by one CTA
+constexpr int kGroupChunk = 4096;
+struct GroupWork {
+  int32_t node, x0, cnt;
+};
+// The largest kappa = s r^2 of a node's groups of 64, 32 and 16 points at which the factored apply is
+// used (see group.cu); below kGroupMin points on either side the difference form runs
+constexpr int kGroupSizes = 3;  // 64, 32, 16
+constexpr float kGroupKappa[kGroupSizes] = {3.f, 2.f, 2.f};
+constexpr int kGroupMin = 32;
 
 struct NodeChunk {
   int32_t node, chunk, x0, cnt;
@@ -176,6 +192,21 @@ struct Task {
   int32_t pad;          // RECOMP: warp groups sharing the task (1, 2, 4, 8); ROW: 1 = rows of CT
 };
 
+// A block of 64 of a directed edge's outputs against all of the neighbour's points, resolved on the host: an item
+// of the factored apply's per-warp queue (five 16-byte words)
+struct FactItem {
+  int64_t slot0;       // the block's first slot
+  int64_t part_off;    // partials of the directed edge
+  int64_t off;         // owner-side vectors (frames)
+  int64_t rev_off;     // the neighbour's operand
+  int64_t coord_nbr;   // the neighbour's coordinates
+  int32_t nrow, n_nbr; // outputs of the block, points of the neighbour
+  int32_t dedge, prob;
+  int32_t gs, pad;     // group size
+  float shi, slo;      // cost scale log2(e) / eps as a two-float
+  int32_t pad2[2];
+};
+
 // A stored-cost (ROW / COL) task with every address resolved on the host, for
 // the bulk-copy staged kernel.  The tile's stage rows are C + r * ld: output
 // rows for ROW tasks, reduction rows for COL tasks.
@@ -206,6 +237,9 @@ struct ApplyArgs {
   const float* coords;
   const float* coords_hi;    // coordinates split hi + lo (hi on the problem's 2^-10 sigma grid)
   const float* coords_lo;
+  const float4* slot_x;      // per slot: coordinates less the group's centre, point index (as int bits)
+  const float2* slot_q;      // per slot: s |x'|^2 as a two-float
+  const float4* grp;         // per 8 slots (at a group's first): 3 x float4, centre, unit, inverse second moments
   const int32_t* exact;      // per problem: 1 = recompute costs with exact squared distances
   int32_t any_exact;         // host: some problem has exact set (selects the kernel instantiation)
   float2* part32;            // FP32 path partials: (frame R, sum) in base 2
@@ -217,6 +251,8 @@ struct ApplyArgs {
   const float* bl;
   const float* arho;         // row normalisers of the absorbed kernels (row side of each edge)
   int32_t* err;              // error word: bit 1 = a bounded wait of a staged kernel ran out
+  const FactItem* items;     // factored kernel: resolved groups (nitems of them), largest first
+  int32_t nitems;
   const StreamTask* stasks;  // staged kernel: resolved stored-cost tasks (ntasks of them)
   int32_t test_stall;        // staged kernel: the producer issues nothing (tests the timeout path)
   const int32_t* fp32_live;  // problems the FP32 kernels still process (not retired, not in a BF16
@@ -338,8 +374,10 @@ struct CheckArgs {
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------
-// slot 0: stored-cost tasks (ROW/COL); slot D (1..3): recomputed squared-Euclidean tasks
+// slot 0: stored-cost tasks (ROW/COL); slot D (1..3): recomputed squared-Euclidean tasks; slot 3 + D: the
+// same in factored form (fact_task.cuh)
 // variant (recomputed costs): 0 = 2 CTAs per SM register budget, 1 = 3 CTAs per SM
+constexpr int kBothForms = 3;  // variant: slots D and 3 + D in one launch
 cudaError_t launch_apply_f32(const ApplyArgs& a, int slot, int variant, int grid, cudaStream_t s);
 // stored-cost (slot 0) tasks with bulk-copy staged rows; one CTA per SM, grid = SM count
 bool apply_tma_available();
@@ -375,6 +413,11 @@ cudaError_t launch_scan_cost(const float* C, int64_t ld, int32_t rows, int32_t c
 cudaError_t launch_transpose_pad(const float* src, int64_t src_ld, int32_t rows, int32_t cols, float* dst,
                                  int64_t dst_ld, cudaStream_t s);
 // coordinates split hi + lo for the exact-distance recomputation (cmax: nprob scratch words)
+cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
+                                 const float* coords, float* out, cudaStream_t s);
+cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
+                               const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
+                               cudaStream_t s);
 cudaError_t launch_split_coords(const float* coords, const NodeD* nodes, int32_t nnodes, const ProbD* probs,
                                 uint32_t* cmax, int32_t nprob, float* hi, float* lo, cudaStream_t s);
 cudaError_t launch_check(const CheckArgs& a, cudaStream_t s);
@@ -390,7 +433,7 @@ cudaError_t noalloc_scratch(float** out, int64_t* capacity_floats);
 int64_t noalloc_scratch_floats_needed(int32_t n_rows, int32_t n_cols);
 cudaError_t launch_edge_apply_noalloc(const float* C, int64_t ld, int32_t n_rows, int32_t n_cols, const double* g,
                                       float shi, float slo, double* m_out, float* scratch, cudaStream_t s);
-constexpr int kApplySlots = 4;
+constexpr int kApplySlots = 7;
 
 }  // namespace treeot
 
