@@ -436,18 +436,3 @@ cudaError_t launch_edge_apply_noalloc(const float* C, int64_t ld, int32_t n_rows
 constexpr int kApplySlots = 7;
 
 }  // namespace treeot
-
-namespace treeot {
-// ---- warm-start MLP kernels (mlp.cu) ---------------------------------------
-cudaError_t mlp_gemm(const void* A, int lda, int ta, const void* B, int ldb, int tb, float* C, int ldc, int M, int N,
-                     int K, const float* bias, int accumulate, cudaStream_t s);
-cudaError_t mlp_gelu_fwd(const float* z, void* a16, int64_t n, cudaStream_t s);
-cudaError_t mlp_gelu_bwd(const float* da, const float* z, void* dz16, float* dz32, int64_t n, cudaStream_t s);
-cudaError_t mlp_to_bf16(const float* x, void* y, int64_t n, cudaStream_t s);
-cudaError_t mlp_input(const float* x, void* y, int64_t rows, int cols, int nlog, float floor_, float scale,
-                      cudaStream_t s);
-cudaError_t mlp_mse(const float* y, const float* t, float* dy32, void* dy16, int64_t n, double* loss, cudaStream_t s);
-cudaError_t mlp_colsum(const float* dz, int M, int N, float* db, cudaStream_t s);
-cudaError_t mlp_adam(float* w, const float* g, float* m1, float* m2, void* w16, int64_t n, float lr, float b1, float b2,
-                     float eps, float c1, float c2, cudaStream_t s);
-}  // namespace treeot

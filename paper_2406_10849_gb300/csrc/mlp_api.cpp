@@ -10,6 +10,7 @@
 
 #include "../../include/tree_ot.h"
 #include "internal.h"
+#include "mlp.h"
 
 using namespace treeot;
 
@@ -19,10 +20,11 @@ struct tree_ot_mlp {
   int64_t off[6] = {};   // W1, b1, W2, b2, W3, b3 in the FP32 parameter vector
   int64_t len[6] = {};
   float *w = nullptr, *g = nullptr, *m1 = nullptr, *m2 = nullptr;  // FP32 master, gradients, Adam moments
-  void* w16 = nullptr;                                             // BF16 copy of the whole vector
+  MlpW16 w16{};  // BF16 copies of the weights; like every BF16 buffer, rows padded with zeros to ld = 8 k
+  int32_t ldi = 0, ldh = 0, ldo = 0;  // padded row strides of in, hid and out columns
   void *x16 = nullptr, *a1 = nullptr, *a2 = nullptr, *dy16 = nullptr, *dz2_16 = nullptr, *dz1_16 = nullptr;
-  float *z1 = nullptr, *z2 = nullptr, *y = nullptr, *dy32 = nullptr, *da2 = nullptr, *dz2_32 = nullptr;
-  float *da1 = nullptr, *dz1_32 = nullptr;
+  float *z1 = nullptr, *z2 = nullptr, *y = nullptr, *dy32 = nullptr, *dz2_32 = nullptr;
+  float* dz1_32 = nullptr;
   double* loss = nullptr;
   int64_t step = 0;
   int32_t nlog = 0;          // input transform: first nlog features -> log(max(x, floor)) * scale
@@ -61,35 +63,62 @@ uint64_t splitmix64(uint64_t& s) {
   return z ^ (z >> 31);
 }
 
-// bf16 pointer arithmetic on the weight copy
-void* w16_at(tree_ot_mlp* m, int t) { return static_cast<char*>(m->w16) + 2 * m->off[t]; }
-
-int forward(tree_ot_mlp* m, const float* x, int32_t B, cudaStream_t s) {
-  MCUDA(mlp_input(x, m->x16, B, m->in, m->nlog, m->log_floor, m->log_scale, s));
-  MCUDA(mlp_gemm(m->x16, m->in, 0, w16_at(m, 0), m->in, 1, m->z1, m->hid, B, m->hid, m->in, m->w + m->off[1], 0, s));
-  MCUDA(mlp_gelu_fwd(m->z1, m->a1, (int64_t)B * m->hid, s));
-  MCUDA(mlp_gemm(m->a1, m->hid, 0, w16_at(m, 2), m->hid, 1, m->z2, m->hid, B, m->hid, m->hid, m->w + m->off[3], 0, s));
-  MCUDA(mlp_gelu_fwd(m->z2, m->a2, (int64_t)B * m->hid, s));
-  MCUDA(mlp_gemm(m->a2, m->hid, 0, w16_at(m, 4), m->hid, 1, m->y, m->out, B, m->out, m->hid, m->w + m->off[5], 0, s));
+int step1(const MlpGemm& a, cudaStream_t s) {
+  MlpStep st{};
+  st.gemm[0] = a;
+  st.ngemm = 1;
+  MCUDA(mlp_step(st, s));
   return TREE_OT_OK;
 }
 
+// y: where the network's output goes (batch x out)
+int forward(tree_ot_mlp* m, const float* x, int32_t B, float* y, cudaStream_t s) {
+  MCUDA(mlp_input(x, m->x16, B, m->in, m->ldi, m->nlog, m->log_floor, m->log_scale, m->loss, s));
+  MlpGemm j = mlp_gemm(m->x16, m->ldi, 0, m->w16.dst[0], m->ldi, 1, m->z1, m->hid, B, m->hid, m->in);
+  j.bias = m->w + m->off[1];
+  j.mode = MLP_GELU;
+  j.H = m->a1;
+  j.ldh = m->ldh;
+  int rc = step1(j, s);
+  if (rc) return rc;
+  j = mlp_gemm(m->a1, m->ldh, 0, m->w16.dst[1], m->ldh, 1, m->z2, m->hid, B, m->hid, m->hid);
+  j.bias = m->w + m->off[3];
+  j.mode = MLP_GELU;
+  j.H = m->a2;
+  j.ldh = m->ldh;
+  if ((rc = step1(j, s))) return rc;
+  j = mlp_gemm(m->a2, m->ldh, 0, m->w16.dst[2], m->ldh, 1, y, m->out, B, m->out, m->hid);
+  j.bias = m->w + m->off[5];
+  return step1(j, s);
+}
+
 int backward(tree_ot_mlp* m, const float* t, int32_t B, cudaStream_t s) {
-  MCUDA(cudaMemsetAsync(m->loss, 0, sizeof(double), s));
-  MCUDA(mlp_mse(m->y, t, m->dy32, m->dy16, (int64_t)B * m->out, m->loss, s));
-  // layer 3: dW3 = dy^T a2, db3 = sum dy, da2 = dy W3
-  MCUDA(mlp_gemm(m->dy16, m->out, 1, m->a2, m->hid, 0, m->g + m->off[4], m->hid, m->out, m->hid, B, nullptr, 0, s));
-  MCUDA(mlp_colsum(m->dy32, B, m->out, m->g + m->off[5], s));
-  MCUDA(mlp_gemm(m->dy16, m->out, 0, w16_at(m, 4), m->hid, 0, m->da2, m->hid, B, m->hid, m->out, nullptr, 0, s));
-  MCUDA(mlp_gelu_bwd(m->da2, m->z2, m->dz2_16, m->dz2_32, (int64_t)B * m->hid, s));
+  MCUDA(mlp_mse(m->y, t, m->dy32, m->dy16, B, m->out, m->ldo, m->loss, s));
+  // layer 3: dW3 = dy^T a2, db3 = sum dy, dz2 = (dy W3) gelu'(z2)
+  MlpStep st{};
+  st.ngemm = 2;
+  st.gemm[0] = mlp_gemm(m->dy16, m->ldo, 0, m->w16.dst[2], m->ldh, 0, m->dz2_32, m->hid, B, m->hid, m->out);
+  st.gemm[0].mode = MLP_GELU_BWD;
+  st.gemm[0].z = m->z2;
+  st.gemm[0].H = m->dz2_16;
+  st.gemm[0].ldh = m->ldh;
+  st.gemm[1] = mlp_gemm(m->dy16, m->ldo, 1, m->a2, m->ldh, 0, m->g + m->off[4], m->hid, m->out, m->hid, B);
+  st.sum = MlpColsum{m->dy32, m->g + m->off[5], B, m->out};
+  MCUDA(mlp_step(st, s));
   // layer 2
-  MCUDA(mlp_gemm(m->dz2_16, m->hid, 1, m->a1, m->hid, 0, m->g + m->off[2], m->hid, m->hid, m->hid, B, nullptr, 0, s));
-  MCUDA(mlp_colsum(m->dz2_32, B, m->hid, m->g + m->off[3], s));
-  MCUDA(mlp_gemm(m->dz2_16, m->hid, 0, w16_at(m, 2), m->hid, 0, m->da1, m->hid, B, m->hid, m->hid, nullptr, 0, s));
-  MCUDA(mlp_gelu_bwd(m->da1, m->z1, m->dz1_16, m->dz1_32, (int64_t)B * m->hid, s));
+  st.gemm[0] = mlp_gemm(m->dz2_16, m->ldh, 0, m->w16.dst[1], m->ldh, 0, m->dz1_32, m->hid, B, m->hid, m->hid);
+  st.gemm[0].mode = MLP_GELU_BWD;
+  st.gemm[0].z = m->z1;
+  st.gemm[0].H = m->dz1_16;
+  st.gemm[0].ldh = m->ldh;
+  st.gemm[1] = mlp_gemm(m->dz2_16, m->ldh, 1, m->a1, m->ldh, 0, m->g + m->off[2], m->hid, m->hid, m->hid, B);
+  st.sum = MlpColsum{m->dz2_32, m->g + m->off[3], B, m->hid};
+  MCUDA(mlp_step(st, s));
   // layer 1
-  MCUDA(mlp_gemm(m->dz1_16, m->hid, 1, m->x16, m->in, 0, m->g + m->off[0], m->in, m->hid, m->in, B, nullptr, 0, s));
-  MCUDA(mlp_colsum(m->dz1_32, B, m->hid, m->g + m->off[1], s));
+  st.ngemm = 1;
+  st.gemm[0] = mlp_gemm(m->dz1_16, m->ldh, 1, m->x16, m->ldi, 0, m->g + m->off[0], m->in, m->hid, m->in, B);
+  st.sum = MlpColsum{m->dz1_32, m->g + m->off[1], B, m->hid};
+  MCUDA(mlp_step(st, s));
   return TREE_OT_OK;
 }
 
@@ -121,19 +150,33 @@ int tree_ot_mlp_create(int32_t in_dim, int32_t hidden, int32_t out_dim, int32_t 
   for (int t = 0; t < 6; ++t) {
     m->off[t] = o;
     m->len[t] = lens[t];
-    o += (lens[t] + 7) / 8 * 8;  // keep every tensor 16-byte aligned in the BF16 copy
+    o += (lens[t] + 7) / 8 * 8;  // every tensor starts at a multiple of 8 floats
   }
   m->nparam = o;
   const int64_t B = max_batch;
   int rc = 0;
+  const auto pad8 = [](int32_t v) { return (v + 7) / 8 * 8; };
+  m->ldi = pad8(in_dim);
+  m->ldh = pad8(hidden);
+  m->ldo = pad8(out_dim);
+  m->w16 = MlpW16{{m->off[0], m->off[2], m->off[4]},
+                  {m->len[0], m->len[2], m->len[4]},
+                  {in_dim, hidden, hidden},
+                  {m->ldi, m->ldh, m->ldh},
+                  {nullptr, nullptr, nullptr}};
+  // BF16 buffers: the padding of a row is never written again after this
+  const auto alloc16 = [&](void** p, int64_t rows, int32_t ld) {
+    if (int e = dalloc(m, p, rows * ld, 2)) return e;
+    return cudaMemset(*p, 0, 2 * (size_t)(rows * ld)) == cudaSuccess ? (int)TREE_OT_OK : mfail(TREE_OT_ERR_CUDA, "cudaMemset (mlp)");
+  };
   if ((rc = dalloc(m, &m->w, o)) || (rc = dalloc(m, &m->g, o)) || (rc = dalloc(m, &m->m1, o)) ||
-      (rc = dalloc(m, &m->m2, o)) || (rc = dalloc(m, &m->w16, o, 2)) || (rc = dalloc(m, &m->x16, B * in_dim, 2)) ||
-      (rc = dalloc(m, &m->a1, B * hidden, 2)) || (rc = dalloc(m, &m->a2, B * hidden, 2)) ||
-      (rc = dalloc(m, &m->dy16, B * out_dim, 2)) || (rc = dalloc(m, &m->dz2_16, B * hidden, 2)) ||
-      (rc = dalloc(m, &m->dz1_16, B * hidden, 2)) || (rc = dalloc(m, &m->z1, B * hidden)) ||
+      (rc = dalloc(m, &m->m2, o)) || (rc = alloc16(&m->w16.dst[0], hidden, m->ldi)) ||
+      (rc = alloc16(&m->w16.dst[1], hidden, m->ldh)) || (rc = alloc16(&m->w16.dst[2], out_dim, m->ldh)) ||
+      (rc = alloc16(&m->x16, B, m->ldi)) || (rc = alloc16(&m->a1, B, m->ldh)) || (rc = alloc16(&m->a2, B, m->ldh)) ||
+      (rc = alloc16(&m->dy16, B, m->ldo)) || (rc = alloc16(&m->dz2_16, B, m->ldh)) ||
+      (rc = alloc16(&m->dz1_16, B, m->ldh)) || (rc = dalloc(m, &m->z1, B * hidden)) ||
       (rc = dalloc(m, &m->z2, B * hidden)) || (rc = dalloc(m, &m->y, B * out_dim)) ||
-      (rc = dalloc(m, &m->dy32, B * out_dim)) || (rc = dalloc(m, &m->da2, B * hidden)) ||
-      (rc = dalloc(m, &m->dz2_32, B * hidden)) || (rc = dalloc(m, &m->da1, B * hidden)) ||
+      (rc = dalloc(m, &m->dy32, B * out_dim)) || (rc = dalloc(m, &m->dz2_32, B * hidden)) ||
       (rc = dalloc(m, &m->dz1_32, B * hidden)) || (rc = dalloc(m, &m->loss, 1))) {
     tree_ot_mlp_destroy(m);
     return rc;
@@ -205,9 +248,7 @@ int tree_ot_mlp_forward(tree_ot_mlp* m, void* stream, const float* x, int32_t ba
   if (rc) return rc;
   if (!y) return mfail(TREE_OT_ERR_ARG, "NULL output");
   cudaStream_t s = (cudaStream_t)stream;
-  if ((rc = forward(m, x, batch, s))) return rc;
-  MCUDA(cudaMemcpyAsync(y, m->y, sizeof(float) * (size_t)batch * m->out, cudaMemcpyDeviceToDevice, s));
-  return TREE_OT_OK;
+  return forward(m, x, batch, y, s);
 }
 
 int tree_ot_mlp_backward(tree_ot_mlp* m, void* stream, const float* x, const float* target, int32_t batch,
@@ -217,7 +258,7 @@ int tree_ot_mlp_backward(tree_ot_mlp* m, void* stream, const float* x, const flo
   if (rc) return rc;
   if (!target) return mfail(TREE_OT_ERR_ARG, "NULL target");
   cudaStream_t s = (cudaStream_t)stream;
-  if ((rc = forward(m, x, batch, s)) || (rc = backward(m, target, batch, s))) return rc;
+  if ((rc = forward(m, x, batch, m->y, s)) || (rc = backward(m, target, batch, s))) return rc;
   if (grads) MCUDA(cudaMemcpyAsync(grads, m->g, sizeof(float) * m->nparam, cudaMemcpyDeviceToDevice, s));
   if (loss) {
     MCUDA(cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -233,7 +274,7 @@ int tree_ot_mlp_train_step(tree_ot_mlp* m, void* stream, const float* x, const f
   if (rc) return rc;
   if (!target || !(lr > 0.0)) return mfail(TREE_OT_ERR_ARG, "NULL target or lr <= 0");
   cudaStream_t s = (cudaStream_t)stream;
-  if ((rc = forward(m, x, batch, s)) || (rc = backward(m, target, batch, s))) return rc;
+  if ((rc = forward(m, x, batch, m->y, s)) || (rc = backward(m, target, batch, s))) return rc;
   m->step += 1;
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - std::pow(b1, (float)m->step), c2 = 1.f - std::pow(b2, (float)m->step);
