@@ -21,7 +21,7 @@
 // The rounded plans are never stored: they are (x, y, err_r, E) plus the
 // potentials, and <C, B^> = <C, F''> + err_r^T C err_c / E.  Entries are the
 // double-float plan entries of the check (FP32 pipe; FP64 handles: FP64), every
-// sum over them is FP64.  Passes over the plans (one CTA per task of 64 rows of
+// sum over them is double-float too, flushed into FP64 (FP64 handles: FP64).  Passes over the plans (one CTA per task of 64 rows of
 // one plan, rows on S), with per-point steps between them:
 //   1  F 1, F^T 1, <C, F>, ||F||_1     -> targets t and c, row scales x
 //   2  F'^T 1                          -> column scales y
@@ -185,6 +185,192 @@ __global__ void __launch_bounds__(256) round_pass_kernel(RoundArgs A) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// Passes 1-4 of FP32 handles.  Entries and costs are pairs of FP32 values already;
+// here every sum over them is one too: products by TwoProd, additions by TwoSum,
+// running sums flushed into FP64 every kFlushCols columns.  A sum then carries a
+// few units of 2^-46 relative (measured by the tests: rounded plans feasible to
+// 1e-13, as with FP64 sums).  GB300 executes an FP64 add or a conversion at 1/70
+// of its FP32 rate, and with FP64 sums those were the passes' whole time (94 M
+// entries in 209 plans: 2.6 / 0.8 / 3.1 / 2.8 ms for passes 1-4).  Row factors
+// (x, err_r) multiply the finished row sums, not the entries.
+// ---------------------------------------------------------------------------
+constexpr int kFlushCols = 32;  // column steps (32 columns each) between flushes
+
+__device__ __forceinline__ void df_acc(DF& s, float v) {  // s += v
+  const DF t = two_sum(s.hi, v);
+  s.hi = t.hi;
+  s.lo += t.lo;
+}
+__device__ __forceinline__ void df_acc(DF& s, DF v) {
+  const DF t = two_sum(s.hi, v.hi);
+  s.hi = t.hi;
+  s.lo += t.lo + v.lo;
+}
+// a (a float) times b
+__device__ __forceinline__ DF df_mul(float a, DF b) {
+  const float p = __fmul_rn(a, b.hi);
+  return {p, fmaf(a, b.lo, fmaf(a, b.hi, -p))};
+}
+__device__ __forceinline__ DF df_mul(DF a, DF b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  return {p, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ DF df_of(double v) {
+  const float h = (float)v;
+  return {h, (float)(v - (double)h)};
+}
+__device__ __forceinline__ double df_to(DF v) { return (double)v.hi + (double)v.lo; }
+
+template <int PASS>
+__global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
+  __shared__ float2 s_col[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int ti = blockIdx.x; ti < A.ntasks; ti += gridDim.x) {
+    const RoundTask t = A.tasks[ti];
+    const DEdgeD d = A.dedges[t.dedge];
+    const EdgeD e = A.edges[d.edge];
+    const ProbD P = A.probs[d.prob];
+    const NodeD nj = A.nodes[d.owner], nk = A.nodes[d.nbr];
+    // cost rows on the owner: C itself (owner = row node), C^T when kept, else C's columns
+    const bool own_rows = d.dir == 0 || e.CT != nullptr;
+    const float* Cm = d.dir == 0 ? e.C : (e.CT ? e.CT : e.C);
+    const int64_t cld = d.dir == 0 ? e.ld : (e.CT ? e.ldt : e.ld);
+    const double cscale = P.cost_kind == 0 ? 1.0 : P.cost_scale;
+    const double kd = cscale * P.inv_eps;
+    const float kh = (float)kd, kl = (float)(kd - (double)kh);
+    const int D = P.dim;
+    float rah[kRndRows], ral[kRndRows], rp[kRndRows][3];
+    DF xr[kRndRows], racc[kRndRows], tacc[kRndRows];
+    double rsum[kRndRows], tsum[kRndRows];
+    bool inf[kRndRows];
+    DF cmax = {0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < kRndRows; ++r) {
+      const int ir = warp * kRndRows + r;
+      const bool on = ir < t.ocount;
+      const int i = t.o0 + (on ? ir : 0);
+      rah[r] = on ? A.ah[d.off + i] : -INFINITY;
+      ral[r] = on ? A.al[d.off + i] : 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        rp[r][k] = (nj.coord_off >= 0 && k < D) ? A.coords[nj.coord_off + (int64_t)i * D + k] : 0.f;
+      if (PASS == 2) xr[r] = on ? df_of(A.xy[d.off + i]) : DF{0.f, 0.f};
+      racc[r] = tacc[r] = {0.f, 0.f};
+      rsum[r] = tsum[r] = 0.0;
+      inf[r] = false;
+    }
+    int step = 0;
+    for (int y0 = 0; y0 < nk.n; y0 += 32) {
+      const int y = y0 + lane;
+      const bool on = y < nk.n;
+      const float bh = on ? A.ah[d.rev_off + y] : -INFINITY;
+      const float bl = on ? A.al[d.rev_off + y] : 0.f;
+      float pb[3] = {0.f, 0.f, 0.f};
+      if (on && nk.coord_off >= 0)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          if (k < D) pb[k] = A.coords[nk.coord_off + (int64_t)y * D + k];
+      DF w = {0.f, 0.f};  // the column's factor: y (pass 3), err_c (pass 4)
+      if (PASS >= 3 && on) {
+        const double ycol = A.xy[d.rev_off + y];
+        // err_c = c - F''^T 1, F''^T 1 = y F'^T 1
+        w = df_of(PASS == 3 ? ycol : fmax(A.tgt[d.rev_off + y] - ycol * A.s2[d.rev_off + y], 0.0));
+      }
+      DF cs = {0.f, 0.f};
+      if (on) {
+#pragma unroll
+        for (int r = 0; r < kRndRows; ++r) {
+          const int ir = warp * kRndRows + r;
+          if (ir >= t.ocount) break;  // warp-uniform
+          const int i = t.o0 + ir;
+          DF c;
+          if (P.cost_kind == 0)
+            c = {own_rows ? Cm[(int64_t)i * cld + y] : Cm[(int64_t)y * cld + i], 0.f};
+          else
+            c = sq_dist_df(D, rp[r], pb);
+          if (PASS == 4) {
+            if (c.hi == INFINITY) {
+              if (w.hi > 0.f) inf[r] = true;
+              continue;
+            }
+            const DF a = {fabsf(c.hi), c.hi < 0.f ? -c.lo : c.lo};
+            if (a.hi > cmax.hi || (a.hi == cmax.hi && a.lo > cmax.lo)) cmax = a;
+            df_acc(tacc[r], df_mul(w, c));
+            continue;
+          }
+          float cu;
+          const float B = plan_entry(rah[r], ral[r], bh, bl, c, kh, kl, cu);
+          if (!(B > 0.f)) continue;  // also where the cost is +inf
+          if (PASS == 1) {
+            df_acc(racc[r], B);
+            df_acc(tacc[r], df_mul(B, c));
+            df_acc(cs, B);
+          } else if (PASS == 2) {
+            df_acc(cs, df_mul(B, xr[r]));
+          } else {
+            const DF b = df_mul(B, w);
+            df_acc(racc[r], b);
+            df_acc(tacc[r], df_mul(b, c));
+          }
+        }
+      }
+      if (PASS <= 2) {  // column sums: combined across the warps, one FP64 atomic per column
+        s_col[warp][lane] = make_float2(cs.hi, cs.lo);
+        __syncthreads();
+        if (warp == 0 && on) {
+          DF v = {0.f, 0.f};
+#pragma unroll
+          for (int q = 0; q < 8; ++q) df_acc(v, DF{s_col[q][lane].x, s_col[q][lane].y});
+          if (v.hi != 0.f) atomicAdd(PASS == 1 ? &A.rsum[d.rev_off + y] : &A.s2[d.rev_off + y], df_to(v));
+        }
+        __syncthreads();
+      }
+      if (PASS != 2 && ++step == kFlushCols) {
+        step = 0;
+#pragma unroll
+        for (int r = 0; r < kRndRows; ++r) {
+          if (PASS != 4) rsum[r] += df_to(racc[r]);
+          tsum[r] += df_to(tacc[r]);
+          racc[r] = tacc[r] = {0.f, 0.f};
+        }
+      }
+    }
+    if (PASS == 2) continue;
+    double tall = 0.0, msum = 0.0;
+#pragma unroll
+    for (int r = 0; r < kRndRows; ++r) {
+      const int ir = warp * kRndRows + r;
+      if (ir >= t.ocount) break;  // warp-uniform
+      double f = cscale;  // the row's factor, with the cost's scale
+      double x = 1.0;
+      if (PASS == 3) x = A.xy[d.off + t.o0 + ir];
+      if (PASS == 4) x = A.er[d.off + t.o0 + ir];
+      f *= x;
+      const double ts = warp_sum_d(tsum[r] + df_to(tacc[r]));
+      if (PASS == 4 && __any_sync(0xffffffffu, inf[r])) {
+        if (x > 0.0) tall += INFINITY;
+      } else if (f != 0.0) {
+        tall += f * ts;
+      }
+      if (PASS == 1 || PASS == 3) {
+        const double row = x * warp_sum_d(rsum[r] + df_to(racc[r]));
+        // each row belongs to one task
+        if (lane == 0) (PASS == 1 ? A.rsum : A.s2)[d.off + t.o0 + ir] = row;
+        msum += row;
+      }
+    }
+    double* acc = A.edge_acc + kRoundAcc * d.edge;
+    if (lane == 0 && tall != 0.0) atomicAdd(&acc[PASS == 1 ? 0 : PASS == 3 ? 1 : 2], tall);
+    if (PASS == 1 && lane == 0 && msum != 0.0) atomicAdd(&acc[5], msum);
+    if (PASS == 4) {
+      const double cm = warp_max_d(df_to(cmax) * cscale);
+      if (lane == 0 && cm > 0.0)
+        atomicMax((unsigned long long*)&acc[4], (unsigned long long)__double_as_longlong(cm));
+    }
+  }
+}
+
 // Per-point steps, one CTA row per directed edge (grid.y), points over grid.x.
 //   STEP 1 (every directed edge): target = the owner's marginal at unit mass (mu_o / sum mu_o,
 //          or the mean of o's plan marginals over the mean of its plans' masses); S side: x.
@@ -249,8 +435,10 @@ template <int PASS>
 void pass(const RoundArgs& a, bool f64, int grid, cudaStream_t s) {
   if (f64)
     round_pass_kernel<PASS, true><<<grid, 256, 0, s>>>(a);
-  else
+  else if constexpr (PASS == 5)
     round_pass_kernel<PASS, false><<<grid, 256, 0, s>>>(a);
+  else
+    round_pass_df_kernel<PASS><<<grid, 256, 0, s>>>(a);
 }
 
 template <int STEP>
