@@ -11,15 +11,19 @@
 //     out[t] = log sum_{r in R} exp( sum_j alpha_j in_j[t, r] )      (R empty: the sum itself)
 // The planner (host) turns one half-step of a colour into a few stages of such
 // ops -- all separators of the colour in each stage, the ops of a stage
-// independent -- and the op kernel runs a stage with one warp per output
-// (lanes over the reduced index) or, without reduced variables, one lane per
-// output.  With k_i the projection onto s n c_i of clique c_i's kernel, cost
+// independent -- and the op kernel runs a stage with a set of lanes per output
+// (over the reduced index) or, without reduced variables, one lane per output.  With k_i the projection onto s n c_i of clique c_i's kernel, cost
 // and its other separator's dual variable and factor m (s's own factor m_s
 // left out of every k_i, so that mu_gamma cancels in v_{l+1}; the same reading
 // as the FP64 oracle), the stages of a half-step are
 //   k_i;  q_2 = (k_1 + k_2)/2;  Pq_i = P_{s n c_i} q_{i-1}, q_i = ((i-1) Pq_i + k_i)/i  (i = 3..l);
 //   Pg = P_gamma q_l;  a_l = q_l - Pg (x) 1;  a_i = q_i + (a_{i+1} - Pq_{i+1}) (x) 1  (i = l-1..2);
 //   u_1 = a_2 - k_1,  u_i = a_i - k_i;   and for l = 1:  u_1 = -(P_gamma k_1) (x) 1.
+// Along a run i0 .. i1 of equal intersections the projections are the identity, so
+// the chain collapses to q_{i1} = ((i0 - 1) Pq_{i0} + k_{i0} + .. + k_{i1}) / i1 and
+// one a per run: the stages are per run, not per clique (every launch of these
+// small stages costs microseconds whatever it computes; a Wasserstein least
+// squares centre of 12 cliques took 36 stages, now 5).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -49,7 +53,9 @@ struct JtIn {
 };
 
 struct JtOp {
-  int32_t nt, nr, nin, pad;
+  int32_t nt, nr, nin;
+  int32_t lanes;  // threads per output: 1 without reduced variables, else 4 .. 32 or a CTA
+  int32_t wide;   // an index may reach 2^31
   int32_t dim[kJtMaxDims];
   int64_t tcount, rcount;
   double* out;  // row-major over the output dims (the last fastest)
@@ -75,6 +81,26 @@ __device__ __forceinline__ double jt_value(const JtOp& op, const int64_t* off) {
   return v;
 }
 
+// adds the offsets of index t over the op's dimensions [k0, k0 + n) (the last fastest)
+__device__ __forceinline__ void jt_offsets(const JtOp& op, int k0, int n, int64_t t, int64_t* off) {
+  if (n == 0) return;
+  if (op.wide) {  // sizes of 2^31 or more: 64-bit divisions
+    for (int k = k0 + n - 1; k >= k0; --k) {
+      const int64_t x = t % op.dim[k];
+      t /= op.dim[k];
+      for (int j = 0; j < op.nin; ++j) off[j] += x * op.in[j].stride[k];
+    }
+    return;
+  }
+  uint32_t rem = (uint32_t)t;
+  for (int k = k0 + n - 1; k > k0; --k) {
+    const uint32_t q = rem / (uint32_t)op.dim[k], x = rem - q * (uint32_t)op.dim[k];
+    rem = q;
+    for (int j = 0; j < op.nin; ++j) off[j] += x * op.in[j].stride[k];
+  }
+  for (int j = 0; j < op.nin; ++j) off[j] += rem * op.in[j].stride[k0];
+}
+
 __device__ __forceinline__ int jt_find(const int64_t* start, int32_t n, int64_t w) {
   int lo = 0, hi = n;  // start[0..n], start[0] = 0
   while (hi - lo > 1) {
@@ -84,69 +110,82 @@ __device__ __forceinline__ int jt_find(const int64_t* start, int32_t n, int64_t 
   return lo;
 }
 
-// one stage of ops; start[o] = the first work unit of op o (a warp per output
-// when the op reduces, a lane per output otherwise), start[nops] = the total
+// one stage of ops; start[o] = the first CTA of op o, start[nops] = the total.  A CTA takes 256 / op.lanes
+// outputs.  The reduction needs one exponential per term and one more per lane: the lanes' maxima meet before
+// their sums do (merging (max, sum) pairs took two FP64 exponentials per shuffle step, most of a stage's
+// time at 1.6 FP64 lanes per clock and SM).
 __global__ void __launch_bounds__(32 * kJtWarps) jt_op_kernel(const JtOp* ops, const int64_t* start, int32_t nops) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * kJtWarps + (threadIdx.x >> 5);
-  if (w >= start[nops]) return;
-  const JtOp& op = ops[jt_find(start, nops, w)];
-  const int64_t unit = w - start[jt_find(start, nops, w)];
-  int64_t t = unit;
-  if (op.rcount == 1) {  // no reduction: one output per lane
-    t = unit * 32 + lane;
-    if (t >= op.tcount) return;
-  }
+  __shared__ double red[2][kJtWarps];
+  const int64_t b = blockIdx.x;
+  const int o = jt_find(start, nops, b);
+  const JtOp& op = ops[o];
+  const int L = op.lanes, sub = threadIdx.x & (L - 1);
+  const int64_t t = (b - start[o]) * (32 * kJtWarps / L) + threadIdx.x / L;
+  const bool on = t < op.tcount;  // the same for all lanes of an output
   int64_t base[kJtMaxIn];
   for (int j = 0; j < kJtMaxIn; ++j) base[j] = 0;
-  int64_t rem = t;
-  for (int k = op.nt - 1; k >= 0; --k) {
-    const int64_t x = rem % op.dim[k];
-    rem /= op.dim[k];
-    for (int j = 0; j < op.nin; ++j) base[j] += x * op.in[j].stride[k];
-  }
-  if (op.rcount == 1) {
-    op.out[t] = jt_value(op, base);
+  jt_offsets(op, 0, op.nt, on ? t : 0, base);
+  if (L == 1) {
+    if (on) op.out[t] = jt_value(op, base);
     return;
   }
   double m = -INFINITY, s = 0.0;
-  for (int64_t r = lane; r < op.rcount; r += 32) {
-    int64_t off[kJtMaxIn];
-    for (int j = 0; j < kJtMaxIn; ++j) off[j] = base[j];
-    int64_t rr = r;
-    for (int k = op.nr - 1; k >= 0; --k) {
-      const int64_t x = rr % op.dim[op.nt + k];
-      rr /= op.dim[op.nt + k];
-      for (int j = 0; j < op.nin; ++j) off[j] += x * op.in[j].stride[op.nt + k];
+  if (on)
+    for (int64_t r = sub; r < op.rcount; r += L) {
+      int64_t off[kJtMaxIn];
+      for (int j = 0; j < kJtMaxIn; ++j) off[j] = base[j];
+      jt_offsets(op, op.nt, op.nr, r, off);
+      const double v = jt_value(op, off);
+      if (v > m) {
+        s = s * exp(m - v) + 1.0;  // (m = -inf: s = 0)
+        m = v;
+      } else if (v > -INFINITY) {
+        s += exp(v - m);
+      }
     }
-    const double v = jt_value(op, off);
-    if (v > m) {
-      s = s * exp(m - v) + 1.0;  // (m = -inf: s = 0)
-      m = v;
-    } else if (v > -INFINITY) {
-      s += exp(v - m);
-    }
+  double M = m;
+  const int w = L < 32 ? L : 32;
+  for (int d = w >> 1; d > 0; d >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, d));
+  const int warp = threadIdx.x >> 5;
+  if (L > 32) {  // block-uniform: the CTA holds one output
+    if ((threadIdx.x & 31) == 0) red[0][warp] = M;
+    __syncthreads();
+    for (int q = 0; q < kJtWarps; ++q) M = fmax(M, red[0][q]);
   }
-  for (int o = 16; o > 0; o >>= 1) {  // merge the lanes' (max, sum) pairs
-    const double m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
-    const double M = fmax(m, m2);
-    if (M > -INFINITY) {
-      s = (m > -INFINITY ? s * exp(m - M) : 0.0) + (m2 > -INFINITY ? s2 * exp(m2 - M) : 0.0);
-      m = M;
-    }
+  s = m > -INFINITY ? (m == M ? s : s * exp(m - M)) : 0.0;
+  for (int d = w >> 1; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  if (L > 32) {
+    if ((threadIdx.x & 31) == 0) red[1][warp] = s;
+    __syncthreads();
+    s = 0.0;
+    for (int q = 0; q < kJtWarps; ++q) s += red[1][q];
   }
-  if (lane == 0) op.out[t] = m > -INFINITY ? m + log(s) : -INFINITY;
+  if (sub == 0 && on) op.out[t] = M > -INFINITY ? M + log(s) : -INFINITY;
 }
 
-// sums over tensors into slots; one CTA per (item, 8192-entry block)
+// exp of one op without reduced variables (a clique's plan from its log terms)
+__global__ void __launch_bounds__(256) jt_plan_kernel(const JtOp* op, double* out) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < op->tcount;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    int64_t base[kJtMaxIn];
+    for (int j = 0; j < kJtMaxIn; ++j) base[j] = 0;
+    jt_offsets(*op, 0, op->nt, t, base);
+    out[t] = exp(jt_value(*op, base));
+  }
+}
+
+constexpr int kJtSumBlock = 1024;  // entries per CTA of the sums
+
+
+// sums over tensors into slots; one CTA per (item, block of kJtSumBlock entries)
 __global__ void __launch_bounds__(256) jt_sum_kernel(const JtSum* items, const int64_t* start, int32_t nitems,
                                                      double* slots) {
   __shared__ double red[8];
   if ((int64_t)blockIdx.x >= start[nitems]) return;
   const int it = jt_find(start, nitems, blockIdx.x);
   const JtSum& q = items[it];
-  const int64_t i0 = (blockIdx.x - start[it]) * 8192;
-  const int64_t i1 = min(q.n, i0 + 8192);
+  const int64_t i0 = (blockIdx.x - start[it]) * kJtSumBlock;
+  const int64_t i1 = min(q.n, i0 + kJtSumBlock);
   double acc = 0.0;
   for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) {
     const double ea = exp(q.a[i]);
@@ -174,11 +213,6 @@ __global__ void jt_residual_finish_kernel(const double* slots, const int32_t* co
   }
   out[0] = sum;
   out[1] = mx;
-}
-
-__global__ void jt_exp_kernel(const double* a, double* out, int64_t n) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = exp(a[i]);
 }
 
 }  // namespace
@@ -322,6 +356,7 @@ JtOp make_op(const tree_ot_jt_handle* h, const Tensor& out, const std::vector<in
     op.dim[k] = h->vsize[dims[k]];
     (k < op.nt ? op.tcount : op.rcount) *= op.dim[k];
   }
+  op.wide = op.tcount >= (int64_t(1) << 31) || op.rcount >= (int64_t(1) << 31) ? 1 : 0;
   op.out = reinterpret_cast<double*>((intptr_t)out.off);
   for (int j = 0; j < op.nin; ++j) {
     const Src& s = ins[j];
@@ -361,8 +396,16 @@ int upload_stage(tree_ot_jt_handle* h, Stage& st, cudaStream_t s) {
   std::vector<int64_t> start(st.ops.size() + 1, 0);
   for (size_t o = 0; o < st.ops.size(); ++o) {
     resolve(h, st.ops[o]);
-    const JtOp& op = st.ops[o];
-    start[o + 1] = start[o] + (op.rcount == 1 ? (op.tcount + 31) / 32 : op.tcount);
+    JtOp& op = st.ops[o];
+    // threads per output: enough for the reduction, a CTA where few outputs reduce over much
+    op.lanes = 1;
+    if (op.rcount > 1) {
+      op.lanes = 4;
+      while (op.lanes < 32 && op.lanes < op.rcount) op.lanes *= 2;
+      if (op.rcount >= 128 && op.tcount <= 2048) op.lanes = 32 * kJtWarps;
+    }
+    const int64_t per = 32 * kJtWarps / op.lanes;
+    start[o + 1] = start[o] + (op.tcount + per - 1) / per;
   }
   st.units = start.back();
   JT_TRY(jt_alloc(h, &st.d_ops, (int64_t)st.ops.size()));
@@ -376,15 +419,14 @@ int upload_stage(tree_ot_jt_handle* h, Stage& st, cudaStream_t s) {
 
 int run_stage(const Stage& st, cudaStream_t s) {
   if (st.ops.empty() || st.units == 0) return TREE_OT_OK;
-  const int64_t blocks = (st.units + kJtWarps - 1) / kJtWarps;
-  jt_op_kernel<<<(unsigned)blocks, 32 * kJtWarps, 0, s>>>(st.d_ops, st.d_start, (int32_t)st.ops.size());
+  jt_op_kernel<<<(unsigned)st.units, 32 * kJtWarps, 0, s>>>(st.d_ops, st.d_start, (int32_t)st.ops.size());
   return jt_cuda(cudaGetLastError(), "junction-tree op launch");
 }
 
 int upload_sums(tree_ot_jt_handle* h, const std::vector<JtSum>& items, JtSum** d_items, int64_t** d_start,
                 int64_t* blocks, cudaStream_t s) {
   std::vector<int64_t> start(items.size() + 1, 0);
-  for (size_t i = 0; i < items.size(); ++i) start[i + 1] = start[i] + (items[i].n + 8191) / 8192;
+  for (size_t i = 0; i < items.size(); ++i) start[i + 1] = start[i] + (items[i].n + kJtSumBlock - 1) / kJtSumBlock;
   *blocks = start.back();
   JT_TRY(jt_alloc(h, d_items, (int64_t)items.size()));
   JT_TRY(jt_alloc(h, d_start, (int64_t)start.size()));
@@ -402,11 +444,12 @@ void plan_half_step(tree_ot_jt_handle* h, int colour, std::vector<Stage>& stages
     int32_t s, l;
     std::vector<std::vector<int32_t>> sets;
     std::vector<int32_t> g;
-    std::vector<Tensor> k, q, Pq, a;
+    std::vector<int32_t> end;            // per run of equal intersections: cliques up to its end
+    std::vector<Tensor> k, q, Pq, a;     // q, Pq, a per run
     Tensor Pg;
   };
   std::vector<SepWork> work;
-  int32_t lmax = 1;
+  size_t runs = 1;
   for (int32_t s = 0; s < h->nsep; ++s) {
     if (h->colour[s] != colour) continue;
     SepWork w;
@@ -414,21 +457,15 @@ void plan_half_step(tree_ot_jt_handle* h, int colour, std::vector<Stage>& stages
     w.l = (int32_t)h->scl[s].size();
     for (int32_t c : h->scl[s]) w.sets.push_back(inter(h->svars[s], h->cvars[c]));
     w.g = h->sgamma[s];
-    lmax = std::max(lmax, w.l);
-    work.push_back(std::move(w));
-  }
-  // temporaries
-  for (SepWork& w : work) {
-    for (int i = 0; i < w.l; ++i) w.k.push_back(new_tensor(h, w.sets[i]));
-    w.q.resize(w.l + 1);
-    w.Pq.resize(w.l + 1);
-    w.a.resize(w.l + 1);
-    for (int i = 2; i <= w.l; ++i) {
-      w.q[i] = new_tensor(h, w.sets[i - 1]);
-      if (i >= 3) w.Pq[i] = new_tensor(h, w.sets[i - 1]);
-      w.a[i] = new_tensor(h, w.sets[i - 1]);
+    for (int i = 0; i < w.l; ++i) {
+      w.k.push_back(new_tensor(h, w.sets[i]));
+      if (i > 0 && w.sets[i] == w.sets[i - 1])
+        w.end.back() = i + 1;
+      else
+        w.end.push_back(i + 1);
     }
-    w.Pg = new_tensor(h, w.g);
+    runs = std::max(runs, w.end.size());
+    work.push_back(std::move(w));
   }
   auto minus = [](const std::vector<int32_t>& a, const std::vector<int32_t>& b) {
     std::vector<int32_t> out;
@@ -451,45 +488,88 @@ void plan_half_step(tree_ot_jt_handle* h, int colour, std::vector<Stage>& stages
       sk.ops.push_back(make_op(h, w.k[i], minus(h->cvars[c], w.sets[i]), ins));
     }
   stages.push_back(std::move(sk));
-  // the geometric chain
-  {
-    Stage st;
-    for (SepWork& w : work)
-      if (w.l >= 2) st.ops.push_back(make_op(h, w.q[2], {}, {src(w.k[0], 0.5), src(w.k[1], 0.5)}));
-    stages.push_back(std::move(st));
+  // the geometric chain, run by run: q = ((i0 - 1) Pq + k_i0 + .. + k_i1) / i1, sums of more than an op's
+  // inputs in rounds of partial sums
+  for (SepWork& w : work) {
+    w.q.resize(w.end.size());
+    w.Pq.resize(w.end.size());
+    w.a.resize(w.end.size());
   }
-  for (int i = 3; i <= lmax; ++i) {
-    Stage sp, sq;
-    for (SepWork& w : work) {
-      if (w.l < i) continue;
-      sp.ops.push_back(make_op(h, w.Pq[i], minus(w.sets[i - 2], w.sets[i - 1]), {src(w.q[i - 1], 1.0)}));
-      sq.ops.push_back(make_op(h, w.q[i], {}, {src(w.Pq[i], (i - 1.0) / i), src(w.k[i - 1], 1.0 / i)}));
+  for (size_t r = 0; r < runs; ++r) {
+    Stage sp;
+    std::vector<std::vector<Src>> terms(work.size());
+    std::deque<Tensor> partial;  // stable addresses: terms point at their variables
+    for (size_t n = 0; n < work.size(); ++n) {
+      SepWork& w = work[n];
+      if (r >= w.end.size()) continue;
+      const int32_t i0 = r ? w.end[r - 1] : 0, i1 = w.end[r];
+      if (i1 == 1) {  // a single clique: q_1 = k_1
+        w.q[r] = w.k[0];
+        continue;
+      }
+      if (r) {
+        w.Pq[r] = new_tensor(h, w.sets[i0]);
+        sp.ops.push_back(make_op(h, w.Pq[r], minus(w.sets[i0 - 1], w.sets[i0]), {src(w.q[r - 1], 1.0)}));
+        terms[n].push_back(src(w.Pq[r], (double)i0 / i1));
+      }
+      for (int32_t i = i0; i < i1; ++i) terms[n].push_back(src(w.k[i], 1.0 / i1));
     }
     stages.push_back(std::move(sp));
-    stages.push_back(std::move(sq));
+    for (bool more = true; more;) {
+      Stage st;
+      more = false;
+      for (size_t n = 0; n < work.size(); ++n) {
+        SepWork& w = work[n];
+        std::vector<Src>& in = terms[n];
+        if (in.empty()) continue;
+        if ((int)in.size() <= kJtMaxIn) {
+          w.q[r] = new_tensor(h, w.sets[w.end[r] - 1]);
+          st.ops.push_back(make_op(h, w.q[r], {}, in));
+          in.clear();
+          continue;
+        }
+        std::vector<Src> next;
+        for (size_t k = 0; k < in.size(); k += kJtMaxIn) {
+          partial.push_back(new_tensor(h, w.sets[w.end[r] - 1]));
+          st.ops.push_back(make_op(h, partial.back(), {},
+                                   std::vector<Src>(in.begin() + k, in.begin() + std::min(in.size(), k + kJtMaxIn))));
+          next.push_back(src(partial.back(), 1.0));
+        }
+        in = std::move(next);
+        more = true;
+      }
+      stages.push_back(std::move(st));
+    }
   }
-  // P_gamma of q_l (or of k_1 when l = 1)
+  // P_gamma of q_l (or of k_1 when l = 1): q_l itself when gamma is the whole intersection
   {
     Stage st;
     for (SepWork& w : work) {
-      const Tensor& top = w.l >= 2 ? w.q[w.l] : w.k[0];
+      const Tensor& top = w.q.back();
+      if (top.vars == w.g) {
+        w.Pg = top;
+        continue;
+      }
+      w.Pg = new_tensor(h, w.g);
       st.ops.push_back(make_op(h, w.Pg, minus(top.vars, w.g), {src(top, 1.0)}));
     }
     stages.push_back(std::move(st));
   }
-  // a_l, then down the chain
-  {
-    Stage st;
-    for (SepWork& w : work)
-      if (w.l >= 2) st.ops.push_back(make_op(h, w.a[w.l], {}, {src(w.q[w.l], 1.0), src(w.Pg, -1.0)}));
-    stages.push_back(std::move(st));
-  }
-  for (int down = 1; down <= lmax - 2; ++down) {
+  // a per run, from the last (which the new duals form themselves: a = q_l - Pg) down
+  for (size_t down = 1; down < runs; ++down) {
     Stage st;
     for (SepWork& w : work) {
-      const int i = w.l - down;
-      if (i < 2) continue;
-      st.ops.push_back(make_op(h, w.a[i], {}, {src(w.q[i], 1.0), src(w.a[i + 1], 1.0), src(w.Pq[i + 1], -1.0)}));
+      if (w.end.size() <= down) continue;
+      const size_t r = w.end.size() - 1 - down;
+      w.a[r] = new_tensor(h, w.sets[w.end[r] - 1]);
+      std::vector<Src> in = {src(w.q[r], 1.0), src(w.Pq[r + 1], -1.0)};
+      if (down == 1) {
+        in.push_back(src(w.q[r + 1], 1.0));
+        in.push_back(src(w.Pg, -1.0));
+      } else {
+        in.push_back(src(w.a[r + 1], 1.0));
+      }
+      st.ops.push_back(make_op(h, w.a[r], {}, in));
     }
     stages.push_back(std::move(st));
   }
@@ -502,9 +582,16 @@ void plan_half_step(tree_ot_jt_handle* h, int colour, std::vector<Stage>& stages
         st.ops.push_back(make_op(h, u[0], {}, {src(w.Pg, -1.0)}));
         continue;
       }
-      st.ops.push_back(make_op(h, u[0], {}, {src(w.a[2], 1.0), src(w.k[0], -1.0)}));
-      for (int i = 2; i <= w.l; ++i)
-        st.ops.push_back(make_op(h, u[i - 1], {}, {src(w.a[i], 1.0), src(w.k[i - 1], -1.0)}));
+      for (size_t r = 0; r < w.end.size(); ++r)
+        for (int32_t i = r ? w.end[r - 1] : 0; i < w.end[r]; ++i) {
+          std::vector<Src> in;
+          if (r + 1 == w.end.size())
+            in = {src(w.q[r], 1.0), src(w.Pg, -1.0)};
+          else
+            in = {src(w.a[r], 1.0)};
+          in.push_back(src(w.k[i], -1.0));
+          st.ops.push_back(make_op(h, u[i], {}, in));
+        }
     }
     stages.push_back(std::move(st));
   }
@@ -758,9 +845,19 @@ int tree_ot_jt_reset(tree_ot_jt_handle* h, void* cuda_stream) {
   set_last_error("");
   if (!h) return jt_fail(TREE_OT_ERR_ARG, "handle is NULL");
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  // the duals, a memset per stretch of neighbours in the arena (one: they are planned first)
+  int64_t b = 0, e = 0;
   for (auto& ds : h->dual)
-    for (const Tensor& t : ds)
-      JT_TRY(jt_cuda(cudaMemsetAsync(h->d_arena + t.off, 0, sizeof(double) * (size_t)t.size, s), "memset"));
+    for (const Tensor& t : ds) {
+      if (t.off == e) {
+        e += t.size;
+        continue;
+      }
+      if (e > b) JT_TRY(jt_cuda(cudaMemsetAsync(h->d_arena + b, 0, sizeof(double) * (size_t)(e - b), s), "memset"));
+      b = t.off;
+      e = b + t.size;
+    }
+  if (e > b) JT_TRY(jt_cuda(cudaMemsetAsync(h->d_arena + b, 0, sizeof(double) * (size_t)(e - b), s), "memset"));
   h->hs = 0;
   return TREE_OT_OK;
 }
@@ -862,10 +959,9 @@ int tree_ot_jt_plan(tree_ot_jt_handle* h, void* cuda_stream, int32_t clique, dou
   set_last_error("");
   if (!h || !plan_out || clique < 0 || clique >= h->ncl) return jt_fail(TREE_OT_ERR_ARG, "bad handle or clique");
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  JT_TRY(run_stage(h->res_stages[0], s));  // every clique's log plan
   const Tensor& t = h->logplan[clique];
   const int blocks = (int)std::min<int64_t>((t.size + 255) / 256, 4096);
-  jt_exp_kernel<<<blocks, 256, 0, s>>>(h->d_arena + t.off, h->d_tmp, t.size);
+  jt_plan_kernel<<<blocks, 256, 0, s>>>(h->res_stages[0].d_ops + clique, h->d_tmp);
   JT_TRY(jt_cuda(cudaGetLastError(), "plan launch"));
   JT_TRY(jt_cuda(cudaMemcpyAsync(plan_out, h->d_tmp, sizeof(double) * (size_t)t.size, cudaMemcpyDeviceToHost, s),
                  "read plan"));
