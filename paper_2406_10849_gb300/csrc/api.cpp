@@ -214,7 +214,8 @@ struct tree_ot_handle {
   DEdgeD* d_dedges = nullptr;
   int32_t* d_node_dedges = nullptr;
   Task* d_tasks[2] = {nullptr, nullptr};
-  NodeChunk* d_chunks[2] = {nullptr, nullptr};
+  NodeChunkD* d_chunks[2] = {nullptr, nullptr};
+  OwnedDEdge* d_owned = nullptr;           // directed edges by owner
   Task* d_check_tasks = nullptr;
   Task* d_btasks[2] = {nullptr, nullptr};
   int32_t* d_queue = nullptr;              // [colour][slot][2] work-queue counters
@@ -482,7 +483,7 @@ NodeArgs node_args(tree_ot_handle* h, int colour, bool retire) {
   a.colour = colour;
   a.nodes = h->d_nodes;
   a.dedges = h->d_dedges;
-  a.node_dedges = h->d_node_dedges;
+  a.owned = h->d_owned;
   a.probs = h->d_probs;
   a.nprob = h->nprob;
   a.done = h->d_done;
@@ -1922,7 +1923,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       (rc = h->alloc(&h->d_node_dedges, (int64_t)h->node_dedges.size())) ||
       (rc = h->alloc(&h->d_tasks[0], h->task_cap[0])) || (rc = h->alloc(&h->d_tasks[1], h->task_cap[1])) ||
       (rc = h->alloc(&h->d_queue, 2 * 2 * kApplySlots)) ||
-      (rc = h->alloc(&h->d_chunks[0], (int64_t)h->chunks[0].size())) ||
+      (rc = h->alloc(&h->d_owned, (int64_t)h->node_dedges.size())) || (rc = h->alloc(&h->d_chunks[0], (int64_t)h->chunks[0].size())) ||
       (rc = h->alloc(&h->d_chunks[1], (int64_t)h->chunks[1].size())) ||
       (rc = h->alloc(&h->d_check_tasks, (int64_t)h->check_tasks.size())) || (rc = h->alloc(&h->d_f, h->vec_len)) ||
       (rc = h->alloc(&h->d_fr, h->vec_len)) || (rc = h->alloc(&h->d_hh, h->vec_len)) ||
@@ -2095,6 +2096,16 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     }
   }
   // plan tables
+  std::vector<OwnedDEdge> owned;
+  for (int32_t di : h->node_dedges) owned.push_back(OwnedDEdge{h->dedges[di], di, 0});
+  std::vector<NodeChunkD> crec[2];
+  for (int c = 0; c < 2; ++c)
+    for (const NodeChunk& k : h->chunks[c]) {
+      const NodeD& nd = h->nodes[k.node];
+      const ProbD& pd = h->probs[nd.prob];
+      crec[c].push_back(NodeChunkD{k.node, k.chunk, k.x0, k.cnt, nd, pd.eps, pd.inv_eps, pd.cost_kind,
+                                   pd.nodes_in_colour[c]});
+    }
   if ((rc = up(h->d_probs, h->probs.data(), sizeof(ProbD) * h->probs.size())) ||
       (rc = up(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size())) ||
       (rc = up(h->d_edges, h->edges.data(), sizeof(EdgeD) * h->edges.size())) ||
@@ -2102,8 +2113,9 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       (rc = up(h->d_node_dedges, h->node_dedges.data(), sizeof(int32_t) * h->node_dedges.size())) ||
       (rc = up(h->d_tasks[0], h->tasks[0].data(), sizeof(Task) * h->tasks[0].size())) ||
       (rc = up(h->d_tasks[1], h->tasks[1].data(), sizeof(Task) * h->tasks[1].size())) ||
-      (rc = up(h->d_chunks[0], h->chunks[0].data(), sizeof(NodeChunk) * h->chunks[0].size())) ||
-      (rc = up(h->d_chunks[1], h->chunks[1].data(), sizeof(NodeChunk) * h->chunks[1].size())) ||
+      (rc = up(h->d_owned, owned.data(), sizeof(OwnedDEdge) * owned.size())) ||
+      (rc = up(h->d_chunks[0], crec[0].data(), sizeof(NodeChunkD) * crec[0].size())) ||
+      (rc = up(h->d_chunks[1], crec[1].data(), sizeof(NodeChunkD) * crec[1].size())) ||
       (rc = up(h->d_check_tasks, h->check_tasks.data(), sizeof(Task) * h->check_tasks.size())))
     return bail(rc);
   if (h->lowp && ((rc = up(h->d_btasks[0], h->btasks[0].data(), sizeof(Task) * h->btasks[0].size())) ||
@@ -2135,31 +2147,28 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       h->node_defer[c] = false;
     else
       h->node_defer[c] = (int64_t)h->chunks[c].size() > 4 * (int64_t)sms;
-    // per problem: the colour's owned directed edges, then its free nodes
+    // per problem the colour's owned directed edges; then the colour's free nodes
     const int32_t np = h->nprob;
-    std::vector<std::vector<int32_t>> dl(np), nl(np);
+    std::vector<std::vector<int32_t>> dl(np);
+    std::vector<int32_t> fn;
     for (size_t j = 0; j < h->nodes.size(); ++j) {
       const NodeD& nd = h->nodes[j];
       if (nd.colour != c) continue;
       for (int32_t i = 0; i < nd.deg; ++i) dl[nd.prob].push_back(h->node_dedges[nd.dedge_begin + i]);
-      if (!nd.fixed) nl[nd.prob].push_back((int32_t)j);
+      if (!nd.fixed) fn.push_back((int32_t)j);
     }
-    // one array: dbeg [np + 1], dedges, nbeg [np + 1], nodes
+    // one array: dbeg [np + 1], dedges, nodes
     std::vector<int32_t> buf(np + 1, 0);
     for (int32_t p = 0; p < np; ++p) {
       buf[p + 1] = buf[p] + (int32_t)dl[p].size();
       buf.insert(buf.end(), dl[p].begin(), dl[p].end());
     }
     const size_t nb = buf.size();
-    buf.resize(nb + np + 1, 0);
-    for (int32_t p = 0; p < np; ++p) {
-      buf[nb + p + 1] = buf[nb + p] + (int32_t)nl[p].size();
-      buf.insert(buf.end(), nl[p].begin(), nl[p].end());
-    }
+    buf.insert(buf.end(), fn.begin(), fn.end());
     if ((rc = h->alloc(&h->d_fin[c], (int64_t)buf.size())) ||
         (rc = up(h->d_fin[c], buf.data(), sizeof(int32_t) * buf.size())))
       return bail(rc);
-    h->fin[c] = FinishList{h->d_fin[c], h->d_fin[c] + (np + 1), h->d_fin[c] + nb, h->d_fin[c] + nb + (np + 1)};
+    h->fin[c] = FinishList{h->d_fin[c], h->d_fin[c] + (np + 1), h->d_fin[c] + nb, (int32_t)fn.size()};
   }
   {
     cudaError_t ce = cudaStreamCreateWithFlags(&h->hstream, cudaStreamNonBlocking);

@@ -85,8 +85,8 @@ __device__ __forceinline__ int node_item(const ForestArgs& F, const NodeArgs& N,
                                          unsigned char* node_sm, double* red) {
   __shared__ int s_go;
   const int tid = threadIdx.x;
-  const NodeChunk c = N.chunks[idx];
-  const int p = N.nodes[c.node].prob;
+  const NodeChunkD c = N.chunks[idx];
+  const int p = c.nd.prob;
   if (tid == 0) {
     const int32_t* cnt = F.cnt + 4 * p;
     int go = 1;

@@ -99,6 +99,20 @@ struct NodeChunk {
   int32_t node, chunk, x0, cnt;
 };
 
+// A chunk with its node and what the update reads of its problem, resolved on
+// the host: one load instead of the chain chunk -> node -> problem.
+struct NodeChunkD {
+  int32_t node, chunk, x0, cnt;
+  NodeD nd;
+  double eps, inv_eps;
+  int32_t cost_kind, in_colour;  // in_colour: the problem's nodes of this colour
+};
+// A directed edge in the order of its owner's list, with its own index
+struct OwnedDEdge {
+  DEdgeD d;
+  int32_t di, pad;
+};
+
 // Node update: points per CTA for a node of n points and degree deg, so that a
 // CTA holds at most `pairs` (edge, point) pairs (a multiple of 32 points when
 // that is at least 32, and at least one point).
@@ -282,13 +296,13 @@ struct AbsorbArgs {
 // h[d] = (f'/eps + log gamma_owner) * log2(e); the apply therefore returns the
 // message plus Z of the neighbour, which the node update subtracts.
 struct NodeArgs {
-  const NodeChunk* chunks;   // CTAs of this launch: (node, chunk) pairs of the colour
+  const NodeChunkD* chunks;  // CTAs of this launch: (node, chunk) pairs of the colour
   int32_t nchunks;
   uint32_t smem;             // dynamic shared memory per CTA (the largest chunk of the colour)
   int32_t colour;
   const NodeD* nodes;
   const DEdgeD* dedges;
-  const int32_t* node_dedges;
+  const OwnedDEdge* owned;   // directed edges by owner: owned[dedge_begin .. dedge_begin + deg)
   const ProbD* probs;
   int32_t nprob;
   int32_t* done;
@@ -339,14 +353,14 @@ struct NodeArgs {
   const FixedChunkD* fixed;  // per chunk of a fixed-leaf launch with deferred bookkeeping (or null)
 };
 
-// Per problem, what node_finish_kernel reads for one colour: the directed
-// edges owned by the colour's nodes (dedges[dbeg[p] .. dbeg[p+1])) and its
-// free nodes (nodes[nbeg[p] .. nbeg[p+1])).
+// What node_finish_kernel reads for one colour: per problem the directed edges
+// owned by the colour's nodes (dedges[dbeg[p] .. dbeg[p+1])), and the colour's
+// free nodes.
 struct FinishList {
   const int32_t* dbeg;
   const int32_t* dedges;
-  const int32_t* nbeg;
-  const int32_t* nodes;
+  const int32_t* nodes;  // the colour's free nodes of all problems
+  int32_t nnodes;
 };
 
 // FP64-grade check of the current potentials.  Per element the exponent

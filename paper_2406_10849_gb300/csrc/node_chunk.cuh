@@ -158,8 +158,9 @@ struct PairWalk {
 };
 
 // FP64 handles: three passes over the chunk's pairs / points in double
-__device__ void chunk_update64(const NodeArgs& A, const NodeD& nd, const NodeChunk& c, const ProbD& P, double* red,
-                               unsigned char* sm, int node_id) {
+__device__ void chunk_update64(const NodeArgs& A, const NodeChunkD& c, double* red, unsigned char* sm) {
+  const NodeD& nd = c.nd;
+  const int node_id = c.node;
   using Q = double;
   const int deg = nd.deg, cnt = c.cnt, np = deg * cnt;
   const NodeSmem L = node_smem_layout(deg, cnt, true);
@@ -174,11 +175,10 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeD& nd, const NodeChu
   Q* s_qb = reinterpret_cast<Q*>(sm + L.qb);
   const int tid = threadIdx.x, lane = tid & 31;
   for (int i = tid; i < deg; i += kNodeThreads) {
-    const int di = A.node_dedges[nd.dedge_begin + i];
-    const DEdgeD d = A.dedges[di];
-    s_de[i] = d;
-    s_zn[i] = A.Z[d.nbr];
-    s_di[i] = di;
+    const OwnedDEdge o = A.owned[nd.dedge_begin + i];
+    s_de[i] = o.d;
+    s_zn[i] = A.Z[o.d.nbr];
+    s_di[i] = o.di;
     s_dr[i] = 0;
     s_r[i] = Q(0);
   }
@@ -198,8 +198,8 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeD& nd, const NodeChu
       const double lg = A.logg[nd.node_off + x];
       const double mu = A.mu[nd.node_off + x];
       // stopping term mu |exp(f/eps + m) - 1| of the previous iterate
-      if (mu > 0.0) r += fabs(mu * exp(fo * P.inv_eps + mi) - mu);
-      A.f[d.off + x] = -P.eps * mi;
+      if (mu > 0.0) r += fabs(mu * exp(fo * c.inv_eps + mi) - mu);
+      A.f[d.off + x] = -c.eps * mi;
       float hi, lo;
       if (lg == -INFINITY) {
         hi = -INFINITY;
@@ -229,7 +229,7 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeD& nd, const NodeChu
       const double mi = merge_pair64(A, d, nd.n, x, s_zn[w.i]);
       s_mi[q] = mi;
       const double fo = A.f[d.off + x];
-      s_q[q] = exp((fo * P.inv_eps - Zold) + mi);
+      s_q[q] = exp((fo * c.inv_eps - Zold) + mi);
     }
   }
   __syncthreads();
@@ -268,7 +268,7 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeD& nd, const NodeChu
         const double mi = s_mi[q];
         r = s_q[q] > s_qb[w.xi] ? s_q[q] - s_qb[w.xi] : s_qb[w.xi] - s_q[q];
         const double g = s_s[w.xi] - mi;
-        A.f[d.off + x] = P.eps * g;
+        A.f[d.off + x] = c.eps * g;
         float hi, lo;
         split2(g * kLog2e, hi, lo);
         A.hh[d.off + x] = hi;
@@ -555,7 +555,7 @@ __device__ __forceinline__ void fixed_chunk_fast(const NodeArgs& A, const FixedC
 // pieces per message, as outside the phase, it gained little and its registers
 // would weigh on every other handle's node update.)
 template <int DEG, bool ONE>
-__device__ __forceinline__ void free_points32(const NodeArgs& A, const NodeD& nd, const NodeChunk& c, double* red,
+__device__ __forceinline__ void free_points32(const NodeArgs& A, const NodeD& nd, const NodeChunkD& c, double* red,
                                               const DEdgeD* s_de, const float2* s_zk, int* s_dr, float* s_r,
                                               const SkEdgeS* s_sk, float2* s_s, bool track, float2 zo, bool& bad) {
   constexpr bool one_piece = ONE;  // the shared-kernel phase: one sum per output
@@ -628,8 +628,9 @@ __device__ __forceinline__ void free_points32(const NodeArgs& A, const NodeD& nd
 // PM: the kernel carries the point-major form for the shared-kernel phase
 // (handles with shared-kernel groups; it needs more registers than the rest)
 template <bool FIXED_ONLY, bool PM = false>
-__device__ void chunk_update32(const NodeArgs& A, const NodeD& nd, const NodeChunk& c, const ProbD& P, double* red,
-                               unsigned char* sm, int node_id) {
+__device__ void chunk_update32(const NodeArgs& A, const NodeChunkD& c, double* red, unsigned char* sm) {
+  const NodeD& nd = c.nd;
+  const int node_id = c.node;
   const int deg = nd.deg, cnt = c.cnt, np = deg * cnt;
   const NodeSmem L = node_smem_layout(deg, cnt, false);
   DEdgeD* s_de = reinterpret_cast<DEdgeD*>(sm + L.de);
@@ -647,13 +648,13 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeD& nd, const NodeChu
   // fix-up's piece); drift from an absorbed base is tracked on stored-cost
   // problems, the only ones absorbed
   const int lp = A.absorbed ? A.lowp[nd.prob] : 0;
-  const bool track = lp == 1 && P.cost_kind == 0;
-  const bool one_piece = lp == 1 && P.cost_kind != 0 && A.sk_ref;
+  const bool track = lp == 1 && c.cost_kind == 0;
+  const bool one_piece = lp == 1 && c.cost_kind != 0 && A.sk_ref;
   for (int i = tid; i < deg; i += kNodeThreads) {
-    const int di = A.node_dedges[nd.dedge_begin + i];
-    const DEdgeD d = A.dedges[di];
-    s_de[i] = d;
-    s_zk[i] = split_l2(A.Z[d.nbr] * kLog2e);
+    const OwnedDEdge o = A.owned[nd.dedge_begin + i];
+    const int di = o.di;
+    s_de[i] = o.d;
+    s_zk[i] = split_l2(A.Z[o.d.nbr] * kLog2e);
     s_di[i] = di;
     s_dr[i] = 0;
     s_r[i] = 0.f;
@@ -680,7 +681,7 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeD& nd, const NodeChu
     v.edge = d.edge;
     v.di = s_di[0];
     v.zk = s_zk[0];
-    v.eps_ln2 = P.eps * kLn2;
+    v.eps_ln2 = c.eps * kLn2;
     v.one_piece = one_piece;
     v.track = track;
     if (one_piece) v.sk = s_sk[0];
@@ -815,24 +816,9 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeD& nd, const NodeChu
   if (__syncthreads_or(bad) && tid == 0) atomicOr(A.err, 1);
 }
 
-// Z_j of a free node from its chunks' (max, sum) pieces of s, and rho_j
-__device__ __forceinline__ void finish_free_node(const NodeArgs& A, int node, const NodeD& nd) {
-  double M = -INFINITY;
-  for (int k = 0; k < nd.nchunks; ++k) M = fmax(M, A.zpart[nd.chunk_base + k].x);
-  double S = 0.0;
-  for (int k = 0; k < nd.nchunks; ++k) {
-    const double2 z = A.zpart[nd.chunk_base + k];
-    S += z.y * exp(z.x - M);
-  }
-  const double Zn = M + log(S);
-  A.Z[node] = Zn;
-  A.rho[node] = -(double)nd.deg * Zn;
-}
-
-// The same, by a whole warp (every lane gets the result): the exponentials of
-// the chunks in parallel lanes, then the sum in chunk order by every lane, so
-// the result is bit-identical to finish_free_node's (FP64 transcendental work
-// by one lane at a time is slow on this GPU).
+// Z_j of a free node from its chunks' (max, sum) pieces of s, and rho_j, by a
+// whole warp: the exponentials of the chunks in parallel lanes, then the sum in
+// chunk order (FP64 transcendental work by one lane at a time is slow on this GPU).
 __device__ __forceinline__ void finish_free_node_warp(const NodeArgs& A, int node, const NodeD& nd, int lane) {
   double M = -INFINITY;
   for (int k = lane; k < nd.nchunks; k += 32) M = fmax(M, A.zpart[nd.chunk_base + k].x);
@@ -858,8 +844,7 @@ __device__ __forceinline__ void finish_free_node_warp(const NodeArgs& A, int nod
 // The stopping quantity of iterate t_now of problem p is complete (rs: the
 // sum of its terms, rm: the largest): phase control and retirement, then the
 // counters of the next launch.
-__device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, const ProbD& P, int64_t t_now,
-                                                     double rs, double rm) {
+__device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, int64_t t_now, double rs, double rm) {
   const double crit = A.tol_kind == 1 ? rm : rs;
   const int lp = A.absorbed ? A.lowp[p] : 0;
   if (lp == 2 && t_now + 1 >= A.lowp_start) {
@@ -869,6 +854,7 @@ __device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, c
     A.lowp_span[2 * p] = t_now + 1;
     A.lowp_best[p] = INFINITY;
     A.lowp_best_t[p] = t_now + 1;
+    const ProbD P = A.probs[p];
     for (int k = 0; k < P.edge_count; ++k) A.drift[P.edge_begin + k] = 1;
   } else if (lp == 1) {
     // the phase's accuracy is enough until the stopping quantity reaches
@@ -887,8 +873,9 @@ __device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, c
       if (A.fp32_live) atomicAdd(A.fp32_live, 1);
     }
   } else if (A.retire && (crit < A.ptol[p] || t_now + 1 >= A.deadline[p])) {
+    A.done_at[p] = t_now + 1;  // before the flag: see node_finish_kernel
+    __threadfence();
     A.done[p] = 1;
-    A.done_at[p] = t_now + 1;
     if (A.fp32_live) atomicSub(A.fp32_live, 1);  // retired: no FP32 apply any more
   }
   A.node_count[p] = 0;
@@ -898,55 +885,71 @@ __device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, c
 }
 
 // One node-update item: chunk c of a node of the active colour at half-step
-// t_now (the number of half-steps done before it).  Unless the launch defers
-// it to node_finish_kernel, thread 0 also does the chunk's arrival
-// bookkeeping: the last chunk of a node merges Z_j and the node's stopping
-// terms; the last node of a problem records the stopping quantity of iterate
-// t_now and (when asked) retires the problem.
+// t_now (the number of half-steps done before it; only thread 0's is read).
+// Unless the launch defers it to node_finish_kernel, warp 0 also does the chunk's
+// arrival bookkeeping: the last chunk of a node merges Z_j and the node's
+// stopping terms; the last node of a problem records the stopping quantity of
+// iterate t_now and (when asked) retires the problem.  This tail is a chain of
+// memory round trips; the warp's lanes take the chunks' exponentials and the
+// owned edges' terms side by side (one thread in turn took 8 of a 1024-point,
+// 8-edge centre's 23 us), and a problem with one node of the colour skips the
+// per-problem counters.
 template <bool F64, bool FIXED_ONLY = false, bool PM = false>
-__device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChunk c, int64_t t_now,
+__device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChunkD& c, int64_t t_now,
                                                 unsigned char* node_sm, double* red) {
-  const NodeD nd = A.nodes[c.node];
+  const NodeD& nd = c.nd;
   const int p = nd.prob;
-  const ProbD P = A.probs[p];
-  const int slot = (int)(t_now % kResidRing);
   const bool skip = A.done[p] != 0;
   if (!skip) {
     if constexpr (F64)
-      chunk_update64(A, nd, c, P, red, node_sm, c.node);
+      chunk_update64(A, c, red, node_sm);
     else
-      chunk_update32<FIXED_ONLY, PM>(A, nd, c, P, red, node_sm, c.node);
+      chunk_update32<FIXED_ONLY, PM>(A, c, red, node_sm);
   }
   if (A.defer) return;  // launch-uniform: the chunk's terms are in resid_acc and zpart
   __syncthreads();
-  if (threadIdx.x != 0) return;
+  if (threadIdx.x >= 32 || skip) return;
+  const int lane = threadIdx.x;
+  int last = 0;
+  if (lane == 0) {
+    __threadfence();
+    last = nd.nchunks == 1 || atomicAdd(&A.node_arrive[c.node], 1) == nd.nchunks - 1;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  // last chunk of this node: finish Z_j and the node's stopping terms
   __threadfence();
-  if (!skip && atomicAdd(&A.node_arrive[c.node], 1) == nd.nchunks - 1) {
-    // last chunk of this node: finish Z_j and the node's stopping terms
+  double nsum = 0.0, nmax = 0.0;
+  for (int i = lane; i < nd.deg; i += 32) {
+    const int di = A.owned[nd.dedge_begin + i].di;
+    // read the chunks' accumulated term and clear it for the next launch
+    const double r = __longlong_as_double(
+        (long long)atomicExch((unsigned long long*)&A.resid_acc[di], 0ull));
+    A.resid_dedge[di] = r;
+    nsum += r;
+    nmax = fmax(nmax, r);
+  }
+  if (!nd.fixed) finish_free_node_warp(A, c.node, nd, lane);
+  nsum = warp_sum_d(nsum);
+  nmax = warp_max_d(nmax);
+  if (lane != 0) return;
+  if (nd.nchunks > 1) A.node_arrive[c.node] = 0;
+  const int slot = (int)(t_now % kResidRing);
+  if (c.in_colour == 1) {
+    A.res_sum[slot * A.nprob + p] = nsum;
+    A.res_max[slot * A.nprob + p] = (unsigned long long)__double_as_longlong(nmax);
+    problem_after_update(A, p, t_now, nsum, nmax);
+    return;
+  }
+  atomicAdd(&A.res_sum[slot * A.nprob + p], nsum);
+  atomicMax(&A.res_max[slot * A.nprob + p], (unsigned long long)__double_as_longlong(nmax));
+  __threadfence();
+  if (atomicAdd(&A.node_count[p], 1) == c.in_colour - 1) {
+    // last node of this problem in this launch: the stopping quantity of iterate t_now is complete
     __threadfence();
-    if (!nd.fixed) finish_free_node(A, c.node, nd);
-    double nsum = 0.0, nmax = 0.0;
-    for (int i = 0; i < nd.deg; ++i) {
-      const int di = A.node_dedges[nd.dedge_begin + i];
-      // read the chunks' accumulated term and clear it for the next launch
-      const double r = __longlong_as_double(
-          (long long)atomicExch((unsigned long long*)&A.resid_acc[di], 0ull));
-      A.resid_dedge[di] = r;
-      nsum += r;
-      nmax = fmax(nmax, r);
-    }
-    A.node_arrive[c.node] = 0;
-    atomicAdd(&A.res_sum[slot * A.nprob + p], nsum);
-    atomicMax(&A.res_max[slot * A.nprob + p], (unsigned long long)__double_as_longlong(nmax));
-    __threadfence();
-    if (atomicAdd(&A.node_count[p], 1) == P.nodes_in_colour[A.colour] - 1) {
-      // last node of this problem in this launch: the stopping quantity of iterate t_now is complete
-      __threadfence();
-      const double rs = *((volatile double*)&A.res_sum[slot * A.nprob + p]);
-      const double rm = __longlong_as_double(
-          (long long)*((volatile unsigned long long*)&A.res_max[slot * A.nprob + p]));
-      problem_after_update(A, p, P, t_now, rs, rm);
-    }
+    const double rs = *((volatile double*)&A.res_sum[slot * A.nprob + p]);
+    const double rm = __longlong_as_double(
+        (long long)*((volatile unsigned long long*)&A.res_max[slot * A.nprob + p]));
+    problem_after_update(A, p, t_now, rs, rm);
   }
 }
 

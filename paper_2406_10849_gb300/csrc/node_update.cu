@@ -34,13 +34,25 @@
 namespace treeot {
 namespace {
 
-// the last CTA of a launch that counts (count_launch) advances the half-step counter
-__device__ __forceinline__ void node_launch_done(const NodeArgs& A) {
-  if (threadIdx.x != 0 || !A.count_launch) return;
-  __threadfence();
-  if (atomicAdd(A.launch_count, 1) == (int)gridDim.x - 1) {
+// The half-step counter advances once every CTA of a counting launch has read
+// it, not when all are done: thread 0 reads it and takes its ticket on the way
+// in (the ticket depends on the value read, so it is taken after), and looks at
+// the ticket on the way out, when it has long arrived.
+struct LaunchTicket {
+  int64_t t_now;
+  int ticket;
+};
+__device__ __forceinline__ LaunchTicket node_launch_begin(const NodeArgs& A) {
+  LaunchTicket k{0, -1};
+  if (threadIdx.x == 0) {
+    k.t_now = *((volatile const int64_t*)A.hs);
+    if (A.count_launch) k.ticket = atomicAdd(A.launch_count, k.t_now < 0 ? 2 : 1);
+  }
+  return k;
+}
+__device__ __forceinline__ void node_launch_end(const NodeArgs& A, const LaunchTicket& k) {
+  if (threadIdx.x == 0 && k.ticket == (int)gridDim.x - 1) {
     *A.launch_count = 0;
-    __threadfence();
     atomicAdd((unsigned long long*)A.hs, 1ull);
   }
 }
@@ -49,10 +61,10 @@ template <bool F64>
 __global__ void __launch_bounds__(kNodeThreads) node_update_kernel(NodeArgs A) {
   extern __shared__ __align__(16) unsigned char node_sm[];
   __shared__ double red[kNodeThreads / 32];
-  const NodeChunk c = A.chunks[blockIdx.x];
-  const int64_t t_now = *((volatile const int64_t*)A.hs);
-  node_chunk_item<F64, false>(A, c, t_now, node_sm, red);
-  node_launch_done(A);
+  const LaunchTicket k = node_launch_begin(A);
+  const NodeChunkD c = A.chunks[blockIdx.x];
+  node_chunk_item<F64, false>(A, c, k.t_now, node_sm, red);
+  node_launch_end(A, k);
 }
 
 // FP32 handles with shared-kernel groups: the same, plus the point-major form
@@ -61,10 +73,10 @@ __global__ void __launch_bounds__(kNodeThreads) node_update_kernel(NodeArgs A) {
 __global__ void __launch_bounds__(kNodeThreads, 3) node_update_sk_kernel(NodeArgs A) {
   extern __shared__ __align__(16) unsigned char node_sm[];
   __shared__ double red[kNodeThreads / 32];
-  const NodeChunk c = A.chunks[blockIdx.x];
-  const int64_t t_now = *((volatile const int64_t*)A.hs);
-  node_chunk_item<false, false, true>(A, c, t_now, node_sm, red);
-  node_launch_done(A);
+  const LaunchTicket k = node_launch_begin(A);
+  const NodeChunkD c = A.chunks[blockIdx.x];
+  node_chunk_item<false, false, true>(A, c, k.t_now, node_sm, red);
+  node_launch_end(A, k);
 }
 
 // chunks of fixed leaves only: without the free-node path the FP32 form fits in
@@ -96,29 +108,36 @@ __global__ void __launch_bounds__(kNodeThreads, 4) node_update_fixed_kernel(Node
       return;
     }
   }
-  const NodeChunk c = A.chunks[blockIdx.x];
-  const int64_t t_now = *((volatile const int64_t*)A.hs);
-  node_chunk_item<F64, true>(A, c, t_now, node_sm, red);
-  node_launch_done(A);
+  const LaunchTicket k = node_launch_begin(A);
+  const NodeChunkD c = A.chunks[blockIdx.x];
+  node_chunk_item<F64, true>(A, c, k.t_now, node_sm, red);
+  node_launch_end(A, k);
 }
 
-// Deferred bookkeeping of one colour's node update, one warp per problem: each
-// owned directed edge's stopping term (summed into resid_acc by the chunks),
-// Z_j of the free nodes from their chunks' pieces, the problem's stopping
-// quantity of iterate t_now, phase control and retirement; the last CTA
-// advances the half-step counter.  The same arithmetic as the last-arrival
-// path of node_chunk_item, run after the chunks' launch instead of on their
-// way out: a chunk then leaves with no fence and no atomic it waits for.
+// Deferred bookkeeping of one colour's node update: a warp per problem (each
+// owned directed edge's stopping term, summed into resid_acc by the chunks; the
+// problem's stopping quantity of iterate t_now, phase control and retirement)
+// and a warp per free node of the colour (Z_j from its chunks' pieces).  The same
+// arithmetic as the last-arrival path of node_chunk_item, run after the chunks'
+// launch instead of on their way out: a chunk then leaves with no fence and no
+// atomic it waits for.  (One warp per problem for all of it walked the problem's
+// nodes in turn: 37 us on 128 trees of up to 32 nodes.)  A node's warp may find its
+// problem retired by this very launch: it then still finishes the node.
 constexpr int kFinishWarps = 8;
 __global__ void __launch_bounds__(32 * kFinishWarps) node_finish_kernel(NodeArgs A, FinishList L) {
   const int lane = threadIdx.x & 31;
-  const int p = blockIdx.x * kFinishWarps + (threadIdx.x >> 5);
-  const int64_t t_now = *((volatile const int64_t*)A.hs);
-  if (p < A.nprob && A.done[p] == 0) {
-    const ProbD P = A.probs[p];
-    if (P.nodes_in_colour[A.colour] > 0) {
+  const int w = blockIdx.x * kFinishWarps + (threadIdx.x >> 5);
+  __shared__ int64_t s_t;
+  const LaunchTicket k = node_launch_begin(A);
+  if (threadIdx.x == 0) s_t = k.t_now;
+  __syncthreads();
+  const int64_t t_now = s_t;
+  if (w < A.nprob) {
+    const int p = w;
+    const int d0 = L.dbeg[p], d1 = L.dbeg[p + 1];
+    if (d1 > d0 && A.done[p] == 0) {
       double nsum = 0.0, nmax = 0.0;
-      for (int i = L.dbeg[p] + lane; i < L.dbeg[p + 1]; i += 32) {
+      for (int i = d0 + lane; i < d1; i += 32) {
         const int di = L.dedges[i];
         const double r = A.resid_acc[di];
         A.resid_acc[di] = 0.0;  // for the next launch
@@ -126,22 +145,26 @@ __global__ void __launch_bounds__(32 * kFinishWarps) node_finish_kernel(NodeArgs
         nsum += r;
         nmax = fmax(nmax, r);
       }
-      for (int i = L.nbeg[p]; i < L.nbeg[p + 1]; ++i) {  // warp-uniform
-        const int node = L.nodes[i];
-        finish_free_node_warp(A, node, A.nodes[node], lane);
-      }
       nsum = warp_sum_d(nsum);
       nmax = warp_max_d(nmax);
       if (lane == 0) {
         const int slot = (int)(t_now % kResidRing);
         A.res_sum[slot * A.nprob + p] = nsum;
         A.res_max[slot * A.nprob + p] = (unsigned long long)__double_as_longlong(nmax);
-        problem_after_update(A, p, P, t_now, nsum, nmax);
+        problem_after_update(A, p, t_now, nsum, nmax);
       }
     }
+  } else if (w - A.nprob < L.nnodes) {
+    const int node = L.nodes[w - A.nprob];
+    const NodeD nd = A.nodes[node];
+    bool live = ((volatile const int32_t*)A.done)[nd.prob] == 0;
+    if (!live) {
+      __threadfence();
+      live = ((volatile const int64_t*)A.done_at)[nd.prob] == t_now + 1;
+    }
+    if (live) finish_free_node_warp(A, node, nd, lane);
   }
-  __syncthreads();
-  node_launch_done(A);
+  node_launch_end(A, k);
 }
 
 // stored potentials of an FP32 handle from the operand the node update keeps:
@@ -217,7 +240,7 @@ cudaError_t launch_node_update(const NodeArgs& a, bool fp64, bool fixed_only, cu
 
 cudaError_t launch_node_finish(const NodeArgs& a, const FinishList& l, cudaStream_t s) {
   if (a.nprob <= 0) return cudaSuccess;
-  const int grid = (a.nprob + kFinishWarps - 1) / kFinishWarps;
+  const int grid = (a.nprob + l.nnodes + kFinishWarps - 1) / kFinishWarps;
   node_finish_kernel<<<grid, 32 * kFinishWarps, 0, s>>>(a, l);
   return cudaGetLastError();
 }
