@@ -220,6 +220,7 @@ struct tree_ot_handle {
   Task* d_btasks[2] = {nullptr, nullptr};
   int32_t* d_queue = nullptr;              // [colour][slot][2] work-queue counters
   int32_t rec_ob = kRecOut;                // recomputed-cost output block (autotuned)
+  int32_t f64_rows = 64;                   // FP64 apply: outputs per task (8 or 64)
   int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
   bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
   std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
@@ -382,9 +383,10 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
     std::vector<Task>& tl = h->tasks[own.colour];
     const bool dense = pd.cost_kind == TREE_OT_COST_DENSE_F32;
     if (h->fp64) {
-      for (int32_t o0 = 0; o0 < own.n; o0 += 64)
+      // a row per warp and task where the GPU has room for it: rows in turn are a chain of latencies
+      for (int32_t o0 = 0; o0 < own.n; o0 += h->f64_rows)
         tl.push_back(Task{(int32_t)di, dense ? (d.dir == 0 ? TASK_ROW : TASK_COL) : TASK_RECOMP, o0,
-                          std::min(64, own.n - o0), 0, nbn.n, 0, 0});
+                          std::min(h->f64_rows, own.n - o0), 0, nbn.n, 0, 0});
     } else if (dense && (d.dir == 0 || h->use_ct)) {
       // rows of C (owner = row node) or of its transpose (owner = column node; pad = 1)
       for (int32_t o0 = 0; o0 < own.n; o0 += 8 * kRowRowsPerWarp)
@@ -1854,6 +1856,14 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   build_apply_tasks(h, 256);
   for (int c = 0; c < 2; ++c) h->task_cap[c] = (int64_t)h->tasks[c].size();
   for (const DEdgeD& d : h->dedges)
+  if (h->fp64) {
+    int64_t rows[2] = {0, 0};
+    for (const DEdgeD& d : h->dedges) rows[h->nodes[d.owner].colour] += h->nodes[d.owner].n;
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (std::max(rows[0], rows[1]) <= (int64_t)64 * 8 * nsm) h->f64_rows = 8;
+  }
     if (!h->fp64 && h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
       h->task_cap[h->nodes[d.owner].colour] += (h->nodes[d.owner].n + 63) / 64;
   build_apply_tasks(h, kRecOut);

