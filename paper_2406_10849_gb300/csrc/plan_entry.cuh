@@ -37,6 +37,32 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
   return {s.hi, s.lo + a.lo + b.lo};
 }
 
+// running sums of (pairs of) floats: s += v with every rounding error kept in s.lo
+__device__ __forceinline__ void df_acc(DF& s, float v) {
+  const DF t = two_sum(s.hi, v);
+  s.hi = t.hi;
+  s.lo += t.lo;
+}
+__device__ __forceinline__ void df_acc(DF& s, DF v) {
+  const DF t = two_sum(s.hi, v.hi);
+  s.hi = t.hi;
+  s.lo += t.lo + v.lo;
+}
+// lo back below half an ulp of hi (|hi| >= |lo|), so that adding to it stays exact to ~2^-48
+__device__ __forceinline__ void df_renorm(DF& s) {
+  const float t = __fadd_rn(s.hi, s.lo);
+  s.lo = __fsub_rn(s.lo, __fsub_rn(t, s.hi));
+  s.hi = t;
+}
+__device__ __forceinline__ double df_to(DF v) { return (double)v.hi + (double)v.lo; }
+// the warp's sum, in every lane (FP64 shuffle sums cost 20 times the FP32 pipe's time per step)
+__device__ __forceinline__ DF warp_sum_df(DF v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+    df_acc(v, DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+  return v;
+}
+
 // squared distance of two D-dimensional FP32 points (D <= 3) as a double-float
 __device__ __forceinline__ DF sq_dist_df(int D, const float* pa, const float* pb) {
   DF c = sq_diff(pa[0], pb[0]);

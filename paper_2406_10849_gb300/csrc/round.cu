@@ -187,26 +187,18 @@ __global__ void __launch_bounds__(256) round_pass_kernel(RoundArgs A) {
 
 // ---------------------------------------------------------------------------
 // Passes 1-4 of FP32 handles.  Entries and costs are pairs of FP32 values already;
-// here every sum over them is one too: products by TwoProd, additions by TwoSum,
-// running sums flushed into FP64 every kFlushCols columns.  A sum then carries a
-// few units of 2^-46 relative (measured by the tests: rounded plans feasible to
+// here every sum over them is one too, across the lanes and warps as well:
+// products by TwoProd, additions by TwoSum, running sums renormalised every
+// kRenormSteps column steps.  A sum then carries a few units of 2^-46 relative (measured by the tests: rounded plans feasible to
 // 1e-13, as with FP64 sums).  GB300 executes an FP64 add or a conversion at 1/70
 // of its FP32 rate, and with FP64 sums those were the passes' whole time (94 M
-// entries in 209 plans: 2.6 / 0.8 / 3.1 / 2.8 ms for passes 1-4).  Row factors
-// (x, err_r) multiply the finished row sums, not the entries.
+// entries in 209 plans: 2.6 / 0.8 / 3.1 / 2.8 ms for passes 1-4; with only the
+// entries' sums in double-float and FP64 across lanes 0.91 / 0.56 / 0.87 / 0.62;
+// now 0.72 / 0.55 / 0.66 / 0.49).  Row factors (x, err_r) multiply the finished
+// row sums, not the entries.
 // ---------------------------------------------------------------------------
-constexpr int kFlushCols = 32;  // column steps (32 columns each) between flushes
+constexpr int kRenormSteps = 32;  // column steps (32 columns each) between renormalisations
 
-__device__ __forceinline__ void df_acc(DF& s, float v) {  // s += v
-  const DF t = two_sum(s.hi, v);
-  s.hi = t.hi;
-  s.lo += t.lo;
-}
-__device__ __forceinline__ void df_acc(DF& s, DF v) {
-  const DF t = two_sum(s.hi, v.hi);
-  s.hi = t.hi;
-  s.lo += t.lo + v.lo;
-}
 // a (a float) times b
 __device__ __forceinline__ DF df_mul(float a, DF b) {
   const float p = __fmul_rn(a, b.hi);
@@ -220,7 +212,6 @@ __device__ __forceinline__ DF df_of(double v) {
   const float h = (float)v;
   return {h, (float)(v - (double)h)};
 }
-__device__ __forceinline__ double df_to(DF v) { return (double)v.hi + (double)v.lo; }
 
 template <int PASS>
 __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
@@ -242,7 +233,6 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
     const int D = P.dim;
     float rah[kRndRows], ral[kRndRows], rp[kRndRows][3];
     DF xr[kRndRows], racc[kRndRows], tacc[kRndRows];
-    double rsum[kRndRows], tsum[kRndRows];
     bool inf[kRndRows];
     DF cmax = {0.f, 0.f};
 #pragma unroll
@@ -257,7 +247,6 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
         rp[r][k] = (nj.coord_off >= 0 && k < D) ? A.coords[nj.coord_off + (int64_t)i * D + k] : 0.f;
       if (PASS == 2) xr[r] = on ? df_of(A.xy[d.off + i]) : DF{0.f, 0.f};
       racc[r] = tacc[r] = {0.f, 0.f};
-      rsum[r] = tsum[r] = 0.0;
       inf[r] = false;
     }
     int step = 0;
@@ -326,39 +315,49 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
         }
         __syncthreads();
       }
-      if (PASS != 2 && ++step == kFlushCols) {
+      if (PASS != 2 && ++step == kRenormSteps) {
         step = 0;
 #pragma unroll
         for (int r = 0; r < kRndRows; ++r) {
-          if (PASS != 4) rsum[r] += df_to(racc[r]);
-          tsum[r] += df_to(tacc[r]);
-          racc[r] = tacc[r] = {0.f, 0.f};
+          df_renorm(racc[r]);
+          df_renorm(tacc[r]);
         }
       }
     }
     if (PASS == 2) continue;
-    double tall = 0.0, msum = 0.0;
+    // row r's sums to lane r: one FP64 conversion for all rows
+    DF row = {0.f, 0.f}, ts = {0.f, 0.f};
+    bool rinf = false;
 #pragma unroll
     for (int r = 0; r < kRndRows; ++r) {
-      const int ir = warp * kRndRows + r;
-      if (ir >= t.ocount) break;  // warp-uniform
-      double f = cscale;  // the row's factor, with the cost's scale
+      if (PASS != 4) {
+        const DF v = warp_sum_df(racc[r]);
+        if (lane == r) row = v;
+      }
+      const DF w = warp_sum_df(tacc[r]);
+      if (lane == r) ts = w;
+      if (PASS == 4 && __any_sync(0xffffffffu, inf[r]) && lane == r) rinf = true;
+    }
+    const int ir = warp * kRndRows + lane;
+    const bool mine = lane < kRndRows && ir < t.ocount;
+    double tall = 0.0, msum = 0.0;
+    if (mine) {
       double x = 1.0;
       if (PASS == 3) x = A.xy[d.off + t.o0 + ir];
       if (PASS == 4) x = A.er[d.off + t.o0 + ir];
-      f *= x;
-      const double ts = warp_sum_d(tsum[r] + df_to(tacc[r]));
-      if (PASS == 4 && __any_sync(0xffffffffu, inf[r])) {
-        if (x > 0.0) tall += INFINITY;
-      } else if (f != 0.0) {
-        tall += f * ts;
+      if (rinf)
+        tall = x > 0.0 ? INFINITY : 0.0;
+      else if (x != 0.0)
+        tall = x * cscale * df_to(ts);
+      if (PASS != 4) {
+        msum = x * df_to(row);
+        (PASS == 1 ? A.rsum : A.s2)[d.off + t.o0 + ir] = msum;  // each row belongs to one task
       }
-      if (PASS == 1 || PASS == 3) {
-        const double row = x * warp_sum_d(rsum[r] + df_to(racc[r]));
-        // each row belongs to one task
-        if (lane == 0) (PASS == 1 ? A.rsum : A.s2)[d.off + t.o0 + ir] = row;
-        msum += row;
-      }
+    }
+#pragma unroll
+    for (int o = kRndRows / 2; o; o >>= 1) {
+      tall += __shfl_xor_sync(0xffffffffu, tall, o);
+      if (PASS == 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
     }
     double* acc = A.edge_acc + kRoundAcc * d.edge;
     if (lane == 0 && tall != 0.0) atomicAdd(&acc[PASS == 1 ? 0 : PASS == 3 ? 1 : 2], tall);
