@@ -62,28 +62,43 @@ __global__ void __launch_bounds__(256) absorb_kernel(AbsorbArgs A) {
       const float ah = A.hh[da.off + x], al = A.hl[da.off + x];
       const float* Crow = e.C + (int64_t)x * e.ld;
       __nv_bfloat16* Krow = reinterpret_cast<__nv_bfloat16*>(e.K) + (int64_t)x * e.ldk;
+      // four columns per lane and step, both passes unrolled so that a lane keeps four 16-byte loads in
+      // flight; the second pass finds the row in L1.  Row pads (columns nb .. ld) hold +inf: no term.
+      // 45 -> 21 us per launch on a 32-node tree of 2048 points per node.
+      const float4* C4 = reinterpret_cast<const float4*>(Crow);
+      const float4* H4 = reinterpret_cast<const float4*>(A.hh + db.off);  // offsets: multiples of 32
+      const float4* L4 = reinterpret_cast<const float4*>(A.hl + db.off);
+      const int n4 = (int)(e.ld >> 2);
       // pass 1: row maximum of A + B - sC (exact grid sums, small final rounding)
       float mx = -kInf;
       if (ah > -kInf) {
-        for (int y = lane; y < e.nb; y += 32) {
-          const float c = Crow[y];
-          float v = fmaf(-c, shi, ah + A.hh[db.off + y]);
-          v = fmaf(-c, slo, v) + (al + A.hl[db.off + y]);
-          mx = fmaxf(mx, v);
+#pragma unroll 4
+        for (int q = lane; q < n4; q += 32) {
+          const float4 c = C4[q], h = H4[q], l = L4[q];
+          const float v0 = fmaf(-c.x, slo, fmaf(-c.x, shi, ah + h.x)) + (al + l.x);
+          const float v1 = fmaf(-c.y, slo, fmaf(-c.y, shi, ah + h.y)) + (al + l.y);
+          const float v2 = fmaf(-c.z, slo, fmaf(-c.z, shi, ah + h.z)) + (al + l.z);
+          const float v3 = fmaf(-c.w, slo, fmaf(-c.w, shi, ah + h.w)) + (al + l.w);
+          mx = fmaxf(mx, fmaxf(fmaxf(v0, v1), fmaxf(v2, v3)));
         }
       }
       mx = warp_max(mx);
       const float rho = mx > -kInf ? quantf(mx) : 0.f;
       // pass 2: Kt = 2^(value - rho) in BF16; padding columns are zero
-      for (int y = lane; y < e.ldk; y += 32) {
-        float k = 0.f;
-        if (y < e.nb && ah > -kInf) {
-          const float c = Crow[y];
-          float v = fmaf(-c, shi, (ah - rho) + A.hh[db.off + y]);
-          v = fmaf(-c, slo, v) + (al + A.hl[db.off + y]);
-          k = ex2(v);
+      const float ar = ah - rho;
+#pragma unroll 4
+      for (int q = lane; q < (int)(e.ldk >> 2); q += 32) {
+        float k0 = 0.f, k1 = 0.f, k2 = 0.f, k3 = 0.f;
+        if (q < n4 && ah > -kInf) {
+          const float4 c = C4[q], h = H4[q], l = L4[q];
+          k0 = ex2(fmaf(-c.x, slo, fmaf(-c.x, shi, ar + h.x)) + (al + l.x));
+          k1 = ex2(fmaf(-c.y, slo, fmaf(-c.y, shi, ar + h.y)) + (al + l.y));
+          k2 = ex2(fmaf(-c.z, slo, fmaf(-c.z, shi, ar + h.z)) + (al + l.z));
+          k3 = ex2(fmaf(-c.w, slo, fmaf(-c.w, shi, ar + h.w)) + (al + l.w));
         }
-        Krow[y] = __float2bfloat16_rn(k);
+        const __nv_bfloat162 b0 = __floats2bfloat162_rn(k0, k1), b1 = __floats2bfloat162_rn(k2, k3);
+        reinterpret_cast<uint2*>(Krow)[q] = make_uint2(*reinterpret_cast<const uint32_t*>(&b0),
+                                                       *reinterpret_cast<const uint32_t*>(&b1));
       }
       if (lane == 0) {
         A.arho[da.off + x] = rho;
