@@ -785,8 +785,11 @@ int reset_state(tree_ot_handle* h, cudaStream_t s) {
     CUDA_TRY(cudaMemsetAsync(h->d_fctl, 0, sizeof(int32_t) * 2, s));
   }
   // apply operand of u = 1: h = log gamma * log2(e)
-  CUDA_TRY(launch_operand(h->d_f, nullptr, h->d_logg, h->d_dedges, h->d_nodes, h->d_probs, (int32_t)h->dedges.size(),
-                          kLog2e, true, h->d_hh, h->d_hl, s));
+  if (h->fp64)
+    CUDA_TRY(launch_operand(h->d_f, nullptr, h->d_logg, h->d_dedges, h->d_nodes, h->d_probs,
+                            (int32_t)h->dedges.size(), kLog2e, true, h->d_hh, h->d_hl, s));
+  else
+    CUDA_TRY(launch_reset_operand(h->d_lgf, h->d_dedges, h->d_nodes, (int32_t)h->dedges.size(), h->d_hh, h->d_hl, s));
   h->f_stale = false;
   // phase of every problem: absorbed BF16 phase (1), waiting for it (2), or FP32 (0)
   CUDA_TRY(cudaMemsetAsync(h->d_absorb_count, 0, sizeof(unsigned long long), s));

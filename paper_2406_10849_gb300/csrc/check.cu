@@ -9,6 +9,7 @@
 // (Dekker's product via FMA), and the sums use Knuth's error-free TwoSum, so
 // the exponent is exact to ~1e-12 before one accurate expf of its high part.
 // Each plan entry then has ~1e-7 relative error with no systematic part.
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -206,6 +207,21 @@ __global__ void operand_kernel(const double* f, const double* Z, const double* l
   }
 }
 
+// apply operand of u = 1 on FP32 handles: log2 gamma, as the plan holds it (formed from the
+// FP64 potentials it took 102 us for 128 trees and 184 us for 500 stars; now 14 and 28)
+__global__ void reset_operand_kernel(const float4* lgf, const DEdgeD* dedges, const NodeD* nodes, int32_t ndedges,
+                                     float* vh, float* vl) {
+  for (int di = blockIdx.x; di < ndedges; di += gridDim.x) {
+    const DEdgeD d = dedges[di];
+    const NodeD nd = nodes[d.owner];
+    for (int x = threadIdx.x; x < nd.n; x += blockDim.x) {
+      const float4 g = nd.fixed ? lgf[nd.node_off + x] : make_float4(0.f, 0.f, 0.f, 0.f);
+      vh[d.off + x] = g.x;
+      vl[d.off + x] = g.y;
+    }
+  }
+}
+
 // batched potential set: pass 0 flags non-finite values, pass 1 writes the
 // normalised potential f' = f + eps Z_owner and records the directed edge for
 // the operand refresh
@@ -367,6 +383,13 @@ cudaError_t launch_operand(const double* f, const double* Z, const double* logg,
     dim3 grid(4, cnt);
     operand_kernel<<<grid, 256, 0, s>>>(f, Z, logg, dedges, nodes, probs, d0, ndedges, scale, quantize, vh, vl);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_reset_operand(const float4* lgf, const DEdgeD* dedges, const NodeD* nodes, int32_t ndedges,
+                                 float* vh, float* vl, cudaStream_t s) {
+  if (ndedges <= 0) return cudaSuccess;
+  reset_operand_kernel<<<std::min(ndedges, 4096), 256, 0, s>>>(lgf, dedges, nodes, ndedges, vh, vl);
   return cudaGetLastError();
 }
 

@@ -415,6 +415,9 @@ cudaError_t launch_materialise_f(const DEdgeD* dedges, int32_t ndedges, const No
 cudaError_t launch_set_potentials(const float* values, int64_t ld, const int32_t* dlist, int32_t count,
                                   const DEdgeD* dedges, const NodeD* nodes, const ProbD* probs, const double* Z,
                                   double* f, DEdgeD* picked, int32_t* bad, bool write, cudaStream_t s);
+// apply operand of u = 1 of an FP32 handle
+cudaError_t launch_reset_operand(const float4* lgf, const DEdgeD* dedges, const NodeD* nodes, int32_t ndedges,
+                                 float* vh, float* vl, cudaStream_t s);
 cudaError_t launch_get_potentials(const int32_t* dlist, int32_t count, const DEdgeD* dedges, const NodeD* nodes,
                                   const ProbD* probs, const double* Z, const double* f, float* values, int64_t ld,
                                   bool centred, cudaStream_t s);
