@@ -1836,7 +1836,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   h->part_len = part_off;
   // node-update chunks: kNodePairs (edge, point) pairs per CTA where a colour has
   // many of them (fewer CTAs, each CTA's metadata loads amortised over more
-  // pairs), kNodePairsSmall where its pairs fill few waves of CTAs anyway
+  // pairs), kNodePairsSmall or kNodePairsTiny where its pairs fill few waves of CTAs anyway
   {
     int64_t pairs[2] = {0, 0};
     for (const NodeD& nd : h->nodes) pairs[nd.colour] += (int64_t)nd.n * std::max(nd.deg, 1);
@@ -1844,7 +1844,9 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     for (int c = 0; c < 2; ++c)
-      h->chunk_pairs[c] = pairs[c] > (int64_t)kNodePairsSmall * 8 * nsm ? kNodePairs : kNodePairsSmall;
+      h->chunk_pairs[c] = pairs[c] > (int64_t)kNodePairsSmall * 8 * nsm  ? kNodePairs
+                          : pairs[c] > (int64_t)kNodePairsTiny * 4 * nsm ? kNodePairsSmall
+                                                                         : kNodePairsTiny;
     for (NodeD& nd : h->nodes) {
       const int32_t cp = node_chunk_points(nd.n, nd.deg, h->chunk_pairs[nd.colour]);
       nd.nchunks = (nd.n + cp - 1) / cp;
@@ -1854,11 +1856,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   }
   h->nzchunks = chunk_base;
 
-  // device task arrays are sized for the finest output blocking the autotuner may pick, in either form
-  // of the recomputed-cost apply (an edge in factored form takes at most n / 64 tasks)
-  build_apply_tasks(h, 256);
-  for (int c = 0; c < 2; ++c) h->task_cap[c] = (int64_t)h->tasks[c].size();
-  for (const DEdgeD& d : h->dedges)
   if (h->fp64) {
     int64_t rows[2] = {0, 0};
     for (const DEdgeD& d : h->dedges) rows[h->nodes[d.owner].colour] += h->nodes[d.owner].n;
@@ -1867,6 +1864,11 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (std::max(rows[0], rows[1]) <= (int64_t)64 * 8 * nsm) h->f64_rows = 8;
   }
+  // device task arrays are sized for the finest output blocking the autotuner may pick, in either form
+  // of the recomputed-cost apply (an edge in factored form takes at most n / 64 tasks)
+  build_apply_tasks(h, 256);
+  for (int c = 0; c < 2; ++c) h->task_cap[c] = (int64_t)h->tasks[c].size();
+  for (const DEdgeD& d : h->dedges)
     if (!h->fp64 && h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
       h->task_cap[h->nodes[d.owner].colour] += (h->nodes[d.owner].n + 63) / 64;
   build_apply_tasks(h, kRecOut);

@@ -35,6 +35,11 @@ constexpr int kNodeThreads = 256;
 // fill the GPU at all (its node update took 0.106 against 0.045 ms).
 constexpr int kNodePairs = 4096;
 constexpr int kNodePairsSmall = 1024;
+// A colour of at most 4 x 256 pairs per SM takes one pair per thread and as many
+// CTAs as there are: the update is then one chain of latencies (a 9-node star of
+// 1024 points: 15.8 us with chunks of 1024 pairs, 12.6 with 256; a 12-node tree
+// of 201 .. 1203 points 17.3 and 14.4).
+constexpr int kNodePairsTiny = 256;
 constexpr int kBfCols = 256;           // BF16 COL task: columns per task (32 lanes x 8)
 constexpr int kBfRowTask = 256;        // BF16 ROW task: rows per task
 constexpr double kGrid = 1024.0;       // apply operands and frames live on a 2^-10 grid
@@ -410,14 +415,14 @@ cudaError_t launch_count_live(const int32_t* done, const int32_t* lowp, int32_t 
 // FP32 handles: the stored potentials f from the operand (hh, hl) and log2 mu
 cudaError_t launch_materialise_f(const DEdgeD* dedges, int32_t ndedges, const NodeD* nodes, const ProbD* probs,
                                  const float4* lgf, const float* hh, const float* hl, double* f, cudaStream_t s);
+// apply operand of u = 1 of an FP32 handle
+cudaError_t launch_reset_operand(const float4* lgf, const DEdgeD* dedges, const NodeD* nodes, int32_t ndedges,
+                                 float* vh, float* vl, cudaStream_t s);
 // v = (f'/eps - Z_owner + log gamma) * scale as FP32 (hi, lo); Z may be null.
 // quantize: hi on the 2^-10 grid (the apply operand), else hi = nearest float.
 cudaError_t launch_set_potentials(const float* values, int64_t ld, const int32_t* dlist, int32_t count,
                                   const DEdgeD* dedges, const NodeD* nodes, const ProbD* probs, const double* Z,
                                   double* f, DEdgeD* picked, int32_t* bad, bool write, cudaStream_t s);
-// apply operand of u = 1 of an FP32 handle
-cudaError_t launch_reset_operand(const float4* lgf, const DEdgeD* dedges, const NodeD* nodes, int32_t ndedges,
-                                 float* vh, float* vl, cudaStream_t s);
 cudaError_t launch_get_potentials(const int32_t* dlist, int32_t count, const DEdgeD* dedges, const NodeD* nodes,
                                   const ProbD* probs, const double* Z, const double* f, float* values, int64_t ld,
                                   bool centred, cudaStream_t s);

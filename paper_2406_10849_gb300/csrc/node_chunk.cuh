@@ -817,23 +817,18 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeChunkD& c, double* r
 }
 
 // Z_j of a free node from its chunks' (max, sum) pieces of s, and rho_j, by a
-// whole warp: the exponentials of the chunks in parallel lanes, then the sum in
-// chunk order (FP64 transcendental work by one lane at a time is slow on this GPU).
+// whole warp, a lane per chunk (FP64 transcendental work by one lane at a time is
+// slow on this GPU).
 __device__ __forceinline__ void finish_free_node_warp(const NodeArgs& A, int node, const NodeD& nd, int lane) {
   double M = -INFINITY;
   for (int k = lane; k < nd.nchunks; k += 32) M = fmax(M, A.zpart[nd.chunk_base + k].x);
   M = warp_max_d(M);
   double S = 0.0;
-  for (int k0 = 0; k0 < nd.nchunks; k0 += 32) {
-    double zy = 0.0, ex = 0.0;
-    if (k0 + lane < nd.nchunks) {
-      const double2 z = A.zpart[nd.chunk_base + k0 + lane];
-      zy = z.y;
-      ex = exp(z.x - M);
-    }
-    const int m = min(32, nd.nchunks - k0);
-    for (int i = 0; i < m; ++i) S += __shfl_sync(0xffffffffu, zy, i) * __shfl_sync(0xffffffffu, ex, i);
+  for (int k = lane; k < nd.nchunks; k += 32) {
+    const double2 z = A.zpart[nd.chunk_base + k];
+    S += z.y * exp(z.x - M);
   }
+  S = warp_sum_d(S);
   if (lane == 0) {
     const double Zn = M + log(S);
     A.Z[node] = Zn;
