@@ -220,7 +220,7 @@ struct tree_ot_handle {
   Task* d_btasks[2] = {nullptr, nullptr};
   int32_t* d_queue = nullptr;              // [colour][slot][2] work-queue counters
   int32_t rec_ob = kRecOut;                // recomputed-cost output block (autotuned)
-  int32_t f64_rows = 64;                   // FP64 apply: outputs per task (8 or 64)
+  int32_t f64_rows = 64;                   // FP64 apply: outputs per task (1 .. 8, or 64)
   int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
   bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
   std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
@@ -383,7 +383,8 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
     std::vector<Task>& tl = h->tasks[own.colour];
     const bool dense = pd.cost_kind == TREE_OT_COST_DENSE_F32;
     if (h->fp64) {
-      // a row per warp and task where the GPU has room for it: rows in turn are a chain of latencies
+      // a row per warp where the GPU has room for it, and as few rows per CTA as there are SMs for: rows in turn
+      // are a chain of latencies, and rows side by side share an SM's 1.6 FP64 lanes per clock
       for (int32_t o0 = 0; o0 < own.n; o0 += h->f64_rows)
         tl.push_back(Task{(int32_t)di, dense ? (d.dir == 0 ? TASK_ROW : TASK_COL) : TASK_RECOMP, o0,
                           std::min(h->f64_rows, own.n - o0), 0, nbn.n, 0, 0});
@@ -1847,6 +1848,11 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       h->chunk_pairs[c] = pairs[c] > (int64_t)kNodePairsSmall * 8 * nsm  ? kNodePairs
                           : pairs[c] > (int64_t)kNodePairsTiny * 4 * nsm ? kNodePairsSmall
                                                                          : kNodePairsTiny;
+    // FP64 runs at 1.6 lanes per clock and SM: below one chunk per SM, the fewer pairs a chunk has the sooner
+    // it is done, down to a warp's
+    if (h->fp64)
+      for (int c = 0; c < 2; ++c)
+        while (h->chunk_pairs[c] > 32 && pairs[c] <= (int64_t)(h->chunk_pairs[c] / 2) * nsm) h->chunk_pairs[c] /= 2;
     for (NodeD& nd : h->nodes) {
       const int32_t cp = node_chunk_points(nd.n, nd.deg, h->chunk_pairs[nd.colour]);
       nd.nchunks = (nd.n + cp - 1) / cp;
@@ -1862,7 +1868,9 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     int dev = 0, nsm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (std::max(rows[0], rows[1]) <= (int64_t)64 * 8 * nsm) h->f64_rows = 8;
+    const int64_t most = std::max(rows[0], rows[1]);
+    if (most <= (int64_t)64 * 8 * nsm)
+      for (h->f64_rows = 1; h->f64_rows < 8 && (int64_t)h->f64_rows * nsm < most;) h->f64_rows *= 2;
   }
   // device task arrays are sized for the finest output blocking the autotuner may pick, in either form
   // of the recomputed-cost apply (an edge in factored form takes at most n / 64 tasks)

@@ -39,9 +39,12 @@ __global__ void __launch_bounds__(kApplyThreads) apply_f64_kernel(ApplyArgs A) {
       const int x = t.o0 + r;
       // four points per lane and step: their loads and exponentials overlap, and a lane's running sum is
       // rescaled at most once per step (rows in turn with one point at a time: 53 us per launch on the
-      // 5-node chain of 64 points, all of it latency; now 8.6)
+      // 5-node chain of 64 points, all of it latency; 8.6 with this, 5.4 with two rows per CTA and the
+      // maximum of a short row first)
       double M = -INFINITY, S = 0.0;
-      for (int y0 = t.r0 + lane; y0 < t.r0 + t.rcount; y0 += 128) {
+      const bool one = t.rcount <= 128;  // a single step: the row's maximum first, no rescaling after
+      for (int yb = t.r0; yb < t.r0 + t.rcount; yb += 128) {  // warp-uniform
+        const int y0 = yb + lane;
         double a[4], m = M;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -51,6 +54,7 @@ __global__ void __launch_bounds__(kApplyThreads) apply_f64_kernel(ApplyArgs A) {
             a[k] = (A.f[d.rev_off + y] - cost_f64(A, e, own, nb, P, t.kind, x, y)) * P.inv_eps + A.logg[nb.node_off + y];
           m = fmax(m, a[k]);
         }
+        if (one) m = warp_max_d(m);
         if (!(m > -INFINITY)) continue;
         if (m > M) S = M > -INFINITY ? S * exp(M - m) : 0.0;
         M = m;
@@ -58,7 +62,7 @@ __global__ void __launch_bounds__(kApplyThreads) apply_f64_kernel(ApplyArgs A) {
         for (int k = 0; k < 4; ++k)
           if (a[k] > -INFINITY) S += a[k] == m ? 1.0 : exp(a[k] - m);
       }
-      const double Mw = warp_max_d(M);
+      const double Mw = one ? M : warp_max_d(M);
       S = (M > -INFINITY) ? (M == Mw ? S : S * exp(M - Mw)) : 0.0;
       S = warp_sum_d(S);
       if (lane == 0) A.part64[d.part_off + (int64_t)t.split * own.n + x] = make_double2(Mw, S);

@@ -44,6 +44,7 @@ __device__ __forceinline__ double merge64(const double2* part, int nsplit, int64
   double M = -INFINITY;
   for (int p = 0; p < nsplit; ++p) M = fmax(M, part[p * stride].x);
   if (!(M > -INFINITY)) return -INFINITY;
+  if (nsplit == 1) return M + log(part[0].y);  // its exponential is that of zero
   double S = 0.0;
   for (int p = 0; p < nsplit; ++p) {
     const double2 v = part[p * stride];
@@ -52,28 +53,30 @@ __device__ __forceinline__ double merge64(const double2* part, int nsplit, int64
   return M + log(S);
 }
 
-// block-wide sum / max of a double (kNodeThreads threads); result valid in all threads
-__device__ double block_sum(double v, double* red) {
-  v = warp_sum_d(v);
+// block-wide sum (valid in thread 0) and max (valid in the warps below nw) of doubles of which only the first
+// nw warps hold any: on this GPU an FP64 instruction occupies an SM's FP64 lanes for 20 clocks per warp, so
+// warps without values stay out
+__device__ double block_sum_d0(double v, double* red, int nw) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < nw) v = warp_sum_d(v);
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  double r = 0.0;
-#pragma unroll
-  for (int i = 0; i < kNodeThreads / 32; ++i) r += red[i];
+  double r = red[0];
+  if (threadIdx.x == 0)
+    for (int i = 1; i < nw; ++i) r += red[i];
   return r;
 }
 
-__device__ double block_max(double v, double* red) {
-  v = warp_max_d(v);
+__device__ double block_max_d(double v, double* red, int nw) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < nw) v = warp_max_d(v);
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  double r = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < kNodeThreads / 32; ++i) r = fmax(r, red[i]);
+  double r = red[0];
+  if (w < nw)
+    for (int i = 1; i < nw; ++i) r = fmax(r, red[i]);
   return r;
 }
 
@@ -174,6 +177,7 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeChunkD& c, double* r
   double* s_s = reinterpret_cast<double*>(sm + L.s);
   Q* s_qb = reinterpret_cast<Q*>(sm + L.qb);
   const int tid = threadIdx.x, lane = tid & 31;
+  const int nw = min((cnt + 31) / 32, kNodeThreads / 32);  // warps with a point
   for (int i = tid; i < deg; i += kNodeThreads) {
     const OwnedDEdge o = A.owned[nd.dedge_begin + i];
     s_de[i] = o.d;
@@ -213,7 +217,7 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeChunkD& c, double* r
       if (track && hi > -INFINITY && fabsf((hi - A.bh[d.off + x]) + (lo - A.bl[d.off + x])) > A.tau) drift = true;
     }
     if (__syncthreads_or(drift) && tid == 0) atomicOr(&A.drift[d.edge], 1);
-    const double rs = block_sum((double)r, red);
+    const double rs = block_sum_d0((double)r, red, nw);
     if (tid == 0) atomicAdd(&A.resid_acc[s_di[0]], rs);
     if (__syncthreads_or(bad) && tid == 0) atomicOr(A.err, 1);
     return;
@@ -249,10 +253,10 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeChunkD& c, double* r
     s_qb[xi] = qsum * (Q)inv_deg;
     smax = fmax(smax, s);
   }
-  smax = block_max(smax, red);  // its barriers also publish s_s and s_qb
+  smax = block_max_d(smax, red, nw);  // its barriers also publish s_s and s_qb
   Q se = Q(0);
   for (int xi = tid; xi < cnt; xi += kNodeThreads) se += exp(s_s[xi] - smax);
-  const double sse = block_sum(se, red);
+  const double sse = block_sum_d0(se, red, nw);
   if (tid == 0) A.zpart[nd.chunk_base + c.chunk] = make_double2(smax, sse);
   // pass 3, pairs: f'_(j,k)/eps = s - m, the next apply's operand, |q_k - mean q|
   {
@@ -279,8 +283,10 @@ __device__ void chunk_update64(const NodeArgs& A, const NodeChunkD& c, double* r
       // per-edge sums: one shared-memory atomic per warp when the warp's pairs share an edge
       const int i0 = __shfl_sync(0xffffffffu, i, 0);
       if (__all_sync(0xffffffffu, i == i0)) {
-        r = warp_sum_d(r);
-        if (lane == 0 && i0 >= 0) atomicAdd(&s_r[i0], r);
+        if (i0 >= 0) {  // warp-uniform
+          r = warp_sum_d(r);
+          if (lane == 0) atomicAdd(&s_r[i0], r);
+        }
       } else if (on) {
         atomicAdd(&s_r[i], r);
       }
