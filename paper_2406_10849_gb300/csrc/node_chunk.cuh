@@ -656,11 +656,13 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeChunkD& c, double* r
   const int lp = A.absorbed ? A.lowp[nd.prob] : 0;
   const bool track = lp == 1 && c.cost_kind == 0;
   const bool one_piece = lp == 1 && c.cost_kind != 0 && A.sk_ref;
+  // the neighbours' normalisers: now, or (pass 1 below) beside the pairs' own loads
+  const bool early = FIXED_ONLY || nd.fixed || (PM && one_piece);
   for (int i = tid; i < deg; i += kNodeThreads) {
     const OwnedDEdge o = A.owned[nd.dedge_begin + i];
     const int di = o.di;
     s_de[i] = o.d;
-    s_zk[i] = split_l2(A.Z[o.d.nbr] * kLog2e);
+    if (early) s_zk[i] = split_l2(A.Z[o.d.nbr] * kLog2e);
     s_di[i] = di;
     s_dr[i] = 0;
     s_r[i] = 0.f;
@@ -742,6 +744,10 @@ __device__ void chunk_update32(const NodeArgs& A, const NodeChunkD& c, double* r
         pv[k] = one_piece ? load_sk_raw(s_sk[pi[k]], x) : load_part2(A.part32 + d.part_off + x, d.nsplit, nd.n);
         oh[k] = A.hh[d.off + x];  // f/eps log2(e) of the previous iterate
         ol[k] = A.hl[d.off + x];
+      }
+      if (qb == 0 && !early) {  // block-uniform
+        for (int i = tid; i < deg; i += kNodeThreads) s_zk[i] = split_l2(A.Z[s_de[i].nbr] * kLog2e);
+        __syncthreads();
       }
 #pragma unroll
       for (int k = 0; k < kIt; ++k) {
@@ -842,12 +848,29 @@ __device__ __forceinline__ void finish_free_node_warp(const NodeArgs& A, int nod
   }
 }
 
+// what problem_after_update compares with; constant while a half-step runs
+struct ProbLimits {
+  double tol;
+  int64_t deadline;
+  int lp;
+};
+__device__ __forceinline__ ProbLimits load_limits(const NodeArgs& A, int p) {
+  ProbLimits l{0.0, 0, 0};
+  if (A.absorbed) l.lp = A.lowp[p];
+  if (A.retire) {
+    l.tol = A.ptol[p];
+    l.deadline = A.deadline[p];
+  }
+  return l;
+}
+
 // The stopping quantity of iterate t_now of problem p is complete (rs: the
 // sum of its terms, rm: the largest): phase control and retirement, then the
 // counters of the next launch.
-__device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, int64_t t_now, double rs, double rm) {
+__device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, int64_t t_now, double rs, double rm,
+                                                     const ProbLimits& lim) {
   const double crit = A.tol_kind == 1 ? rm : rs;
-  const int lp = A.absorbed ? A.lowp[p] : 0;
+  const int lp = lim.lp;
   if (lp == 2 && t_now + 1 >= A.lowp_start) {
     // enter the low-precision phase: absorb every edge of the problem next
     A.lowp[p] = 1;
@@ -873,7 +896,7 @@ __device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, i
       A.lowp_span[2 * p + 1] = t_now + 1;
       if (A.fp32_live) atomicAdd(A.fp32_live, 1);
     }
-  } else if (A.retire && (crit < A.ptol[p] || t_now + 1 >= A.deadline[p])) {
+  } else if (A.retire && (crit < lim.tol || t_now + 1 >= lim.deadline)) {
     A.done_at[p] = t_now + 1;  // before the flag: see node_finish_kernel
     __threadfence();
     A.done[p] = 1;
@@ -887,14 +910,14 @@ __device__ __forceinline__ void problem_after_update(const NodeArgs& A, int p, i
 
 // One node-update item: chunk c of a node of the active colour at half-step
 // t_now (the number of half-steps done before it; only thread 0's is read).
-// Unless the launch defers it to node_finish_kernel, warp 0 also does the chunk's
-// arrival bookkeeping: the last chunk of a node merges Z_j and the node's
-// stopping terms; the last node of a problem records the stopping quantity of
-// iterate t_now and (when asked) retires the problem.  This tail is a chain of
-// memory round trips; the warp's lanes take the chunks' exponentials and the
-// owned edges' terms side by side (one thread in turn took 8 of a 1024-point,
-// 8-edge centre's 23 us), and a problem with one node of the colour skips the
-// per-problem counters.
+// Unless the launch defers it to node_finish_kernel, the chunk's first two warps
+// also do its arrival bookkeeping: the last chunk of a node merges Z_j (warp 1)
+// and the node's stopping terms (warp 0); the last node of a problem records the
+// stopping quantity of iterate t_now and (when asked) retires the problem.  Both
+// are chains of memory round trips and FP64 exponentials, so they run side by
+// side, and their lanes take the chunks and the owned edges side by side (one
+// thread in turn took 8 of a 1024-point, 8-edge centre's 23 us).  A problem with
+// one node of the colour skips the per-problem counters.
 template <bool F64, bool FIXED_ONLY = false, bool PM = false>
 __device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChunkD& c, int64_t t_now,
                                                 unsigned char* node_sm, double* red) {
@@ -907,18 +930,24 @@ __device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChu
     else
       chunk_update32<FIXED_ONLY, PM>(A, c, red, node_sm);
   }
-  if (A.defer) return;  // launch-uniform: the chunk's terms are in resid_acc and zpart
+  if (A.defer || skip) return;  // block-uniform; deferred: the chunk's terms are in resid_acc and zpart
+  __shared__ int s_last;
   __syncthreads();
-  if (threadIdx.x >= 32 || skip) return;
-  const int lane = threadIdx.x;
-  int last = 0;
-  if (lane == 0) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp > 1) return;
+  if (threadIdx.x == 0) {
     __threadfence();
-    last = nd.nchunks == 1 || atomicAdd(&A.node_arrive[c.node], 1) == nd.nchunks - 1;
+    s_last = nd.nchunks == 1 || atomicAdd(&A.node_arrive[c.node], 1) == nd.nchunks - 1;
   }
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
-  // last chunk of this node: finish Z_j and the node's stopping terms
+  asm volatile("bar.sync 1, 64;" ::: "memory");  // warps 0 and 1
+  if (!s_last) return;
+  // last chunk of this node: warp 1 finishes Z_j, warp 0 the node's stopping terms
   __threadfence();
+  if (warp == 1) {
+    if (!nd.fixed) finish_free_node_warp(A, c.node, nd, lane);
+    return;
+  }
+  const ProbLimits lim = load_limits(A, p);  // on their way beside the terms
   double nsum = 0.0, nmax = 0.0;
   for (int i = lane; i < nd.deg; i += 32) {
     const int di = A.owned[nd.dedge_begin + i].di;
@@ -929,7 +958,6 @@ __device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChu
     nsum += r;
     nmax = fmax(nmax, r);
   }
-  if (!nd.fixed) finish_free_node_warp(A, c.node, nd, lane);
   nsum = warp_sum_d(nsum);
   nmax = warp_max_d(nmax);
   if (lane != 0) return;
@@ -938,7 +966,7 @@ __device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChu
   if (c.in_colour == 1) {
     A.res_sum[slot * A.nprob + p] = nsum;
     A.res_max[slot * A.nprob + p] = (unsigned long long)__double_as_longlong(nmax);
-    problem_after_update(A, p, t_now, nsum, nmax);
+    problem_after_update(A, p, t_now, nsum, nmax, lim);
     return;
   }
   atomicAdd(&A.res_sum[slot * A.nprob + p], nsum);
@@ -950,7 +978,7 @@ __device__ __forceinline__ void node_chunk_item(const NodeArgs& A, const NodeChu
     const double rs = *((volatile double*)&A.res_sum[slot * A.nprob + p]);
     const double rm = __longlong_as_double(
         (long long)*((volatile unsigned long long*)&A.res_max[slot * A.nprob + p]));
-    problem_after_update(A, p, t_now, rs, rm);
+    problem_after_update(A, p, t_now, rs, rm, lim);
   }
 }
 

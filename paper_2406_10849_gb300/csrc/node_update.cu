@@ -57,8 +57,10 @@ __device__ __forceinline__ void node_launch_end(const NodeArgs& A, const LaunchT
   }
 }
 
+// three CTAs per SM (96 registers without the cap, hence two: 45 barycenters of
+// about 1000 chunks took 19.0 us per launch)
 template <bool F64>
-__global__ void __launch_bounds__(kNodeThreads) node_update_kernel(NodeArgs A) {
+__global__ void __launch_bounds__(kNodeThreads, F64 ? 2 : 3) node_update_kernel(NodeArgs A) {
   extern __shared__ __align__(16) unsigned char node_sm[];
   __shared__ double red[kNodeThreads / 32];
   const LaunchTicket k = node_launch_begin(A);
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps) node_finish_kernel(NodeArgs
         const int slot = (int)(t_now % kResidRing);
         A.res_sum[slot * A.nprob + p] = nsum;
         A.res_max[slot * A.nprob + p] = (unsigned long long)__double_as_longlong(nmax);
-        problem_after_update(A, p, t_now, nsum, nmax);
+        problem_after_update(A, p, t_now, nsum, nmax, load_limits(A, p));
       }
     }
   } else if (w - A.nprob < L.nnodes) {
