@@ -37,6 +37,8 @@
 
 #include "../../include/tree_ot.h"
 #include "internal.h"
+#include "pdl.h"
+#include "ptx.cuh"
 
 namespace treeot {
 namespace {
@@ -116,6 +118,7 @@ __device__ __forceinline__ int jt_find(const int64_t* start, int32_t n, int64_t 
 // time at 1.6 FP64 lanes per clock and SM).
 __global__ void __launch_bounds__(32 * kJtWarps) jt_op_kernel(const JtOp* ops, const int64_t* start, int32_t nops) {
   __shared__ double red[2][kJtWarps];
+  pdl_trigger();
   const int64_t b = blockIdx.x;
   const int o = jt_find(start, nops, b);
   const JtOp& op = ops[o];
@@ -125,6 +128,7 @@ __global__ void __launch_bounds__(32 * kJtWarps) jt_op_kernel(const JtOp* ops, c
   int64_t base[kJtMaxIn];
   for (int j = 0; j < kJtMaxIn; ++j) base[j] = 0;
   jt_offsets(op, 0, op.nt, on ? t : 0, base);
+  pdl_wait();  // plan data up to here, tensors from here
   if (L == 1) {
     if (on) op.out[t] = jt_value(op, base);
     return;
@@ -419,8 +423,12 @@ int upload_stage(tree_ot_jt_handle* h, Stage& st, cudaStream_t s) {
 
 int run_stage(const Stage& st, cudaStream_t s) {
   if (st.ops.empty() || st.units == 0) return TREE_OT_OK;
-  jt_op_kernel<<<(unsigned)st.units, 32 * kJtWarps, 0, s>>>(st.d_ops, st.d_start, (int32_t)st.ops.size());
-  return jt_cuda(cudaGetLastError(), "junction-tree op launch");
+  const JtOp* ops = st.d_ops;
+  const int64_t* start = st.d_start;
+  int32_t nops = (int32_t)st.ops.size();
+  void* args[] = {&ops, &start, &nops};
+  return jt_cuda(launch_pdl(reinterpret_cast<const void*>(jt_op_kernel), (int)st.units, 32 * kJtWarps, 0, s, args),
+                 "junction-tree op launch");
 }
 
 int upload_sums(tree_ot_jt_handle* h, const std::vector<JtSum>& items, JtSum** d_items, int64_t** d_start,

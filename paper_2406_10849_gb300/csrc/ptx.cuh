@@ -47,6 +47,14 @@ __device__ __forceinline__ uint4 ldg_stream_u4(const uint4* p) {
   return v;
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_pdl (pdl.h) may start while its predecessor in
+// the stream still runs: pdl_trigger() lets the successor's CTAs in as SM resources allow, and pdl_wait()
+// returns once every predecessor has completed and its writes are visible.  Every such kernel waits before it
+// touches anything a launch may have written (so completion is transitive along the stream); only plan data,
+// written once at create, is read before.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
