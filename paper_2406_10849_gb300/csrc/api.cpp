@@ -1449,7 +1449,7 @@ int setup_shared_kernels(tree_ot_handle* h, cudaStream_t s) {
         (rc = h->alloc(&khi, (int64_t)mp * kd)) ||
         (rc = h->alloc(&klo, (int64_t)mp * kd)) || (rc = h->alloc(&vhi, maxc * kd)) ||
         (rc = h->alloc(&vlo, maxc * kd)) || (rc = h->alloc(&sout, maxc * align_up(own.n, 32))) ||
-        (rc = h->alloc(&benv, ((maxc + kSkEnvCols - 1) / kSkEnvCols) * kd)) ||
+        (rc = h->alloc(&benv, ((maxc + kSkEnvColsMin - 1) / kSkEnvColsMin) * kd)) ||
         (rc = h->alloc(&dc[0], (int64_t)g.cols[0].size())) ||
         (rc = h->alloc(&dc[1], (int64_t)g.cols[1].size())) || (rc = h->alloc(&fix_count, 1)) ||
         (rc = h->alloc(&fix_list, (int64_t)own.n * maxc)))

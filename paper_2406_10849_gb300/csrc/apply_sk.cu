@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "pdl.h"
 #include "ptx.cuh"
 #include "sk.h"
 
@@ -128,7 +129,9 @@ __global__ void __launch_bounds__(256) sk_envelope1_kernel(SkArgs A) {
   __shared__ float s_part[8][kEnvBatch];
   __shared__ float s_m[kEnvBatch];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * kEnvCols, nc = min(kEnvCols, A.ncols - c0);
+  pdl_trigger();
+  pdl_wait();
+  const int c0 = blockIdx.x * A.env_cols, nc = min(A.env_cols, A.ncols - c0);
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.fix_count = 0;  // the previous fix-up is done
   const int y0 = 4 * (int)threadIdx.x;
   float e[4] = {-kInf, -kInf, -kInf, -kInf};
@@ -188,6 +191,8 @@ __global__ void __launch_bounds__(256) sk_envelope1_kernel(SkArgs A) {
 // CTA, its eight warps taking every eighth CTA's row
 __global__ void __launch_bounds__(256) sk_envelope_reduce_kernel(SkArgs A, int32_t nblk) {
   __shared__ float s_m[8][33];
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int y = blockIdx.x * 32 + lane;
   float m = -kInf;
@@ -309,6 +314,8 @@ __device__ __forceinline__ void sk_vbuild_cols(const SkArgs& A, int blk) {
 // both operand builds in one launch (they read the same envelope and nothing
 // of each other): CTAs [0, mp) build rows of K', the rest columns of V'
 __global__ void __launch_bounds__(256) sk_kvbuild_kernel(SkArgs A) {
+  pdl_trigger();
+  pdl_wait();
   if ((int)blockIdx.x < A.mp)  // block-uniform
     sk_kbuild_row(A, blockIdx.x);
   else
@@ -1012,6 +1019,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // the sum of 2^(term - frame) with the recomputed-cost apply's argument
 __global__ void __launch_bounds__(256) sk_fixup_kernel(SkArgs A) {
   __shared__ float red[8];
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nfix = *A.fix_count;
   for (int w = blockIdx.x; w < nfix; w += gridDim.x) {  // block-uniform
@@ -1169,19 +1178,31 @@ bool sk_encode_maps(const SkArgs& a, SkMaps* m) {
   return true;
 }
 
-cudaError_t launch_sk(const SkArgs& a, const SkMaps* maps, cudaStream_t s, cudaEvent_t before_product,
+cudaError_t launch_sk(const SkArgs& args, const SkMaps* maps, cudaStream_t s, cudaEvent_t before_product,
                       cudaEvent_t after_product) {
+  SkArgs a = args;
   if (a.ncols <= 0) return cudaSuccess;
   if (a.use_tc && !maps) return cudaErrorInvalidValue;
   if (!(a.use_tc ? sk_tc_ready(a.tc_pair) : sk_gemm_ready())) return cudaErrorInvalidConfiguration;
-  const int nenv = (a.ncols + kEnvCols - 1) / kEnvCols;
+  void* kargs[] = {&a, nullptr};
+  cudaError_t le = cudaSuccess;
   if (a.ny <= 4 * 256 && a.benv) {
-    sk_envelope1_kernel<<<nenv, 256, 0, s>>>(a);
-    sk_envelope_reduce_kernel<<<(a.ny + 31) / 32, 256, 0, s>>>(a, nenv);
+    // columns per CTA: 32 amortise a CTA's partial envelope, but 4000 columns are then 125 CTAs, less than one
+    // per SM, each walking its columns in turn (26.5 us); below two per SM a CTA takes one batch of 8 (envelope and
+    // its reduction together 30 -> 23 us; with the overlapped launches 7.02 -> 6.40 ms for 32 half-steps of
+    // 500 stars, 6.60 without them)
+    a.env_cols = a.ncols > 2 * 152 * kEnvCols ? kEnvCols : kEnvBatch;
+    int32_t nenv = (a.ncols + a.env_cols - 1) / a.env_cols;
+    kargs[1] = &nenv;
+    le = launch_pdl(reinterpret_cast<const void*>(sk_envelope1_kernel), nenv, 256, 0, s, kargs);
+    if (le == cudaSuccess)
+      le = launch_pdl(reinterpret_cast<const void*>(sk_envelope_reduce_kernel), (a.ny + 31) / 32, 256, 0, s, kargs);
   } else {
-    sk_envelope_kernel<<<nenv, 256, 0, s>>>(a);
+    sk_envelope_kernel<<<(a.ncols + kEnvCols - 1) / kEnvCols, 256, 0, s>>>(a);
   }
-  sk_kvbuild_kernel<<<a.mp + (a.ncols + 7) / 8, 256, 0, s>>>(a);
+  if (le == cudaSuccess)
+    le = launch_pdl(reinterpret_cast<const void*>(sk_kvbuild_kernel), a.mp + (a.ncols + 7) / 8, 256, 0, s, kargs);
+  if (le != cudaSuccess) return le;
   if (before_product) cudaEventRecord(before_product, s);
   const dim3 grid(a.mp / kSkTileM, (a.ncols + kSkTileN - 1) / kSkTileN);
   if (a.use_tc && a.tc_pair) {
@@ -1216,8 +1237,9 @@ cudaError_t launch_sk(const SkArgs& a, const SkMaps* maps, cudaStream_t s, cudaE
     sk_gemm_kernel<<<grid, kSkThreads, kSkSmem, s>>>(a);
   }
   if (after_product) cudaEventRecord(after_product, s);
-  sk_fixup_kernel<<<152 * 8, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  le = cudaGetLastError();
+  if (le != cudaSuccess) return le;
+  return launch_pdl(reinterpret_cast<const void*>(sk_fixup_kernel), 152 * 8, 256, 0, s, kargs);
 }
 
 cudaError_t launch_sk_reset(float* b, int32_t kd, cudaStream_t s) {
