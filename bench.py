@@ -255,7 +255,9 @@ def sfu_peak(sms: int, mhz: float) -> float:
 # FP32-pipe lane operations per element the recomputed-cost apply needs by the
 # survey's algorithmic count (2-D points): the squared distance (two differences,
 # a square and an FMA), the argument (operand minus frame, scale), the sum --
-# about 8 -- beside one ex2 on the MUFU.
+# about 8 -- beside one ex2 on the MUFU.  Edges in factored form need fewer (the
+# difference is taken per group of outputs): there the MUFU is the bound, and
+# the fraction of its rate (sfu_frac) the figure to read.
 RECOMP_ALG_OPS_PER_ELEM = 8.0
 
 
@@ -328,7 +330,7 @@ def bench_batched(dev, stream, steps: int, warmup: int, converge: bool, num_tree
         "edge_applies_per_s": total_apply * steps / (t_max / 1e3), "ms_per_step": t_max / steps,
         "apply_ms": apply_ms, "node_update_ms": prof["node_update"][0] / steps,
         "elements_per_s": elem_rate,
-        "roofline": {"bound": "alu", "kernel": "apply_recomp_kernel<2>",
+        "roofline": {"bound": "alu", "kernel": "apply_fact_kernel<2>, apply_recomp_kernel<2>",
                      "achieved": RECOMP_ALG_OPS_PER_ELEM * elem_rate / 1e12, "peak": peak / 1e12, "unit": "Tops/s",
                      "frac": RECOMP_ALG_OPS_PER_ELEM * elem_rate / peak,
                      "ops_per_element": RECOMP_ALG_OPS_PER_ELEM,
