@@ -162,6 +162,13 @@ typedef struct tree_ot_problem {
                                        each CTA holding half of a tile's V' operand); the
                                        same sums, for comparison                           */
 
+/* Test hook: bits 24..27 of flags fix the form of the factored recomputed-cost
+ * apply instead of the autotuner's choice, so that a test can say which kernel
+ * it compares: 0 off, else 1 + split + 4 * both with 2^split (split 0..3) warps
+ * sharing a block of 64 outputs and both = 1 for both forms' tasks in one
+ * launch (only where the handle's recomputed costs have one dimension). */
+#define TREE_OT_TEST_APPLY_SHIFT 24
+
 #define TREE_OT_TOL_SUM          0  /* the paper's stopping sum (Bipartite Iterative Scaling) */
 #define TREE_OT_TOL_MAX          1  /* the largest single term of that sum                 */
 
@@ -401,7 +408,12 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * colour c's node update finishes its bookkeeping in an extra launch
  * (TREE_OT_OPT_NODE_DEFER), [15] the shared-kernel BF16 phase's product: 0
  * no shared-kernel group, 1 mma.sync, 2 tcgen05 with one CTA per 128-row tile,
- * 3 tcgen05 over CTA pairs (TREE_OT_OPT_SK_ONE_CTA, TREE_OT_OPT_SK_MMA_SYNC). */
+ * 3 tcgen05 over CTA pairs (TREE_OT_OPT_SK_ONE_CTA, TREE_OT_OPT_SK_MMA_SYNC),
+ * [16] directed edges whose recomputed-cost apply has the factored form, [17]
+ * log2 of the warps that share a block of its outputs, [18] 1 when its tasks and
+ * the difference form's run in one launch, [19] groups of outputs that it has
+ * summed by the difference form since create (read from the device, after
+ * everything queued before: only when nstats > 19). */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);
 
 /* Launch timing (no paper counterpart: measurement support).  While enabled,

@@ -253,6 +253,7 @@ struct tree_ot_handle {
   float *d_hh = nullptr, *d_hl = nullptr, *d_ah = nullptr, *d_al = nullptr, *d_coords = nullptr;
   float4 *d_slot_x = nullptr, *d_grp = nullptr;  // compact groups of the support points (group.cu)
   float2* d_slot_q = nullptr;
+  unsigned long long* d_fallbacks = nullptr;  // groups the factored apply has summed by the difference form
   float *d_coords_hi = nullptr, *d_coords_lo = nullptr;  // coordinates split hi + lo (exact distances)
   uint32_t* d_cmax = nullptr;              // per problem max |coordinate| (split scratch)
   int32_t* d_exact = nullptr;              // per problem: exact squared distances (recomputed costs)
@@ -464,6 +465,7 @@ ApplyArgs apply_args(tree_ot_handle* h, int colour) {
   a.slot_x = h->d_slot_x;
   a.slot_q = h->d_slot_q;
   a.grp = h->d_grp;
+  a.fallbacks = h->d_fallbacks;
   a.exact = h->d_exact;
   a.any_exact = h->any_exact;
   a.part32 = h->d_part32;
@@ -1379,8 +1381,10 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   }
   if (rc == TREE_OT_OK && slots > 0 &&
       !((rc = h->alloc(&h->d_slot_x, slots)) || (rc = h->alloc(&h->d_slot_q, slots)) ||
-        (rc = h->alloc(&h->d_grp, 3 * (slots / 8))))) {
-    e = cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s);
+        (rc = h->alloc(&h->d_grp, 3 * (slots / 8))) || (rc = h->alloc(&h->d_fallbacks, 1)))) {
+    e = cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
       e = launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
                              h->d_grp, s);
@@ -2207,7 +2211,12 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   // the autotuners time the FP32 kernels: no problem in a BF16 phase meanwhile
   CUDA_TRY(cudaMemsetAsync(h->d_lowp, 0, sizeof(int32_t) * h->nprob, s));
   if ((rc = recount_live(h, s))) return bail(rc);
-  if (o.autotune && !h->fp64 && (rc = autotune_recompute(h, s))) return bail(rc);
+  if (const uint32_t form = (o.flags >> TREE_OT_TEST_APPLY_SHIFT) & 15u) {
+    const int32_t split = (int32_t)((form - 1) & 3u), both = (int32_t)((form - 1) >> 2);
+    if (!h->fp64 && (rc = apply_tune(h, TuneCfg{kRecOut, 0, 0, split, both && one_dimension(h) ? 1 : 0}, s))) return bail(rc);
+  } else if (o.autotune && !h->fp64 && (rc = autotune_recompute(h, s))) {
+    return bail(rc);
+  }
   if (!h->fp64) {
     if ((rc = upload_stream_tasks(h, s))) return bail(rc);
     if (o.flags & (TREE_OT_OPT_DENSE_TMA | TREE_OT_OPT_TEST_STALL)) {
@@ -2787,7 +2796,14 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
     for (int c = 0; c < 2; ++c)
       if (g.args[c].ncols > 0)
         sk_form = std::max<int64_t>(sk_form, g.args[c].use_tc ? (g.args[c].tc_pair ? 3 : 2) : 1);
-  const int64_t v[16] = {(int64_t)h->dedges.size(),
+  int64_t fact_edges = 0;
+  for (const DEdgeD& d : h->dedges) fact_edges += fact_edge(h, d);
+  unsigned long long fallbacks = 0;
+  if (nstats > 19 && h->d_fallbacks) {
+    CUDA_TRY(cudaDeviceSynchronize());
+    CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
+  }
+  const int64_t v[20] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2802,8 +2818,12 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         (int64_t)h->dense_tma,
                         (int64_t)h->persistent,
                         (int64_t)((h->node_defer[0] ? 1 : 0) | (h->node_defer[1] ? 2 : 0)),
-                        sk_form};
-  for (int32_t i = 0; i < nstats && i < 16; ++i) stats[i] = v[i];
+                        sk_form,
+                        fact_edges,
+                        (int64_t)h->fact_split,
+                        (int64_t)(h->both_forms ? 1 : 0),
+                        (int64_t)fallbacks};
+  for (int32_t i = 0; i < nstats && i < 20; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

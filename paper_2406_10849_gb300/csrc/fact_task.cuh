@@ -498,6 +498,7 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
       const unsigned m = GS == 64 ? bad[0] | bad[1]
                                   : (g * GS < 32 ? bad[0] : bad[1]) & (((GS < 32 ? 1u << (GS & 31) : 0u) - 1u) << ((g * GS) & 31));
       if (!m) continue;  // warp-uniform
+      if (lane == 0 && share == 0) atomicAdd(A.fallbacks, 1ull);
       float4 rw[4];
       float2 so[4];
 #pragma unroll

@@ -259,6 +259,7 @@ struct ApplyArgs {
   const float4* slot_x;      // per slot: coordinates less the group's centre, point index (as int bits)
   const float2* slot_q;      // per slot: s |x'|^2 as a two-float
   const float4* grp;         // per 8 slots (at a group's first): 3 x float4, centre, unit, inverse second moments
+  unsigned long long* fallbacks;  // factored form: groups summed by the difference form instead
   const int32_t* exact;      // per problem: 1 = recompute costs with exact squared distances
   int32_t any_exact;         // host: some problem has exact set (selects the kernel instantiation)
   float2* part32;            // FP32 path partials: (frame R, sum) in base 2

@@ -283,7 +283,7 @@ class _Marshalled:
 def options(precision="fp32", tol=1e-6, tol_kind="sum", max_half_steps=100000, check_every=32, use_graph=True,
             apply_mode="auto", refine_tol=None, absorb_tau=None, lowp_start=None, autotune=None,
             dense_kernel="auto", exact_dist=False, transpose=True, test_stall=False, sk_product="auto",
-            persistent=False, node_finish="auto") -> Options:
+            persistent=False, node_finish="auto", test_apply=None) -> Options:
     """tree_ot_options with the defaults of tree_ot_default_options; dense_kernel picks the
     stored-cost apply ("auto": the autotuner's choice, "tma": bulk-copy staged, "ldg": plain loads);
     exact_dist: recompute squared distances exactly from the first half-step;
@@ -294,7 +294,9 @@ def options(precision="fp32", tol=1e-6, tol_kind="sum", max_half_steps=100000, c
     sk_product: the shared-kernel BF16 phase's product ("auto": tcgen05 over CTA pairs where
     available, "one_cta": tcgen05 with one CTA per 128-row tile, "mma": the legacy mma.sync kernel);
     node_finish: where the node update's bookkeeping runs ("auto": by chunk count per colour,
-    "defer": an extra launch after the chunks, "arrive": the last-arriving chunk)."""
+    "defer": an extra launch after the chunks, "arrive": the last-arriving chunk);
+    test_apply: test hook, (split, both) fixes the form of the factored recomputed-cost apply
+    (TREE_OT_TEST_APPLY_SHIFT)."""
     load()
     o = Options()
     _lib.tree_ot_default_options(C.byref(o))
@@ -316,6 +318,9 @@ def options(precision="fp32", tol=1e-6, tol_kind="sum", max_half_steps=100000, c
     o.flags = ({"auto": 0, "tma": 1, "ldg": 2}[dense_kernel] | (4 if exact_dist else 0) | (0 if transpose else 8)
                | (16 if test_stall else 0) | {"auto": 0, "mma": 32, "one_cta": 512}[sk_product] | (64 if persistent else 0)
                | {"auto": 0, "defer": 128, "arrive": 256}[node_finish])
+    if test_apply is not None:
+        split, both = test_apply
+        o.flags |= (1 + int(split) + 4 * int(both)) << 24
     return o
 
 
@@ -507,12 +512,13 @@ class Solver:
             self.set_potential(prob, 2 * e + 1, f[(int(b), int(a))])
 
     def plan_stats(self) -> dict:
-        st = (C.c_int64 * 16)()
-        _check(_lib.tree_ot_plan_stats(self.h, st, 16))
+        st = (C.c_int64 * 20)()
+        _check(_lib.tree_ot_plan_stats(self.h, st, 20))
         keys = ["directed_edges", "edges", "elements_per_half_step", "matrix_bytes_per_half_step",
                 "apply_tasks_c0", "apply_tasks_c1", "device_bytes", "node_ctas_c0", "node_ctas_c1",
                 "recompute_output_block", "recompute_ctas_per_sm", "recompute_variant", "dense_tma",
-                "persistent", "node_defer", "sk_product"]
+                "persistent", "node_defer", "sk_product", "factored_edges", "factored_split", "both_forms",
+                "factored_fallbacks"]
         return dict(zip(keys, [int(x) for x in st]))
 
 

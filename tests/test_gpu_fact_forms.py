@@ -1,0 +1,80 @@
+"""Every form of the factored recomputed-cost apply, fixed by a test option instead of the
+autotuner's timing: one warp per block of outputs or 2, 4, 8 warps sharing it, in a launch of its
+own or in one with the difference form, and its fallback for frames that moved far.  Group sizes
+64, 32 and 16, 1 to 3 dimensions, neighbours with fewer stages of 64 points than warps sharing them."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import tree_ot as O
+from test_gpu_fact import cloud_star
+from test_gpu_parity import marginal_gap, rel_err
+
+FORMS = [(split, both) for both in (0, 1) for split in range(4)]
+SHAPES = {
+    # (sizes, dim, eps)
+    "few_stages_1d": ((65, 32, 33, 63, 64, 129), 1, 0.2),
+    "few_stages_3d": ((66, 32, 33, 64, 130), 3, 0.5),
+    "sizes_64_32_16_and_difference_2d": ((900, 300, 150, 700, 1100), 2, 0.01),
+    "chunks_1d": ((4097, 70, 33), 1, 0.01),
+    "many_points_2d": ((70, 4133, 513), 2, 0.02),
+}
+
+
+def solver(T, p, split, both, **kw):
+    s = T.Solver([p], T.options(test_apply=(split, both), **kw))
+    st = s.plan_stats()
+    assert st["factored_split"] == split and st["both_forms"] == both
+    return s
+
+
+@pytest.mark.parametrize("exact", [False, True])
+@pytest.mark.parametrize("split,both", FORMS)
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_iterates(name, split, both, exact):
+    import paper_2406_10849_gb300 as T
+    T.load()
+    n, dim, eps = SHAPES[name]
+    p = cloud_star(n, dim, eps, seed=21)
+    with solver(T, p, split, both, exact_dist=exact) as s:
+        if not exact:
+            assert s.plan_stats()["factored_edges"] > 0
+        for steps in (2, 3):
+            s.reset()
+            s.half_steps(steps)
+            got = s.potentials(0)
+            ref = O.run_half_steps(p, steps)
+            assert rel_err(got, ref, p.eps) <= 1e-4
+            assert marginal_gap(p, got, ref) <= 1e-6  # the bar of every FP32 iterate
+
+
+@pytest.mark.parametrize("split,both", FORMS)
+@pytest.mark.parametrize("n,dim,eps", [((400, 300, 260), 1, 0.002), ((1300, 33, 64, 2200), 2, 0.005),
+                                       ((700, 900, 40), 3, 0.05)])
+def test_fallback_of_far_frames(n, dim, eps, split, both):
+    """Potentials that jump by hundreds of eps from point to point: frames far from the messages, sums out of
+    the FP32 range.  Those groups are summed by the difference form, and the count shows that it ran.
+
+    Bound on a message, in nats: a cost formed in FP32 has a relative error of (dim + 2) 2^-24, and with such
+    potentials the largest costs count; 64 units of 2^-24 for the argument's, the exponential's and the sum's
+    roundings.  Two half-steps, and a node's mean over its edges: three times that."""
+    import paper_2406_10849_gb300 as T
+    T.load()
+    p = cloud_star(n, dim, eps, seed=3)
+    rng = np.random.default_rng(0)
+    f = {}
+    for a, b in np.asarray(p.edges):
+        for j, k in ((int(a), int(b)), (int(b), int(a))):
+            f[(j, k)] = 200.0 * eps * (2.0 * rng.random(int(p.n[j])) - 1.0)
+    ref = O.run_half_steps(p, 2, f)
+    with solver(T, p, split, both) as s:
+        assert s.plan_stats()["factored_edges"] > 0
+        s.set_potentials(f)
+        before = s.plan_stats()["factored_fallbacks"]
+        s.half_steps(2)
+        assert s.plan_stats()["factored_fallbacks"] > before
+        got = s.potentials(0)
+    worst = max(float(O.cost(p, int(a), int(b)).max()) for a, b in np.asarray(p.edges))
+    bound = ((dim + 2) * worst / eps + 64.0) * 2.0 ** -24
+    assert max(float(np.abs(got[k] - ref[k]).max()) for k in ref) / eps <= 3.0 * bound
