@@ -86,21 +86,22 @@ __device__ __forceinline__ void add_to(float& s, float& l, float v) {
 
 // A lane's four outputs summed by the difference form over the points [y0, y1) of its slice (every
 // kSlices-th), each relative to its own maximum: the fallback of a group whose frames do not fit.  Two passes
-// (maximum, sum) over points staged in the warp's shared memory, 64 at a time.  out: frames in, (frame, sum) out.
+// (maximum, sum) over points staged in the warp's shared memory, 64 at a time.  A stage's terms are summed in
+// FP32 (32 at most) and the stages as a two-float.  out: frames in, (frame, sum) out.
 template <int D>
 __device__ __noinline__ void fact_slow(const ApplyArgs& A, const float4* rows, int64_t coord_own, int64_t coord_nbr,
                                        int64_t h_off, int y0, int y1, int slice, int slices, float shi, float slo,
                                        float4* stage, float2* out) {
   float* wts = reinterpret_cast<float*>(stage + 64);
   const int lane = threadIdx.x & 31;
-  float px[4][D], cm[4], R[4], acc[4];
+  float px[4][D], cm[4], R[4], S[4], Sl[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int row = __float_as_int(rows[r].w);
 #pragma unroll
     for (int k = 0; k < D; ++k) px[r][k] = A.coords[coord_own + (int64_t)row * D + k];
     cm[r] = -kInf;
-    acc[r] = 0.f;
+    S[r] = Sl[r] = 0.f;
     R[r] = out[r].x;
   }
   for (int pass = 0; pass < 2; ++pass) {
@@ -116,6 +117,7 @@ __device__ __noinline__ void fact_slow(const ApplyArgs& A, const float4* rows, i
         stage[lane + 32 * h] = make_float4(q[0], D > 1 ? q[D > 1 ? 1 : 0] : 0.f, D > 2 ? q[D > 2 ? 2 : 0] : 0.f, hh);
       }
       __syncwarp();
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 2
       for (int i = slice; i < 64; i += slices) {
         const float4 q = stage[i];
@@ -139,6 +141,9 @@ __device__ __noinline__ void fact_slow(const ApplyArgs& A, const float4* rows, i
             acc[r] = fmaf(ex2(t), w, acc[r]);
         }
       }
+      if (pass == 1)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) add_to(S[r], Sl[r], acc[r]);
     }
     if (pass == 0)
 #pragma unroll
@@ -146,7 +151,7 @@ __device__ __noinline__ void fact_slow(const ApplyArgs& A, const float4* rows, i
         if (cm[r] > -kInf) R[r] += quant(cm[r]);
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) out[r] = make_float2(R[r], acc[r]);
+  for (int r = 0; r < 4; ++r) out[r] = make_float2(R[r], S[r] + Sl[r]);
   __syncwarp();
 }
 

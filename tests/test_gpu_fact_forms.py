@@ -78,3 +78,37 @@ def test_fallback_of_far_frames(n, dim, eps, split, both):
     worst = max(float(O.cost(p, int(a), int(b)).max()) for a, b in np.asarray(p.edges))
     bound = ((dim + 2) * worst / eps + 64.0) * 2.0 ** -24
     assert max(float(np.abs(got[k] - ref[k]).max()) for k in ref) / eps <= 3.0 * bound
+
+
+@pytest.mark.parametrize("split", range(4))
+@pytest.mark.parametrize("n,dim", [(8200, 1), (6001, 2), (4096, 3)])
+def test_fallback_sums_long_supports(n, dim, split):
+    """A message shifted by hundreds of binades since the last half-step: every group's sum over a long support
+    comes from the fallback.  rms error in nats: a cost's FP32 rounding, (dim + 2) 2^-24 of it, weighted by the
+    terms, and 4 units of 2^-24 for the exponential, the operand and the sum."""
+    import gen
+    import paper_2406_10849_gb300 as T
+    T.load()
+    rng = np.random.default_rng(dim)
+    coords = [rng.random((k, dim)).astype(np.float32) for k in (n, 300, 64)]
+    marg = {1: rng.dirichlet(np.ones(300)), 2: rng.dirichlet(np.ones(64))}
+    p = gen.TreeProblem(name="long", edges=gen.star_edges(2), n=np.array([n, 300, 64], np.int32),
+                        fixed=np.array([False, True, True]), marginals={k: m / m.sum() for k, m in marg.items()},
+                        eps=0.5, coords=coords, cost_scale=1.0)
+    with solver(T, p, split, 0) as s:
+        s.half_steps(3)
+        f = s.potentials(0)
+        f[(0, 1)] = f[(0, 1)] + 150.0 * p.eps
+        s.set_potentials(f)
+        f = s.potentials(0)
+        before = s.plan_stats()["factored_fallbacks"]
+        s.half_steps(1)
+        assert s.plan_stats()["factored_fallbacks"] - before >= 300 // 64
+        got = s.potentials(0)[(1, 0)] / p.eps
+    C = O.cost(p, 1, 0) / p.eps
+    a = f[(0, 1)][None, :] / p.eps - C
+    top = a.max(1, keepdims=True)
+    w = np.exp(a - top)
+    err = got + top[:, 0] + np.log(w.sum(1))
+    bound = ((dim + 2) * (w * C).sum(1) / w.sum(1) + 4.0) * 2.0 ** -24
+    assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(np.mean(bound ** 2))
