@@ -412,8 +412,10 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * [16] directed edges whose recomputed-cost apply has the factored form, [17]
  * log2 of the warps that share a block of its outputs, [18] 1 when its tasks and
  * the difference form's run in one launch, [19] groups of outputs that it has
- * summed by the difference form since create (read from the device, after
- * everything queued before: only when nstats > 19). */
+ * summed by the difference form since create because their frames did not fit
+ * (read from the device, after everything queued before: only when nstats > 19),
+ * [20] points of the factored edges' nodes in groups too wide for the factored
+ * form (always summed by the difference form). */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);
 
 /* Launch timing (no paper counterpart: measurement support).  While enabled,

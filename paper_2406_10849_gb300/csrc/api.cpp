@@ -222,6 +222,7 @@ struct tree_ot_handle {
   int32_t rec_ob = kRecOut;                // recomputed-cost output block (autotuned)
   int32_t f64_rows = 64;                   // FP64 apply: outputs per task (1 .. 8, or 64)
   int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
+  int64_t wide_points = 0;                 // points of factored nodes in groups that take the difference form
   bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
   std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
   int32_t item_begin[2][4] = {}, item_count[2][4] = {};  // per dimension
@@ -1105,7 +1106,7 @@ int tune_applies(tree_ot_handle* h, cudaStream_t s, cudaEvent_t e0, cudaEvent_t 
     RC_TRY(upload_tasks(h, s));
     RC_TRY(time_applies(h, s, APPLY_FACT, e0, e1, &ms));
     if (ms > 1.3f * best) break;  // more warps per group only get slower from here
-    if (ms < best) {
+    if (ms < 0.95f * best) {  // fewer warps at equal times: the persistent launch prefers them
       best = ms;
       cfg->split = lw;
     }
@@ -1337,8 +1338,8 @@ int plan_shared_kernels(tree_ot_handle* h, const tree_ot_problem* probs, int32_t
 }
 
 // Compact groups of the support points of squared-Euclidean problems (group.cu): measures the groups of
-// 64, 32, 16 and 8 points of every node, picks each node's size by kGroupKappa, sorts the points and sets the
-// directed edges in factored form to a single reduction split (nodes and dedges are uploaded again after).
+// 64, 32 and 16 points of every node, picks each node's size by the share of wide groups, sorts the points and
+// sets the directed edges in factored form to a single reduction split (nodes and dedges are uploaded again after).
 int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   if (h->fp64) return TREE_OT_OK;
   std::vector<GroupWork> work;
@@ -1350,29 +1351,37 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   }
   if (work.empty()) return TREE_OT_OK;
   GroupWork* d_work = nullptr;
-  float* d_meas = nullptr;
-  std::vector<float> meas(kGroupSizes * work.size());
+  int32_t *d_meas = nullptr, *d_wide = nullptr;
+  std::vector<int32_t> block_wide;  // per block of 64 slots: outputs in wide groups
+  std::vector<int32_t> meas(kGroupSizes * work.size());
   const int32_t nw = (int32_t)work.size();
   cudaError_t e = cudaMalloc((void**)&d_work, sizeof(GroupWork) * work.size());
-  if (e == cudaSuccess) e = cudaMalloc((void**)&d_meas, sizeof(float) * meas.size());
+  if (e == cudaSuccess) e = cudaMalloc((void**)&d_meas, sizeof(int32_t) * meas.size());
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_work, work.data(), sizeof(GroupWork) * work.size(), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, d_meas, s);
+  if (e == cudaSuccess) e = launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, d_meas, s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(meas.data(), d_meas, sizeof(float) * meas.size(), cudaMemcpyDeviceToHost, s);
+    e = cudaMemcpyAsync(meas.data(), d_meas, sizeof(int32_t) * meas.size(), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   int rc = e == cudaSuccess ? TREE_OT_OK : cuda_fail(e, "measuring the point groups");
-  int64_t slots = 0;
+  // large: more than four blocks of 64 outputs per colour for each of the GPU's 16 warps per SM
+  int64_t blocks = 0, slots = 0;
+  for (const GroupWork& w : work) blocks += (int64_t)((w.cnt + 63) / 64) * h->nodes[w.node].deg;
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const bool many = blocks > (int64_t)2 * 4 * 16 * nsm;
   for (size_t i = 0; rc == TREE_OT_OK && i < work.size();) {
     NodeD& nd = h->nodes[work[i].node];
-    double r2[kGroupSizes] = {};
+    int64_t wide[kGroupSizes] = {};
     size_t k = i;
     for (; k < work.size() && work[k].node == work[i].node; ++k)
-      for (int v = 0; v < kGroupSizes; ++v) r2[v] += meas[kGroupSizes * k + v];
-    for (int v = 0; v < kGroupSizes && nd.gs == 0; ++v) {
-      const int32_t gs = 64 >> v, ng = (nd.n + gs - 1) / gs;
-      if (h->probs[nd.prob].s2_scaled * (r2[v] / ng) <= kGroupKappa[v]) nd.gs = gs;
-    }
+      for (int v = 0; v < kGroupSizes; ++v) wide[v] += meas[kGroupSizes * k + v];
+    for (int v = 0; v < kGroupSizes && nd.gs == 0; ++v)
+      if (wide[v] * kGroupWide[many ? 0 : 1] <= nd.n) {
+        nd.gs = 64 >> v;
+        h->wide_points += wide[v];
+      }
     if (nd.gs) {
       nd.slot_off = slots;
       slots += align_up(nd.n, 64);
@@ -1382,15 +1391,21 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   if (rc == TREE_OT_OK && slots > 0 &&
       !((rc = h->alloc(&h->d_slot_x, slots)) || (rc = h->alloc(&h->d_slot_q, slots)) ||
         (rc = h->alloc(&h->d_grp, 3 * (slots / 8))) || (rc = h->alloc(&h->d_fallbacks, 1)))) {
-    e = cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s);
+    block_wide.assign((size_t)(slots / 64), 0);
+    e = cudaMalloc((void**)&d_wide, sizeof(int32_t) * block_wide.size());
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_wide, 0, sizeof(int32_t) * block_wide.size(), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
       e = launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
-                             h->d_grp, s);
+                             h->d_grp, d_wide, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(block_wide.data(), d_wide, sizeof(int32_t) * block_wide.size(), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) rc = cuda_fail(e, "building the point groups");
   }
+  cudaFree(d_wide);
   cudaFree(d_work);
   cudaFree(d_meas);
   if (rc) return rc;
@@ -1420,9 +1435,11 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   for (int c = 0; c < 2; ++c) {
     auto& v = h->items[c];
     auto dim = [&](const FactItem& x) { return h->probs[x.prob].dim; };
+    // an output of a wide group takes about three times the time of the others
+    auto cost = [&](const FactItem& x) { return (int64_t)(x.nrow + 2 * block_wide[(size_t)(x.slot0 / 64)]) * x.n_nbr; };
     std::stable_sort(v.begin(), v.end(), [&](const FactItem& x, const FactItem& y) {
       if (dim(x) != dim(y)) return dim(x) < dim(y);
-      return (int64_t)x.nrow * x.n_nbr > (int64_t)y.nrow * y.n_nbr;
+      return cost(x) > cost(y);
     });
     for (const FactItem& x : v) ++h->item_count[c][dim(x)];
     for (int k = 1; k < 4; ++k) h->item_begin[c][k] = h->item_begin[c][k - 1] + h->item_count[c][k - 1];
@@ -2803,7 +2820,7 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
   }
-  const int64_t v[20] = {(int64_t)h->dedges.size(),
+  const int64_t v[21] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2822,8 +2839,9 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         fact_edges,
                         (int64_t)h->fact_split,
                         (int64_t)(h->both_forms ? 1 : 0),
-                        (int64_t)fallbacks};
-  for (int32_t i = 0; i < nstats && i < 20; ++i) stats[i] = v[i];
+                        (int64_t)fallbacks,
+                        h->wide_points};
+  for (int32_t i = 0; i < nstats && i < 21; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

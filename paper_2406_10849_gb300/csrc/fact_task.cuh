@@ -23,9 +23,9 @@
 // x'_k Y_k, of size s r |y'|; cy comes from a least-squares slope of the
 // previous messages' frames over the group, which makes y' of the significant
 // terms small (the spread of the targets, not the transport distance).  The
-// planner uses this form only where s r^2 (r: half the longer side of the
-// groups) is small enough that the result is at least as accurate as the
-// difference form (see group.cu).
+// planner marks groups where s r^2 (r: the largest coordinate of x') is too large
+// for the result to be at least as accurate as the difference form's; those are
+// summed by that form (see group.cu).
 //
 // Range.  One frame F per group: an output's sum is about 2^(b(x) - F), b the
 // previous message's frame less off(x).  F lies kFactRoom binades above the
@@ -257,6 +257,7 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
   FactRaw<D> raw;  // the first stage, in flight during the set-up
   fact_load<D>(A, it.coord_nbr, it.rev_off, min(y, last), raw);
   bool good[2];  // the lane's two outputs: r = 0, 1 -> lane + 32 r
+  bool wide[2] = {false, false};  // of a group too wide for the factored form
   {
     float xp[2][D], frm[2], v[2];
     float2 off[2];
@@ -281,6 +282,8 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
       if (NG > 1 || r == 0) {  // one group over both outputs of every lane: worked out once
         const float4* gr = A.grp + 3 * ((it.slot0 + g * GS) / 8);
         const float4 g0 = gr[0], g1 = gr[1], g2 = gr[2];
+        wide[r] = g2.z != 0.f;
+        if (NG == 1) wide[1] = wide[0];
         // slope of the frames over the group: 2s (cy - c)
         const float vref = __shfl_sync(0xffffffffu, NG == 1 ? v[0] : v[r], lane & ~(kSpan - 1));
         float gs[D], e[D];
@@ -355,8 +358,11 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
         lo[r] = fmaxf(lo[r], __shfl_xor_sync(0xffffffffu, lo[r], o));
       }
       const float F = hi[r] > -kInf ? quant(hi[r]) + kFactRoom : 0.f;
-      good[r] = !(hi[r] + lo[r] > kFactSpread);
-      if ((lane & (kSpan - 1)) == 0) gc[8 * ((lane + 32 * r) / GS)] = F;
+      good[r] = !(hi[r] + lo[r] > kFactSpread) && !wide[r];
+      if ((lane & (kSpan - 1)) == 0) {
+        gc[8 * ((lane + 32 * r) / GS)] = F;
+        gc[8 * ((lane + 32 * r) / GS) + 7] = wide[r] ? 1.f : 0.f;
+      }
       // frame F + off back on the grid, and what it leaves over, for the end
       const float2 fs = two_sum(F, off[r].x);
       const float q = quant(fs.x);
@@ -368,6 +374,12 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
 #pragma unroll 1
   for (int g = 0; g < NG; ++g) {
     if (g * GS >= nrow) break;  // warp-uniform
+    if (gc[8 * g + 7] != 0.f) {  // warp-uniform: a wide group's sums come from the fallback below
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (slice == 0) sums[g * GS + ll + kLanes * r] = make_float2(0.f, 0.f);
+      continue;
+    }
     // (x, x) pairs, opaque so that they stay in registers instead of being rebuilt before every use
     uint64_t X[4][D];
 #pragma unroll
@@ -503,7 +515,7 @@ __device__ __forceinline__ void fact_block(const ApplyArgs& A, const FactItem& i
       const unsigned m = GS == 64 ? bad[0] | bad[1]
                                   : (g * GS < 32 ? bad[0] : bad[1]) & (((GS < 32 ? 1u << (GS & 31) : 0u) - 1u) << ((g * GS) & 31));
       if (!m) continue;  // warp-uniform
-      if (lane == 0 && share == 0) atomicAdd(A.fallbacks, 1ull);
+      if (lane == 0 && share == 0 && gc[8 * g + 7] == 0.f) atomicAdd(A.fallbacks, 1ull);
       float4 rw[4];
       float2 so[4];
 #pragma unroll

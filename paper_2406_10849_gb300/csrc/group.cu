@@ -4,24 +4,38 @@
 //
 // Sort-tile-recursive order: the points of a chunk (at most 4096, in their
 // given order) are sorted along the first coordinate into slabs, each slab along
-// the second into tiles (and along the third), a tile holding one group.  One
+// the second into tiles (and along the third), a tile holding one group.  Slabs
+// and tiles hold whole groups, as even in number as they divide: with the
+// remainder in a last narrow slab its few groups spanned the slab's whole
+// length (2048 uniform points in the square: one group in 16 had 6 times the
+// mean's squared extent, now the widest has twice).  One
 // CTA per chunk, a bitonic sort of 64-bit keys (segment, coordinate, index) in
 // shared memory; a support of more than 4096 points is grouped chunk by chunk,
 // its groups as compact as those of 4096 points spread over the same region.
 //
-// Which size.  The factored form's error grows with kappa = s r^2 (s = scale
-// log2(e) / eps, r^2 the mean over the groups of the squared half of a group's
-// longer side), the difference form's with the squared transport distance.
-// Measured on the GPU against FP64 iterates (rms error of the potentials in
-// units of eps after 2 and 6 half-steps, random trees of 64..900 points, D = 1..3,
-// eps 0.004..0.05, geometric mean over 27 shapes): difference form 1.35e-7;
-// factored within kappa limits 2, 2, 2: 1.21e-7; 4, 3, 3: 1.33e-7, but single
-// shapes then lose up to 1.8x (2-D, 900 points, eps 0.004), all of them through
-// groups of 32 and 16 above 2.  The iterates' floor (largest marginal error after
-// 1600-3000 half-steps): 2.4e-7 -> 1.4e-7 on 16 x 16 stars, 1.2e-7 -> 0.7e-7 on 2-D
-// clouds at eps 0.02, 1.0e-7 -> 0.6e-7 on 1-D barycenters.  A node takes the
-// largest group size within its limit (larger groups share a staged value among
-// more outputs), and the difference form if none is.
+// Which groups.  The factored form's error grows with kappa = s r^2 of the
+// output's own group (s = scale log2(e) / eps, r the largest coordinate
+// difference to the group's centre), the difference form's with the squared
+// transport distance.  Measured on the GPU against FP64 messages of the same
+// potentials (uniform, radially concentrated and outlier-ridden supports of 400 to 4096
+// points, D = 1..3, eps 0.002..0.03; rms and largest error of the message in
+// nats, by the kappa of the output's group, factored against difference form):
+//   kappa    <= 1             1..2            2..4            5..6            8..10           > 20
+//   rms      0.7e-7 / 1.2e-7  0.8e-7 / 1.2e-7 0.9e-7 / 1.2e-7 0.9e-7 / 1.2e-7 1.1e-7 / 1.2e-7 5.9e-7 / 1.5e-7
+//   largest  4.0e-7 / 5.9e-7  3.9e-7 / 5.6e-7 5.3e-7 / 5.3e-7 1.3e-6 / 0.6e-6 1.2e-6 / 0.9e-6 8.5e-6 / 1.5e-6
+// A group takes the factored form up to kappa = 4 (groups of 16 in three
+// dimensions up to 2: 1.3e-7 against 1.1e-7 between 2 and 4), where neither error
+// is larger than the difference form's; a wider one is summed by the difference
+// form (the fallback in fact_task.cuh, about four times a group's time).  A node
+// takes the largest group size (larger groups share a staged value among more
+// outputs) that leaves few enough of its points in wide groups, and the
+// difference form throughout if none does: an eighth of them on a large handle,
+// whose per-warp queue takes the costlier blocks first (128 trees of 128-2048
+// points, 16 half-steps, shares of 1/32, 1/16, 1/8: 11.23, 11.05, 10.91 ms), a 32nd on
+// a small one, where a CTA waits for its slowest warp (64 trees of 64-512 points,
+// 32 half-steps, 1/32 and 1/8: 1.71, 1.82 ms).  (With the limit on the node's mean
+// kappa instead, single groups of clustered supports ran factored at kappa 40
+// and beyond.)
 #include <cmath>
 
 #include "internal.h"
@@ -54,12 +68,15 @@ __device__ void bitonic_sort(uint64_t* k, int m) {
   __syncthreads();
 }
 
-// the smallest q with q^p >= v (small integers)
+// the p-th root of v to the nearest integer (p = 2 or 3, small v >= 1)
 __device__ __forceinline__ int iroot(int v, int p) {
   int q = 1;
-  while ((p == 2 ? q * q : q * q * q) < v) ++q;
+  while ((p == 2 ? (2 * q + 1) * (2 * q + 1) / 4 : (2 * q + 1) * (2 * q + 1) * (2 * q + 1) / 8) < v) ++q;
   return q;
 }
+
+// part k of n groups in S parts begins at group k n / S; the part that holds group g
+__device__ __forceinline__ int part_of(int g, int n, int S) { return ((g + 1) * S - 1) / n; }
 
 // key order of the chunk's points for groups of gs; on return the low 16 bits
 // of keys[i] are the chunk-relative index of the i-th point
@@ -70,20 +87,18 @@ __device__ void str_order(const float* x, int D, int cnt, int m, int gs, uint64_
   if (D == 1) return;
   const int ng = (cnt + gs - 1) / gs;
   const int S = iroot(ng, D);
-  const int per = (ng + S - 1) / S * gs;  // points per slab
   for (int i = threadIdx.x; i < cnt; i += kGroupThreads) {
     const uint32_t idx = (uint32_t)keys[i] & 0xffffu;
-    keys[i] = ((uint64_t)(i / per) << 48) | ((uint64_t)float_key(x[(int64_t)idx * D + 1]) << 16) | idx;
+    const int slab = part_of(i / gs, ng, S);
+    keys[i] = ((uint64_t)slab << 48) | ((uint64_t)float_key(x[(int64_t)idx * D + 1]) << 16) | idx;
   }
   bitonic_sort(keys, m);
   if (D == 2) return;
   for (int i = threadIdx.x; i < cnt; i += kGroupThreads) {
     const uint32_t idx = (uint32_t)keys[i] & 0xffffu;
-    const int slab = i / per, in = i - slab * per;
-    const int ng2 = (min(per, cnt - slab * per) + gs - 1) / gs;
-    const int S2 = iroot(ng2, 2);
-    const int p2 = (ng2 + S2 - 1) / S2 * gs;
-    const uint64_t seg = (uint64_t)slab * 64 + in / p2;
+    const int slab = part_of(i / gs, ng, S);
+    const int g0 = slab * ng / S, ng2 = (slab + 1) * ng / S - g0;
+    const uint64_t seg = (uint64_t)slab * 64 + part_of(i / gs - g0, ng2, iroot(ng2, 2));
     keys[i] = (seg << 48) | ((uint64_t)float_key(x[(int64_t)idx * D + 2]) << 16) | idx;
   }
   bitonic_sort(keys, m);
@@ -95,43 +110,57 @@ __device__ __forceinline__ int pow2_at_least(int n) {
   return m;
 }
 
-// sum over the chunk's groups of (half the longer side)^2, for every group size
+// the grid of split_coords_kernel
+__device__ __forceinline__ float grid_unit(float cm) {
+  int e = 0;
+  if (cm > 0.f) (void)frexpf(cm, &e);
+  return ldexpf(1.f, e - 10);
+}
+
+// the centre of the points keys[i0 .. i1): their mean, on the grid
+__device__ __forceinline__ void group_centre(const float* x, int D, const uint64_t* keys, int i0, int i1, float unit,
+                                             float* c) {
+  for (int k = 0; k < D; ++k) {
+    float sum = 0.f;
+    for (int i = i0; i < i1; ++i) sum += x[(int64_t)((uint32_t)keys[i] & 0xffffu) * D + k];
+    if (i1 > i0) c[k] = rintf(sum / (float)(i1 - i0) / unit) * unit;
+  }
+}
+
+// too wide for the factored form: kappa = s r^2 above the limit (false for no points)
+__device__ __forceinline__ bool group_wide(int gs, int D, float s, float r) {
+  return !(s * r * r <= (gs == 16 && D == 3 ? kGroupKappa16 : kGroupKappa));
+}
+
+// the points of the chunk that lie in wide groups, for every group size
 __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const GroupWork* work, const NodeD* nodes,
                                                                       const ProbD* probs, const float* coords,
-                                                                      float* out) {
+                                                                      const uint32_t* cmax, int32_t* out) {
   __shared__ uint64_t keys[kGroupChunk];
-  __shared__ float part[kGroupThreads];
+  __shared__ int s_wide;
   const GroupWork w = work[blockIdx.x];
   const NodeD nd = nodes[w.node];
   const int D = probs[nd.prob].dim;
+  const float s = probs[nd.prob].s2_scaled;
   const float* x = coords + nd.coord_off + (int64_t)w.x0 * D;
+  const float unit = grid_unit(__uint_as_float(cmax[nd.prob]));
   const int m = pow2_at_least(w.cnt);
   for (int v = 0; v < kGroupSizes; ++v) {
     const int gs = 64 >> v;
     str_order(x, D, w.cnt, m, gs, keys);
-    const int ng = (w.cnt + gs - 1) / gs;
-    float r2 = 0.f;
-    for (int g = threadIdx.x; g < ng; g += kGroupThreads) {
-      float side = 0.f;
-      for (int k = 0; k < D; ++k) {
-        float lo = INFINITY, hi = -INFINITY;
-        for (int i = g * gs; i < min((g + 1) * gs, w.cnt); ++i) {
-          const float c = x[(int64_t)((uint32_t)keys[i] & 0xffffu) * D + k];
-          lo = fminf(lo, c);
-          hi = fmaxf(hi, c);
-        }
-        side = fmaxf(side, hi - lo);
-      }
-      r2 += 0.25f * side * side;
-    }
-    part[threadIdx.x] = r2;
+    if (threadIdx.x == 0) s_wide = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      float s = 0.f;
-      for (int i = 0; i < kGroupThreads; ++i) s += part[i];
-      out[kGroupSizes * blockIdx.x + v] = s;
+    for (int g = threadIdx.x; g < (w.cnt + gs - 1) / gs; g += kGroupThreads) {
+      const int i0 = g * gs, i1 = min(i0 + gs, w.cnt);
+      float c[3] = {0.f, 0.f, 0.f}, r = 0.f;
+      group_centre(x, D, keys, i0, i1, unit, c);
+      for (int i = i0; i < i1; ++i)
+        for (int k = 0; k < D; ++k)
+          r = fmaxf(r, fabsf(x[(int64_t)((uint32_t)keys[i] & 0xffffu) * D + k] - c[k]));
+      if (group_wide(gs, D, s, r)) atomicAdd(&s_wide, i1 - i0);
     }
     __syncthreads();
+    if (threadIdx.x == 0) out[kGroupSizes * blockIdx.x + v] = s_wide;
   }
 }
 
@@ -139,7 +168,7 @@ __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const Grou
 __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupWork* work, const NodeD* nodes,
                                                                     const ProbD* probs, const float* coords,
                                                                     const uint32_t* cmax, float4* slot_x,
-                                                                    float2* slot_q, float4* grp) {
+                                                                    float2* slot_q, float4* grp, int32_t* block_wide) {
   __shared__ uint64_t keys[kGroupChunk];
   const GroupWork w = work[blockIdx.x];
   const NodeD nd = nodes[w.node];
@@ -149,21 +178,15 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
   const double s = probs[nd.prob].cost_scale * kLog2e * probs[nd.prob].inv_eps;
   const float* x = coords + nd.coord_off + (int64_t)w.x0 * D;
   str_order(x, D, w.cnt, pow2_at_least(w.cnt), gs, keys);
-  const float cm = __uint_as_float(cmax[nd.prob]);
-  int e = 0;
-  if (cm > 0.f) (void)frexpf(cm, &e);
-  const float unit = ldexpf(1.f, e - 10);  // the grid of split_coords_kernel
+  const float unit = grid_unit(__uint_as_float(cmax[nd.prob]));
   // a chunk but the last holds a multiple of 64 points; pads run to the end of the last block of 64
   const int slots = (w.cnt + 63) / 64 * 64;
   for (int g = threadIdx.x; g < slots / gs; g += kGroupThreads) {
     const int i0 = g * gs, i1 = min(i0 + gs, w.cnt);
     float c[3] = {0.f, 0.f, 0.f};
     float M[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // second moments 00 01 02 11 12 22
-    for (int k = 0; k < D; ++k) {
-      float sum = 0.f;
-      for (int i = i0; i < i1; ++i) sum += x[(int64_t)((uint32_t)keys[i] & 0xffffu) * D + k];
-      if (i1 > i0) c[k] = rintf(sum / (float)(i1 - i0) / unit) * unit;
-    }
+    float far = 0.f;  // the largest coordinate difference to the centre
+    group_centre(x, D, keys, i0, i1, unit, c);
     for (int i = i0; i < i0 + gs; ++i) {
       const uint32_t idx = (uint32_t)keys[min(i, w.cnt - 1)] & 0xffffu;  // pads repeat the last point
       float d[3] = {0.f, 0.f, 0.f};
@@ -172,6 +195,7 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
         for (int k = 0; k < D; ++k) {
           const float v = x[(int64_t)idx * D + k];
           d[k] = v - c[k];
+          far = fmaxf(far, fabsf(d[k]));
           const double dd = (double)v - (double)c[k];
           q += dd * dd;
         }
@@ -204,24 +228,26 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
     float4* r = grp + 3 * ((nd.slot_off + w.x0 + i0) / 8);
     r[0] = make_float4(c[0], c[1], c[2], unit);
     r[1] = make_float4(I[0], I[1], I[2], I[3]);
-    r[2] = make_float4(I[4], I[5], 0.f, 0.f);
+    const bool wide = i1 > i0 && group_wide(gs, D, probs[nd.prob].s2_scaled, far);
+    r[2] = make_float4(I[4], I[5], wide ? 1.f : 0.f, 0.f);
+    if (wide) atomicAdd(&block_wide[(nd.slot_off + w.x0 + i0) / 64], i1 - i0);
   }
 }
 
 }  // namespace
 
 cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, float* out, cudaStream_t s) {
+                                 const float* coords, const uint32_t* cmax, int32_t* out, cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  group_measure_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, out);
+  group_measure_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
                                const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
-                               cudaStream_t s) {
+                               int32_t* block_wide, cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  group_build_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, slot_x, slot_q, grp);
+  group_build_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, slot_x, slot_q, grp, block_wide);
   return cudaGetLastError();
 }
 

@@ -94,10 +94,12 @@ constexpr int kGroupChunk = 4096;
 struct GroupWork {
   int32_t node, x0, cnt;
 };
-// The largest kappa = s r^2 of a node's groups of 64, 32 and 16 points at which the factored apply is
-// used (see group.cu); below kGroupMin points on either side the difference form runs
+// The largest kappa = s r^2 of a group (64, 32 or 16 points) that takes the factored form, and the largest share
+// 1 / kGroupWide of a node's points in wider groups, on large handles and on others (see group.cu); below
+// kGroupMin points on either side the difference form runs
 constexpr int kGroupSizes = 3;  // 64, 32, 16
-constexpr float kGroupKappa[kGroupSizes] = {3.f, 2.f, 2.f};
+constexpr float kGroupKappa = 4.f, kGroupKappa16 = 2.f;  // (groups of 16 in three dimensions)
+constexpr int kGroupWide[2] = {8, 32};
 constexpr int kGroupMin = 32;
 
 struct NodeChunk {
@@ -258,7 +260,7 @@ struct ApplyArgs {
   const float* coords_lo;
   const float4* slot_x;      // per slot: coordinates less the group's centre, point index (as int bits)
   const float2* slot_q;      // per slot: s |x'|^2 as a two-float
-  const float4* grp;         // per 8 slots (at a group's first): 3 x float4, centre, unit, inverse second moments
+  const float4* grp;         // per 8 slots (at a group's first): 3 x float4, centre, unit, inverse second moments, 1 = wide
   unsigned long long* fallbacks;  // factored form: groups summed by the difference form instead
   const int32_t* exact;      // per problem: 1 = recompute costs with exact squared distances
   int32_t any_exact;         // host: some problem has exact set (selects the kernel instantiation)
@@ -437,10 +439,10 @@ cudaError_t launch_transpose_pad(const float* src, int64_t src_ld, int32_t rows,
                                  int64_t dst_ld, cudaStream_t s);
 // coordinates split hi + lo for the exact-distance recomputation (cmax: nprob scratch words)
 cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, float* out, cudaStream_t s);
+                                 const float* coords, const uint32_t* cmax, int32_t* out, cudaStream_t s);
 cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
                                const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
-                               cudaStream_t s);
+                               int32_t* block_wide, cudaStream_t s);
 cudaError_t launch_split_coords(const float* coords, const NodeD* nodes, int32_t nnodes, const ProbD* probs,
                                 uint32_t* cmax, int32_t nprob, float* hi, float* lo, cudaStream_t s);
 cudaError_t launch_check(const CheckArgs& a, cudaStream_t s);
