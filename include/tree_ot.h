@@ -415,7 +415,8 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * summed by the difference form since create because their frames did not fit
  * (read from the device, after everything queued before: only when nstats > 19),
  * [20] points of the factored edges' nodes in groups too wide for the factored
- * form (always summed by the difference form). */
+ * form (always summed by the difference form), [21] the most reduction splits of
+ * a factored edge. */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);
 
 /* Launch timing (no paper counterpart: measurement support).  While enabled,

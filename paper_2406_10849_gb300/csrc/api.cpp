@@ -369,6 +369,11 @@ bool fact_edge(const tree_ot_handle* h, const DEdgeD& d) {
   return h->nodes[d.owner].gs > 0 && h->nodes[d.nbr].n >= kGroupMin;
 }
 
+// points of the neighbour per reduction split of a factored edge
+int32_t fact_split_points(int32_t n_nbr, int32_t nsplit) {
+  return (int32_t)align_up((n_nbr + nsplit - 1) / nsplit, 64);
+}
+
 // Apply tasks of both colours, grouped by kernel slot.  rec_ob: largest output
 // block of a recomputed-cost task (256, 512 or 1024 outputs); a task with fewer
 // outputs runs its CTA as G warp groups splitting the reduction points.
@@ -402,15 +407,17 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
           tl.push_back(Task{(int32_t)di, TASK_COL, o0, std::min(kColCols, own.n - o0), s * kColRows,
                             std::min(kColRows, nbn.n - s * kColRows), s, 0});
     } else if (fact_edge(h, d)) {
-      // slots of the owner's groups against all of the neighbour's points, 2^split warps of a CTA per block of 64;
-      // the exact-distance kernel reads the same range as plain outputs, with G warp groups of at most
+      // slots of the owner's groups against a split of the neighbour's points, 2^split warps of a CTA per block of
+      // 64; the exact-distance kernel reads the same range as plain outputs, with G warp groups of at most
       // 1024 / G outputs
-      const int32_t ob = (8 >> h->fact_split) * 64;
+      const int32_t ob = (8 >> h->fact_split) * 64, per = fact_split_points(nbn.n, d.nsplit);
       for (int32_t o0 = 0; o0 < own.n; o0 += ob) {
         const int32_t oc = std::min(ob, own.n - o0);
         int32_t G = 1;
         while (G < 8 && kRecOut / (2 * G) >= oc) G *= 2;
-        tl.push_back(Task{(int32_t)di, TASK_FACT + h->fact_split, o0, oc, 0, nbn.n, 0, G});
+        for (int32_t s = 0; s < d.nsplit; ++s)
+          tl.push_back(Task{(int32_t)di, TASK_FACT + h->fact_split, o0, oc, s * per, std::min(per, nbn.n - s * per), s,
+                            G});
       }
     } else {
       for (int32_t o0 = 0; o0 < own.n; o0 += rec_ob) {
@@ -1339,7 +1346,7 @@ int plan_shared_kernels(tree_ot_handle* h, const tree_ot_problem* probs, int32_t
 
 // Compact groups of the support points of squared-Euclidean problems (group.cu): measures the groups of
 // 64, 32 and 16 points of every node, picks each node's size by the share of wide groups, sorts the points and
-// sets the directed edges in factored form to a single reduction split (nodes and dedges are uploaded again after).
+// sets the reduction splits of the directed edges in factored form (nodes and dedges are uploaded again after).
 int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   if (h->fp64) return TREE_OT_OK;
   std::vector<GroupWork> work;
@@ -1409,28 +1416,42 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   cudaFree(d_work);
   cudaFree(d_meas);
   if (rc) return rc;
+  // Points a warp may walk for its block of 64 outputs: an even share of the colour's work over the GPU's 16 warps
+  // per SM, half as much again, at least 256.  Up to 8 warps share a block's points; beyond that the reduction is
+  // split, its pieces merged by the node update (a leaf of 64 points at a centre of 65536, D = 2: 116 us per
+  // half-step without splits, 602 without the autotuner; 33 and 34 with them).  Without the autotuner, a block gets as many warps as its longest walk asks for.
+  double warp_run[2] = {0.0, 0.0};
+  for (const DEdgeD& d : h->dedges)
+    if (fact_edge(h, d))
+      warp_run[h->nodes[d.owner].colour] += (double)((h->nodes[d.owner].n + 63) / 64) * h->nodes[d.nbr].n;
+  for (double& w : warp_run) w = std::max(256.0, 1.5 * w / (16.0 * nsm));
   for (size_t di = 0; di < h->dedges.size(); ++di) {
     DEdgeD& d = h->dedges[di];
     if (!fact_edge(h, d)) continue;
-    d.nsplit = 1;
     const NodeD &own = h->nodes[d.owner], &nbn = h->nodes[d.nbr];
     const ProbD& pd = h->probs[d.prob];
-    for (int32_t o0 = 0; o0 < own.n; o0 += 64) {
-      FactItem it{};
-      it.slot0 = own.slot_off + o0;
-      it.part_off = d.part_off;
-      it.off = d.off;
-      it.rev_off = d.rev_off;
-      it.coord_nbr = nbn.coord_off;
-      it.nrow = std::min(64, own.n - o0);
-      it.n_nbr = nbn.n;
-      it.dedge = (int32_t)di;
-      it.prob = d.prob;
-      it.gs = own.gs;
-      it.shi = pd.s2_scaled;
-      it.slo = pd.s2_scaled_lo;
-      h->items[own.colour].push_back(it);
-    }
+    const double run = warp_run[own.colour];
+    d.nsplit = std::max(1, std::min((nbn.n + kRecRed - 1) / kRecRed, (int32_t)std::ceil(nbn.n / (8.0 * run))));
+    const int32_t per = fact_split_points(nbn.n, d.nsplit);
+    d.nsplit = (nbn.n + per - 1) / per;
+    while (h->fact_split < 3 && per > run * (1 << h->fact_split)) ++h->fact_split;  // until the autotuner times it
+    for (int32_t o0 = 0; o0 < own.n; o0 += 64)
+      for (int32_t k = 0; k < d.nsplit; ++k) {
+        FactItem it{};
+        it.slot0 = own.slot_off + o0;
+        it.part_off = d.part_off + (int64_t)k * own.n;
+        it.off = d.off;
+        it.rev_off = d.rev_off + (int64_t)k * per;
+        it.coord_nbr = nbn.coord_off + (int64_t)k * per * pd.dim;
+        it.nrow = std::min(64, own.n - o0);
+        it.n_nbr = std::min(per, nbn.n - k * per);
+        it.dedge = (int32_t)di;
+        it.prob = d.prob;
+        it.gs = own.gs;
+        it.shi = pd.s2_scaled;
+        it.slo = pd.s2_scaled_lo;
+        h->items[own.colour].push_back(it);
+      }
   }
   for (int c = 0; c < 2; ++c) {
     auto& v = h->items[c];
@@ -1448,7 +1469,6 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
     CUDA_TRY(cudaMemcpyAsync(h->d_items[c], v.data(), sizeof(FactItem) * v.size(), cudaMemcpyHostToDevice, s));
   }
   CUDA_TRY(cudaStreamSynchronize(s));
-  build_apply_tasks(h, kRecOut);
   return TREE_OT_OK;
 }
 
@@ -1893,14 +1913,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     if (most <= (int64_t)64 * 8 * nsm)
       for (h->f64_rows = 1; h->f64_rows < 8 && (int64_t)h->f64_rows * nsm < most;) h->f64_rows *= 2;
   }
-  // device task arrays are sized for the finest output blocking the autotuner may pick, in either form
-  // of the recomputed-cost apply (an edge in factored form takes at most n / 64 tasks)
-  build_apply_tasks(h, 256);
-  for (int c = 0; c < 2; ++c) h->task_cap[c] = (int64_t)h->tasks[c].size();
-  for (const DEdgeD& d : h->dedges)
-    if (!h->fp64 && h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
-      h->task_cap[h->nodes[d.owner].colour] += (h->nodes[d.owner].n + 63) / 64;
-  build_apply_tasks(h, kRecOut);
   // absorbed BF16 phase: apply tasks per colour and absorption blocks (stored-cost edges only)
   h->lowp = o.apply_mode == TREE_OT_APPLY_BF16 && !h->fp64;
   if (h->lowp) {
@@ -1965,7 +1977,6 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   if ((rc = h->alloc(&h->d_probs, num_probs)) || (rc = h->alloc(&h->d_nodes, NN)) ||
       (rc = h->alloc(&h->d_edges, NE)) || (rc = h->alloc(&h->d_dedges, ND)) ||
       (rc = h->alloc(&h->d_node_dedges, (int64_t)h->node_dedges.size())) ||
-      (rc = h->alloc(&h->d_tasks[0], h->task_cap[0])) || (rc = h->alloc(&h->d_tasks[1], h->task_cap[1])) ||
       (rc = h->alloc(&h->d_queue, 2 * 2 * kApplySlots)) ||
       (rc = h->alloc(&h->d_owned, (int64_t)h->node_dedges.size())) || (rc = h->alloc(&h->d_chunks[0], (int64_t)h->chunks[0].size())) ||
       (rc = h->alloc(&h->d_chunks[1], (int64_t)h->chunks[1].size())) ||
@@ -2042,6 +2053,19 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
                                         num_probs, h->d_coords_hi, h->d_coords_lo, s);
     if (e != cudaSuccess) return bail(cuda_fail(e, "coordinate split"));
     if ((rc = plan_groups(h, s))) return bail(rc);
+  }
+  {
+    // device task arrays are sized for the finest blocking the autotuner may pick: output blocks of 256 of the
+    // difference form, of 64 of the factored one
+    const int32_t split = h->fact_split;
+    h->fact_split = 3;
+    build_apply_tasks(h, 256);
+    for (int c = 0; c < 2; ++c) {
+      h->task_cap[c] = (int64_t)h->tasks[c].size();
+      if ((rc = h->alloc(&h->d_tasks[c], h->task_cap[c]))) return bail(rc);
+    }
+    h->fact_split = split;
+    build_apply_tasks(h, kRecOut);
   }
   if ((rc = setup_shared_kernels(h, s))) return bail(rc);
   if (!h->fp64) {  // host-resolved records of the fixed leaves' chunks, per colour
@@ -2813,14 +2837,18 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
     for (int c = 0; c < 2; ++c)
       if (g.args[c].ncols > 0)
         sk_form = std::max<int64_t>(sk_form, g.args[c].use_tc ? (g.args[c].tc_pair ? 3 : 2) : 1);
-  int64_t fact_edges = 0;
-  for (const DEdgeD& d : h->dedges) fact_edges += fact_edge(h, d);
+  int64_t fact_edges = 0, fact_splits = 0;
+  for (const DEdgeD& d : h->dedges)
+    if (fact_edge(h, d)) {
+      ++fact_edges;
+      fact_splits = std::max<int64_t>(fact_splits, d.nsplit);
+    }
   unsigned long long fallbacks = 0;
   if (nstats > 19 && h->d_fallbacks) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
   }
-  const int64_t v[21] = {(int64_t)h->dedges.size(),
+  const int64_t v[22] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2840,8 +2868,9 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         (int64_t)h->fact_split,
                         (int64_t)(h->both_forms ? 1 : 0),
                         (int64_t)fallbacks,
-                        h->wide_points};
-  for (int32_t i = 0; i < nstats && i < 21; ++i) stats[i] = v[i];
+                        h->wide_points,
+                        fact_splits};
+  for (int32_t i = 0; i < nstats && i < 22; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

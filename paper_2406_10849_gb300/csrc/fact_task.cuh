@@ -577,11 +577,11 @@ __device__ void fact_task(const ApplyArgs& A, const Task& t, float* sm) {
     it.slot0 += b * 64;
     it.nrow = min(64, t.ocount - b * 64);
   }
-  it.part_off = d.part_off;
+  it.part_off = d.part_off + (int64_t)t.split * own.n;
   it.off = d.off;
-  it.rev_off = d.rev_off;
-  it.coord_nbr = nbn.coord_off;
-  it.n_nbr = nbn.n;
+  it.rev_off = d.rev_off + t.r0;
+  it.coord_nbr = nbn.coord_off + (int64_t)t.r0 * D;
+  it.n_nbr = t.rcount;
   it.dedge = t.dedge;
   it.shi = A.probs[d.prob].s2_scaled;
   it.slo = A.probs[d.prob].s2_scaled_lo;

@@ -213,7 +213,7 @@ struct Task {
   int32_t pad;          // RECOMP: warp groups sharing the task (1, 2, 4, 8); ROW: 1 = rows of CT
 };
 
-// A block of 64 of a directed edge's outputs against all of the neighbour's points, resolved on the host: an item
+// A block of 64 of a directed edge's outputs against a split of the neighbour's points, resolved on the host: an item
 // of the factored apply's per-warp queue (five 16-byte words)
 struct FactItem {
   int64_t slot0;       // the block's first slot
@@ -221,7 +221,7 @@ struct FactItem {
   int64_t off;         // owner-side vectors (frames)
   int64_t rev_off;     // the neighbour's operand
   int64_t coord_nbr;   // the neighbour's coordinates
-  int32_t nrow, n_nbr; // outputs of the block, points of the neighbour
+  int32_t nrow, n_nbr; // outputs of the block, points of the split (a multiple of 64 before the last)
   int32_t dedge, prob;
   int32_t gs, pad;     // group size
   float shi, slo;      // cost scale log2(e) / eps as a two-float

@@ -112,3 +112,28 @@ def test_fallback_sums_long_supports(n, dim, split):
     err = got + top[:, 0] + np.log(w.sum(1))
     bound = ((dim + 2) * (w * C).sum(1) / w.sum(1) + 4.0) * 2.0 ** -24
     assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(np.mean(bound ** 2))
+
+
+@pytest.mark.parametrize("tune", [False, True])
+@pytest.mark.parametrize("n,dim,eps,splits", [
+    ((64, 16384, 33), 2, 0.05, True), ((16385, 64, 65), 1, 0.05, True), ((130, 9001), 3, 0.5, True),
+    ((70, 8255, 40), 2, 0.05, True), ((1024, 1024, 1024), 2, 0.01, False)])
+def test_long_reductions_are_split(n, dim, eps, splits, tune):
+    """Edges between a short and a long support: the long reduction is shared by the eight warps of a CTA and
+    split over CTAs, where an even one keeps a single piece; splits that end in a partial stage or an odd point."""
+    import paper_2406_10849_gb300 as T
+    T.load()
+    p = cloud_star(n, dim, eps, seed=8)
+    with T.Solver([p], T.options(autotune=tune)) as s:
+        st = s.plan_stats()
+        assert st["factored_edges"] > 0
+        assert (st["factored_splits"] > 1) == splits
+        if splits and not tune:
+            assert st["factored_split"] == 3
+        for steps in (2, 3):
+            s.reset()
+            s.half_steps(steps)
+            got = s.potentials(0)
+            ref = O.run_half_steps(p, steps)
+            assert rel_err(got, ref, p.eps) <= 1e-4
+            assert marginal_gap(p, got, ref) <= 1e-6  # the bar of every FP32 iterate
