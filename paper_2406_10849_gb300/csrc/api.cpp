@@ -173,6 +173,22 @@ void treeot::set_last_error(const std::string& msg) { g_err = msg; }
 // the handle
 // ---------------------------------------------------------------------------
 
+// What an apply and a node update read of a handle's exact-distance plan: while some problem runs with exact squared
+// distances, every recomputed cost takes the difference form with its own reduction splits (in place of the
+// factored form's)
+struct ExactPlan {
+  std::vector<DEdgeD> dedges;  // empty: the handle has no factored edges, its one plan serves both
+  std::vector<Task> tasks[2];
+  int32_t slot_begin[2][kApplySlots] = {}, slot_count[2][kApplySlots] = {};
+  int32_t rec_ob = kRecOut;
+  DEdgeD* d_dedges = nullptr;
+  OwnedDEdge* d_owned = nullptr;
+  FixedChunkD* d_fixed[2] = {nullptr, nullptr};
+  Task* d_tasks[2] = {nullptr, nullptr};
+  int32_t* d_fcnt = nullptr;   // item counts of the persistent launch
+  bool ready = false;          // the device arrays are filled (on the first use)
+};
+
 struct tree_ot_handle {
   tree_ot_options opt{};
   bool fp64 = false;
@@ -222,6 +238,7 @@ struct tree_ot_handle {
   int32_t rec_ob = kRecOut;                // recomputed-cost output block (autotuned)
   int32_t f64_rows = 64;                   // FP64 apply: outputs per task (1 .. 8, or 64)
   int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
+  ExactPlan xplan;
   int64_t wide_points = 0;                 // points of factored nodes in groups that take the difference form
   bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
   std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
@@ -377,17 +394,22 @@ int32_t fact_split_points(int32_t n_nbr, int32_t nsplit) {
 // Apply tasks of both colours, grouped by kernel slot.  rec_ob: largest output
 // block of a recomputed-cost task (256, 512 or 1024 outputs); a task with fewer
 // outputs runs its CTA as G warp groups splitting the reduction points.
-void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
+// exact: the exact-distance plan, all of it in the difference form.
+void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob, bool exact = false) {
+  std::vector<Task>* tasks = exact ? h->xplan.tasks : h->tasks;
+  auto* slot_begin = exact ? h->xplan.slot_begin : h->slot_begin;
+  auto* slot_count = exact ? h->xplan.slot_count : h->slot_count;
   for (int c = 0; c < 2; ++c) {
-    h->tasks[c].clear();
-    for (int s2 = 0; s2 < kApplySlots; ++s2) h->slot_begin[c][s2] = h->slot_count[c][s2] = 0;
+    tasks[c].clear();
+    for (int s2 = 0; s2 < kApplySlots; ++s2) slot_begin[c][s2] = slot_count[c][s2] = 0;
   }
-  for (size_t di = 0; di < h->dedges.size(); ++di) {
-    const DEdgeD& d = h->dedges[di];
+  const std::vector<DEdgeD>& dedges = exact ? h->xplan.dedges : h->dedges;
+  for (size_t di = 0; di < dedges.size(); ++di) {
+    const DEdgeD& d = dedges[di];
     const NodeD& own = h->nodes[d.owner];
     const NodeD& nbn = h->nodes[d.nbr];
     const ProbD& pd = h->probs[d.prob];
-    std::vector<Task>& tl = h->tasks[own.colour];
+    std::vector<Task>& tl = tasks[own.colour];
     const bool dense = pd.cost_kind == TREE_OT_COST_DENSE_F32;
     if (h->fp64) {
       // a row per warp where the GPU has room for it, and as few rows per CTA as there are SMs for: rows in turn
@@ -406,18 +428,14 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
         for (int32_t o0 = 0; o0 < own.n; o0 += kColCols)
           tl.push_back(Task{(int32_t)di, TASK_COL, o0, std::min(kColCols, own.n - o0), s * kColRows,
                             std::min(kColRows, nbn.n - s * kColRows), s, 0});
-    } else if (fact_edge(h, d)) {
-      // slots of the owner's groups against a split of the neighbour's points, 2^split warps of a CTA per block of
-      // 64; the exact-distance kernel reads the same range as plain outputs, with G warp groups of at most
-      // 1024 / G outputs
+    } else if (!exact && fact_edge(h, d)) {
+      // slots of the owner's groups against a split of the neighbour's points, 2^split warps of a CTA per block of 64
       const int32_t ob = (8 >> h->fact_split) * 64, per = fact_split_points(nbn.n, d.nsplit);
       for (int32_t o0 = 0; o0 < own.n; o0 += ob) {
         const int32_t oc = std::min(ob, own.n - o0);
-        int32_t G = 1;
-        while (G < 8 && kRecOut / (2 * G) >= oc) G *= 2;
         for (int32_t s = 0; s < d.nsplit; ++s)
           tl.push_back(Task{(int32_t)di, TASK_FACT + h->fact_split, o0, oc, s * per, std::min(per, nbn.n - s * per), s,
-                            G});
+                            0});
       }
     } else {
       for (int32_t o0 = 0; o0 < own.n; o0 += rec_ob) {
@@ -438,26 +456,117 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob) {
       return (int)h->probs[h->dedges[t.dedge].prob].dim + (t.kind >= TASK_FACT ? 3 : 0);
     };
     auto cost_of = [&](const Task& t) { return (int64_t)t.ocount * t.rcount; };
-    std::stable_sort(h->tasks[c].begin(), h->tasks[c].end(), [&](const Task& x, const Task& y) {
+    std::stable_sort(tasks[c].begin(), tasks[c].end(), [&](const Task& x, const Task& y) {
       const int sx = slot_of(x), sy = slot_of(y);
       if (sx != sy) return sx < sy;
       return sx != 0 && cost_of(x) > cost_of(y);
     });
-    for (const Task& t : h->tasks[c]) h->slot_count[c][slot_of(t)] += 1;
+    for (const Task& t : tasks[c]) slot_count[c][slot_of(t)] += 1;
     int32_t b = 0;
     for (int s2 = 0; s2 < kApplySlots; ++s2) {
-      h->slot_begin[c][s2] = b;
-      b += h->slot_count[c][s2];
+      slot_begin[c][s2] = b;
+      b += slot_count[c][s2];
     }
   }
-  h->rec_ob = rec_ob;
+  if (!exact) h->rec_ob = rec_ob;
+}
+
+// the exact-distance plan is in use
+bool exact_plan(const tree_ot_handle* h) { return h->any_exact && !h->xplan.dedges.empty(); }
+
+// items per problem and colour of the persistent launch: apply tasks, node-update chunks
+std::vector<int32_t> forest_counts(const tree_ot_handle* h, const std::vector<Task>* tasks) {
+  std::vector<int32_t> cnt(4 * (size_t)h->nprob, 0);
+  for (int c = 0; c < 2; ++c) {
+    for (const Task& t : tasks[c]) ++cnt[4 * h->dedges[t.dedge].prob + c];
+    for (const NodeChunk& ch : h->chunks[c]) ++cnt[4 * h->nodes[ch.node].prob + 2 + c];
+  }
+  return cnt;
+}
+
+std::vector<OwnedDEdge> owned_records(const tree_ot_handle* h, const std::vector<DEdgeD>& dedges) {
+  std::vector<OwnedDEdge> owned;
+  for (int32_t di : h->node_dedges) owned.push_back(OwnedDEdge{dedges[di], di, 0});
+  return owned;
+}
+
+// host-resolved records of the fixed leaves' chunks of a colour
+int fixed_records(const tree_ot_handle* h, const std::vector<DEdgeD>& dedges, int c, cudaStream_t s,
+                  std::vector<FixedChunkD>* out) {
+  std::vector<SkRefD> skref(dedges.size(), SkRefD{nullptr, nullptr, nullptr});
+  if (h->d_skref) {
+    CUDA_TRY(cudaMemcpyAsync(skref.data(), h->d_skref, sizeof(SkRefD) * skref.size(), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+  }
+  for (int32_t k = 0; k < h->nfixed_chunks[c]; ++k) {
+    const NodeChunk& ch = h->chunks[c][k];
+    const NodeD& nd = h->nodes[ch.node];
+    const int32_t di = h->node_dedges[nd.dedge_begin];
+    const DEdgeD& d = dedges[di];
+    const ProbD& pd = h->probs[nd.prob];
+    out->push_back(FixedChunkD{d.off, d.part_off, nd.node_off, ch.node, ch.x0, ch.cnt, nd.n, nd.prob, di, d.nbr, d.edge,
+                               d.nsplit, pd.cost_kind, pd.eps * 0.69314718055994530942, skref[di]});
+  }
+  return TREE_OT_OK;
+}
+
+// The exact-distance plan: directed edges with the difference form's reduction splits, and the largest output
+// block that gives every SM two tasks.  Its device memory is taken at create (plan_exact) and filled when the
+// certification first asks for exact distances (fill_exact).
+int plan_exact(tree_ot_handle* h, int nsm) {
+  ExactPlan& x = h->xplan;
+  bool any = false;
+  for (const DEdgeD& d : h->dedges) any = any || fact_edge(h, d);
+  if (!any) return TREE_OT_OK;
+  x.dedges = h->dedges;
+  for (DEdgeD& d : x.dedges)
+    if (fact_edge(h, d)) d.nsplit = (h->nodes[d.nbr].n + kRecRed - 1) / kRecRed;
+  int64_t count[2] = {0, 0};
+  for (x.rec_ob = kRecOut;; x.rec_ob /= 2) {
+    count[0] = count[1] = 0;
+    for (const DEdgeD& d : x.dedges)
+      if (h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
+        count[h->nodes[d.owner].colour] += (int64_t)((h->nodes[d.owner].n + x.rec_ob - 1) / x.rec_ob) * d.nsplit;
+    if (x.rec_ob == 256 || std::max(count[0], count[1]) >= 2 * nsm) break;
+  }
+  for (int c = 0; c < 2; ++c) {
+    for (const Task& t : h->tasks[c]) count[c] += t.kind < TASK_RECOMP;  // stored costs: as they are
+    RC_TRY(h->alloc(&x.d_tasks[c], count[c]));
+    RC_TRY(h->alloc(&x.d_fixed[c], h->nfixed_chunks[c]));
+  }
+  RC_TRY(h->alloc(&x.d_dedges, (int64_t)x.dedges.size()));
+  RC_TRY(h->alloc(&x.d_owned, (int64_t)h->node_dedges.size()));
+  if (h->opt.flags & TREE_OT_OPT_PERSISTENT) RC_TRY(h->alloc(&x.d_fcnt, 4 * (int64_t)h->nprob));
+  return TREE_OT_OK;
+}
+
+int fill_exact(tree_ot_handle* h, cudaStream_t s) {
+  ExactPlan& x = h->xplan;
+  if (x.ready || x.dedges.empty()) return TREE_OT_OK;
+  build_apply_tasks(h, x.rec_ob, true);
+  auto up = [&](auto* dst, const auto& v) {
+    return v.empty() ? cudaSuccess : cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, s);
+  };
+  CUDA_TRY(up(x.d_dedges, x.dedges));
+  CUDA_TRY(up(x.d_owned, owned_records(h, x.dedges)));
+  for (int c = 0; c < 2; ++c) {
+    std::vector<FixedChunkD> fr;
+    RC_TRY(fixed_records(h, x.dedges, c, s, &fr));
+    CUDA_TRY(up(x.d_fixed[c], fr));
+    CUDA_TRY(up(x.d_tasks[c], x.tasks[c]));
+  }
+  if (x.d_fcnt) CUDA_TRY(up(x.d_fcnt, forest_counts(h, x.tasks)));
+  CUDA_TRY(cudaStreamSynchronize(s));
+  x.ready = true;
+  return TREE_OT_OK;
 }
 
 ApplyArgs apply_args(tree_ot_handle* h, int colour) {
   ApplyArgs a{};
-  a.tasks = h->d_tasks[colour];
-  a.ntasks = (int32_t)h->tasks[colour].size();
-  a.dedges = h->d_dedges;
+  const bool x = exact_plan(h);
+  a.tasks = x ? h->xplan.d_tasks[colour] : h->d_tasks[colour];
+  a.ntasks = (int32_t)(x ? h->xplan.tasks : h->tasks)[colour].size();
+  a.dedges = x ? h->xplan.d_dedges : h->d_dedges;
   a.edges = h->d_edges;
   a.nodes = h->d_nodes;
   a.probs = h->d_probs;
@@ -495,8 +604,8 @@ NodeArgs node_args(tree_ot_handle* h, int colour, bool retire) {
   a.smem = h->node_smem[colour];
   a.colour = colour;
   a.nodes = h->d_nodes;
-  a.dedges = h->d_dedges;
-  a.owned = h->d_owned;
+  a.dedges = exact_plan(h) ? h->xplan.d_dedges : h->d_dedges;
+  a.owned = exact_plan(h) ? h->xplan.d_owned : h->d_owned;
   a.probs = h->d_probs;
   a.nprob = h->nprob;
   a.done = h->d_done;
@@ -586,11 +695,14 @@ int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, ApplySet set = A
     prof_span(h, TREE_OT_PROF_APPLY_FP64, p0, prof_mark(h, s));
     return TREE_OT_OK;
   }
+  const Task* tasks = a.tasks;
+  const int32_t* slot_begin = (exact_plan(h) ? h->xplan.slot_begin : h->slot_begin)[colour];
+  const int32_t* slot_count = (exact_plan(h) ? h->xplan.slot_count : h->slot_count)[colour];
   for (int slot = 0; slot < kApplySlots; ++slot) {
-    const int32_t cnt = h->slot_count[colour][slot];
+    const int32_t cnt = slot_count[slot];
     if (cnt == 0) continue;
     if (set != APPLY_ALL && set != (slot == 0 ? APPLY_STORED : slot <= 3 ? APPLY_DIFF : APPLY_FACT)) continue;
-    a.tasks = h->d_tasks[colour] + h->slot_begin[colour][slot];
+    a.tasks = tasks + slot_begin[slot];
     a.ntasks = cnt;
     a.queue = h->d_queue + 2 * (colour * kApplySlots + slot);
     const int p0 = prof_mark(h, s);
@@ -606,18 +718,18 @@ int launch_apply(tree_ot_handle* h, int colour, cudaStream_t s, ApplySet set = A
     int work = cnt, variant = slot == 0 ? 0 : h->rec_variant;
     // both forms in one launch: slot 3 + D's tasks follow slot D's (no other dimension in the handle)
     const bool both = h->both_forms && set == APPLY_ALL && !a.any_exact && slot > 0;
-    if (both && slot > 3 && h->slot_count[colour][slot - 3] > 0) continue;  // taken by that launch
-    if (both && slot <= 3 && h->slot_count[colour][slot + 3] > 0) {
-      a.ntasks += h->slot_count[colour][slot + 3];
+    if (both && slot > 3 && slot_count[slot - 3] > 0) continue;  // taken by that launch
+    if (both && slot <= 3 && slot_count[slot + 3] > 0) {
+      a.ntasks += slot_count[slot + 3];
       work = a.ntasks;
       variant = kBothForms;
       cap = h->rec_grid[0][slot];
     } else if (slot > 3) {
       variant = h->fact_split > 0 ? 1 : 0;
-      cap = a.any_exact ? h->rec_grid[0][slot - 3] : h->rec_grid[variant][slot];
+      cap = h->rec_grid[variant][slot];
       a.items = h->d_items[colour] + h->item_begin[colour][slot - 3];
       a.nitems = h->item_count[colour][slot - 3];
-      if (!a.any_exact && variant == 0) work = (a.nitems + 3) / 4;  // four warps per CTA
+      if (variant == 0) work = (a.nitems + 3) / 4;  // four warps per CTA
     }
     const int grid = std::max(1, std::min<int>(work, cap));
     cudaError_t e = launch_apply_f32(a, slot, variant, grid, s);
@@ -658,12 +770,13 @@ int launch_update(tree_ot_handle* h, int colour, bool retire, cudaStream_t s) {
   // first) when they fill the GPU on their own, or when there is nothing else;
   // otherwise one launch takes every chunk (two half-empty launches back to
   // back cost more than the leaner kernel saves).
+  const FixedChunkD* fixed = exact_plan(h) ? h->xplan.d_fixed[colour] : h->d_fixed[colour];
   const bool all_fixed = nf > 0 && nf == nall;
   const bool split = nf > 0 && nf < nall && nf >= 4 * h->sms;
   if (split) {
     a.nchunks = nf;
     a.count_launch = 0;
-    a.fixed = defer ? h->d_fixed[colour] : nullptr;
+    a.fixed = defer ? fixed : nullptr;
     e = launch_node_update(a, h->fp64, true, s);
     a.fixed = nullptr;
   }
@@ -672,7 +785,7 @@ int launch_update(tree_ot_handle* h, int colour, bool retire, cudaStream_t s) {
     a.chunks = h->d_chunks[colour] + first;
     a.nchunks = nall - first;
     a.count_launch = defer ? 0 : 1;
-    a.fixed = (all_fixed && defer) ? h->d_fixed[colour] : nullptr;
+    a.fixed = (all_fixed && defer) ? fixed : nullptr;
     e = launch_node_update(a, h->fp64, all_fixed, s);
     a.fixed = nullptr;
   }
@@ -701,12 +814,10 @@ int launch_forest_chunk(tree_ot_handle* h, int G, bool retire, cudaStream_t s) {
   ForestArgs f{};
   for (int c = 0; c < 2; ++c) {
     f.ap[c] = apply_args(h, c);
-    f.ap[c].tasks = h->d_tasks[c] + h->slot_begin[c][h->forest_D];
-    // the factored tasks follow the others: no other dimension's lie between
-    f.ap[c].ntasks = h->slot_count[c][h->forest_D] + h->slot_count[c][h->forest_D + 3];
+    // every task: one dimension, the factored ones after the others
     f.nd[c] = node_args(h, c, retire);
   }
-  f.cnt = h->d_fcnt;
+  f.cnt = exact_plan(h) ? h->xplan.d_fcnt : h->d_fcnt;
   f.app_done = h->d_fdone;
   f.nod_done = h->d_fdone + h->nprob;
   f.ctl = h->d_fctl;
@@ -1348,7 +1459,8 @@ int plan_shared_kernels(tree_ot_handle* h, const tree_ot_problem* probs, int32_t
 // 64, 32 and 16 points of every node, picks each node's size by the share of wide groups, sorts the points and
 // sets the reduction splits of the directed edges in factored form (nodes and dedges are uploaded again after).
 int plan_groups(tree_ot_handle* h, cudaStream_t s) {
-  if (h->fp64) return TREE_OT_OK;
+  // exact distances from the first half-step: the difference form throughout
+  if (h->fp64 || (h->opt.flags & TREE_OT_OPT_EXACT_DIST)) return TREE_OT_OK;
   std::vector<GroupWork> work;
   for (size_t j = 0; j < h->nodes.size(); ++j) {
     const NodeD& nd = h->nodes[j];
@@ -1585,12 +1697,7 @@ int setup_forest(tree_ot_handle* h, cudaStream_t s) {
     }
   }
   if (D == 0) return TREE_OT_OK;
-  std::vector<int32_t> cnt(4 * (size_t)h->nprob, 0);
-  for (int c = 0; c < 2; ++c) {
-    for (int32_t i = 0; i < h->slot_count[c][D] + h->slot_count[c][D + 3]; ++i)
-      ++cnt[4 * h->dedges[h->tasks[c][h->slot_begin[c][D] + i].dedge].prob + c];
-    for (const NodeChunk& ch : h->chunks[c]) ++cnt[4 * h->nodes[ch.node].prob + 2 + c];
-  }
+  const std::vector<int32_t> cnt = forest_counts(h, h->tasks);
   if (!h->d_fcnt) {
     int rc = 0;
     if ((rc = h->alloc(&h->d_fcnt, 4 * (int64_t)h->nprob)) || (rc = h->alloc(&h->d_fdone, 2 * (int64_t)h->nprob)) ||
@@ -2066,26 +2173,16 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     }
     h->fact_split = split;
     build_apply_tasks(h, kRecOut);
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if ((rc = plan_exact(h, nsm))) return bail(rc);
   }
   if ((rc = setup_shared_kernels(h, s))) return bail(rc);
   if (!h->fp64) {  // host-resolved records of the fixed leaves' chunks, per colour
-    std::vector<SkRefD> skref(h->dedges.size(), SkRefD{nullptr, nullptr, nullptr});
-    if (h->d_skref) {
-      cudaError_t ce = cudaMemcpyAsync(skref.data(), h->d_skref, sizeof(SkRefD) * skref.size(), cudaMemcpyDeviceToHost, s);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-      if (ce != cudaSuccess) return bail(cuda_fail(ce, "read shared-kernel references"));
-    }
     for (int c = 0; c < 2; ++c) {
       std::vector<FixedChunkD> fr;
-      for (int32_t k = 0; k < h->nfixed_chunks[c]; ++k) {
-        const NodeChunk& ch = h->chunks[c][k];
-        const NodeD& nd = h->nodes[ch.node];
-        const int32_t di = h->node_dedges[nd.dedge_begin];
-        const DEdgeD& d = h->dedges[di];
-        const ProbD& pd = h->probs[nd.prob];
-        fr.push_back(FixedChunkD{d.off, d.part_off, nd.node_off, ch.node, ch.x0, ch.cnt, nd.n, nd.prob, di, d.nbr,
-                                 d.edge, d.nsplit, pd.cost_kind, pd.eps * 0.69314718055994530942, skref[di]});
-      }
+      if ((rc = fixed_records(h, h->dedges, c, s, &fr))) return bail(rc);
       if (fr.empty()) continue;
       if ((rc = h->alloc(&h->d_fixed[c], (int64_t)fr.size()))) return bail(rc);
       const cudaError_t ce =
@@ -2164,8 +2261,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     }
   }
   // plan tables
-  std::vector<OwnedDEdge> owned;
-  for (int32_t di : h->node_dedges) owned.push_back(OwnedDEdge{h->dedges[di], di, 0});
+  const std::vector<OwnedDEdge> owned = owned_records(h, h->dedges);
   std::vector<NodeChunkD> crec[2];
   for (int c = 0; c < 2; ++c)
     for (const NodeChunk& k : h->chunks[c]) {
@@ -2430,6 +2526,7 @@ int tree_ot_solve(tree_ot_handle* h, void* cuda_stream, tree_ot_result* results)
       const int32_t any = *std::max_element(h->h_exact.begin(), h->h_exact.end());
       CUDA_TRY(cudaMemcpyAsync(h->d_exact, h->h_exact.data(), sizeof(int32_t) * h->nprob, cudaMemcpyHostToDevice, s));
       if (any != h->any_exact) {
+        if (any) RC_TRY(fill_exact(h, s));
         h->any_exact = any;
         if (use_graph) {
           if (h->graph) cudaGraphExecDestroy(h->graph);
@@ -2848,7 +2945,7 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
   }
-  const int64_t v[22] = {(int64_t)h->dedges.size(),
+  const int64_t v[23] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2869,8 +2966,9 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         (int64_t)(h->both_forms ? 1 : 0),
                         (int64_t)fallbacks,
                         h->wide_points,
-                        fact_splits};
-  for (int32_t i = 0; i < nstats && i < 22; ++i) stats[i] = v[i];
+                        fact_splits,
+                        (int64_t)(exact_plan(h) ? 1 : 0)};
+  for (int32_t i = 0; i < nstats && i < 23; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

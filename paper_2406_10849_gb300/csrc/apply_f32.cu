@@ -242,15 +242,14 @@ __global__ void __launch_bounds__(kApplyThreads, 2) apply_dense_kernel(ApplyArgs
 // Tasks come from a work queue (an atomic counter; tasks are sorted by cost on
 // the host), so uneven edges of a batch of trees balance across the CTAs.  The
 // last CTA to leave resets the counter for the next launch.
-// MODE 0: the difference form alone.  MODE 1: both forms' tasks, and some
-// problems run the exact-distance variant (A.exact).  MODE 2: both forms' tasks
-// in one launch, for handles whose two launches would each leave the GPU half
+// MODE 0: the difference form alone.  MODE 1: the same where some problems run
+// the exact-distance variant (A.exact).  MODE 2: both forms' tasks in one launch, for handles whose two launches would each leave the GPU half
 // empty (the autotuner times it).  Instantiated separately so that the plain
 // kernel keeps its register budget.
 template <int D, int MINB, int MODE>
 __global__ void __launch_bounds__(kApplyThreads, MINB) apply_recomp_kernel(ApplyArgs A) {
   // 24 KB of the difference form's staging; the factored form's where it runs (28 KB)
-  __shared__ __align__(16) float sm[MODE == 0 ? 24 * kApplyThreads : kFactSmemFloats];
+  __shared__ __align__(16) float sm[MODE == 2 ? kFactSmemFloats : 24 * kApplyThreads];
   __shared__ int s_ti;
   // every problem retired or in a BF16 phase: nothing to apply (the same for every CTA; the
   // work queue is then untouched and stays reset)
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(kApplyThreads, MINB) apply_recomp_kernel(Apply
     if (A.done[prob] || A.lowp[prob] == 1) continue;  // retired, or in a BF16 phase
     if (MODE == 1 && A.exact[prob])  // block-uniform: refined past the plain recomputation's floor
       recomp_task_exact<D>(A, t, sm);
-    else if (MODE != 0 && t.kind >= TASK_FACT)
+    else if (MODE == 2 && t.kind >= TASK_FACT)
       fact_dispatch<D>(A, t, sm);
     else
       recomp_task<D>(A, t, sm);
@@ -503,9 +502,7 @@ cudaError_t launch_apply_f32(const ApplyArgs& a, int slot, int variant, int grid
   if (slot == 0) {
     apply_dense_kernel<<<grid, kApplyThreads, 0, s>>>(a);
   } else if (a.any_exact) {
-    // rare (after certification): the 2-CTA register budget, whatever the tuned variant; takes both
-    // forms' tasks
-    if (slot > 3) slot -= 3;
+    // rare (after certification): the 2-CTA register budget, whatever the tuned variant
     if (slot == 1) apply_recomp_kernel<1, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
     if (slot == 2) apply_recomp_kernel<2, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
     if (slot == 3) apply_recomp_kernel<3, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);

@@ -137,3 +137,42 @@ def test_long_reductions_are_split(n, dim, eps, splits, tune):
             ref = O.run_half_steps(p, steps)
             assert rel_err(got, ref, p.eps) <= 1e-4
             assert marginal_gap(p, got, ref) <= 1e-6  # the bar of every FP32 iterate
+
+
+def test_exact_distances_take_the_difference_form():
+    """With exact squared distances from the start nothing is factored, and the reduction is cut into pieces of
+    512 points as for every difference-form apply: 4 blocks of 1024 outputs x 8 pieces for each of the two leaves."""
+    import paper_2406_10849_gb300 as T
+    T.load()
+    p = cloud_star((4096, 4096, 4000), 2, 0.05, seed=4)
+    with T.Solver([p], T.options(exact_dist=True, autotune=False)) as s:
+        st = s.plan_stats()
+        assert st["factored_edges"] == 0
+        assert st["apply_tasks_c0"] == 2 * 4 * 8 and st["apply_tasks_c1"] == 2 * 4 * 8
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_certification_switches_to_the_exact_plan_and_back(persistent):
+    """16 x 16 stars certified at 1.2e-7: where the plain costs stop short of it, the handle goes on with exact
+    distances, the difference form and its own splits; a reset brings the factored form back, bit for bit."""
+    import gen
+    import paper_2406_10849_gb300 as T
+    T.load()
+    probs = gen.warmstart_stars(9_000_000, 16, side=16, eps=0.005)
+    with T.Solver(probs, T.options(tol=1.2e-7, tol_kind="max", max_half_steps=6000, autotune=False,
+                                   persistent=persistent)) as s:
+        assert s.plan_stats()["factored_edges"] > 0
+        s.half_steps(6)
+        first = [s.potentials(i) for i in (0, 9)]
+        s.reset()
+        rc, res = s.solve()
+        assert s.plan_stats()["exact_plan"] == 1
+        assert rc == 0
+        for i in (0, 9):
+            assert O.final_check(probs[i], s.potentials(i))["max_marginal_l1"] <= 1.5e-7
+        s.reset()
+        assert s.plan_stats()["exact_plan"] == 0
+        s.half_steps(6)
+        for i, f in zip((0, 9), first):
+            again = s.potentials(i)
+            assert all(np.array_equal(f[k], again[k]) for k in again)
