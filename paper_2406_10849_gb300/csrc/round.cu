@@ -283,7 +283,8 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
               if (w.hi > 0.f) inf[r] = true;
               continue;
             }
-            const DF a = {fabsf(c.hi), c.hi < 0.f ? -c.lo : c.lo};
+            DF a = {fabsf(c.hi), c.hi < 0.f ? -c.lo : c.lo};
+            df_renorm(a);  // a distance's low part may exceed an ulp of its high part: compare sums, not parts
             if (a.hi > cmax.hi || (a.hi == cmax.hi && a.lo > cmax.lo)) cmax = a;
             df_acc(tacc[r], df_mul(w, c));
             continue;
