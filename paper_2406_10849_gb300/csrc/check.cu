@@ -25,13 +25,13 @@ namespace {
 // stay in the lanes' registers until the task ends, column sums are combined
 // across the warps in shared memory and added to the column marginal with one
 // FP64 atomic per column and task.  Sums inside a task use Kahan compensation;
-// across lanes and warps they are double-float (in FP64 those few additions per
-// column and row took almost as long as the entries: 94 M entries took 1.07 ms,
-// now 0.66).
+// across lanes and warps they are three floats (plan_entry.cuh), or FP64 where
+// one leaves the FP32 range (in FP64 those few additions per column and row took
+// almost as long as the entries).
 // COL tasks belong to the FP64 check and are skipped here.
 constexpr int kChkRows = 8;  // rows per warp
 
-__global__ void __launch_bounds__(256) check_kernel(CheckArgs A) {
+__global__ void __launch_bounds__(256, 2) check_kernel(CheckArgs A) {
   __shared__ float s_col[8][32];
   __shared__ float s_cmp[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -97,28 +97,44 @@ __global__ void __launch_bounds__(256) check_kernel(CheckArgs A) {
       s_col[warp][lane] = cs;
       s_cmp[warp][lane] = cc;
       __syncthreads();
-      if (warp == 0 && on) {  // double-float across the warps, one conversion per column
-        DF v = {0.f, 0.f};
+      if (warp == 0 && on) {
+        TF v = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int w = 0; w < 8; ++w) df_acc(v, DF{s_col[w][lane], -s_cmp[w][lane]});
-        if (v.hi != 0.f) atomicAdd(&A.marg[b_off + y], df_to(v));
+        for (int w = 0; w < 8; ++w) tf_acc(v, s_col[w][lane], -s_cmp[w][lane]);
+        double sum = tf_to(v);
+        if (!tf_finite(v)) {  // out of the FP32 range: in FP64
+          sum = 0.0;
+          for (int w = 0; w < 8; ++w) sum += (double)s_col[w][lane] - (double)s_cmp[w][lane];
+        }
+        if (sum != 0.0) atomicAdd(&A.marg[b_off + y], sum);
       }
       __syncthreads();
     }
-    // row r's sum to lane r, the task's sums to every lane: double-float, then one conversion each
-    DF mine = {0.f, 0.f}, mass = {0.f, 0.f}, tc = {0.f, 0.f};
+    TF row[kChkRows], trn[kChkRows];
 #pragma unroll
     for (int r = 0; r < kChkRows; ++r) {
-      const DF row = warp_sum_df(DF{rs[r], -rc[r]});
-      if (lane == r) mine = row;
-      df_acc(mass, row);
-      df_acc(tc, warp_sum_df(DF{ts[r], -tcmp[r]}));
+      row[r] = {rs[r], -rc[r], 0.f};
+      trn[r] = {ts[r], -tcmp[r], 0.f};
     }
-    if (lane < kChkRows && warp * kChkRows + lane < t.ocount)
-      A.marg[a_off + t.o0 + warp * kChkRows + lane] = df_to(mine);
-    if (lane == 0 && (tc.hi != 0.f || mass.hi != 0.f)) {
-      atomicAdd(&A.edge_tc[d.edge], df_to(tc));
-      atomicAdd(&A.edge_mass[d.edge], df_to(mass));
+    const TF rsum = warp_rows_sum(row), tsum = warp_rows_sum(trn);
+    double mass = tf_to(rsum), tc = tf_to(tsum);
+    const int mine = lane >> 2;
+    if (__any_sync(0xffffffffu, !tf_finite(rsum) || !tf_finite(tsum)))
+#pragma unroll
+      for (int r = 0; r < kChkRows; ++r) {
+        const double m = warp_sum_d((double)rs[r] - (double)rc[r]), c = warp_sum_d((double)ts[r] - (double)tcmp[r]);
+        if (r == mine) mass = m, tc = c;
+      }
+    if (warp * kChkRows + mine >= t.ocount) mass = tc = 0.0;
+    else if ((lane & 3) == 0) A.marg[a_off + t.o0 + warp * kChkRows + mine] = mass;
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) {  // the warp's rows
+      mass += __shfl_xor_sync(0xffffffffu, mass, o);
+      tc += __shfl_xor_sync(0xffffffffu, tc, o);
+    }
+    if (lane == 0 && (tc != 0.0 || mass != 0.0)) {
+      atomicAdd(&A.edge_tc[d.edge], tc);
+      atomicAdd(&A.edge_mass[d.edge], mass);
     }
   }
 }

@@ -37,30 +37,65 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
   return {s.hi, s.lo + a.lo + b.lo};
 }
 
-// running sums of (pairs of) floats: s += v with every rounding error kept in s.lo
-__device__ __forceinline__ void df_acc(DF& s, float v) {
-  const DF t = two_sum(s.hi, v);
-  s.hi = t.hi;
-  s.lo += t.lo;
-}
-__device__ __forceinline__ void df_acc(DF& s, DF v) {
-  const DF t = two_sum(s.hi, v.hi);
-  s.hi = t.hi;
-  s.lo += t.lo + v.lo;
-}
 // lo back below half an ulp of hi (|hi| >= |lo|), so that adding to it stays exact to ~2^-48
 __device__ __forceinline__ void df_renorm(DF& s) {
   const float t = __fadd_rn(s.hi, s.lo);
   s.lo = __fsub_rn(s.lo, __fsub_rn(t, s.hi));
   s.hi = t;
 }
-__device__ __forceinline__ double df_to(DF v) { return (double)v.hi + (double)v.lo; }
-// the warp's sum, in every lane (FP64 shuffle sums cost 20 times the FP32 pipe's time per step)
-__device__ __forceinline__ DF warp_sum_df(DF v) {
+
+// Running sums as three floats: every rounding error of the first is summed in the second, the second's in the
+// third.  A sum of n terms carries about n^2 2^-72 relative, less than one FP64 addition (2^-53) for any support
+// here, where pairs of floats would leave n 2^-48; FP64 itself runs at 1/70 of the FP32 rate.
+struct TF {
+  float a, b, c;
+};
+__device__ __forceinline__ void tf_acc(TF& s, float v) {  // s += v
+  const DF t = two_sum(s.a, v), u = two_sum(s.b, t.lo);
+  s = {t.hi, u.hi, s.c + u.lo};
+}
+__device__ __forceinline__ void tf_acc(TF& s, float p, float m) {  // s += p + m
+  const DF t = two_sum(s.a, p), u = two_sum(s.b, t.lo), v = two_sum(u.hi, m);
+  s = {t.hi, v.hi, s.c + (u.lo + v.lo)};
+}
+__device__ __forceinline__ void tf_acc(TF& s, TF v) {
+  tf_acc(s, v.a, v.b);
+  s.c += v.c;
+}
+__device__ __forceinline__ double tf_to(TF s) { return (double)s.a + ((double)s.b + (double)s.c); }
+__device__ __forceinline__ TF tf_of(double v) {
+  const float a = (float)v;
+  const double r = v - (double)a;
+  const float b = (float)r;
+  return {a, b, (float)(r - (double)b)};
+}
+// x v as three floats, x v.a exactly (as long as it neither overflows nor falls below 2^-102)
+__device__ __forceinline__ TF tf_mul(float x, TF v) {
+  const float p = __fmul_rn(x, v.a), q = __fmul_rn(x, v.b);
+  const DF m = two_sum(fmaf(x, v.a, -p), q);
+  return {p, m.hi, fmaf(x, v.c, m.lo + fmaf(x, v.b, -q))};
+}
+// finite: no sum on the way to it overflowed (an overflow leaves inf or NaN in every part that follows)
+__device__ __forceinline__ bool tf_finite(TF s) { return fabsf(s.a) <= 3.4028235e38f; }
+
+// Sums of eight per-lane values across the warp: the lanes trade halves of their values, so that each step adds half
+// as many; every lane ends with the sum of value lane / 4.
+__device__ __forceinline__ TF warp_rows_sum(TF (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  auto trade = [](TF keep, TF give, int o) {
+    tf_acc(keep, TF{__shfl_xor_sync(0xffffffffu, give.a, o), __shfl_xor_sync(0xffffffffu, give.b, o),
+                    __shfl_xor_sync(0xffffffffu, give.c, o)});
+    return keep;
+  };
 #pragma unroll
-  for (int o = 16; o; o >>= 1)
-    df_acc(v, DF{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
-  return v;
+  for (int h = 4; h >= 1; h >>= 1) {
+    const int o = 4 * h;
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < h; ++i) v[i] = trade(up ? v[i + h] : v[i], up ? v[i] : v[i + h], o);
+  }
+  v[0] = trade(v[0], v[0], 2);
+  return trade(v[0], v[0], 1);
 }
 
 // squared distance of two D-dimensional FP32 points (D <= 3) as a double-float

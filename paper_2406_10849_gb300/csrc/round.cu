@@ -21,7 +21,7 @@
 // The rounded plans are never stored: they are (x, y, err_r, E) plus the
 // potentials, and <C, B^> = <C, F''> + err_r^T C err_c / E.  Entries are the
 // double-float plan entries of the check (FP32 pipe; FP64 handles: FP64), every
-// sum over them is double-float too, flushed into FP64 (FP64 handles: FP64).  Passes over the plans (one CTA per task of 64 rows of
+// sum over them is three floats (FP64 handles: FP64).  Passes over the plans (one CTA per task of 64 rows of
 // one plan, rows on S), with per-point steps between them:
 //   1  F 1, F^T 1, <C, F>, ||F||_1     -> targets t and c, row scales x
 //   2  F'^T 1                          -> column scales y
@@ -186,36 +186,99 @@ __global__ void __launch_bounds__(256) round_pass_kernel(RoundArgs A) {
 }
 
 // ---------------------------------------------------------------------------
-// Passes 1-4 of FP32 handles.  Entries and costs are pairs of FP32 values already;
-// here every sum over them is one too, across the lanes and warps as well:
-// products by TwoProd, additions by TwoSum, running sums renormalised every
-// kRenormSteps column steps.  A sum then carries a few units of 2^-46 relative (measured by the tests: rounded plans feasible to
-// 1e-13, as with FP64 sums).  GB300 executes an FP64 add or a conversion at 1/70
-// of its FP32 rate, and with FP64 sums those were the passes' whole time (94 M
-// entries in 209 plans: 2.6 / 0.8 / 3.1 / 2.8 ms for passes 1-4; with only the
-// entries' sums in double-float and FP64 across lanes 0.91 / 0.56 / 0.87 / 0.62;
-// now 0.72 / 0.55 / 0.66 / 0.49).  Row factors (x, err_r) multiply the finished
-// row sums, not the entries.
+// Passes 1-4 of FP32 handles.  Entries are FP32 values, costs pairs of them; the factors x, y and err_c and every
+// sum over entries are three floats (TF, plan_entry.cuh): GB300 executes an FP64 add or a conversion at 1/70 of its
+// FP32 rate, and with FP64 sums those were the passes' whole time (check and rounding of 94 M entries in 209 plans:
+// 11.8 ms with FP64 sums, 4.5 with pairs of floats, which keep 2^-46 instead of 2^-53, 5.3 with three).  Row factors
+// (x, err_r) multiply the finished row sums, not the entries.
+//
+// Accuracy: products of an entry with a factor are exact to 2^-70, sums to n^2 2^-72, both below FP64's own
+// rounding; products with a cost to 2^-47 each, independent between the entries they are summed over.
+//
+// Range: products would lose their low parts below 2^-102 and overflow above 2^128, where FP64 does neither.  So
+// factors are scaled by powers of two: x by 2^kUp in pass 2 (B x <= t <= 1 for every entry of a row), y and err_c
+// (at most 1) by 2^kMid in passes 3 and 4, and costs by the power of two next to their scale / eps (by 2^kCost more
+// in pass 1).  A sum that overflows all the same (it is then inf or NaN) is formed again in FP64, a row at a
+// time or a column of the task's rows.
 // ---------------------------------------------------------------------------
-constexpr int kRenormSteps = 32;  // column steps (32 columns each) between renormalisations
+constexpr int kUp = 100, kMid = 64, kCost = 32;
 
-// a (a float) times b
-__device__ __forceinline__ DF df_mul(float a, DF b) {
-  const float p = __fmul_rn(a, b.hi);
-  return {p, fmaf(a, b.lo, fmaf(a, b.hi, -p))};
+// the exponent of the power of two that scales costs: that of kd = scale / eps, within a float's range
+__device__ __forceinline__ int cost_exp(double kd) { return max(-120, min(120, ilogb(kd))); }
+
+// one plan of a task, what every entry of it takes
+struct RoundPlan {
+  const float* C;      // stored costs, rows on the owner when own_rows
+  int64_t ld;
+  bool own_rows, stored;
+  double cscale;
+  float kh, kl;
+  int D;
+};
+
+__device__ __forceinline__ DF round_cost(const RoundPlan& p, int i, int y, const float* pa, const float* pb) {
+  if (p.stored) return {p.own_rows ? p.C[(int64_t)i * p.ld + y] : p.C[(int64_t)y * p.ld + i], 0.f};
+  return sq_dist_df(p.D, pa, pb);
 }
-__device__ __forceinline__ DF df_mul(DF a, DF b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  return {p, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)))};
+
+__device__ __forceinline__ void round_point(const RoundArgs& A, const NodeD& nd, int D, int i, float* p) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = (nd.coord_off >= 0 && k < D) ? A.coords[nd.coord_off + (int64_t)i * D + k] : 0.f;
 }
-__device__ __forceinline__ DF df_of(double v) {
-  const float h = (float)v;
-  return {h, (float)(v - (double)h)};
+
+// err_c = c - F''^T 1, F''^T 1 = y F'^T 1
+__device__ __forceinline__ double round_errc(const RoundArgs& A, int64_t k) {
+  return fmax(A.tgt[k] - A.xy[k] * A.s2[k], 0.0);
+}
+
+// Row i's sums in FP64, by the whole warp: the entries' (pass 1: B, pass 3: B y) and those times the costs (pass 4:
+// err_c C).
+template <int PASS>
+__device__ __noinline__ void round_row_fp64(const RoundArgs& A, const RoundPlan& p, const DEdgeD& d, const NodeD& nj,
+                                            const NodeD& nk, int i, double& row, double& cost) {
+  float pa[3], pb[3];
+  round_point(A, nj, p.D, i, pa);
+  row = cost = 0.0;
+  for (int y = threadIdx.x & 31; y < nk.n; y += 32) {
+    round_point(A, nk, p.D, y, pb);
+    const DF c = round_cost(p, i, y, pa, pb);
+    const double C = ((double)c.hi + (double)c.lo) * p.cscale;
+    if (PASS == 4) {
+      const double w = round_errc(A, d.rev_off + y);
+      if (w > 0.0) cost += w * C;
+      continue;
+    }
+    float cu;
+    const double B = plan_entry(A.ah[d.off + i], A.al[d.off + i], A.ah[d.rev_off + y], A.al[d.rev_off + y], c, p.kh, p.kl, cu);
+    const double b = PASS == 3 ? B * A.xy[d.rev_off + y] : B;
+    row += b;
+    if (b > 0.0) cost += b * C;
+  }
+  row = warp_sum_d(row);
+  cost = warp_sum_d(cost);
+}
+
+// Column y's sum over rows [i0, i1) in FP64 (pass 1: B, pass 2: x B)
+template <int PASS>
+__device__ __noinline__ double round_col_fp64(const RoundArgs& A, const RoundPlan& p, const DEdgeD& d, const NodeD& nj,
+                                              const NodeD& nk, int i0, int i1, int y) {
+  float pa[3], pb[3];
+  round_point(A, nk, p.D, y, pb);
+  double sum = 0.0;
+  for (int i = i0; i < i1; ++i) {
+    round_point(A, nj, p.D, i, pa);
+    float cu;
+    const double B = plan_entry(A.ah[d.off + i], A.al[d.off + i], A.ah[d.rev_off + y], A.al[d.rev_off + y],
+                                round_cost(p, i, y, pa, pb), p.kh, p.kl, cu);
+    sum += PASS == 2 ? A.xy[d.off + i] * B : B;
+  }
+  return sum;
 }
 
 template <int PASS>
-__global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
-  __shared__ float2 s_col[8][32];
+__global__ void __launch_bounds__(256, 2) round_pass_tf_kernel(RoundArgs A) {
+  __shared__ float4 s_row[8 * kRndRows][2];  // (a hi, a lo, x coordinates 0, 1), (coordinate 2, x as three floats)
+  __shared__ float s_col[2][3][8][32];       // alternate steps: one barrier each
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int ti = blockIdx.x; ti < A.ntasks; ti += gridDim.x) {
     const RoundTask t = A.tasks[ti];
@@ -224,139 +287,140 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
     const ProbD P = A.probs[d.prob];
     const NodeD nj = A.nodes[d.owner], nk = A.nodes[d.nbr];
     // cost rows on the owner: C itself (owner = row node), C^T when kept, else C's columns
-    const bool own_rows = d.dir == 0 || e.CT != nullptr;
-    const float* Cm = d.dir == 0 ? e.C : (e.CT ? e.CT : e.C);
-    const int64_t cld = d.dir == 0 ? e.ld : (e.CT ? e.ldt : e.ld);
-    const double cscale = P.cost_kind == 0 ? 1.0 : P.cost_scale;
-    const double kd = cscale * P.inv_eps;
-    const float kh = (float)kd, kl = (float)(kd - (double)kh);
-    const int D = P.dim;
-    float rah[kRndRows], ral[kRndRows], rp[kRndRows][3];
-    DF xr[kRndRows], racc[kRndRows], tacc[kRndRows];
-    bool inf[kRndRows];
-    DF cmax = {0.f, 0.f};
-#pragma unroll
-    for (int r = 0; r < kRndRows; ++r) {
-      const int ir = warp * kRndRows + r;
+    RoundPlan p;
+    p.stored = P.cost_kind == 0;
+    p.own_rows = d.dir == 0 || e.CT != nullptr;
+    p.C = d.dir == 0 ? e.C : (e.CT ? e.CT : e.C);
+    p.ld = d.dir == 0 ? e.ld : (e.CT ? e.ldt : e.ld);
+    p.cscale = p.stored ? 1.0 : P.cost_scale;
+    p.D = P.dim;
+    const double kd = p.cscale * P.inv_eps;
+    p.kh = (float)kd;
+    p.kl = (float)(kd - (double)p.kh);
+    const int ce = cost_exp(kd) + (PASS == 1 ? kCost : 0);
+    const float cmul = ldexpf(1.f, max(-126, min(126, ce)));
+    const double cunit = 1.0 / (double)cmul;
+    __syncthreads();  // the last task's rows are read
+    for (int ir = threadIdx.x; ir < 8 * kRndRows; ir += 256) {
       const bool on = ir < t.ocount;
       const int i = t.o0 + (on ? ir : 0);
-      rah[r] = on ? A.ah[d.off + i] : -INFINITY;
-      ral[r] = on ? A.al[d.off + i] : 0.f;
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        rp[r][k] = (nj.coord_off >= 0 && k < D) ? A.coords[nj.coord_off + (int64_t)i * D + k] : 0.f;
-      if (PASS == 2) xr[r] = on ? df_of(A.xy[d.off + i]) : DF{0.f, 0.f};
-      racc[r] = tacc[r] = {0.f, 0.f};
-      inf[r] = false;
+      float q[3];
+      round_point(A, nj, p.D, i, q);
+      const TF x = PASS == 2 && on ? tf_of(ldexp(A.xy[d.off + i], kUp)) : TF{0.f, 0.f, 0.f};
+      s_row[ir][0] = make_float4(on ? A.ah[d.off + i] : -INFINITY, on ? A.al[d.off + i] : 0.f, q[0], q[1]);
+      s_row[ir][1] = make_float4(q[2], x.a, x.b, x.c);
     }
+    __syncthreads();
+    TF racc[kRndRows], tacc[kRndRows];
+#pragma unroll
+    for (int r = 0; r < kRndRows; ++r) racc[r] = tacc[r] = {0.f, 0.f, 0.f};
+    unsigned inf = 0;  // rows with an infinite cost of positive weight (pass 4)
+    DF cmax = {0.f, 0.f};
+    const int nrows = min(kRndRows, t.ocount - warp * kRndRows);  // the warp's rows (may be negative)
     int step = 0;
-    for (int y0 = 0; y0 < nk.n; y0 += 32) {
+    for (int y0 = 0; y0 < nk.n; y0 += 32, ++step) {
       const int y = y0 + lane;
       const bool on = y < nk.n;
       const float bh = on ? A.ah[d.rev_off + y] : -INFINITY;
       const float bl = on ? A.al[d.rev_off + y] : 0.f;
       float pb[3] = {0.f, 0.f, 0.f};
-      if (on && nk.coord_off >= 0)
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-          if (k < D) pb[k] = A.coords[nk.coord_off + (int64_t)y * D + k];
-      DF w = {0.f, 0.f};  // the column's factor: y (pass 3), err_c (pass 4)
-      if (PASS >= 3 && on) {
-        const double ycol = A.xy[d.rev_off + y];
-        // err_c = c - F''^T 1, F''^T 1 = y F'^T 1
-        w = df_of(PASS == 3 ? ycol : fmax(A.tgt[d.rev_off + y] - ycol * A.s2[d.rev_off + y], 0.0));
-      }
-      DF cs = {0.f, 0.f};
+      if (on) round_point(A, nk, p.D, y, pb);
+      TF w = {0.f, 0.f, 0.f};  // the column's factor: y (pass 3), err_c (pass 4)
+      if (PASS == 3 && on) w = tf_of(ldexp(A.xy[d.rev_off + y], kMid));
+      if (PASS == 4 && on) w = tf_of(ldexp(round_errc(A, d.rev_off + y), kMid));
+      TF cs = {0.f, 0.f, 0.f};
       if (on) {
 #pragma unroll
         for (int r = 0; r < kRndRows; ++r) {
-          const int ir = warp * kRndRows + r;
-          if (ir >= t.ocount) break;  // warp-uniform
-          const int i = t.o0 + ir;
-          DF c;
-          if (P.cost_kind == 0)
-            c = {own_rows ? Cm[(int64_t)i * cld + y] : Cm[(int64_t)y * cld + i], 0.f};
-          else
-            c = sq_dist_df(D, rp[r], pb);
+          if (r >= nrows) break;  // warp-uniform
+          const int i = t.o0 + warp * kRndRows + r;
+          const float4 q0 = s_row[warp * kRndRows + r][0], q1 = s_row[warp * kRndRows + r][1];
+          const float pa[3] = {q0.z, q0.w, q1.x};
+          const DF c = round_cost(p, i, y, pa, pb);
           if (PASS == 4) {
             if (c.hi == INFINITY) {
-              if (w.hi > 0.f) inf[r] = true;
+              if (w.a > 0.f) inf |= 1u << r;
               continue;
             }
             DF a = {fabsf(c.hi), c.hi < 0.f ? -c.lo : c.lo};
             df_renorm(a);  // a distance's low part may exceed an ulp of its high part: compare sums, not parts
             if (a.hi > cmax.hi || (a.hi == cmax.hi && a.lo > cmax.lo)) cmax = a;
-            df_acc(tacc[r], df_mul(w, c));
+            const float ch = c.hi * cmul, cl = c.lo * cmul, g = __fmul_rn(w.a, ch);
+            tf_acc(tacc[r], g, fmaf(w.b, ch, fmaf(w.a, cl, fmaf(w.a, ch, -g))));
             continue;
           }
           float cu;
-          const float B = plan_entry(rah[r], ral[r], bh, bl, c, kh, kl, cu);
+          const float B = plan_entry(q0.x, q0.y, bh, bl, c, p.kh, p.kl, cu);
           if (!(B > 0.f)) continue;  // also where the cost is +inf
+          if (PASS == 2) {
+            tf_acc(cs, tf_mul(B, TF{q1.y, q1.z, q1.w}));
+            continue;
+          }
+          const float ch = c.hi * cmul, cl = c.lo * cmul;
           if (PASS == 1) {
-            df_acc(racc[r], B);
-            df_acc(tacc[r], df_mul(B, c));
-            df_acc(cs, B);
-          } else if (PASS == 2) {
-            df_acc(cs, df_mul(B, xr[r]));
+            tf_acc(racc[r], B);
+            const float g = __fmul_rn(B, ch);
+            tf_acc(tacc[r], g, fmaf(B, cl, fmaf(B, ch, -g)));
+            tf_acc(cs, B);
           } else {
-            const DF b = df_mul(B, w);
-            df_acc(racc[r], b);
-            df_acc(tacc[r], df_mul(b, c));
+            const TF b = tf_mul(B, w);
+            tf_acc(racc[r], b);
+            const float g = __fmul_rn(b.a, ch);
+            tf_acc(tacc[r], g, fmaf(b.b, ch, fmaf(b.a, cl, fmaf(b.a, ch, -g))));
           }
         }
       }
-      if (PASS <= 2) {  // column sums: combined across the warps, one FP64 atomic per column
-        s_col[warp][lane] = make_float2(cs.hi, cs.lo);
-        __syncthreads();
-        if (warp == 0 && on) {
-          DF v = {0.f, 0.f};
+      if (PASS <= 2) {  // column sums: combined across the warps (in turn), one FP64 atomic per column
+        const int buf = step & 1;
+        s_col[buf][0][warp][lane] = cs.a;
+        s_col[buf][1][warp][lane] = cs.b;
+        s_col[buf][2][warp][lane] = cs.c;
+        double* col = PASS == 1 ? A.rsum : A.s2;
+        if (__syncthreads_or(!(fabsf(cs.a) <= 1e37f))) {  // eight such sums stay in range; else in FP64
+          if (on && nrows > 0) {
+            const int i0 = t.o0 + warp * kRndRows;
+            atomicAdd(&col[d.rev_off + y], round_col_fp64<PASS>(A, p, d, nj, nk, i0, i0 + nrows, y));
+          }
+        } else if (warp == (step & 7) && on) {
+          TF v = {0.f, 0.f, 0.f};
 #pragma unroll
-          for (int q = 0; q < 8; ++q) df_acc(v, DF{s_col[q][lane].x, s_col[q][lane].y});
-          if (v.hi != 0.f) atomicAdd(PASS == 1 ? &A.rsum[d.rev_off + y] : &A.s2[d.rev_off + y], df_to(v));
-        }
-        __syncthreads();
-      }
-      if (PASS != 2 && ++step == kRenormSteps) {
-        step = 0;
-#pragma unroll
-        for (int r = 0; r < kRndRows; ++r) {
-          df_renorm(racc[r]);
-          df_renorm(tacc[r]);
+          for (int q = 0; q < 8; ++q) tf_acc(v, TF{s_col[buf][0][q][lane], s_col[buf][1][q][lane], s_col[buf][2][q][lane]});
+          if (v.a != 0.f) atomicAdd(&col[d.rev_off + y], PASS == 2 ? ldexp(tf_to(v), -kUp) : tf_to(v));
         }
       }
     }
     if (PASS == 2) continue;
-    // row r's sums to lane r: one FP64 conversion for all rows
-    DF row = {0.f, 0.f}, ts = {0.f, 0.f};
-    bool rinf = false;
-#pragma unroll
-    for (int r = 0; r < kRndRows; ++r) {
-      if (PASS != 4) {
-        const DF v = warp_sum_df(racc[r]);
-        if (lane == r) row = v;
-      }
-      const DF w = warp_sum_df(tacc[r]);
-      if (lane == r) ts = w;
-      if (PASS == 4 && __any_sync(0xffffffffu, inf[r]) && lane == r) rinf = true;
+    const TF rs = PASS != 4 ? warp_rows_sum(racc) : TF{0.f, 0.f, 0.f}, ts = warp_rows_sum(tacc);
+    const int r = lane >> 2, ir = warp * kRndRows + r;
+    double row = tf_to(rs), cost = tf_to(ts) * cunit * p.cscale;
+    if (PASS == 3) row = ldexp(row, -kMid);
+    if (PASS >= 3) cost = ldexp(cost, -kMid);
+    // rows whose sums left the range
+    const unsigned off = __ballot_sync(0xffffffffu, r < nrows && (!tf_finite(rs) || !tf_finite(ts)));
+#pragma unroll 1
+    for (int k = 0; k < nrows; ++k) {
+      if (!(off >> 4 * k & 1u)) continue;  // warp-uniform
+      double a, b;
+      round_row_fp64<PASS>(A, p, d, nj, nk, t.o0 + warp * kRndRows + k, a, b);
+      if (r == k) row = a, cost = b;
     }
-    const int ir = warp * kRndRows + lane;
-    const bool mine = lane < kRndRows && ir < t.ocount;
+    if (PASS == 4) inf = __reduce_or_sync(0xffffffffu, inf);
     double tall = 0.0, msum = 0.0;
-    if (mine) {
+    if ((lane & 3) == 0 && r < nrows) {
       double x = 1.0;
       if (PASS == 3) x = A.xy[d.off + t.o0 + ir];
       if (PASS == 4) x = A.er[d.off + t.o0 + ir];
-      if (rinf)
+      if (inf >> r & 1)
         tall = x > 0.0 ? INFINITY : 0.0;
       else if (x != 0.0)
-        tall = x * cscale * df_to(ts);
+        tall = x * cost;
       if (PASS != 4) {
-        msum = x * df_to(row);
+        msum = x * row;
         (PASS == 1 ? A.rsum : A.s2)[d.off + t.o0 + ir] = msum;  // each row belongs to one task
       }
     }
 #pragma unroll
-    for (int o = kRndRows / 2; o; o >>= 1) {
+    for (int o = 16; o >= 4; o >>= 1) {  // lanes 0, 4, 8, .. hold the rows
       tall += __shfl_xor_sync(0xffffffffu, tall, o);
       if (PASS == 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
     }
@@ -364,7 +428,7 @@ __global__ void __launch_bounds__(256, 2) round_pass_df_kernel(RoundArgs A) {
     if (lane == 0 && tall != 0.0) atomicAdd(&acc[PASS == 1 ? 0 : PASS == 3 ? 1 : 2], tall);
     if (PASS == 1 && lane == 0 && msum != 0.0) atomicAdd(&acc[5], msum);
     if (PASS == 4) {
-      const double cm = warp_max_d(df_to(cmax) * cscale);
+      const double cm = warp_max_d(((double)cmax.hi + (double)cmax.lo) * p.cscale);
       if (lane == 0 && cm > 0.0)
         atomicMax((unsigned long long*)&acc[4], (unsigned long long)__double_as_longlong(cm));
     }
@@ -438,7 +502,7 @@ void pass(const RoundArgs& a, bool f64, int grid, cudaStream_t s) {
   else if constexpr (PASS == 5)
     round_pass_kernel<PASS, false><<<grid, 256, 0, s>>>(a);
   else
-    round_pass_df_kernel<PASS><<<grid, 256, 0, s>>>(a);
+    round_pass_tf_kernel<PASS><<<grid, 256, 0, s>>>(a);
 }
 
 template <int STEP>
