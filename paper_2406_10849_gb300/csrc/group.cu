@@ -199,8 +199,10 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
           const double dd = (double)v - (double)c[k];
           q += dd * dd;
         }
-      M[0] += d[0] * d[0], M[1] += d[0] * d[1], M[2] += d[0] * d[2];
-      M[3] += d[1] * d[1], M[4] += d[1] * d[2], M[5] += d[2] * d[2];
+      // in units of the grid: the coordinates' own unit may put squares, and a determinant of them, out of range
+      const float e0 = d[0] / unit, e1 = d[1] / unit, e2 = d[2] / unit;
+      M[0] += e0 * e0, M[1] += e0 * e1, M[2] += e0 * e2;
+      M[3] += e1 * e1, M[4] += e1 * e2, M[5] += e2 * e2;
       // s |x'|^2 as a two-float, its high part on the 2^-10 grid
       q *= s;
       const float qh = (float)(rint(q * kGrid) / kGrid);
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
       slot_q[at] = make_float2(qh, (float)(q - (double)qh));
     }
     // inverse of the second moments (with a small ridge; zero for a single place)
-    const float ridge = 1e-3f * (M[0] + M[3] + M[5]) / D + 1e-30f;
+    const float ridge = 1e-3f * (M[0] + M[3] + M[5]) / D;
     float I[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const float a = M[0] + ridge, d1 = M[3] + ridge, f = M[5] + ridge;
     if (D == 1) {
@@ -223,8 +225,10 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
       I[0] = A00 / det, I[1] = A01 / det, I[2] = A02 / det;
       I[3] = (a * f - M[2] * M[2]) / det, I[4] = (M[1] * M[2] - a * M[4]) / det, I[5] = (a * d1 - M[1] * M[1]) / det;
     }
-    for (int k = 0; k < 6; ++k)
-      if (!isfinite(I[k]) || ridge < 1e-25f) I[k] = 0.f;
+    for (int k = 0; k < 6; ++k) {
+      I[k] = I[k] / unit / unit;
+      if (!isfinite(I[k])) I[k] = 0.f;
+    }
     float4* r = grp + 3 * ((nd.slot_off + w.x0 + i0) / 8);
     r[0] = make_float4(c[0], c[1], c[2], unit);
     r[1] = make_float4(I[0], I[1], I[2], I[3]);

@@ -71,3 +71,27 @@ def test_wide_groups_are_counted():
             st = s.plan_stats()
         assert st["factored_edges"] == 2
         assert lo <= st["wide_points"] <= hi
+
+
+@pytest.mark.parametrize("k", [-24, 24])
+@pytest.mark.parametrize("dim", [1, 2, 3])
+def test_coordinates_in_other_units(dim, k):
+    """Coordinates times 2^k, the cost scale divided by 2^(2 k): the same problem, every step of it scaled by a power
+    of two, so the iterates agree bit for bit."""
+    import gen
+    import paper_2406_10849_gb300 as T
+    T.load()
+    rng = np.random.default_rng(dim)
+    coords = [rng.random((n, dim)).astype(np.float32) for n in (700, 500, 900)]
+    marg = {j: rng.dirichlet(np.ones(n)) for j, n in ((1, 500), (2, 900))}
+    out = []
+    for unit in (1.0, 2.0 ** k):
+        p = gen.TreeProblem(name="units", edges=gen.star_edges(2), n=np.array([700, 500, 900], np.int32),
+                            fixed=np.array([False, True, True]), marginals={j: m / m.sum() for j, m in marg.items()},
+                            eps=0.1, coords=[c * np.float32(unit) for c in coords], cost_scale=unit ** -2.0)
+        with T.Solver([p], T.options(autotune=False)) as s:
+            assert s.plan_stats()["factored_edges"] == 4
+            s.half_steps(4)
+            out.append(s.potentials(0))
+    for key in out[0]:
+        assert np.array_equal(out[0][key], out[1][key]), key
