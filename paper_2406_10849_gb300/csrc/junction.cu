@@ -181,9 +181,9 @@ __global__ void __launch_bounds__(256) jt_plan_kernel(const JtOp* op, double* ou
 constexpr int kJtSumBlock = 1024;  // entries per CTA of the sums
 
 
-// sums over tensors into slots; one CTA per (item, block of kJtSumBlock entries)
+// sums over tensors, one CTA and one partial sum per (item, block of kJtSumBlock entries)
 __global__ void __launch_bounds__(256) jt_sum_kernel(const JtSum* items, const int64_t* start, int32_t nitems,
-                                                     double* slots) {
+                                                     double* part) {
   __shared__ double red[8];
   if ((int64_t)blockIdx.x >= start[nitems]) return;
   const int it = jt_find(start, nitems, blockIdx.x);
@@ -201,7 +201,25 @@ __global__ void __launch_bounds__(256) jt_sum_kernel(const JtSum* items, const i
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += red[w];
-    atomicAdd(&slots[q.slot], t);
+    part[blockIdx.x] = t;
+  }
+}
+
+// the slots from the items' partial sums, one CTA per slot, in an order that does not change from run to run
+__global__ void __launch_bounds__(256) jt_slot_kernel(const JtSum* items, const int64_t* start, int32_t nitems,
+                                                      const double* part, double* slots) {
+  __shared__ double red[8];
+  double acc = 0.0;
+  for (int it = 0; it < nitems; ++it)  // few, sorted as planned
+    if (items[it].slot == (int)blockIdx.x)
+      for (int64_t b = start[it] + threadIdx.x; b < start[it + 1]; b += 256) acc += part[b];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    slots[blockIdx.x] = t;
   }
 }
 
@@ -260,6 +278,7 @@ struct tree_ot_jt_handle {
   int64_t arena_len = 0, cost_len = 0;
   double* d_arena = nullptr;
   float* d_cost = nullptr;
+  double* d_part = nullptr;    // partial sums, one per CTA of jt_sum_kernel
   double* d_slots = nullptr;   // 2 per separator
   int32_t* d_constrained = nullptr;
   double* d_res = nullptr;     // (sum, max)
@@ -839,6 +858,7 @@ int tree_ot_jt_create(const tree_ot_jt_problem* p, void* cuda_stream, tree_ot_jt
   if ((rc = upload_sums(h, h->res_sums, &h->d_res_sums, &h->d_res_start, &h->res_blocks, s)) ||
       (rc = upload_sums(h, h->tc_sums, &h->d_tc_sums, &h->d_tc_start, &h->tc_blocks, s)))
     return bail(rc);
+  if ((rc = jt_alloc(h, &h->d_part, std::max(h->res_blocks, h->tc_blocks)))) return bail(rc);
   if ((rc = jt_cuda(cudaStreamSynchronize(s), "cudaStreamSynchronize(create)"))) return bail(rc);
   *out = h;
   return TREE_OT_OK;
@@ -929,10 +949,11 @@ int tree_ot_jt_residual(tree_ot_jt_handle* h, void* cuda_stream, double* sum, do
   if (!h || !sum || !max) return jt_fail(TREE_OT_ERR_ARG, "NULL argument");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   for (const Stage& st : h->res_stages) JT_TRY(run_stage(st, s));
-  JT_TRY(jt_cuda(cudaMemsetAsync(h->d_slots, 0, sizeof(double) * (2 * (size_t)h->nsep + 1), s), "memset"));
   if (h->res_blocks > 0)
     jt_sum_kernel<<<(unsigned)h->res_blocks, 256, 0, s>>>(h->d_res_sums, h->d_res_start, (int32_t)h->res_sums.size(),
-                                                           h->d_slots);
+                                                           h->d_part);
+  jt_slot_kernel<<<2 * h->nsep, 256, 0, s>>>(h->d_res_sums, h->d_res_start, (int32_t)h->res_sums.size(), h->d_part,
+                                             h->d_slots);
   jt_residual_finish_kernel<<<1, 32, 0, s>>>(h->d_slots, h->d_constrained, h->nsep, h->d_res);
   JT_TRY(jt_cuda(cudaGetLastError(), "residual launch"));
   double r[2];
@@ -981,10 +1002,10 @@ int tree_ot_jt_transport_cost(tree_ot_jt_handle* h, void* cuda_stream, double* t
   if (!h || !tc) return jt_fail(TREE_OT_ERR_ARG, "NULL argument");
   cudaStream_t s = (cudaStream_t)cuda_stream;
   JT_TRY(run_stage(h->res_stages[0], s));
-  JT_TRY(jt_cuda(cudaMemsetAsync(h->d_slots, 0, sizeof(double), s), "memset"));
   if (h->tc_blocks > 0)
     jt_sum_kernel<<<(unsigned)h->tc_blocks, 256, 0, s>>>(h->d_tc_sums, h->d_tc_start, (int32_t)h->tc_sums.size(),
-                                                          h->d_slots);
+                                                          h->d_part);
+  jt_slot_kernel<<<1, 256, 0, s>>>(h->d_tc_sums, h->d_tc_start, (int32_t)h->tc_sums.size(), h->d_part, h->d_slots);
   JT_TRY(jt_cuda(cudaGetLastError(), "transport cost launch"));
   JT_TRY(jt_cuda(cudaMemcpyAsync(tc, h->d_slots, sizeof(double), cudaMemcpyDeviceToHost, s), "read cost"));
   return jt_cuda(cudaStreamSynchronize(s), "cudaStreamSynchronize(cost)");
