@@ -513,7 +513,7 @@ int fixed_records(const tree_ot_handle* h, const std::vector<DEdgeD>& dedges, in
 // The exact-distance plan: directed edges with the difference form's reduction splits, and the largest output
 // block that gives every SM two tasks.  Its device memory is taken at create (plan_exact) and filled when the
 // certification first asks for exact distances (fill_exact).
-int plan_exact(tree_ot_handle* h, int nsm) {
+int plan_exact(tree_ot_handle* h) {
   ExactPlan& x = h->xplan;
   bool any = false;
   for (const DEdgeD& d : h->dedges) any = any || fact_edge(h, d);
@@ -527,7 +527,7 @@ int plan_exact(tree_ot_handle* h, int nsm) {
     for (const DEdgeD& d : x.dedges)
       if (h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
         count[h->nodes[d.owner].colour] += (int64_t)((h->nodes[d.owner].n + x.rec_ob - 1) / x.rec_ob) * d.nsplit;
-    if (x.rec_ob == 256 || std::max(count[0], count[1]) >= 2 * nsm) break;
+    if (x.rec_ob == 256 || std::max(count[0], count[1]) >= 2 * h->sms) break;
   }
   for (int c = 0; c < 2; ++c) {
     for (const Task& t : h->tasks[c]) count[c] += t.kind < TASK_RECOMP;  // stored costs: as they are
@@ -1486,10 +1486,7 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   // large: more than four blocks of 64 outputs per colour for each of the GPU's 16 warps per SM
   int64_t blocks = 0, slots = 0;
   for (const GroupWork& w : work) blocks += (int64_t)((w.cnt + 63) / 64) * h->nodes[w.node].deg;
-  int dev = 0, nsm = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const bool many = blocks > (int64_t)2 * 4 * 16 * nsm;
+  const bool many = blocks > (int64_t)2 * 4 * 16 * h->sms;
   for (size_t i = 0; rc == TREE_OT_OK && i < work.size();) {
     NodeD& nd = h->nodes[work[i].node];
     int64_t wide[kGroupSizes] = {};
@@ -1536,7 +1533,7 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   for (const DEdgeD& d : h->dedges)
     if (fact_edge(h, d))
       warp_run[h->nodes[d.owner].colour] += (double)((h->nodes[d.owner].n + 63) / 64) * h->nodes[d.nbr].n;
-  for (double& w : warp_run) w = std::max(256.0, 1.5 * w / (16.0 * nsm));
+  for (double& w : warp_run) w = std::max(256.0, 1.5 * w / (16.0 * h->sms));
   for (size_t di = 0; di < h->dedges.size(); ++di) {
     DEdgeD& d = h->dedges[di];
     if (!fact_edge(h, d)) continue;
@@ -1642,6 +1639,7 @@ int setup_shared_kernels(tree_ot_handle* h, cudaStream_t s) {
       a.fix_count = fix_count;
       a.fix_list = fix_list;
       a.err = h->d_err;
+      a.sms = h->sms;
       a.use_tc = !(h->opt.flags & TREE_OT_OPT_SK_MMA_SYNC) && sk_tc_available() ? 1 : 0;
       a.tc_pair = a.use_tc && !(h->opt.flags & TREE_OT_OPT_SK_ONE_CTA) && sk_tc_pair_available() ? 1 : 0;
     }
@@ -1869,6 +1867,12 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   h->opt = o;
   h->fp64 = o.precision == TREE_OT_PREC_FP64;
   h->nprob = num_probs;
+  {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) h->sms = 1;
+    cudaGetLastError();
+  }
   int rc = TREE_OT_OK;
   // Stored costs: the column owner's apply reduces down columns, which streams
   // short row pieces at a large stride.  When the device has the room, each edge
@@ -1989,9 +1993,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   {
     int64_t pairs[2] = {0, 0};
     for (const NodeD& nd : h->nodes) pairs[nd.colour] += (int64_t)nd.n * std::max(nd.deg, 1);
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = h->sms;
     for (int c = 0; c < 2; ++c)
       h->chunk_pairs[c] = pairs[c] > (int64_t)kNodePairsSmall * 8 * nsm  ? kNodePairs
                           : pairs[c] > (int64_t)kNodePairsTiny * 4 * nsm ? kNodePairsSmall
@@ -2013,9 +2015,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   if (h->fp64) {
     int64_t rows[2] = {0, 0};
     for (const DEdgeD& d : h->dedges) rows[h->nodes[d.owner].colour] += h->nodes[d.owner].n;
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nsm = h->sms;
     const int64_t most = std::max(rows[0], rows[1]);
     if (most <= (int64_t)64 * 8 * nsm)
       for (h->f64_rows = 1; h->f64_rows < 8 && (int64_t)h->f64_rows * nsm < most;) h->f64_rows *= 2;
@@ -2173,10 +2173,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
     }
     h->fact_split = split;
     build_apply_tasks(h, kRecOut);
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if ((rc = plan_exact(h, nsm))) return bail(rc);
+    if ((rc = plan_exact(h))) return bail(rc);
   }
   if ((rc = setup_shared_kernels(h, s))) return bail(rc);
   if (!h->fp64) {  // host-resolved records of the fixed leaves' chunks, per colour
@@ -2295,10 +2292,7 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   }
   if (bad) return bail(fail(TREE_OT_ERR_NONFINITE, "a dense cost holds NaN or -inf"));
 
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  h->sms = sms;
+  const int sms = h->sms;
   for (int slot = 0; slot < kApplySlots; ++slot) {
     h->apply_grid[slot] = sms * apply_ctas_per_sm(slot, 0);
     for (int v = 0; v < 2; ++v) h->rec_grid[v][slot] = sms * apply_ctas_per_sm(slot, v);

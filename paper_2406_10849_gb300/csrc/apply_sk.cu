@@ -1191,7 +1191,7 @@ cudaError_t launch_sk(const SkArgs& args, const SkMaps* maps, cudaStream_t s, cu
     // per SM, each walking its columns in turn (26.5 us); below two per SM a CTA takes one batch of 8 (envelope and
     // its reduction together 30 -> 23 us; with the overlapped launches 7.02 -> 6.40 ms for 32 half-steps of
     // 500 stars, 6.60 without them)
-    a.env_cols = a.ncols > 2 * 152 * kEnvCols ? kEnvCols : kEnvBatch;
+    a.env_cols = a.ncols > 2 * a.sms * kEnvCols ? kEnvCols : kEnvBatch;
     int32_t nenv = (a.ncols + a.env_cols - 1) / a.env_cols;
     kargs[1] = &nenv;
     le = launch_pdl(reinterpret_cast<const void*>(sk_envelope1_kernel), nenv, 256, 0, s, kargs);
@@ -1239,7 +1239,7 @@ cudaError_t launch_sk(const SkArgs& args, const SkMaps* maps, cudaStream_t s, cu
   if (after_product) cudaEventRecord(after_product, s);
   le = cudaGetLastError();
   if (le != cudaSuccess) return le;
-  return launch_pdl(reinterpret_cast<const void*>(sk_fixup_kernel), 152 * 8, 256, 0, s, kargs);
+  return launch_pdl(reinterpret_cast<const void*>(sk_fixup_kernel), a.sms * 8, 256, 0, s, kargs);
 }
 
 cudaError_t launch_sk_reset(float* b, int32_t kd, cudaStream_t s) {

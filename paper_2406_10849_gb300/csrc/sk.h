@@ -62,6 +62,7 @@ struct SkArgs {
   const float* yc;        // column (neighbour) support, ny x dim
   float s_hi, s_lo;       // scale log2(e) / eps as a two-float
   float* b;               // [kd] envelope; -inf between uses
+  int32_t sms;            // the GPU's SMs (grid and block rules)
   int32_t env_cols;       // columns per CTA of the one-pass envelope kernel (set per launch)
   float* benv;            // [ceil(ncols / kSkEnvColsMin)][kd] per-CTA envelopes of the one-pass envelope kernel
   float* cmax;            // [ncols] column maxima M_j (-inf: inactive)
