@@ -201,10 +201,12 @@ typedef struct tree_ot_options {
     double refine_tol;        /* default 1e-5                                            */
     double absorb_tau;        /* default 48                                              */
     int32_t lowp_start;       /* default 16                                              */
-    int32_t autotune;         /* 1 (default): at create, time the recomputed-cost apply for
-                                 each tile shape (output block 256/512/1024, CTAs per SM)
-                                 and keep the fastest, cached per problem shape; and time
-                                 the two stored-cost kernels (see TREE_OT_OPT_DENSE_*)  */
+    int32_t autotune;         /* 1 (default): at create, time the recomputed-cost apply and
+                                 keep the fastest: output block 256/512/1024 and CTAs per SM
+                                 of the difference form, warps per block of the factored one,
+                                 and one launch for both against one each; cached per sizes
+                                 and forms.  And time the two stored-cost kernels (see
+                                 TREE_OT_OPT_DENSE_*)                                   */
 } tree_ot_options;
 
 /* ---- per-problem result ------------------------------------------------- */
@@ -418,7 +420,8 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * form (always summed by the difference form), [21] the most reduction splits of
  * a factored edge, [22] 1 while some problem runs with exact squared distances
  * (after a certification asked for them) and every recomputed cost of the handle
- * therefore takes the difference form. */
+ * therefore takes the difference form, [23] configurations of the recomputed-cost
+ * apply that create timed (0: none to choose, or found for these sizes before). */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);
 
 /* Launch timing (no paper counterpart: measurement support).  While enabled,

@@ -239,6 +239,8 @@ struct tree_ot_handle {
   int32_t f64_rows = 64;                   // FP64 apply: outputs per task (1 .. 8, or 64)
   int32_t fact_split = 0;                  // factored apply: log2 of the warps per block of 64 outputs (autotuned)
   ExactPlan xplan;
+  int32_t timed_configs = 0;               // configurations of the recomputed-cost apply timed at create
+  bool small_mixed = false;                // some but not all of the recomputed costs factored, on a small handle
   int64_t wide_points = 0;                 // points of factored nodes in groups that take the difference form
   bool both_forms = false;                 // both forms' tasks in one launch (autotuned; one dimension only)
   std::vector<FactItem> items[2];          // per colour: blocks of the factored apply, by dimension, largest first
@@ -386,6 +388,18 @@ bool fact_edge(const tree_ot_handle* h, const DEdgeD& d) {
   return h->nodes[d.owner].gs > 0 && h->nodes[d.nbr].n >= kGroupMin;
 }
 
+// v in ascending order of key(x), equal keys in their given order (sorts 16-byte pairs instead of the records)
+template <class T, class K>
+void sort_by_key(std::vector<T>& v, K key) {
+  std::vector<std::pair<uint64_t, uint32_t>> k(v.size());
+  for (size_t i = 0; i < v.size(); ++i) k[i] = {key(v[i]), (uint32_t)i};
+  if (std::is_sorted(k.begin(), k.end())) return;
+  std::sort(k.begin(), k.end());
+  std::vector<T> out(v.size());
+  for (size_t i = 0; i < v.size(); ++i) out[i] = v[k[i].second];
+  v.swap(out);
+}
+
 // points of the neighbour per reduction split of a factored edge
 int32_t fact_split_points(int32_t n_nbr, int32_t nsplit) {
   return (int32_t)align_up((n_nbr + nsplit - 1) / nsplit, 64);
@@ -456,10 +470,9 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob, bool exact = false) {
       return (int)h->probs[h->dedges[t.dedge].prob].dim + (t.kind >= TASK_FACT ? 3 : 0);
     };
     auto cost_of = [&](const Task& t) { return (int64_t)t.ocount * t.rcount; };
-    std::stable_sort(tasks[c].begin(), tasks[c].end(), [&](const Task& x, const Task& y) {
-      const int sx = slot_of(x), sy = slot_of(y);
-      if (sx != sy) return sx < sy;
-      return sx != 0 && cost_of(x) > cost_of(y);
+    sort_by_key(tasks[c], [&](const Task& x) {
+      const uint64_t slot = (uint64_t)slot_of(x) << 56;
+      return slot ? slot + ((1ull << 48) - (uint64_t)cost_of(x)) : slot;
     });
     for (const Task& t : tasks[c]) slot_count[c][slot_of(t)] += 1;
     int32_t b = 0;
@@ -1164,8 +1177,12 @@ uint64_t shape_signature(const tree_ot_handle* h) {
     mix((uint64_t)h->nodes[d.nbr].n);
     mix((uint64_t)h->probs[d.prob].dim);
     mix((uint64_t)h->nodes[d.owner].colour);
-    mix((uint64_t)h->nodes[d.owner].gs);
   }
+  // which forms the handle has, but not which edge has which: new points of the same sizes find the entry
+  bool form[2] = {false, false};
+  for (const DEdgeD& d : h->dedges)
+    if (h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID) form[fact_edge(h, d)] = true;
+  mix(form[0] + 2 * form[1]);
   return sig;
 }
 
@@ -1181,6 +1198,7 @@ int upload_tasks(tree_ot_handle* h, cudaStream_t s) {
 
 // one timing of both colours' applies with the current configuration (warm-up, then two of each)
 int time_applies(tree_ot_handle* h, cudaStream_t s, ApplySet set, cudaEvent_t e0, cudaEvent_t e1, float* ms) {
+  ++h->timed_configs;
   for (int rep = 0; rep < 3; ++rep) {
     if (rep == 1) CUDA_TRY(cudaEventRecord(e0, s));
     RC_TRY(launch_apply(h, 0, s, set));
@@ -1230,22 +1248,22 @@ int tune_applies(tree_ot_handle* h, cudaStream_t s, cudaEvent_t e0, cudaEvent_t 
     }
   }
   h->fact_split = cfg->split;
-  // difference form: output block, register budget and grid
+  // difference form: register budget and grid with blocks of 1024, then the block
   best = 1e30f;
-  for (int32_t ob : {1024, 512, 256}) {
-    if (!diff) break;
-    build_apply_tasks(h, ob);
-    RC_TRY(upload_tasks(h, s));
-    for (int32_t v = 0; v < 3; ++v) {
-      h->grid_mult = v == 2 ? 1 : 0;
-      h->rec_variant = v == 1 ? 1 : 0;
-      RC_TRY(time_applies(h, s, APPLY_DIFF, e0, e1, &ms));
-      if (ms < best) {
-        best = ms;
-        cfg->ob = ob;
-        cfg->gm = h->grid_mult;
-        cfg->variant = h->rec_variant;
-      }
+  for (int32_t k = 0; diff && k < 5; ++k) {
+    const int32_t ob = k < 3 ? 1024 : k == 3 ? 512 : 256;
+    if (k == 0 || k > 2) {
+      build_apply_tasks(h, ob);
+      RC_TRY(upload_tasks(h, s));
+    }
+    h->grid_mult = k < 3 ? (k == 2 ? 1 : 0) : cfg->gm;
+    h->rec_variant = k < 3 ? (k == 1 ? 1 : 0) : cfg->variant;
+    RC_TRY(time_applies(h, s, APPLY_DIFF, e0, e1, &ms));
+    if (ms < best) {
+      best = ms;
+      cfg->ob = ob;
+      cfg->gm = h->grid_mult;
+      cfg->variant = h->rec_variant;
     }
   }
   if (!diff || !fact || !one_dimension(h)) return TREE_OT_OK;
@@ -1253,7 +1271,7 @@ int tune_applies(tree_ot_handle* h, cudaStream_t s, cudaEvent_t e0, cudaEvent_t 
   RC_TRY(apply_tune(h, *cfg, s));
   float two = 0.f;
   RC_TRY(time_applies(h, s, APPLY_ALL, e0, e1, &two));
-  if (two > 0.4f) return TREE_OT_OK;  // 0.1 ms per apply: both launches fill the GPU
+  if (two > 1.0f) return TREE_OT_OK;  // 0.25 ms per apply: both launches fill the GPU
   const TuneCfg sep = *cfg;
   h->both_forms = true;
   for (int32_t ob : {1024, 512, 256})
@@ -1262,12 +1280,14 @@ int tune_applies(tree_ot_handle* h, cudaStream_t s, cudaEvent_t e0, cudaEvent_t 
       build_apply_tasks(h, ob);
       RC_TRY(upload_tasks(h, s));
       RC_TRY(time_applies(h, s, APPLY_ALL, e0, e1, &ms));
-      if (ms > 1.5f * two) break;
-      if (ms < (cfg->both ? best : two)) {
+      const float now = cfg->both ? best : two;
+      if (ms < now) {
         best = ms;
         cfg->ob = ob;
         cfg->split = lw;
         cfg->both = 1;
+      } else if (ms > 1.1f * now) {
+        break;  // more warps per block only get slower from here
       }
     }
   if (!cfg->both) *cfg = sep;
@@ -1469,32 +1489,32 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
       work.push_back(GroupWork{(int32_t)j, x0, std::min(kGroupChunk, nd.n - x0)});
   }
   if (work.empty()) return TREE_OT_OK;
+  // large: more than four blocks of 64 outputs per colour for each of the GPU's 16 warps per SM
+  int64_t blocks = 0;
+  for (const GroupWork& w : work) blocks += (int64_t)((w.cnt + 63) / 64) * h->nodes[w.node].deg;
+  const bool many = blocks > (int64_t)2 * 4 * 16 * h->sms;
+  const int32_t share = kGroupWide[many ? 0 : 1];
   GroupWork* d_work = nullptr;
   int32_t *d_meas = nullptr, *d_wide = nullptr;
   std::vector<int32_t> block_wide;  // per block of 64 slots: outputs in wide groups
   std::vector<int32_t> meas(kGroupSizes * work.size());
   const int32_t nw = (int32_t)work.size();
-  cudaError_t e = cudaMalloc((void**)&d_work, sizeof(GroupWork) * work.size());
-  if (e == cudaSuccess) e = cudaMalloc((void**)&d_meas, sizeof(int32_t) * meas.size());
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_work, work.data(), sizeof(GroupWork) * work.size(), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, d_meas, s);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(meas.data(), d_meas, sizeof(int32_t) * meas.size(), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  int rc = e == cudaSuccess ? TREE_OT_OK : cuda_fail(e, "measuring the point groups");
-  // large: more than four blocks of 64 outputs per colour for each of the GPU's 16 warps per SM
-  int64_t blocks = 0, slots = 0;
-  for (const GroupWork& w : work) blocks += (int64_t)((w.cnt + 63) / 64) * h->nodes[w.node].deg;
-  const bool many = blocks > (int64_t)2 * 4 * 16 * h->sms;
-  for (size_t i = 0; rc == TREE_OT_OK && i < work.size();) {
+  // (small tables, kept with the handle: freeing them here would wait for the device)
+  RC_TRY(h->alloc(&d_work, (int64_t)work.size()));
+  RC_TRY(h->alloc(&d_meas, (int64_t)meas.size()));
+  CUDA_TRY(cudaMemcpyAsync(d_work, work.data(), sizeof(GroupWork) * work.size(), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, share, d_meas, s));
+  CUDA_TRY(cudaMemcpyAsync(meas.data(), d_meas, sizeof(int32_t) * meas.size(), cudaMemcpyDeviceToHost, s));
+  CUDA_TRY(cudaStreamSynchronize(s));
+  int64_t slots = 0;
+  for (size_t i = 0; i < work.size();) {
     NodeD& nd = h->nodes[work[i].node];
     int64_t wide[kGroupSizes] = {};
     size_t k = i;
     for (; k < work.size() && work[k].node == work[i].node; ++k)
       for (int v = 0; v < kGroupSizes; ++v) wide[v] += meas[kGroupSizes * k + v];
     for (int v = 0; v < kGroupSizes && nd.gs == 0; ++v)
-      if (wide[v] * kGroupWide[many ? 0 : 1] <= nd.n) {
+      if (wide[v] * share <= nd.n) {
         nd.gs = 64 >> v;
         h->wide_points += wide[v];
       }
@@ -1504,27 +1524,20 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
     }
     i = k;
   }
-  if (rc == TREE_OT_OK && slots > 0 &&
-      !((rc = h->alloc(&h->d_slot_x, slots)) || (rc = h->alloc(&h->d_slot_q, slots)) ||
-        (rc = h->alloc(&h->d_grp, 3 * (slots / 8))) || (rc = h->alloc(&h->d_fallbacks, 1)))) {
-    block_wide.assign((size_t)(slots / 64), 0);
-    e = cudaMalloc((void**)&d_wide, sizeof(int32_t) * block_wide.size());
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_wide, 0, sizeof(int32_t) * block_wide.size(), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-      e = launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
-                             h->d_grp, d_wide, s);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(block_wide.data(), d_wide, sizeof(int32_t) * block_wide.size(), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) rc = cuda_fail(e, "building the point groups");
-  }
-  cudaFree(d_wide);
-  cudaFree(d_work);
-  cudaFree(d_meas);
-  if (rc) return rc;
+  if (slots == 0) return TREE_OT_OK;
+  block_wide.assign((size_t)(slots / 64), 0);
+  RC_TRY(h->alloc(&h->d_slot_x, slots));
+  RC_TRY(h->alloc(&h->d_slot_q, slots));
+  RC_TRY(h->alloc(&h->d_grp, 3 * (slots / 8)));
+  RC_TRY(h->alloc(&h->d_fallbacks, 1));
+  RC_TRY(h->alloc(&d_wide, (int64_t)block_wide.size()));
+  CUDA_TRY(cudaMemsetAsync(d_wide, 0, sizeof(int32_t) * block_wide.size(), s));
+  CUDA_TRY(cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s));
+  CUDA_TRY(cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
+                              h->d_grp, d_wide, s));
+  CUDA_TRY(cudaMemcpyAsync(block_wide.data(), d_wide, sizeof(int32_t) * block_wide.size(), cudaMemcpyDeviceToHost, s));
+  CUDA_TRY(cudaStreamSynchronize(s));
   // Points a warp may walk for its block of 64 outputs: an even share of the colour's work over the GPU's 16 warps
   // per SM, half as much again, at least 256.  Up to 8 warps share a block's points; beyond that the reduction is
   // split, its pieces merged by the node update (a leaf of 64 points at a centre of 65536, D = 2: 116 us per
@@ -1562,15 +1575,20 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
         h->items[own.colour].push_back(it);
       }
   }
+  {
+    int64_t fact = 0, rec = 0;
+    for (const DEdgeD& d : h->dedges) {
+      fact += fact_edge(h, d);
+      rec += h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID;
+    }
+    h->small_mixed = !many && fact > 0 && fact < rec;
+  }
   for (int c = 0; c < 2; ++c) {
     auto& v = h->items[c];
     auto dim = [&](const FactItem& x) { return h->probs[x.prob].dim; };
     // an output of a wide group takes about three times the time of the others
     auto cost = [&](const FactItem& x) { return (int64_t)(x.nrow + 2 * block_wide[(size_t)(x.slot0 / 64)]) * x.n_nbr; };
-    std::stable_sort(v.begin(), v.end(), [&](const FactItem& x, const FactItem& y) {
-      if (dim(x) != dim(y)) return dim(x) < dim(y);
-      return cost(x) > cost(y);
-    });
+    sort_by_key(v, [&](const FactItem& x) { return ((uint64_t)dim(x) << 56) + ((1ull << 48) - (uint64_t)cost(x)); });
     for (const FactItem& x : v) ++h->item_count[c][dim(x)];
     for (int k = 1; k < 4; ++k) h->item_begin[c][k] = h->item_begin[c][k - 1] + h->item_count[c][k - 1];
     if (v.empty()) continue;
@@ -2164,15 +2182,21 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
   {
     // device task arrays are sized for the finest blocking the autotuner may pick: output blocks of 256 of the
     // difference form, of 64 of the factored one
-    const int32_t split = h->fact_split;
-    h->fact_split = 3;
-    build_apply_tasks(h, 256);
-    for (int c = 0; c < 2; ++c) {
-      h->task_cap[c] = (int64_t)h->tasks[c].size();
-      if ((rc = h->alloc(&h->d_tasks[c], h->task_cap[c]))) return bail(rc);
-    }
-    h->fact_split = split;
     build_apply_tasks(h, kRecOut);
+    int64_t cap[2] = {0, 0};
+    for (int c = 0; c < 2; ++c)
+      for (const Task& k : h->tasks[c]) cap[c] += h->fp64 || k.kind < TASK_RECOMP;
+    for (const DEdgeD& d : h->dedges)
+      if (!h->fp64 && h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID) {
+        const int32_t ob = fact_edge(h, d) ? 64 : 256;
+        cap[h->nodes[d.owner].colour] += (int64_t)((h->nodes[d.owner].n + ob - 1) / ob) * d.nsplit;
+      }
+    for (int c = 0; c < 2; ++c) {
+      h->task_cap[c] = cap[c];
+      if ((rc = h->alloc(&h->d_tasks[c], cap[c]))) return bail(rc);
+    }
+    // without the autotuner: both forms of a small handle in one launch
+    h->both_forms = h->small_mixed && one_dimension(h);
     if ((rc = plan_exact(h))) return bail(rc);
   }
   if ((rc = setup_shared_kernels(h, s))) return bail(rc);
@@ -2198,11 +2222,12 @@ int tree_ot_create(const tree_ot_problem* probs, int32_t num_probs, const tree_o
       for (int32_t x = 0; x < nd.n; ++x) {
         const double v = h->mu[j][x];
         mu[nd.node_off + x] = v;
-        lg[nd.node_off + x] = v > 0.0 ? std::log(v) : -INFINITY;
+        const double lv = v > 0.0 ? std::log(v) : -INFINITY;
+        lg[nd.node_off + x] = lv;
         // log2 mu as (hi on the 2^-10 grid, lo), as the device splits values
         float4& g = lgf[nd.node_off + x];
         if (v > 0.0) {
-          const double l2 = std::log(v) * kLog2e;
+          const double l2 = lv * kLog2e;
           const float hi = std::rint((float)l2 * 1024.f) * (1.f / 1024.f);
           g = float4{hi, (float)(l2 - (double)hi), (float)v, 0.f};
         } else {
@@ -2939,7 +2964,7 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
   }
-  const int64_t v[23] = {(int64_t)h->dedges.size(),
+  const int64_t v[24] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2961,8 +2986,9 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         (int64_t)fallbacks,
                         h->wide_points,
                         fact_splits,
-                        (int64_t)(exact_plan(h) ? 1 : 0)};
-  for (int32_t i = 0; i < nstats && i < 23; ++i) stats[i] = v[i];
+                        (int64_t)(exact_plan(h) ? 1 : 0),
+                        (int64_t)h->timed_configs};
+  for (int32_t i = 0; i < nstats && i < 24; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

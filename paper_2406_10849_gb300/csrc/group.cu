@@ -78,13 +78,16 @@ __device__ __forceinline__ int iroot(int v, int p) {
 // part k of n groups in S parts begins at group k n / S; the part that holds group g
 __device__ __forceinline__ int part_of(int g, int n, int S) { return ((g + 1) * S - 1) / n; }
 
-// key order of the chunk's points for groups of gs; on return the low 16 bits
+// the chunk's points in order of their first coordinate; on return the low 16 bits
 // of keys[i] are the chunk-relative index of the i-th point
-__device__ void str_order(const float* x, int D, int cnt, int m, int gs, uint64_t* keys) {
+__device__ void first_order(const float* x, int D, int cnt, int m, uint64_t* keys) {
   for (int i = threadIdx.x; i < m; i += kGroupThreads)
     keys[i] = i < cnt ? ((uint64_t)float_key(x[(int64_t)i * D]) << 16) | (uint32_t)i : ~0ull;
   bitonic_sort(keys, m);
-  if (D == 1) return;
+}
+
+// from there the order for groups of gs (D > 1; in one dimension the first order is it)
+__device__ void str_order(const float* x, int D, int cnt, int m, int gs, uint64_t* keys) {
   const int ng = (cnt + gs - 1) / gs;
   const int S = iroot(ng, D);
   for (int i = threadIdx.x; i < cnt; i += kGroupThreads) {
@@ -132,11 +135,14 @@ __device__ __forceinline__ bool group_wide(int gs, int D, float s, float r) {
   return !(s * r * r <= (gs == 16 && D == 3 ? kGroupKappa16 : kGroupKappa));
 }
 
-// the points of the chunk that lie in wide groups, for every group size
+// The points of the chunk that lie in wide groups, for every group size; a node of a single chunk stops at the
+// first size that leaves few enough of them (a 1 / share; the sizes after it count as wide throughout)
 __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const GroupWork* work, const NodeD* nodes,
                                                                       const ProbD* probs, const float* coords,
-                                                                      const uint32_t* cmax, int32_t* out) {
+                                                                      const uint32_t* cmax, int32_t share,
+                                                                      int32_t* out) {
   __shared__ uint64_t keys[kGroupChunk];
+  __shared__ uint16_t first[kGroupChunk];
   __shared__ int s_wide;
   const GroupWork w = work[blockIdx.x];
   const NodeD nd = nodes[w.node];
@@ -145,9 +151,23 @@ __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const Grou
   const float* x = coords + nd.coord_off + (int64_t)w.x0 * D;
   const float unit = grid_unit(__uint_as_float(cmax[nd.prob]));
   const int m = pow2_at_least(w.cnt);
+  bool found = false;
+  first_order(x, D, w.cnt, m, keys);
+  if (D > 1)
+    for (int i = threadIdx.x; i < w.cnt; i += kGroupThreads) first[i] = (uint16_t)keys[i];
   for (int v = 0; v < kGroupSizes; ++v) {
     const int gs = 64 >> v;
-    str_order(x, D, w.cnt, m, gs, keys);
+    if (found) {  // block-uniform
+      if (threadIdx.x == 0) out[kGroupSizes * blockIdx.x + v] = w.cnt;
+      continue;
+    }
+    if (D > 1) {
+      __syncthreads();
+      if (v > 0)
+        for (int i = threadIdx.x; i < m; i += kGroupThreads) keys[i] = i < w.cnt ? first[i] : ~0ull;
+      __syncthreads();
+      str_order(x, D, w.cnt, m, gs, keys);
+    }
     if (threadIdx.x == 0) s_wide = 0;
     __syncthreads();
     for (int g = threadIdx.x; g < (w.cnt + gs - 1) / gs; g += kGroupThreads) {
@@ -161,6 +181,8 @@ __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const Grou
     }
     __syncthreads();
     if (threadIdx.x == 0) out[kGroupSizes * blockIdx.x + v] = s_wide;
+    found = w.cnt == nd.n && s_wide * share <= w.cnt;
+    __syncthreads();
   }
 }
 
@@ -177,7 +199,8 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
   const int D = probs[nd.prob].dim;
   const double s = probs[nd.prob].cost_scale * kLog2e * probs[nd.prob].inv_eps;
   const float* x = coords + nd.coord_off + (int64_t)w.x0 * D;
-  str_order(x, D, w.cnt, pow2_at_least(w.cnt), gs, keys);
+  first_order(x, D, w.cnt, pow2_at_least(w.cnt), keys);
+  if (D > 1) str_order(x, D, w.cnt, pow2_at_least(w.cnt), gs, keys);
   const float unit = grid_unit(__uint_as_float(cmax[nd.prob]));
   // a chunk but the last holds a multiple of 64 points; pads run to the end of the last block of 64
   const int slots = (w.cnt + 63) / 64 * 64;
@@ -241,9 +264,10 @@ __global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupW
 }  // namespace
 
 cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, const uint32_t* cmax, int32_t* out, cudaStream_t s) {
+                                 const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
+                                 cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  group_measure_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, out);
+  group_measure_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, share, out);
   return cudaGetLastError();
 }
 

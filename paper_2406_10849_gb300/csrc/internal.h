@@ -439,7 +439,8 @@ cudaError_t launch_transpose_pad(const float* src, int64_t src_ld, int32_t rows,
                                  int64_t dst_ld, cudaStream_t s);
 // coordinates split hi + lo for the exact-distance recomputation (cmax: nprob scratch words)
 cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, const uint32_t* cmax, int32_t* out, cudaStream_t s);
+                                 const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
+                                 cudaStream_t s);
 cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
                                const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
                                int32_t* block_wide, cudaStream_t s);

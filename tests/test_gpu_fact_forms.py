@@ -176,3 +176,23 @@ def test_certification_switches_to_the_exact_plan_and_back(persistent):
         for i, f in zip((0, 9), first):
             again = s.potentials(i)
             assert all(np.array_equal(f[k], again[k]) for k in again)
+
+
+def test_new_points_of_known_sizes_are_not_timed_again():
+    """The autotuner's choice is kept per sizes and forms: another batch of points and eps on the same trees, which
+    groups its points differently, takes it over."""
+    import gen
+    import paper_2406_10849_gb300 as T
+    T.load()
+    timed = []
+    for seed in range(4):
+        rng = np.random.default_rng(seed)
+        probs = []
+        for n in ((333, 301, 77), (205, 411, 1033, 90)):
+            p = cloud_star(n, 2, float(np.exp(rng.uniform(np.log(0.01), np.log(0.03)))), seed=seed)
+            probs.append(p)
+        with T.Solver(probs, T.options()) as s:
+            st = s.plan_stats()
+        assert 0 < st["factored_edges"] < st["directed_edges"]
+        timed.append(st["timed_configs"])
+    assert timed[0] > 0 and timed[1:] == [0, 0, 0]
