@@ -47,7 +47,8 @@ def plans_of(s, p):
 @pytest.mark.parametrize("steps", [1, 6])
 def test_feasible_to_fp64_rounding(T, n, kind, steps):
     """Fixed marginals of the rounded plans in L1, in units of 2^-53: one rounding each for the target, the scales x
-    and y, err_r, err_c, E and the entry's products, and the sums of this test (pairwise) beside them: at most 8."""
+    and y, err_r, err_c, E and the entry's products, and the sums of this test (pairwise) beside them: 8; and one
+    for every FP64 addition of a task of 64 rows to a column's sum, in an order that changes from run to run."""
     rng = np.random.default_rng(n)
     p = gen.random_tree_problem(rng, 4, n_range=(n, n + 13), eps_range=(0.05, 0.05), D=2, name="gap")
     p.cost_kind = kind
@@ -60,7 +61,7 @@ def test_feasible_to_fp64_rounding(T, n, kind, steps):
         for j, q in ((int(a), plan.sum(1)), (int(b), plan.sum(0))):
             if p.fixed[j]:
                 worst = max(worst, float(np.abs(q - p.marginals[j] / p.marginals[j].sum()).sum()))
-    assert worst <= 8.0 * 2.0 ** -53
+    assert worst <= (8.0 + (n + 13 + 63) // 64) * 2.0 ** -53
 
 
 @pytest.mark.parametrize("k", [-90, 90])
