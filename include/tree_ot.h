@@ -421,7 +421,8 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * a factored edge, [22] 1 while some problem runs with exact squared distances
  * (after a certification asked for them) and every recomputed cost of the handle
  * therefore takes the difference form, [23] configurations of the recomputed-cost
- * apply that create timed (0: none to choose, or found for these sizes before). */
+ * apply that create timed (0: none to choose, or found for these sizes before),
+ * [24] to [26] nodes whose points lie in groups of 64, 32 and 16. */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);
 
 /* Launch timing (no paper counterpart: measurement support).  While enabled,

@@ -2959,12 +2959,15 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
       ++fact_edges;
       fact_splits = std::max<int64_t>(fact_splits, d.nsplit);
     }
+  int64_t grouped[kGroupSizes] = {};
+  for (const NodeD& nd : h->nodes)
+    for (int v = 0; v < kGroupSizes; ++v) grouped[v] += nd.gs == 64 >> v;
   unsigned long long fallbacks = 0;
   if (nstats > 19 && h->d_fallbacks) {
     CUDA_TRY(cudaDeviceSynchronize());
     CUDA_TRY(cudaMemcpy(&fallbacks, h->d_fallbacks, sizeof(fallbacks), cudaMemcpyDeviceToHost));
   }
-  const int64_t v[24] = {(int64_t)h->dedges.size(),
+  const int64_t v[27] = {(int64_t)h->dedges.size(),
                         (int64_t)h->edges.size(),
                         h->elems,
                         h->matrix_bytes,
@@ -2987,8 +2990,11 @@ int tree_ot_plan_stats(tree_ot_handle* h, int64_t* stats, int32_t nstats) {
                         h->wide_points,
                         fact_splits,
                         (int64_t)(exact_plan(h) ? 1 : 0),
-                        (int64_t)h->timed_configs};
-  for (int32_t i = 0; i < nstats && i < 24; ++i) stats[i] = v[i];
+                        (int64_t)h->timed_configs,
+                        grouped[0],
+                        grouped[1],
+                        grouped[2]};
+  for (int32_t i = 0; i < nstats && i < 27; ++i) stats[i] = v[i];
   return TREE_OT_OK;
 }
 

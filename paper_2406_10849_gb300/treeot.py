@@ -512,13 +512,14 @@ class Solver:
             self.set_potential(prob, 2 * e + 1, f[(int(b), int(a))])
 
     def plan_stats(self) -> dict:
-        st = (C.c_int64 * 24)()
-        _check(_lib.tree_ot_plan_stats(self.h, st, 24))
+        st = (C.c_int64 * 27)()
+        _check(_lib.tree_ot_plan_stats(self.h, st, 27))
         keys = ["directed_edges", "edges", "elements_per_half_step", "matrix_bytes_per_half_step",
                 "apply_tasks_c0", "apply_tasks_c1", "device_bytes", "node_ctas_c0", "node_ctas_c1",
                 "recompute_output_block", "recompute_ctas_per_sm", "recompute_variant", "dense_tma",
                 "persistent", "node_defer", "sk_product", "factored_edges", "factored_split", "both_forms",
-                "factored_fallbacks", "wide_points", "factored_splits", "exact_plan", "timed_configs"]
+                "factored_fallbacks", "wide_points", "factored_splits", "exact_plan", "timed_configs",
+                "nodes_in_64", "nodes_in_32", "nodes_in_16"]
         return dict(zip(keys, [int(x) for x in st]))
 
 

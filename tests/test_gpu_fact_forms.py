@@ -196,3 +196,26 @@ def test_new_points_of_known_sizes_are_not_timed_again():
         assert 0 < st["factored_edges"] < st["directed_edges"]
         timed.append(st["timed_configs"])
     assert timed[0] > 0 and timed[1:] == [0, 0, 0]
+
+
+@pytest.mark.parametrize("split", range(4))
+@pytest.mark.parametrize("n,dim,eps,clustered,sizes", [
+    ((900, 700, 450, 1300, 260), 1, 0.002, False, (64, 32, 16)),
+    ((577, 1215, 1480, 802, 940, 1895), 2, 0.01, False, (64, 32, 16)),
+    ((900, 700, 450, 1300), 3, 0.05, False, (64, 32)), ((1470, 40), 3, 0.05, True, (16,))])
+def test_group_sizes(n, dim, eps, clustered, sizes, split):
+    """Nodes of every group size in every dimension, each with one and several warps per block."""
+    import paper_2406_10849_gb300 as T
+    T.load()
+    p = cloud_star(n, dim, eps, seed=21, clustered=clustered)
+    with solver(T, p, split, 0) as s:
+        st = s.plan_stats()
+        for gs in sizes:
+            assert st[f"nodes_in_{gs}"] > 0, gs
+        for steps in (2, 3):
+            s.reset()
+            s.half_steps(steps)
+            got = s.potentials(0)
+            ref = O.run_half_steps(p, steps)
+            assert rel_err(got, ref, p.eps) <= 1e-4
+            assert marginal_gap(p, got, ref) <= 1e-6  # the bar of every FP32 iterate
