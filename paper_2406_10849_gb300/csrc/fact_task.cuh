@@ -18,8 +18,8 @@
 //
 // Accuracy.  Differences are taken on the 2^-10 sigma coordinate grid of
 // split_coords_kernel: |y - c|^2 is exact up to its small low part, A lives on
-// the 2^-10 grid of the operands, and what is left of it (|e| <= 2^-11) is the
-// term's weight w = 2^e.  The remaining roundings are those of the products
+// the 2^-10 grid of the operands, and what is left of it, with the operand's low
+// part (|e| <= 2^-10 together), is the term's weight w = 2^e.  The remaining roundings are those of the products
 // x'_k Y_k, of size s r |y'|; cy comes from a least-squares slope of the
 // previous messages' frames over the group, which makes y' of the significant
 // terms small (the spread of the targets, not the transport distance).  The

@@ -30,7 +30,7 @@ int forest_ctas_per_sm(int D, bool exact, int minb, uint32_t smem) {
                  : D == 2 ? forest_kernel_ptr<2>(exact, minb)
                  : D == 3 ? forest_kernel_ptr<3>(exact, minb) : nullptr;
   if (!fn) return 0;
-  // static (24 KB of apply staging) plus dynamic shared memory may pass the default 48 KB
+  // static (28 KB of apply staging) plus dynamic shared memory may pass the default 48 KB
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kApplyThreads, smem) != cudaSuccess) return 0;
