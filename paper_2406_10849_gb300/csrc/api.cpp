@@ -341,15 +341,36 @@ struct tree_ot_handle {
   double last_wall_ms = 0.0;
   std::vector<int32_t> last_status;
 
+  // Device memory that lives as long as the handle.  A plan has some seventy tables, most of a few KB, and a
+  // cudaMalloc takes about 3 us: small ones come from slabs of 256 KB, then twice the last up to 4 MB, each table
+  // on a 256-byte boundary.
+  char* slab = nullptr;
+  size_t slab_left = 0, slab_next = (size_t)1 << 18;
+
   template <class T>
   int alloc(T** p, int64_t count) {
     *p = nullptr;
     if (count <= 0) count = 1;
-    const size_t bytes = sizeof(T) * (size_t)count;
-    cudaError_t e = cudaMalloc((void**)p, bytes);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-    owned.push_back(*p);
-    device_bytes += (int64_t)bytes;
+    const size_t bytes = sizeof(T) * (size_t)count, room = (bytes + 255) / 256 * 256;
+    const bool small = room <= slab_next / 2 || room <= slab_left;
+    if (!small || room > slab_left) {
+      void* q = nullptr;
+      const size_t take = small ? slab_next : bytes;
+      cudaError_t e = cudaMalloc(&q, take);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
+      owned.push_back(q);
+      device_bytes += (int64_t)take;
+      if (!small) {
+        *p = static_cast<T*>(q);
+        return TREE_OT_OK;
+      }
+      slab = static_cast<char*>(q);
+      slab_left = take;
+      slab_next = std::min(slab_next * 2, (size_t)1 << 22);
+    }
+    *p = reinterpret_cast<T*>(slab);
+    slab += room;
+    slab_left -= room;
     return TREE_OT_OK;
   }
 };
