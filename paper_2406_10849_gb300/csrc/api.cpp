@@ -1503,11 +1503,16 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   // exact distances from the first half-step: the difference form throughout
   if (h->fp64 || (h->opt.flags & TREE_OT_OPT_EXACT_DIST)) return TREE_OT_OK;
   std::vector<GroupWork> work;
+  int64_t slots = 0;
+  bool chunked = false;  // a node of several chunks
   for (size_t j = 0; j < h->nodes.size(); ++j) {
-    const NodeD& nd = h->nodes[j];
+    NodeD& nd = h->nodes[j];
     if (nd.coord_off < 0 || nd.n < kGroupMin || h->probs[nd.prob].cost_kind != TREE_OT_COST_SQEUCLID) continue;
+    nd.slot_off = slots;
+    slots += align_up(nd.n, 64);
     for (int32_t x0 = 0; x0 < nd.n; x0 += kGroupChunk)
-      work.push_back(GroupWork{(int32_t)j, x0, std::min(kGroupChunk, nd.n - x0)});
+      work.push_back(GroupWork{(int32_t)j, x0, std::min(kGroupChunk, nd.n - x0), 0, nd.slot_off + x0});
+    chunked = chunked || nd.n > kGroupChunk;
   }
   if (work.empty()) return TREE_OT_OK;
   // large: more than four blocks of 64 outputs per colour for each of the GPU's 16 warps per SM
@@ -1515,50 +1520,44 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
   for (const GroupWork& w : work) blocks += (int64_t)((w.cnt + 63) / 64) * h->nodes[w.node].deg;
   const bool many = blocks > (int64_t)2 * 4 * 16 * h->sms;
   const int32_t share = kGroupWide[many ? 0 : 1];
-  GroupWork* d_work = nullptr;
-  int32_t *d_meas = nullptr, *d_wide = nullptr;
-  std::vector<int32_t> block_wide;  // per block of 64 slots: outputs in wide groups
-  std::vector<int32_t> meas(kGroupSizes * work.size());
   const int32_t nw = (int32_t)work.size();
-  // (small tables, kept with the handle: freeing them here would wait for the device)
-  RC_TRY(h->alloc(&d_work, (int64_t)work.size()));
-  RC_TRY(h->alloc(&d_meas, (int64_t)meas.size()));
+  GroupWork* d_work = nullptr;
+  int32_t* d_counts = nullptr;
+  // per chunk and size the points in wide groups, then per block of 64 slots its outputs in wide groups
+  std::vector<int32_t> counts(kGroupSizes * work.size() + (size_t)(slots / 64), 0);
+  const int32_t* block_wide = counts.data() + kGroupSizes * work.size();
+  RC_TRY(h->alloc(&d_work, nw));
+  RC_TRY(h->alloc(&d_counts, (int64_t)counts.size()));
+  RC_TRY(h->alloc(&h->d_slot_x, slots));
+  RC_TRY(h->alloc(&h->d_slot_q, slots));
+  RC_TRY(h->alloc(&h->d_grp, 3 * (slots / 8)));
+  RC_TRY(h->alloc(&h->d_fallbacks, 1));
+  const GroupTables tables{h->d_slot_x, h->d_slot_q, h->d_grp, d_counts + kGroupSizes * work.size()};
+  CUDA_TRY(cudaMemsetAsync(d_counts, 0, sizeof(int32_t) * counts.size(), s));
+  CUDA_TRY(cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s));
   CUDA_TRY(cudaMemcpyAsync(d_work, work.data(), sizeof(GroupWork) * work.size(), cudaMemcpyHostToDevice, s));
-  CUDA_TRY(launch_group_measure(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, share, d_meas, s));
-  CUDA_TRY(cudaMemcpyAsync(meas.data(), d_meas, sizeof(int32_t) * meas.size(), cudaMemcpyDeviceToHost, s));
+  CUDA_TRY(launch_group_plan(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, share, d_counts, tables, s));
+  CUDA_TRY(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int32_t) * counts.size(), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  int64_t slots = 0;
   for (size_t i = 0; i < work.size();) {
     NodeD& nd = h->nodes[work[i].node];
     int64_t wide[kGroupSizes] = {};
     size_t k = i;
     for (; k < work.size() && work[k].node == work[i].node; ++k)
-      for (int v = 0; v < kGroupSizes; ++v) wide[v] += meas[kGroupSizes * k + v];
+      for (int v = 0; v < kGroupSizes; ++v) wide[v] += counts[kGroupSizes * k + v];
     for (int v = 0; v < kGroupSizes && nd.gs == 0; ++v)
       if (wide[v] * share <= nd.n) {
         nd.gs = 64 >> v;
         h->wide_points += wide[v];
       }
-    if (nd.gs) {
-      nd.slot_off = slots;
-      slots += align_up(nd.n, 64);
-    }
     i = k;
   }
-  if (slots == 0) return TREE_OT_OK;
-  block_wide.assign((size_t)(slots / 64), 0);
-  RC_TRY(h->alloc(&h->d_slot_x, slots));
-  RC_TRY(h->alloc(&h->d_slot_q, slots));
-  RC_TRY(h->alloc(&h->d_grp, 3 * (slots / 8)));
-  RC_TRY(h->alloc(&h->d_fallbacks, 1));
-  RC_TRY(h->alloc(&d_wide, (int64_t)block_wide.size()));
-  CUDA_TRY(cudaMemsetAsync(d_wide, 0, sizeof(int32_t) * block_wide.size(), s));
-  CUDA_TRY(cudaMemsetAsync(h->d_fallbacks, 0, sizeof(unsigned long long), s));
-  CUDA_TRY(cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s));
-  CUDA_TRY(launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, h->d_slot_x, h->d_slot_q,
-                              h->d_grp, d_wide, s));
-  CUDA_TRY(cudaMemcpyAsync(block_wide.data(), d_wide, sizeof(int32_t) * block_wide.size(), cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(cudaStreamSynchronize(s));
+  if (chunked) {  // the sizes of these nodes follow from all of their chunks
+    CUDA_TRY(cudaMemcpyAsync(h->d_nodes, h->nodes.data(), sizeof(NodeD) * h->nodes.size(), cudaMemcpyHostToDevice, s));
+    CUDA_TRY(launch_group_build(d_work, nw, h->d_nodes, h->d_probs, h->d_coords, h->d_cmax, tables, s));
+    CUDA_TRY(cudaMemcpyAsync(counts.data(), d_counts, sizeof(int32_t) * counts.size(), cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+  }
   // Points a warp may walk for its block of 64 outputs: an even share of the colour's work over the GPU's 16 warps
   // per SM, half as much again, at least 256.  Up to 8 warps share a block's points; beyond that the reduction is
   // split, its pieces merged by the node update (a leaf of 64 points at a centre of 65536, D = 2: 116 us per
@@ -1616,7 +1615,6 @@ int plan_groups(tree_ot_handle* h, cudaStream_t s) {
     RC_TRY(h->alloc(&h->d_items[c], (int64_t)v.size()));
     CUDA_TRY(cudaMemcpyAsync(h->d_items[c], v.data(), sizeof(FactItem) * v.size(), cudaMemcpyHostToDevice, s));
   }
-  CUDA_TRY(cudaStreamSynchronize(s));
   return TREE_OT_OK;
 }
 

@@ -135,12 +135,92 @@ __device__ __forceinline__ bool group_wide(int gs, int D, float s, float r) {
   return !(s * r * r <= (gs == 16 && D == 3 ? kGroupKappa16 : kGroupKappa));
 }
 
-// The points of the chunk that lie in wide groups, for every group size; a node of a single chunk stops at the
-// first size that leaves few enough of them (a 1 / share; the sizes after it count as wide throughout)
-__global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const GroupWork* work, const NodeD* nodes,
-                                                                      const ProbD* probs, const float* coords,
-                                                                      const uint32_t* cmax, int32_t share,
-                                                                      int32_t* out) {
+// slots and group records of a chunk in groups of gs, its points in the order of keys
+__device__ void build_groups(const GroupWork& w, const ProbD& P, const float* x, const uint64_t* keys, int gs,
+                             float unit, const GroupTables& T) {
+  const int D = P.dim;
+  const double s = P.cost_scale * kLog2e * P.inv_eps;
+  // a chunk but the last holds a multiple of 64 points; pads run to the end of the last block of 64
+  const int slots = (w.cnt + 63) / 64 * 64;
+  for (int g = threadIdx.x; g < slots / gs; g += kGroupThreads) {
+    const int i0 = g * gs, i1 = min(i0 + gs, w.cnt);
+    float c[3] = {0.f, 0.f, 0.f};
+    float M[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // second moments 00 01 02 11 12 22
+    float far = 0.f;  // the largest coordinate difference to the centre
+    group_centre(x, D, keys, i0, i1, unit, c);
+    for (int i = i0; i < i0 + gs; ++i) {
+      const uint32_t idx = (uint32_t)keys[min(i, w.cnt - 1)] & 0xffffu;  // pads repeat the last point
+      float d[3] = {0.f, 0.f, 0.f};
+      double q = 0.0;
+      if (i < i1)
+        for (int k = 0; k < D; ++k) {
+          const float v = x[(int64_t)idx * D + k];
+          d[k] = v - c[k];
+          far = fmaxf(far, fabsf(d[k]));
+          const double dd = (double)v - (double)c[k];
+          q += dd * dd;
+        }
+      // in units of the grid: the coordinates' own unit may put squares, and a determinant of them, out of range
+      const float e0 = d[0] / unit, e1 = d[1] / unit, e2 = d[2] / unit;
+      M[0] += e0 * e0, M[1] += e0 * e1, M[2] += e0 * e2;
+      M[3] += e1 * e1, M[4] += e1 * e2, M[5] += e2 * e2;
+      // s |x'|^2 as a two-float, its high part on the 2^-10 grid
+      q *= s;
+      const float qh = (float)(rint(q * kGrid) / kGrid);
+      const int64_t at = w.slot + i;
+      T.slot_x[at] = make_float4(d[0], d[1], d[2], __int_as_float(w.x0 + (int)idx));
+      T.slot_q[at] = make_float2(qh, (float)(q - (double)qh));
+    }
+    // inverse of the second moments (with a small ridge; zero for a single place)
+    const float ridge = 1e-3f * (M[0] + M[3] + M[5]) / D;
+    float I[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float a = M[0] + ridge, d1 = M[3] + ridge, f = M[5] + ridge;
+    if (D == 1) {
+      I[0] = 1.f / a;
+    } else if (D == 2) {
+      const float det = a * d1 - M[1] * M[1];
+      I[0] = d1 / det, I[1] = -M[1] / det, I[2] = a / det;
+    } else {
+      const float A00 = d1 * f - M[4] * M[4], A01 = M[2] * M[4] - M[1] * f, A02 = M[1] * M[4] - M[2] * d1;
+      const float det = a * A00 + M[1] * A01 + M[2] * A02;
+      I[0] = A00 / det, I[1] = A01 / det, I[2] = A02 / det;
+      I[3] = (a * f - M[2] * M[2]) / det, I[4] = (M[1] * M[2] - a * M[4]) / det, I[5] = (a * d1 - M[1] * M[1]) / det;
+    }
+    for (int k = 0; k < 6; ++k) {
+      I[k] = I[k] / unit / unit;
+      if (!isfinite(I[k])) I[k] = 0.f;
+    }
+    float4* r = T.grp + 3 * ((w.slot + i0) / 8);
+    r[0] = make_float4(c[0], c[1], c[2], unit);
+    r[1] = make_float4(I[0], I[1], I[2], I[3]);
+    const bool wide = i1 > i0 && group_wide(gs, D, P.s2_scaled, far);
+    r[2] = make_float4(I[4], I[5], wide ? 1.f : 0.f, 0.f);
+    if (wide) atomicAdd(&T.block_wide[(w.slot + i0) / 64], i1 - i0);
+  }
+}
+
+// the chunks of nodes with several, once the host has chosen the node's size (nd.gs; 0: none)
+__global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupWork* work, const NodeD* nodes,
+                                                                    const ProbD* probs, const float* coords,
+                                                                    const uint32_t* cmax, GroupTables T) {
+  __shared__ uint64_t keys[kGroupChunk];
+  const GroupWork w = work[blockIdx.x];
+  const NodeD nd = nodes[w.node];
+  if (nd.gs == 0 || w.cnt == nd.n) return;  // block-uniform
+  const ProbD P = probs[nd.prob];
+  const float* x = coords + nd.coord_off + (int64_t)w.x0 * P.dim;
+  first_order(x, P.dim, w.cnt, pow2_at_least(w.cnt), keys);
+  if (P.dim > 1) str_order(x, P.dim, w.cnt, pow2_at_least(w.cnt), nd.gs, keys);
+  build_groups(w, P, x, keys, nd.gs, grid_unit(__uint_as_float(cmax[nd.prob])), T);
+}
+
+// The points of the chunk that lie in wide groups, for every group size.  A node of a single chunk stops at the
+// first size that leaves few enough of them (a 1 / share; the sizes after it count as wide throughout) and builds
+// its groups there and then: a second launch, and the host's choice before it, would add some 60 us to every create.
+__global__ void __launch_bounds__(kGroupThreads) group_plan_kernel(const GroupWork* work, const NodeD* nodes,
+                                                                   const ProbD* probs, const float* coords,
+                                                                   const uint32_t* cmax, int32_t share, int32_t* out,
+                                                                   GroupTables T) {
   __shared__ uint64_t keys[kGroupChunk];
   __shared__ uint16_t first[kGroupChunk];
   __shared__ int s_wide;
@@ -183,99 +263,24 @@ __global__ void __launch_bounds__(kGroupThreads) group_measure_kernel(const Grou
     if (threadIdx.x == 0) out[kGroupSizes * blockIdx.x + v] = s_wide;
     found = w.cnt == nd.n && s_wide * share <= w.cnt;
     __syncthreads();
-  }
-}
-
-// slots and group records of a chunk whose node takes groups of nd.gs
-__global__ void __launch_bounds__(kGroupThreads) group_build_kernel(const GroupWork* work, const NodeD* nodes,
-                                                                    const ProbD* probs, const float* coords,
-                                                                    const uint32_t* cmax, float4* slot_x,
-                                                                    float2* slot_q, float4* grp, int32_t* block_wide) {
-  __shared__ uint64_t keys[kGroupChunk];
-  const GroupWork w = work[blockIdx.x];
-  const NodeD nd = nodes[w.node];
-  const int gs = nd.gs;
-  if (gs == 0) return;
-  const int D = probs[nd.prob].dim;
-  const double s = probs[nd.prob].cost_scale * kLog2e * probs[nd.prob].inv_eps;
-  const float* x = coords + nd.coord_off + (int64_t)w.x0 * D;
-  first_order(x, D, w.cnt, pow2_at_least(w.cnt), keys);
-  if (D > 1) str_order(x, D, w.cnt, pow2_at_least(w.cnt), gs, keys);
-  const float unit = grid_unit(__uint_as_float(cmax[nd.prob]));
-  // a chunk but the last holds a multiple of 64 points; pads run to the end of the last block of 64
-  const int slots = (w.cnt + 63) / 64 * 64;
-  for (int g = threadIdx.x; g < slots / gs; g += kGroupThreads) {
-    const int i0 = g * gs, i1 = min(i0 + gs, w.cnt);
-    float c[3] = {0.f, 0.f, 0.f};
-    float M[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // second moments 00 01 02 11 12 22
-    float far = 0.f;  // the largest coordinate difference to the centre
-    group_centre(x, D, keys, i0, i1, unit, c);
-    for (int i = i0; i < i0 + gs; ++i) {
-      const uint32_t idx = (uint32_t)keys[min(i, w.cnt - 1)] & 0xffffu;  // pads repeat the last point
-      float d[3] = {0.f, 0.f, 0.f};
-      double q = 0.0;
-      if (i < i1)
-        for (int k = 0; k < D; ++k) {
-          const float v = x[(int64_t)idx * D + k];
-          d[k] = v - c[k];
-          far = fmaxf(far, fabsf(d[k]));
-          const double dd = (double)v - (double)c[k];
-          q += dd * dd;
-        }
-      // in units of the grid: the coordinates' own unit may put squares, and a determinant of them, out of range
-      const float e0 = d[0] / unit, e1 = d[1] / unit, e2 = d[2] / unit;
-      M[0] += e0 * e0, M[1] += e0 * e1, M[2] += e0 * e2;
-      M[3] += e1 * e1, M[4] += e1 * e2, M[5] += e2 * e2;
-      // s |x'|^2 as a two-float, its high part on the 2^-10 grid
-      q *= s;
-      const float qh = (float)(rint(q * kGrid) / kGrid);
-      const int64_t at = nd.slot_off + w.x0 + i;
-      slot_x[at] = make_float4(d[0], d[1], d[2], __int_as_float(w.x0 + (int)idx));
-      slot_q[at] = make_float2(qh, (float)(q - (double)qh));
-    }
-    // inverse of the second moments (with a small ridge; zero for a single place)
-    const float ridge = 1e-3f * (M[0] + M[3] + M[5]) / D;
-    float I[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const float a = M[0] + ridge, d1 = M[3] + ridge, f = M[5] + ridge;
-    if (D == 1) {
-      I[0] = 1.f / a;
-    } else if (D == 2) {
-      const float det = a * d1 - M[1] * M[1];
-      I[0] = d1 / det, I[1] = -M[1] / det, I[2] = a / det;
-    } else {
-      const float A00 = d1 * f - M[4] * M[4], A01 = M[2] * M[4] - M[1] * f, A02 = M[1] * M[4] - M[2] * d1;
-      const float det = a * A00 + M[1] * A01 + M[2] * A02;
-      I[0] = A00 / det, I[1] = A01 / det, I[2] = A02 / det;
-      I[3] = (a * f - M[2] * M[2]) / det, I[4] = (M[1] * M[2] - a * M[4]) / det, I[5] = (a * d1 - M[1] * M[1]) / det;
-    }
-    for (int k = 0; k < 6; ++k) {
-      I[k] = I[k] / unit / unit;
-      if (!isfinite(I[k])) I[k] = 0.f;
-    }
-    float4* r = grp + 3 * ((nd.slot_off + w.x0 + i0) / 8);
-    r[0] = make_float4(c[0], c[1], c[2], unit);
-    r[1] = make_float4(I[0], I[1], I[2], I[3]);
-    const bool wide = i1 > i0 && group_wide(gs, D, probs[nd.prob].s2_scaled, far);
-    r[2] = make_float4(I[4], I[5], wide ? 1.f : 0.f, 0.f);
-    if (wide) atomicAdd(&block_wide[(nd.slot_off + w.x0 + i0) / 64], i1 - i0);
+    if (found) build_groups(w, probs[nd.prob], x, keys, gs, unit, T);  // block-uniform; only reads keys
   }
 }
 
 }  // namespace
 
-cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
-                                 cudaStream_t s) {
+cudaError_t launch_group_plan(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
+                              const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
+                              const GroupTables& t, cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  group_measure_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, share, out);
+  group_plan_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, share, out, t);
   return cudaGetLastError();
 }
 
 cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                               const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
-                               int32_t* block_wide, cudaStream_t s) {
+                               const float* coords, const uint32_t* cmax, const GroupTables& t, cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  group_build_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, slot_x, slot_q, grp, block_wide);
+  group_build_kernel<<<nwork, kGroupThreads, 0, s>>>(work, nodes, probs, coords, cmax, t);
   return cudaGetLastError();
 }
 

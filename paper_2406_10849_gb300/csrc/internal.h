@@ -92,7 +92,15 @@ struct NodeD {
 // A chunk of at most kGroupChunk consecutive points of a node, sorted into compact groups by one CTA
 constexpr int kGroupChunk = 4096;
 struct GroupWork {
-  int32_t node, x0, cnt;
+  int32_t node, x0, cnt, pad;
+  int64_t slot;  // the chunk's first slot
+};
+// what the grouping writes (see ApplyArgs); block_wide: outputs in wide groups per block of 64 slots
+struct GroupTables {
+  float4* slot_x;
+  float2* slot_q;
+  float4* grp;
+  int32_t* block_wide;
 };
 // The largest kappa = s r^2 of a group (64, 32 or 16 points) that takes the factored form, and the largest share
 // 1 / kGroupWide of a node's points in wider groups, on large handles and on others (see group.cu); below
@@ -438,12 +446,11 @@ cudaError_t launch_scan_cost(const float* C, int64_t ld, int32_t rows, int32_t c
 cudaError_t launch_transpose_pad(const float* src, int64_t src_ld, int32_t rows, int32_t cols, float* dst,
                                  int64_t dst_ld, cudaStream_t s);
 // coordinates split hi + lo for the exact-distance recomputation (cmax: nprob scratch words)
-cudaError_t launch_group_measure(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                                 const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
-                                 cudaStream_t s);
+cudaError_t launch_group_plan(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
+                              const float* coords, const uint32_t* cmax, int32_t share, int32_t* out,
+                              const GroupTables& t, cudaStream_t s);
 cudaError_t launch_group_build(const GroupWork* work, int32_t nwork, const NodeD* nodes, const ProbD* probs,
-                               const float* coords, const uint32_t* cmax, float4* slot_x, float2* slot_q, float4* grp,
-                               int32_t* block_wide, cudaStream_t s);
+                               const float* coords, const uint32_t* cmax, const GroupTables& t, cudaStream_t s);
 cudaError_t launch_split_coords(const float* coords, const NodeD* nodes, int32_t nnodes, const ProbD* probs,
                                 uint32_t* cmax, int32_t nprob, float* hi, float* lo, cudaStream_t s);
 cudaError_t launch_check(const CheckArgs& a, cudaStream_t s);
