@@ -219,3 +219,24 @@ def test_group_sizes(n, dim, eps, clustered, sizes, split):
             ref = O.run_half_steps(p, steps)
             assert rel_err(got, ref, p.eps) <= 1e-4
             assert marginal_gap(p, got, ref) <= 1e-6  # the bar of every FP32 iterate
+
+
+@pytest.mark.parametrize("split", range(4))
+def test_persistent_launch_of_split_reductions(split):
+    """The persistent launch runs the same tasks, with several reduction splits per edge, wide groups and both forms:
+    the same bits as per-half-step launches."""
+    import paper_2406_10849_gb300 as T
+    T.load()
+    probs = [cloud_star((64, 16384, 33), 2, 0.05, seed=1), cloud_star((300, 257, 45), 2, 0.003, seed=2),
+             cloud_star((600, 333, 64), 2, 0.01, seed=3, clustered=True)]
+    out = []
+    for persistent in (False, True):
+        with T.Solver(probs, T.options(autotune=False, persistent=persistent, test_apply=(split, 0))) as s:
+            st = s.plan_stats()
+            assert st["factored_splits"] > 1 and st["persistent"] == (2 if persistent else 0)
+            assert 0 < st["factored_edges"] < st["directed_edges"]
+            s.half_steps(5)
+            out.append([s.potentials(i) for i in range(3)])
+    for a, b in zip(*out):
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
