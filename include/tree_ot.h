@@ -112,8 +112,8 @@ typedef struct tree_ot_problem {
  * |x - y|^2 alone perturbs C/eps enough to hold some iterates ~1e-7..1e-6 (max
  * marginal L1) away from the solution at small eps.  Problems the certification
  * (see tree_ot_solve) finds stuck above tol continue with exactly formed squared
- * distances (coordinates split hi + lo, ~1.8x the FP32 work per element), the
- * handle's other problems meanwhile with plainly recomputed ones; this bit uses the exact form from the first half-step for every such problem. */
+ * distances (coordinates split hi + lo, ~1.8x the FP32 work per element); this
+ * bit uses the exact form from the first half-step for every such problem. */
 #define TREE_OT_OPT_EXACT_DIST   4u
 /* Stored costs: when the device has room (free memory above twice the matrices'
  * size plus 1 GiB) every edge also keeps its cost transposed, so the column
@@ -419,8 +419,8 @@ int tree_ot_get_potentials_batch(tree_ot_handle *h, void *cuda_stream, int32_t c
  * [20] points of the factored edges' nodes in groups too wide for the factored
  * form (always summed by the difference form), [21] the most reduction splits of
  * a factored edge, [22] 1 while some problem runs with exact squared distances
- * (after a certification asked for them) and every recomputed cost of the handle
- * therefore takes the difference form, [23] configurations of the recomputed-cost
+ * (after a certification asked for them) and its recomputed costs therefore take
+ * the difference form, [23] configurations of the recomputed-cost
  * apply that create timed (0: none to choose, or found for these sizes before),
  * [24] to [26] nodes whose points lie in groups of 64, 32 and 16. */
 int tree_ot_plan_stats(tree_ot_handle *h, int64_t *stats, int32_t nstats);

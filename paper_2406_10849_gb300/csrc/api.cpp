@@ -173,8 +173,8 @@ void treeot::set_last_error(const std::string& msg) { g_err = msg; }
 // the handle
 // ---------------------------------------------------------------------------
 
-// What an apply and a node update read of a handle's exact-distance plan: while some problem runs with exact squared
-// distances, every recomputed cost takes the difference form with its own reduction splits (in place of the
+// What an apply and a node update read of a handle's exact-distance plan: while some problems run with exact squared
+// distances, their recomputed costs take the difference form with its own reduction splits (in place of the
 // factored form's)
 struct ExactPlan {
   std::vector<DEdgeD> dedges;  // empty: the handle has no factored edges, its one plan serves both
@@ -186,7 +186,6 @@ struct ExactPlan {
   FixedChunkD* d_fixed[2] = {nullptr, nullptr};
   Task* d_tasks[2] = {nullptr, nullptr};
   int32_t* d_fcnt = nullptr;   // item counts of the persistent launch
-  bool ready = false;          // the device arrays are filled (on the first use)
 };
 
 struct tree_ot_handle {
@@ -429,7 +428,7 @@ int32_t fact_split_points(int32_t n_nbr, int32_t nsplit) {
 // Apply tasks of both colours, grouped by kernel slot.  rec_ob: largest output
 // block of a recomputed-cost task (256, 512 or 1024 outputs); a task with fewer
 // outputs runs its CTA as G warp groups splitting the reduction points.
-// exact: the exact-distance plan, all of it in the difference form.
+// exact: the exact-distance plan, whose problems with exact distances take the difference form.
 void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob, bool exact = false) {
   std::vector<Task>* tasks = exact ? h->xplan.tasks : h->tasks;
   auto* slot_begin = exact ? h->xplan.slot_begin : h->slot_begin;
@@ -463,7 +462,7 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob, bool exact = false) {
         for (int32_t o0 = 0; o0 < own.n; o0 += kColCols)
           tl.push_back(Task{(int32_t)di, TASK_COL, o0, std::min(kColCols, own.n - o0), s * kColRows,
                             std::min(kColRows, nbn.n - s * kColRows), s, 0});
-    } else if (!exact && fact_edge(h, d)) {
+    } else if (fact_edge(h, d) && !(exact && h->h_exact[d.prob])) {
       // slots of the owner's groups against a split of the neighbour's points, 2^split warps of a CTA per block of 64
       const int32_t ob = (8 >> h->fact_split) * 64, per = fact_split_points(nbn.n, d.nsplit);
       for (int32_t o0 = 0; o0 < own.n; o0 += ob) {
@@ -473,8 +472,9 @@ void build_apply_tasks(tree_ot_handle* h, int32_t rec_ob, bool exact = false) {
                             0});
       }
     } else {
-      for (int32_t o0 = 0; o0 < own.n; o0 += rec_ob) {
-        const int32_t oc = std::min(rec_ob, own.n - o0);
+      const int32_t ob = exact && fact_edge(h, d) ? h->xplan.rec_ob : rec_ob;
+      for (int32_t o0 = 0; o0 < own.n; o0 += ob) {
+        const int32_t oc = std::min(ob, own.n - o0);
         int32_t G = 1;
         while (G < 8 && kRecOut / (2 * G) >= oc) G *= 2;
         for (int32_t s = 0; s < d.nsplit; ++s)
@@ -544,28 +544,31 @@ int fixed_records(const tree_ot_handle* h, const std::vector<DEdgeD>& dedges, in
   return TREE_OT_OK;
 }
 
-// The exact-distance plan: directed edges with the difference form's reduction splits, and the largest output
-// block that gives every SM two tasks.  Its device memory is taken at create (plan_exact) and filled when the
-// certification first asks for exact distances (fill_exact).
+// The exact-distance plan: directed edges, those of problems with exact distances with the difference form's
+// reduction splits, and for these the largest output block that would give every SM two tasks.  Its device memory
+// is taken at create (plan_exact) and filled whenever the certification asks for exact distances (fill_exact).
 int plan_exact(tree_ot_handle* h) {
   ExactPlan& x = h->xplan;
   bool any = false;
   for (const DEdgeD& d : h->dedges) any = any || fact_edge(h, d);
   if (!any) return TREE_OT_OK;
   x.dedges = h->dedges;
-  for (DEdgeD& d : x.dedges)
-    if (fact_edge(h, d)) d.nsplit = (h->nodes[d.nbr].n + kRecRed - 1) / kRecRed;
-  int64_t count[2] = {0, 0};
-  for (x.rec_ob = kRecOut;; x.rec_ob /= 2) {
-    count[0] = count[1] = 0;
-    for (const DEdgeD& d : x.dedges)
-      if (h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
-        count[h->nodes[d.owner].colour] += (int64_t)((h->nodes[d.owner].n + x.rec_ob - 1) / x.rec_ob) * d.nsplit;
-    if (x.rec_ob == 256 || std::max(count[0], count[1]) >= 2 * h->sms) break;
+  auto splits = [&](const DEdgeD& d) { return (h->nodes[d.nbr].n + kRecRed - 1) / kRecRed; };
+  auto blocks = [&](const DEdgeD& d, int32_t ob) { return (int64_t)((h->nodes[d.owner].n + ob - 1) / ob); };
+  for (x.rec_ob = kRecOut; x.rec_ob > 256; x.rec_ob /= 2) {
+    int64_t count[2] = {0, 0};
+    for (const DEdgeD& d : h->dedges)
+      if (fact_edge(h, d)) count[h->nodes[d.owner].colour] += blocks(d, x.rec_ob) * splits(d);
+    if (std::max(count[0], count[1]) >= 2 * h->sms) break;
   }
+  int64_t cap[2] = {0, 0};  // the finest tasks of either form
+  for (const DEdgeD& d : h->dedges)
+    if (h->probs[d.prob].cost_kind == TREE_OT_COST_SQEUCLID)
+      cap[h->nodes[d.owner].colour] += fact_edge(h, d) ? std::max(blocks(d, x.rec_ob) * splits(d), blocks(d, 64) * d.nsplit)
+                                                       : blocks(d, 256) * d.nsplit;
   for (int c = 0; c < 2; ++c) {
-    for (const Task& t : h->tasks[c]) count[c] += t.kind < TASK_RECOMP;  // stored costs: as they are
-    RC_TRY(h->alloc(&x.d_tasks[c], count[c]));
+    for (const Task& t : h->tasks[c]) cap[c] += t.kind < TASK_RECOMP;  // stored costs: as they are
+    RC_TRY(h->alloc(&x.d_tasks[c], cap[c]));
     RC_TRY(h->alloc(&x.d_fixed[c], h->nfixed_chunks[c]));
   }
   RC_TRY(h->alloc(&x.d_dedges, (int64_t)x.dedges.size()));
@@ -574,24 +577,31 @@ int plan_exact(tree_ot_handle* h) {
   return TREE_OT_OK;
 }
 
+// the plan for the problems that h_exact names
 int fill_exact(tree_ot_handle* h, cudaStream_t s) {
   ExactPlan& x = h->xplan;
-  if (x.ready || x.dedges.empty()) return TREE_OT_OK;
-  build_apply_tasks(h, x.rec_ob, true);
+  if (x.dedges.empty()) return TREE_OT_OK;
+  for (size_t di = 0; di < x.dedges.size(); ++di) {
+    DEdgeD& d = x.dedges[di];
+    d.nsplit = h->dedges[di].nsplit;
+    if (fact_edge(h, d) && h->h_exact[d.prob]) d.nsplit = (h->nodes[d.nbr].n + kRecRed - 1) / kRecRed;
+  }
+  build_apply_tasks(h, h->rec_ob, true);
   auto up = [&](auto* dst, const auto& v) {
     return v.empty() ? cudaSuccess : cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, s);
   };
+  const std::vector<OwnedDEdge> owned = owned_records(h, x.dedges);
+  const std::vector<int32_t> cnt = forest_counts(h, x.tasks);
+  std::vector<FixedChunkD> fr[2];
   CUDA_TRY(up(x.d_dedges, x.dedges));
-  CUDA_TRY(up(x.d_owned, owned_records(h, x.dedges)));
+  CUDA_TRY(up(x.d_owned, owned));
   for (int c = 0; c < 2; ++c) {
-    std::vector<FixedChunkD> fr;
-    RC_TRY(fixed_records(h, x.dedges, c, s, &fr));
-    CUDA_TRY(up(x.d_fixed[c], fr));
+    RC_TRY(fixed_records(h, x.dedges, c, s, &fr[c]));
+    CUDA_TRY(up(x.d_fixed[c], fr[c]));
     CUDA_TRY(up(x.d_tasks[c], x.tasks[c]));
   }
-  if (x.d_fcnt) CUDA_TRY(up(x.d_fcnt, forest_counts(h, x.tasks)));
+  if (x.d_fcnt) CUDA_TRY(up(x.d_fcnt, cnt));
   CUDA_TRY(cudaStreamSynchronize(s));
-  x.ready = true;
   return TREE_OT_OK;
 }
 
@@ -2529,7 +2539,7 @@ int tree_ot_solve(tree_ot_handle* h, void* cuda_stream, tree_ot_result* results)
       }
       return ring_sum[slot * h->nprob + p];
     };
-    bool resume = false;
+    bool resume = false, more_exact = false;
     std::fill(resumed.begin(), resumed.end(), 0);
     for (int p = 0; p < h->nprob; ++p) {
       if (!h->h_done[p]) continue;
@@ -2541,6 +2551,7 @@ int tree_ot_solve(tree_ot_handle* h, void* cuda_stream, tree_ot_result* results)
                             !h->h_exact[p];
       if (!(got < 0.99 * prev_got[p]) && !to_exact) continue;
       if (to_exact) h->h_exact[p] = 1;
+      more_exact = more_exact || to_exact;
       prev_got[p] = got;
       // next threshold: the FP32 quantity it retired on, scaled by how far the check missed
       const double crit = retired_on(p);
@@ -2563,7 +2574,7 @@ int tree_ot_solve(tree_ot_handle* h, void* cuda_stream, tree_ot_result* results)
     {
       const int32_t any = *std::max_element(h->h_exact.begin(), h->h_exact.end());
       CUDA_TRY(cudaMemcpyAsync(h->d_exact, h->h_exact.data(), sizeof(int32_t) * h->nprob, cudaMemcpyHostToDevice, s));
-      if (any != h->any_exact) {
+      if (any != h->any_exact || (more_exact && !h->xplan.dedges.empty())) {  // other tasks, other launches
         if (any) RC_TRY(fill_exact(h, s));
         h->any_exact = any;
         if (use_graph) {

@@ -322,7 +322,8 @@ __global__ void __launch_bounds__(kFactThreads, kFactCtas) apply_fact_kernel(App
     if (lane == 0) ticket = atomicAdd(&A.queue[0], 1);
     if (nxt < A.nitems && lane < kWords) word = reinterpret_cast<const int32_t*>(A.items + nxt)[lane];
     const FactItem& it = *reinterpret_cast<const FactItem*>(s_rec[warp]);
-    if (!A.done[it.prob] && A.lowp[it.prob] != 1) {  // not retired, nor in a BF16 phase
+    // not retired, nor in a BF16 phase, nor with exact distances (the plan then holds other tasks for it)
+    if (!A.done[it.prob] && A.lowp[it.prob] != 1 && !(A.any_exact && A.exact[it.prob])) {
       if (it.gs == 64)
         fact_block<D, 64, false>(A, it, sm, warp, 0);
       else if (it.gs == 32)
@@ -501,7 +502,7 @@ cudaError_t launch_apply_f32(const ApplyArgs& a, int slot, int variant, int grid
   if (a.ntasks <= 0) return cudaSuccess;
   if (slot == 0) {
     apply_dense_kernel<<<grid, kApplyThreads, 0, s>>>(a);
-  } else if (a.any_exact) {
+  } else if (a.any_exact && slot <= 3) {
     // rare (after certification): the 2-CTA register budget, whatever the tuned variant
     if (slot == 1) apply_recomp_kernel<1, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);
     if (slot == 2) apply_recomp_kernel<2, 2, 1><<<grid, kApplyThreads, 0, s>>>(a);

@@ -67,7 +67,7 @@ __device__ __forceinline__ int apply_item(const ForestArgs& F, const ApplyArgs& 
   if (go == 1) {
     if (EXACT && A.exact[p])
       recomp_task_exact<D>(A, task, sm);
-    else if (!EXACT && task.kind >= TASK_FACT)  // an exact-distance plan has the difference form alone
+    else if (task.kind >= TASK_FACT)
       fact_dispatch<D>(A, task, sm);
     else
       recomp_task<D>(A, task, sm);
