@@ -32,9 +32,12 @@ namespace {
 constexpr int kChkRows = 8;  // rows per warp
 
 __global__ void __launch_bounds__(256, 2) check_kernel(CheckArgs A) {
-  __shared__ float s_col[8][32];
-  __shared__ float s_cmp[8][32];
+  // column sums of alternate steps (counted through all tasks): a step needs one barrier, since the warp that reads
+  // a buffer reaches the next step's before any warp writes that buffer again
+  __shared__ float s_col[2][8][32];
+  __shared__ float s_cmp[2][8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int step = 0;
   for (int ti = blockIdx.x; ti < A.ntasks; ti += gridDim.x) {
     const Task t = A.tasks[ti];
     if (t.kind != TASK_ROW) continue;  // block-uniform
@@ -63,7 +66,7 @@ __global__ void __launch_bounds__(256, 2) check_kernel(CheckArgs A) {
       for (int k = 0; k < 3; ++k) rp[r][k] = (na.coord_off >= 0 && k < D) ? A.coords[na.coord_off + (int64_t)x * D + k] : 0.f;
       rs[r] = rc[r] = ts[r] = tcmp[r] = 0.f;
     }
-    for (int y0 = 0; y0 < e.nb; y0 += 32) {
+    for (int y0 = 0; y0 < e.nb; y0 += 32, ++step) {
       const int y = y0 + lane;
       const bool on = y < e.nb;
       const float bh = on ? A.ah[b_off + y] : -INFINITY;
@@ -94,21 +97,21 @@ __global__ void __launch_bounds__(256, 2) check_kernel(CheckArgs A) {
           cs = t1;
         }
       }
-      s_col[warp][lane] = cs;
-      s_cmp[warp][lane] = cc;
+      float(*col)[32] = s_col[step & 1], (*cmp)[32] = s_cmp[step & 1];
+      col[warp][lane] = cs;
+      cmp[warp][lane] = cc;
       __syncthreads();
-      if (warp == 0 && on) {
+      if (warp == (step & 7) && on) {  // the warps in turn
         TF v = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int w = 0; w < 8; ++w) tf_acc(v, s_col[w][lane], -s_cmp[w][lane]);
+        for (int w = 0; w < 8; ++w) tf_acc(v, col[w][lane], -cmp[w][lane]);
         double sum = tf_to(v);
         if (!tf_finite(v)) {  // out of the FP32 range: in FP64
           sum = 0.0;
-          for (int w = 0; w < 8; ++w) sum += (double)s_col[w][lane] - (double)s_cmp[w][lane];
+          for (int w = 0; w < 8; ++w) sum += (double)col[w][lane] - (double)cmp[w][lane];
         }
         if (sum != 0.0) atomicAdd(&A.marg[b_off + y], sum);
       }
-      __syncthreads();
     }
     TF row[kChkRows], trn[kChkRows];
 #pragma unroll

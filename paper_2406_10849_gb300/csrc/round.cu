@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256) round_pass_kernel(RoundArgs A) {
 // Passes 1-4 of FP32 handles.  Entries are FP32 values, costs pairs of them; the factors x, y and err_c and every
 // sum over entries are three floats (TF, plan_entry.cuh): GB300 executes an FP64 add or a conversion at 1/70 of its
 // FP32 rate, and with FP64 sums those were the passes' whole time (check and rounding of 94 M entries in 209 plans:
-// 11.8 ms with FP64 sums, 4.5 with pairs of floats, which keep 2^-46 instead of 2^-53, 5.3 with three).  Row factors
+// 11.8 ms with FP64 sums, 4.5 with pairs of floats, which keep 2^-46 instead of 2^-53, 5.2 with three).  Row factors
 // (x, err_r) multiply the finished row sums, not the entries.
 //
 // Accuracy: products of an entry with a factor are exact to 2^-70, sums to n^2 2^-72, both below FP64's own
